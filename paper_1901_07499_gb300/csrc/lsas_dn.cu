@@ -469,8 +469,8 @@ __global__ void __launch_bounds__(128 * kTcSlots, 2) dn_tc_kernel(const float* _
 // every step) and fp32 Adam.  Three passes per step:
 //  * forward (dn_tc_train_kernel<false>): the inference tile loop of
 //    dn_tc_kernel, which also stores each ReLU output r1, r2, r3 exactly as
-//    the next layer consumed it (bf16, [R][N][32]) and, at the network
-//    output, dy = 2 (y - t) / n and the tile's sum of (y - t)^2;
+//    the next layer consumed it (bf16) and, at the network output,
+//    dy = 2 (y - t) / n and the tile's sum of (y - t)^2;
 //  * data gradients (dn_tc_train_kernel<true>): the same tile loop over
 //    three convolutions with transposed, flipped weights (g3 = conv(dy; W4'),
 //    g2 = conv(g3; W3'), g1 = conv(g2; W2'), W'[c][o][k] = W[o][c][4 - k}),
@@ -483,7 +483,19 @@ __global__ void __launch_bounds__(128 * kTcSlots, 2) dn_tc_kernel(const float* _
 //    copies of the layer input in shared memory; per-block partial sums are
 //    added in block order.  The two layers with two-channel sides (1 and 4)
 //    and the biases reduce on the CUDA cores from the same bf16 tensors.
-constexpr int kTrAct = 32;   // channels of a stored activation row (bf16)
+// A stored tensor is [R][4][N + 4][8] bf16: four planes of eight channels per
+// row, so that the threads of a warp (consecutive positions) write and read
+// consecutive 16-byte pieces, with two zero positions at either end of a
+// plane (the convolutions' zero padding).
+constexpr int kTrPad = 2;    // zero positions at either end of a plane
+__host__ __device__ __forceinline__ size_t tr_plane(int R, int N) {   // elements of one tensor
+  return static_cast<size_t>(R) * 32 * (N + 2 * kTrPad);
+}
+// element offset of position q of channel chunk 0 of row r; chunk kc adds kc * tr_chunk(N)
+__device__ __forceinline__ size_t tr_at(int r, int N, int q) {
+  return (static_cast<size_t>(r) * 4 * (N + 2 * kTrPad) + q + kTrPad) * 8;
+}
+__device__ __forceinline__ size_t tr_chunk(int N) { return static_cast<size_t>(N + 2 * kTrPad) * 8; }
 
 // Backward weight image: layer-1 slot = W4' (2 -> 32), layer-2 slot = W3',
 // layer-3 slot = W2', zero biases and layer-4 slot, the constant operand.
@@ -569,7 +581,8 @@ __global__ void __launch_bounds__(128 * kTcSlots, 2) dn_tc_train_kernel(
   bool ok = mbar_wait_bounded(smem_u32(&bars[0]), 0);
   if (!ok) latch(status, kStTimeout);
   uint32_t phase = slot == 0 ? 1u : 0u;
-  const size_t plane = static_cast<size_t>(R) * N * kTrAct;   // one stored tensor (elements)
+  const size_t plane = tr_plane(R, N);   // one stored tensor (elements)
+  const size_t chunk = tr_chunk(N);
   for (int tile = blockIdx.x * kTcSlots + slot; tile < tiles; tile += stride) {
     const int r = tile / tiles_row;
     const int s0 = (tile % tiles_row) * kTcValid - kTcFirst;   // position of MMA row 0
@@ -588,7 +601,7 @@ __global__ void __launch_bounds__(128 * kTcSlots, 2) dn_tc_train_kernel(
     const int q = s0 + u;                                     // position of MMA row u
     const bool inside = q >= 0 && q < N;
     const bool mine = u >= kTcFirst && u < kTcFirst + kTcValid && inside;   // stored by this tile
-    const size_t rowoff = (static_cast<size_t>(r) * N + q) * kTrAct;
+    const size_t rowoff = tr_at(r, N, q);
     auto issue_wait = [&](int layer) {
       fence_proxy_async();
       tmem_fence_before();
@@ -630,7 +643,7 @@ __global__ void __launch_bounds__(128 * kTcSlots, 2) dn_tc_train_kernel(
         uint4 mk[4];
         if (BWD) {
 #pragma unroll
-          for (int kc = 0; kc < 4; ++kc) mk[kc] = *reinterpret_cast<const uint4*>(mask_src + rowoff + 8 * kc);
+          for (int kc = 0; kc < 4; ++kc) mk[kc] = *reinterpret_cast<const uint4*>(mask_src + rowoff + kc * chunk);
         }
 #pragma unroll
         for (int kc = 0; kc < 4; ++kc) {
@@ -651,7 +664,16 @@ __global__ void __launch_bounds__(128 * kTcSlots, 2) dn_tc_train_kernel(
       for (int kc = 0; kc < 4; ++kc) *reinterpret_cast<uint4*>(act + kc * kTcLbo + (u + 2) * 16) = w[kc];
       if (mine) {
 #pragma unroll
-        for (int kc = 0; kc < 4; ++kc) *reinterpret_cast<uint4*>(out + rowoff + 8 * kc) = w[kc];
+        for (int kc = 0; kc < 4; ++kc) *reinterpret_cast<uint4*>(out + rowoff + kc * chunk) = w[kc];
+        // the row's first and last position also write its zero pads
+        if (q == 0 || q == N - 1) {
+          const long pad = q == 0 ? -16 : 8;
+#pragma unroll
+          for (int kc = 0; kc < 4; ++kc) {
+            uint4* z = reinterpret_cast<uint4*>(out + rowoff + kc * chunk + pad);
+            z[0] = z[1] = make_uint4(0u, 0u, 0u, 0u);
+          }
+        }
       }
     };
     float d[32];
@@ -699,7 +721,7 @@ __global__ void __launch_bounds__(128 * kTcSlots, 2) dn_tc_train_kernel(
 constexpr int kTrSmem = kTcSmem + 64;   // + per-slot loss partials of four warps
 
 // Weight gradient of a 32 -> 32 layer on tcgen05.  A: the layer's input
-// r [R][N][32] bf16; G: the gradient at its output g [R][N][32] bf16.  A
+// r, G: the gradient at its output g (stored bf16 tensors).  A
 // block of 128 threads takes tiles of 128 positions of one row; per tile it
 // stores G as the MN-major B operand (K = position, N = 32 output channels)
 // and five copies of A shifted by the five taps as the MN-major A operand
@@ -707,15 +729,16 @@ constexpr int kTrSmem = kTcSmem + 64;   // + per-slot loss partials of four warp
 // position q0 + p + k - 2), then one thread issues, per 16 positions, an
 // M = 128 MMA over copies 0-3 and one over copies 1-4 (its last 32 rows are
 // tap 4).  The accumulators stay in TMEM across the block's tiles; at the
-// end the block writes its partial sums wpart[block][k][c][o] and bias
-// partials bpart[block][o].
+// end the block writes its partial sums, a row [k][c][o] then the bias
+// partials [o].
 constexpr int kWgCopy = 128 * 16;                          // one channel chunk of one copy
 constexpr int kWgA = 0, kWgG = kWgA + 5 * 4 * kWgCopy;     // 40 KB of copies, 8 KB of G
+constexpr int kWgPart = 5 * 32 * 32 + 32;                  // one block's partials (floats)
 constexpr int kWgSmem = kWgG + 4 * kWgCopy + 16 + 16 + 4 * 32 * 4;
 __global__ void __launch_bounds__(128) dn_tc_wgrad_kernel(const __nv_bfloat16* __restrict__ G,
                                                          const __nv_bfloat16* __restrict__ A,
                                                          int R, int N, float* __restrict__ wpart,
-                                                         float* __restrict__ bpart, int* status) {
+                                                         int* status) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int u = threadIdx.x, warp = u >> 5, lane = u & 31;
   unsigned char* acp = smem + kWgA;
@@ -744,13 +767,12 @@ __global__ void __launch_bounds__(128) dn_tc_wgrad_kernel(const __nv_bfloat16* _
   bool ok = true, first = true;
   for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     const int r = tile / tiles_row, q0 = (tile % tiles_row) * 128;
-    const size_t rbase = static_cast<size_t>(r) * N;
     // G row u (position q0 + u): B operand and the bias sums
     {
-      const uint4* src = reinterpret_cast<const uint4*>(G + (rbase + q0 + u) * kTrAct);
+      const __nv_bfloat16* src = G + tr_at(r, N, q0 + u);
 #pragma unroll
       for (int kc = 0; kc < 4; ++kc) {
-        const uint4 w = src[kc];
+        const uint4 w = *reinterpret_cast<const uint4*>(src + kc * tr_chunk(N));
         *reinterpret_cast<uint4*>(gsm + kc * kWgCopy + u * 16) = w;
         const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&w);
 #pragma unroll
@@ -761,14 +783,10 @@ __global__ void __launch_bounds__(128) dn_tc_wgrad_kernel(const __nv_bfloat16* _
     for (int i = u; i < 132; i += 128) {
       const int qa = q0 - 2 + i;
       uint4 w[4];
-      if (qa >= 0 && qa < N) {
-        const uint4* src = reinterpret_cast<const uint4*>(A + (rbase + qa) * kTrAct);
+      const __nv_bfloat16* src = A + tr_at(r, N, qa);   // pads of zeros beyond the row's ends
 #pragma unroll
-        for (int kc = 0; kc < 4; ++kc) w[kc] = src[kc];
-      } else {
-#pragma unroll
-        for (int kc = 0; kc < 4; ++kc) w[kc] = make_uint4(0u, 0u, 0u, 0u);
-      }
+      for (int kc = 0; kc < 4; ++kc)
+        w[kc] = *reinterpret_cast<const uint4*>(src + kc * tr_chunk(N));
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
         const int pr = i - k;
@@ -804,7 +822,7 @@ __global__ void __launch_bounds__(128) dn_tc_wgrad_kernel(const __nv_bfloat16* _
     tmem_fence_after();
   }
   // partial sums of this block: row 32 k + c of D1 (taps 0-3), rows 96 + c of D2 (tap 4)
-  float* wp = wpart + static_cast<size_t>(blockIdx.x) * 5 * 32 * 32;
+  float* wp = wpart + static_cast<size_t>(blockIdx.x) * kWgPart;
   {
     float v[32];
     if (!first) {
@@ -835,7 +853,7 @@ __global__ void __launch_bounds__(128) dn_tc_wgrad_kernel(const __nv_bfloat16* _
   }
   __syncthreads();
   if (u < 32)
-    bpart[static_cast<size_t>(blockIdx.x) * 32 + u] =
+    wp[5120 + u] =
         ((bred[u] + bred[32 + u]) + bred[64 + u]) + bred[96 + u];
   tmem_fence_before();
   __syncthreads();
@@ -843,63 +861,200 @@ __global__ void __launch_bounds__(128) dn_tc_wgrad_kernel(const __nv_bfloat16* _
   if (warp == 0) tmem_dealloc(*tbase, 64);
 }
 
-// dW[o][c][k] = sum over blocks of wpart[b][k][c][o]; db[o] likewise (block order)
-__global__ void dn_wgrad_reduce_kernel(const float* __restrict__ wpart, const float* __restrict__ bpart,
-                                       int blocks, float* __restrict__ dW, float* __restrict__ db) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;   // (o, c, k) of dW
-  if (i < 32 * 32 * 5) {
-    const int k = i % 5, c = (i / 5) % 32, o = i / 160;
-    float s = 0.f;
-    for (int b = 0; b < blocks; ++b) s += wpart[(static_cast<size_t>(b) * 5 + k) * 1024 + c * 32 + o];
-    dW[i] = s;
-  } else if (i < 32 * 32 * 5 + 32) {
-    const int o = i - 32 * 32 * 5;
-    float s = 0.f;
-    for (int b = 0; b < blocks; ++b) s += bpart[static_cast<size_t>(b) * 32 + o];
-    db[o] = s;
+// Weight gradient of a layer with a two-channel side on the CUDA cores:
+// layer 4 (T = dy fp32 [R][2][N], B = r3) or layer 1 (T = x0, B = g1), B a
+// stored bf16 tensor:
+//   layer 4: dW[j][c][k] = sum_q B[c][q] T[j][q + 2 - k], db[j] = sum_q T[j][q]
+//   layer 1: dW[c][j][k] = sum_q B[c][q] T[j][q + k - 2], db[c] = sum_q B[c][q]
+// Bound by the FMA pipe (320 FMAs a position) and by one pass over B.  A warp
+// takes one 8-channel chunk of a 128-position tile; a lane keeps the 80 sums
+// of its chunk in registers over four consecutive positions per tile, so a
+// position's 8 channels come in one 16-byte load and its 10 shifted T values
+// from two 8-value register windows.  Blocks of 4 chunks x 2 tiles walk the
+// tiles and write one row of partial sums each (kSdPart floats: [j][k][c],
+// then the biases); dn_reduce_kernel adds the rows in order.  Before, one
+// block per (output, input) channel pair re-read both tensors with 2-byte
+// strided loads on 64 of the SMs: 749 + 659 us at 256 rows of 1024, against
+// 17.6 us for both layers in this one launch.
+constexpr int kSdThreads = 256;
+constexpr int kSdPart = 320 + 32;
+__global__ void __launch_bounds__(kSdThreads, 2) dn_tc_side_kernel(
+    const float* __restrict__ dy, const __nv_bfloat16* __restrict__ r3,
+    const float* __restrict__ x0, const __nv_bfloat16* __restrict__ g1, int R, int N,
+    float* __restrict__ part4, float* __restrict__ part1) {
+  __shared__ float comb[4][88];
+  const bool layer4 = blockIdx.y == 0;
+  const float* __restrict__ T = layer4 ? dy : x0;
+  const __nv_bfloat16* __restrict__ B = layer4 ? r3 : g1;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int kc = warp & 3, sub = warp >> 2;
+  const int tiles_row = N / 128, tiles = R * tiles_row;
+  float2 acc[2][kDnK][4];
+  float2 bacc[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    bacc[i] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int k = 0; k < kDnK; ++k) acc[j][k][i] = make_float2(0.f, 0.f);
+  }
+  for (int tile = 2 * blockIdx.x + sub; tile < tiles; tile += 2 * gridDim.x) {
+    const int r = tile / tiles_row, q = (tile % tiles_row) * 128 + 4 * lane;
+    // windows of T: positions q - 2 .. q + 5 (zero outside the row)
+    float w[2][8];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const float* t = T + (static_cast<size_t>(r) * 2 + j) * N + q;
+      const float4 c = *reinterpret_cast<const float4*>(t);
+      const float2 a = q > 0 ? *reinterpret_cast<const float2*>(t - 2) : make_float2(0.f, 0.f);
+      const float2 d = q + 4 < N ? *reinterpret_cast<const float2*>(t + 4) : make_float2(0.f, 0.f);
+      w[j][0] = a.x; w[j][1] = a.y;
+      w[j][2] = c.x; w[j][3] = c.y; w[j][4] = c.z; w[j][5] = c.w;
+      w[j][6] = d.x; w[j][7] = d.y;
+    }
+    const uint4* b = reinterpret_cast<const uint4*>(B + tr_at(r, N, q) + kc * tr_chunk(N));
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint4 v = b[i];
+      const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+      float2 x[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        x[e] = make_float2(__uint_as_float(u[e] << 16), __uint_as_float(u[e] & 0xFFFF0000u));
+      if (layer4) {
+        if (kc == 0) bacc[0] = cadd(bacc[0], make_float2(w[0][2 + i], w[1][2 + i]));
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) bacc[e] = cadd(bacc[e], x[e]);
+      }
+      // tap index kk walks the window upwards: k = 4 - kk for layer 4, kk for layer 1
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int kk = 0; kk < kDnK; ++kk) {
+          const float2 tv = make_float2(w[j][i + kk], w[j][i + kk]);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) acc[j][kk][e] = __ffma2_rn(x[e], tv, acc[j][kk][e]);
+        }
+    }
+  }
+  // lanes (butterfly), then the block's two tile lanes of each chunk
+  float v[88];
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int kk = 0; kk < kDnK; ++kk)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        v[(j * kDnK + kk) * 8 + 2 * e] = acc[j][kk][e].x;
+        v[(j * kDnK + kk) * 8 + 2 * e + 1] = acc[j][kk][e].y;
+      }
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    v[80 + 2 * e] = bacc[e].x;
+    v[81 + 2 * e] = bacc[e].y;
+  }
+#pragma unroll
+  for (int i = 0; i < 88; ++i) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], off);
+  }
+  if (sub == 1 && lane == 0) {
+#pragma unroll
+    for (int i = 0; i < 88; ++i) comb[kc][i] = v[i];
+  }
+  __syncthreads();
+  if (sub == 0 && lane == 0) {
+    float* out = (layer4 ? part4 : part1) + static_cast<size_t>(blockIdx.x) * kSdPart;
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int kk = 0; kk < kDnK; ++kk)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const int k = layer4 ? 4 - kk : kk, i = (j * kDnK + kk) * 8 + e;
+          out[(j * kDnK + k) * 32 + 8 * kc + e] = v[i] + comb[kc][i];
+        }
+    if (!layer4 || kc == 0) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) out[320 + 8 * kc + e] = v[80 + e] + comb[kc][80 + e];
+    }
   }
 }
 
-// Weight gradient of a layer with a two-channel side on the CUDA cores, from
-// the training pass's tensors: layer 4 (G = dy fp32 [R][2][N], A = r3 bf16
-// [R][N][32]) or layer 1 (G = g1 bf16 [R][N][32], A = x0 fp32 [R][2][N]).
-// One block per (o, c), fixed-order tree (as dn_wgrad_kernel).
-template <bool LAYER4>
-__global__ void __launch_bounds__(kDnGradThreads) dn_wgrad_side_kernel(
-    const float* __restrict__ f32, const __nv_bfloat16* __restrict__ b16, int R, int N,
-    float* __restrict__ dW, float* __restrict__ db) {
-  __shared__ float red[kDnK + 1][kDnGradThreads];
-  const int o = blockIdx.x, c = blockIdx.y, t = threadIdx.x;
-  const int cin = LAYER4 ? 32 : 2;
-  float acc[kDnK + 1] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  const size_t total = static_cast<size_t>(R) * N;
-  for (size_t i = t; i < total; i += kDnGradThreads) {
-    const int r = static_cast<int>(i / N), p = static_cast<int>(i % N);
-    const float g = LAYER4 ? f32[(static_cast<size_t>(r) * 2 + o) * N + p]
-                           : __bfloat162float(b16[(static_cast<size_t>(r) * N + p) * kTrAct + o]);
-#pragma unroll
-    for (int k = 0; k < kDnK; ++k) {
-      const int qq = p + k - 2;
-      float v = 0.f;
-      if (qq >= 0 && qq < N)
-        v = LAYER4 ? __bfloat162float(b16[(static_cast<size_t>(r) * N + qq) * kTrAct + c])
-                   : f32[(static_cast<size_t>(r) * 2 + c) * N + qq];
-      acc[k] = fmaf(g, v, acc[k]);
-    }
-    acc[kDnK] += g;
-  }
-#pragma unroll
-  for (int k = 0; k <= kDnK; ++k) red[k][t] = acc[k];
-  __syncthreads();
-  for (int s = kDnGradThreads / 2; s > 0; s >>= 1) {
-    if (t < s) {
-#pragma unroll
-      for (int k = 0; k <= kDnK; ++k) red[k][t] += red[k][t + s];
-    }
+// Sums the blocks' partial rows of every weight gradient and the loss
+// partials, in a fixed order, in one launch.  A block takes 32 columns of one
+// layer's rows: 8 slices of consecutive rows are added side by side (a serial
+// chain of rows / 8 coalesced loads), then the slices in order.  (One thread
+// per column over 1024 rows took 78 us a layer and one thread over every tile
+// 32 us for the loss; this launch takes 9 us at 512 rows.)
+struct DnReduceLayer {
+  const float* part;   // [rows][stride]
+  int rows, stride;
+  float* dW;
+  float* db;
+};
+struct DnReduceArgs {
+  DnReduceLayer l[4];   // layers 3 and 2 (32 -> 32: [k][c][o], then [o]), 4 and 1 ([j][k][c], bias)
+  const float* loss_part;
+  int loss_n;
+  size_t n;
+  float* loss;
+};
+constexpr int kRdBig = (5120 + 32) / 32, kRdSide = kSdPart / 32;
+constexpr int kRdBlocks = 2 * kRdBig + 2 * kRdSide + 1;
+__global__ void __launch_bounds__(256) dn_reduce_kernel(const DnReduceArgs a) {
+  __shared__ float red[8][33];
+  const int t = threadIdx.x, col32 = t & 31, slice = t >> 5;
+  int b = blockIdx.x;
+  if (b == kRdBlocks - 1) {   // the loss: strided sums, then a tree
+    __shared__ float ls[256];
+    float s = 0.f;
+    for (int i = t; i < a.loss_n; i += 256) s += a.loss_part[i];
+    ls[t] = s;
     __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+      if (t < w) ls[t] += ls[t + w];
+      __syncthreads();
+    }
+    if (t == 0) *a.loss = ls[0] / static_cast<float>(a.n);
+    return;
   }
-  if (t < kDnK) dW[(o * cin + c) * kDnK + t] = red[t][0];
-  if (t == 0 && c == 0) db[o] = red[kDnK][0];
+  int layer;
+  if (b < 2 * kRdBig) {
+    layer = b / kRdBig;
+    b %= kRdBig;
+  } else {
+    b -= 2 * kRdBig;
+    layer = 2 + b / kRdSide;
+    b %= kRdSide;
+  }
+  const DnReduceLayer l = a.l[layer];
+  const int col = b * 32 + col32;
+  const int per = (l.rows + 7) / 8;
+  const int lo = slice * per, hi = min(l.rows, lo + per);
+  float s = 0.f;
+#pragma unroll 8
+  for (int i = lo; i < hi; ++i) s += l.part[static_cast<size_t>(i) * l.stride + col];
+  red[slice][col32] = s;
+  __syncthreads();
+  if (slice != 0) return;
+#pragma unroll
+  for (int i = 1; i < 8; ++i) s += red[i][col32];
+  if (layer < 2) {
+    if (col < 5120) {
+      const int k = col / 1024, c = (col / 32) % 32, o = col % 32;
+      l.dW[(o * 32 + c) * kDnK + k] = s;
+    } else {
+      l.db[col - 5120] = s;
+    }
+  } else if (col < 320) {
+    const int j = col / 160, k = (col / 32) % 5, c = col % 32;
+    l.dW[(layer == 2 ? j * 32 + c : c * 2 + j) * kDnK + k] = s;
+  } else if (layer == 3 || col < 322) {
+    l.db[col - 320] = s;
+  }
 }
 
 // ------------------------------------------- LS estimate fused with the refinement
@@ -1083,28 +1238,33 @@ __global__ void __launch_bounds__(128 * kTcSlots, 1) dn_ls_tc_kernel(const KPara
 // so that it keeps the buffer's alignment); x0, t, y, dy [R][2][N]; a1, a2,
 // a3, g1, g2 [R][32][N]; rms [R]; transposed weights [5120]; loss partials.
 // The tensor-core training pass also keeps the backward weight image, the
-// bf16 parameters, the weight-gradient block partials of the two 32 -> 32
-// layers (wp), and stores its bf16 tensors r1..r3 from a1 on and g3, g2, g1
-// from g1 on ([R][N][32] each, three to a pair of fp32 regions); its per-tile
+// bf16 parameters, the block partials of the weight gradients (wp: two
+// 32 -> 32 layers, then the two with two-channel sides), and stores its bf16 tensors r1..r3 from a1 on and g3, g2, g1
+// from g1 on (tr_plane elements each, three to a pair of fp32 regions: 192 of
+// the pair's 256 R N bytes plus the pads' 768 R); its per-tile
 // loss partials go to y.
 struct DnWork {
   float *img, *bimg, *pb, *wp, *x0, *tt, *y, *dy, *a1, *a2, *a3, *g1, *g2, *rms, *wt, *part;
 };
 constexpr int kPbFloats = (kDnParams / 2 + 4) / 4 * 4;
-constexpr int kWgPart = 5 * 32 * 32 + 32;                  // one block's partials (floats)
+// partial rows of each weight gradient: at most two blocks per SM write one
+constexpr int kMaxParts = 512;
 static int wg_blocks(int R, int N) {
-  const int t = R * (N / 128);
-  return t < 1024 ? t : 1024;
+  const long t = static_cast<long>(R) * (N / 128);
+  return t < kMaxParts ? static_cast<int>(t) : kMaxParts;
+}
+static size_t part_floats(int R, int N) {
+  return 2 * static_cast<size_t>(wg_blocks(R, N)) * (kWgPart + kSdPart);
 }
 size_t dn_work_floats(int R, int N) {
-  return 2 * kTcImgFloats + kPbFloats + 2 * static_cast<size_t>(wg_blocks(R, N)) * kWgPart +
+  return 2 * kTcImgFloats + kPbFloats + part_floats(R, N) +
          static_cast<size_t>(R) * N * (4 * 2 + 5 * 32) + R + 5120 + kDnLossBlocks;
 }
 static DnWork dn_work(float* w, int R, int N) {
   DnWork d;
   const size_t s2 = static_cast<size_t>(R) * 2 * N, s32 = static_cast<size_t>(R) * 32 * N;
   d.img = w; d.bimg = w + kTcImgFloats; d.pb = d.bimg + kTcImgFloats;
-  d.wp = d.pb + kPbFloats; d.x0 = d.wp + 2 * static_cast<size_t>(wg_blocks(R, N)) * kWgPart;
+  d.wp = d.pb + kPbFloats; d.x0 = d.wp + part_floats(R, N);
   d.tt = d.x0 + s2; d.y = d.tt + s2; d.dy = d.y + s2;
   d.a1 = d.dy + s2; d.a2 = d.a1 + s32; d.a3 = d.a2 + s32; d.g1 = d.a3 + s32; d.g2 = d.g1 + s32;
   d.rms = d.g2 + s32; d.wt = d.rms + R; d.part = d.wt + 5120;
@@ -1238,29 +1398,35 @@ cudaError_t dn_grad_tc(const float* P32, const float2* Hls, const float2* Ht, in
   const int grid = want < sms * 2 ? want : sms * 2;
   auto* acts = reinterpret_cast<__nv_bfloat16*>(d.a1);
   auto* grads = reinterpret_cast<__nv_bfloat16*>(d.g1);
-  const size_t plane = static_cast<size_t>(R) * N * kTrAct;
+  const size_t plane = tr_plane(R, N);
   dn_tc_train_kernel<false><<<grid, 128 * kTcSlots, kTrSmem, st>>>(
       d.img, d.x0, d.tt, R, N, 2.0f / static_cast<float>(n), acts, nullptr, d.dy, d.y, status);
-  dn_loss_final_kernel<<<1, 32, 0, st>>>(d.y, tiles, n, loss);
   dn_tc_train_kernel<true><<<grid, 128 * kTcSlots, kTrSmem, st>>>(
       d.bimg, d.dy, nullptr, R, N, 0.f, acts, grads, nullptr, nullptr, status);
-  const int wgb = wg_blocks(R, N);
+  const int parts = wg_blocks(R, N);
+  const int wgb = parts;
   float* wp3 = d.wp;
-  float* wp2 = d.wp + static_cast<size_t>(wgb) * kWgPart;
+  float* wp2 = wp3 + static_cast<size_t>(parts) * kWgPart;
+  float* sp4 = wp2 + static_cast<size_t>(parts) * kWgPart;
+  float* sp1 = sp4 + static_cast<size_t>(parts) * kSdPart;
   // layer 3: G = g3, A = r2; layer 2: G = g2, A = r1
-  dn_tc_wgrad_kernel<<<wgb, 128, kWgSmem, st>>>(grads, acts + plane, R, N, wp3,
-                                                wp3 + static_cast<size_t>(wgb) * 5120, status);
-  dn_tc_wgrad_kernel<<<wgb, 128, kWgSmem, st>>>(grads + plane, acts, R, N, wp2,
-                                                wp2 + static_cast<size_t>(wgb) * 5120, status);
-  dn_wgrad_reduce_kernel<<<(5120 + 32 + 127) / 128, 128, 0, st>>>(
-      wp3, wp3 + static_cast<size_t>(wgb) * 5120, wgb, grad + kOffW3, grad + kOffB3);
-  dn_wgrad_reduce_kernel<<<(5120 + 32 + 127) / 128, 128, 0, st>>>(
-      wp2, wp2 + static_cast<size_t>(wgb) * 5120, wgb, grad + kOffW2, grad + kOffB2);
-  // layer 4: G = dy, A = r3; layer 1: G = g1, A = x0
-  dn_wgrad_side_kernel<true><<<dim3(2, 32), kDnGradThreads, 0, st>>>(d.dy, acts + 2 * plane, R, N,
-                                                                    grad + kOffW4, grad + kOffB4);
-  dn_wgrad_side_kernel<false><<<dim3(32, 2), kDnGradThreads, 0, st>>>(d.x0, grads + 2 * plane, R, N,
-                                                                     grad + kOffW1, grad + kOffB1);
+  dn_tc_wgrad_kernel<<<wgb, 128, kWgSmem, st>>>(grads, acts + plane, R, N, wp3, status);
+  dn_tc_wgrad_kernel<<<wgb, 128, kWgSmem, st>>>(grads + plane, acts, R, N, wp2, status);
+  // layer 4: T = dy, B = r3; layer 1: T = x0, B = g1
+  const int ptiles = R * (N / 128);
+  const int sdw = (ptiles + 1) / 2, sdb = sdw < sms && sdw < parts ? sdw : (sms < parts ? sms : parts);
+  dn_tc_side_kernel<<<dim3(sdb, 2), kSdThreads, 0, st>>>(d.dy, acts + 2 * plane, d.x0,
+                                                         grads + 2 * plane, R, N, sp4, sp1);
+  DnReduceArgs a;
+  a.l[0] = {wp3, wgb, kWgPart, grad + kOffW3, grad + kOffB3};
+  a.l[1] = {wp2, wgb, kWgPart, grad + kOffW2, grad + kOffB2};
+  a.l[2] = {sp4, sdb, kSdPart, grad + kOffW4, grad + kOffB4};
+  a.l[3] = {sp1, sdb, kSdPart, grad + kOffW1, grad + kOffB1};
+  a.loss_part = d.y;
+  a.loss_n = tiles;
+  a.n = n;
+  a.loss = loss;
+  dn_reduce_kernel<<<kRdBlocks, 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 
