@@ -4,7 +4,7 @@
 // Per antenna row of N subcarriers: normalise H_LS by its RMS, run a residual
 // 1-D convolutional network over subcarriers (2 -> 32 -> 32 -> 32 -> 2
 // channels, kernel 5, ReLU, output added to the input), denormalise.  The
-// same kernels train it: forward with cached pre-activations, mean squared
+// same kernels train it: forward with stored ReLU outputs, mean squared
 // error against the normalised true channel, backward (data gradients as
 // forward convolutions with transposed, flipped weights and ReLU masks;
 // weight gradients as fixed-order block reductions) and Adam.  Inference can
@@ -29,96 +29,507 @@ constexpr int kOffW1 = 0, kOffB1 = 320, kOffW2 = 352, kOffB2 = 5472, kOffW3 = 55
 __device__ __forceinline__ float to_f(float v) { return v; }
 __device__ __forceinline__ float to_f(__nv_bfloat16 v) { return __bfloat162float(v); }
 
-// out[r][o][p] = mask? (pre[r][o][p] > 0) * (b[o] + sum_c sum_k W[o][c][k] in'[r][c][p+k-2]) + res
-// with in' = relu(in) when relu_in.  grid (R, N / kDnPos), kDnPos threads.
-template <int CIN, int COUT, typename WT>
-__global__ void __launch_bounds__(kDnPos) dn_conv_kernel(const float* __restrict__ in,
-                                                         const WT* __restrict__ W,
-                                                         const WT* __restrict__ b, int relu_in,
-                                                         const float* __restrict__ pre,
-                                                         const float* __restrict__ res,
+// FP32 network on the CUDA cores.  Activations are stored after their ReLU
+// (r > 0 is the backward's mask), [R][C][N]; every kernel works on tiles of
+// kDnPos positions of one row.
+//
+// Weights as the kernels read them (dn_setup_kernel), so that the outputs a
+// thread keeps lie next to each other: forward layers 1 to 3 [in][k][out],
+// layer 4 [in][out][k]; data gradients W'[out][in][k] = W[in][out][4 - k] of
+// layers 4, 3 and 2 as forward convolutions, [in][k][out].
+constexpr int kFw1 = 0, kFw2 = kFw1 + 320, kFw3 = kFw2 + 5120, kFw4 = kFw3 + 5120;
+constexpr int kBw4 = kFw4 + 320, kBw3 = kBw4 + 320, kBw2 = kBw3 + 5120;
+constexpr int kBias = kBw2 + 5120, kWtFloats = kBias + 100;   // b1, b2, b3, b4 (two, two unused)
+
+template <typename WT>
+__device__ __forceinline__ void fp32_weights(const WT* __restrict__ P, float* __restrict__ wt,
+                                             int first, int step) {
+  for (int e = first; e < kWtFloats; e += step) {
+    int src;
+    if (e < kFw2) {                                  // [j][k][o]
+      src = kOffW1 + ((e % 32) * 2 + e / 160) * kDnK + (e / 32) % kDnK;
+    } else if (e < kFw4) {                           // [c][k][o]
+      const int f = (e - kFw2) % 5120;
+      src = (e < kFw3 ? kOffW2 : kOffW3) + ((f % 32) * 32 + f / 160) * kDnK + (f / 32) % kDnK;
+    } else if (e < kBw4) {                           // [c][j][k]
+      const int f = e - kFw4;
+      src = kOffW4 + (((f / kDnK) % 2) * 32 + f / 10) * kDnK + f % kDnK;
+    } else if (e < kBw3) {                           // [j][k][c]
+      const int f = e - kBw4;
+      src = kOffW4 + ((f / 160) * 32 + f % 32) * kDnK + 4 - (f / 32) % kDnK;
+    } else if (e < kBias) {                          // [o][k][c]
+      const int f = (e - kBw3) % 5120;
+      src = (e < kBw2 ? kOffW3 : kOffW2) + ((f / 160) * 32 + f % 32) * kDnK + 4 - (f / 32) % kDnK;
+    } else {
+      const int f = e - kBias, l = f / 32;
+      src = (l == 0 ? kOffB1 : l == 1 ? kOffB2 : l == 2 ? kOffB3 : kOffB4) + (f % 32) % (l < 3 ? 32 : 2);
+    }
+    wt[e] = to_f(P[src]);
+  }
+}
+
+// positions q - 2 .. q + 5 of a row (q a multiple of 4), zero outside [0, N)
+__device__ __forceinline__ void window8(const float* __restrict__ row, int q, int N, float (&w)[8]) {
+  const float4 c = *reinterpret_cast<const float4*>(row + q);
+  const float2 a = q > 0 ? *reinterpret_cast<const float2*>(row + q - 2) : make_float2(0.f, 0.f);
+  const float2 d = q + 4 < N ? *reinterpret_cast<const float2*>(row + q + 4) : make_float2(0.f, 0.f);
+  w[0] = a.x; w[1] = a.y;
+  w[2] = c.x; w[3] = c.y; w[4] = c.z; w[5] = c.w;
+  w[6] = d.x; w[7] = d.y;
+}
+
+__device__ __forceinline__ void cp_async(uint32_t dst, const void* src, bool on, int bytes) {
+  // bytes is 8 or 16; zero-fills when off
+  if (bytes == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(on ? 16 : 0)
+                 : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(on ? 8 : 0)
+                 : "memory");
+}
+
+__device__ __forceinline__ float4 relu4(float4 v) {
+  return make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f));
+}
+// v where m > 0, else 0
+__device__ __forceinline__ float4 mask4(float4 v, float4 m) {
+  return make_float4(m.x > 0.f ? v.x : 0.f, m.y > 0.f ? v.y : 0.f, m.z > 0.f ? v.z : 0.f,
+                     m.w > 0.f ? v.w : 0.f);
+}
+
+// 2 -> 32 channels: layer 1 (bias and ReLU) or the data gradient of layer 4
+// (masked by the stored layer output).  Bound by writing the 32 channels: a
+// warp takes four of them and a lane four positions, inputs and outputs in
+// 16-byte pieces.  256 rows of 1024: 9 us against 19.6 us for one position a
+// thread with scalar shared-memory operands.
+template <bool BWD>
+__global__ void __launch_bounds__(256) dn_conv_in_kernel(const float* __restrict__ in,
+                                                         const float* __restrict__ wt,
+                                                         const float* __restrict__ bias,
+                                                         const float* __restrict__ mask,
                                                          float* __restrict__ out, int N) {
-  __shared__ float ws[COUT * CIN * kDnK];
-  __shared__ float xs[CIN][kDnPos + kDnK - 1];
-  const int r = blockIdx.x;
-  const int p0 = blockIdx.y * kDnPos;
-  const int t = threadIdx.x;
-  for (int i = t; i < COUT * CIN * kDnK; i += kDnPos) ws[i] = to_f(W[i]);
-  const float* inr = in + static_cast<size_t>(r) * CIN * N;
-  for (int i = t; i < CIN * (kDnPos + kDnK - 1); i += kDnPos) {
-    const int c = i / (kDnPos + kDnK - 1), j = i % (kDnPos + kDnK - 1);
-    const int p = p0 + j - 2;
-    float v = (p >= 0 && p < N) ? inr[static_cast<size_t>(c) * N + p] : 0.f;
-    if (relu_in) v = fmaxf(v, 0.f);
-    xs[c][j] = v;
-  }
-  __syncthreads();
-  float acc[COUT];
+  __shared__ __align__(16) float ws[320];
+  const int tiles_row = N / kDnPos;
+  const int r = blockIdx.x / tiles_row;
+  const int lane = threadIdx.x & 31, ch = (threadIdx.x >> 5) * 4;
+  const int q = (blockIdx.x % tiles_row) * kDnPos + 4 * lane;
+  for (int i = threadIdx.x; i < 320; i += 256) ws[i] = wt[i];
+  float w[2][8];
+  window8(in + static_cast<size_t>(r) * 2 * N, q, N, w[0]);
+  window8(in + (static_cast<size_t>(r) * 2 + 1) * N, q, N, w[1]);
+  float acc[4][4];   // [channel][position]
 #pragma unroll
-  for (int o = 0; o < COUT; ++o) acc[o] = b ? to_f(b[o]) : 0.f;
-#pragma unroll 4
-  for (int c = 0; c < CIN; ++c) {
+  for (int o = 0; o < 4; ++o)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[o][i] = BWD ? 0.f : bias[ch + o];
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
 #pragma unroll
     for (int k = 0; k < kDnK; ++k) {
-      const float x = xs[c][t + k];
+      const float4 v = *reinterpret_cast<const float4*>(ws + (j * kDnK + k) * 32 + ch);
+      const float vv[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-      for (int o = 0; o < COUT; ++o) acc[o] = fmaf(ws[(o * CIN + c) * kDnK + k], x, acc[o]);
+      for (int o = 0; o < 4; ++o)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[o][i] = fmaf(vv[o], w[j][i + k], acc[o][i]);
     }
-  }
-  const size_t base = static_cast<size_t>(r) * COUT * N + p0 + t;
 #pragma unroll
-  for (int o = 0; o < COUT; ++o) {
-    float v = acc[o];
-    if (pre) v = pre[base + static_cast<size_t>(o) * N] > 0.f ? v : 0.f;
-    if (res) v += res[base + static_cast<size_t>(o) * N];
-    out[base + static_cast<size_t>(o) * N] = v;
+  for (int o = 0; o < 4; ++o) {
+    const size_t at = (static_cast<size_t>(r) * 32 + ch + o) * N + q;
+    float4 v = make_float4(acc[o][0], acc[o][1], acc[o][2], acc[o][3]);
+    v = BWD ? mask4(v, *reinterpret_cast<const float4*>(mask + at)) : relu4(v);
+    *reinterpret_cast<float4*>(out + at) = v;
   }
 }
 
-// W'[c][o][k] = W[o][c][4 - k]: data gradient of a conv as a forward conv.
-__global__ void dn_wt_kernel(const float* W, float* Wt, int cin, int cout) {
-  const int n = cin * cout * kDnK;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const int k = i % kDnK, o = (i / kDnK) % cout, c = i / (kDnK * cout);
-    Wt[i] = W[(o * cin + c) * kDnK + (kDnK - 1 - k)];
-  }
-}
-
-// dW[o][c][k] = sum_r sum_p dout[r][o][p] in'[r][c][p + k - 2] and, for
-// c = 0, db[o] = sum dout[r][o][p].  One block per (o, c), fixed-order tree.
-constexpr int kDnGradThreads = 256;
-__global__ void __launch_bounds__(kDnGradThreads) dn_wgrad_kernel(
-    const float* __restrict__ dout, const float* __restrict__ in, int relu_in, int cin, int cout,
-    int R, int N, float* __restrict__ dW, float* __restrict__ db) {
-  __shared__ float red[kDnK + 1][kDnGradThreads];
-  const int o = blockIdx.x, c = blockIdx.y, t = threadIdx.x;
-  float acc[kDnK + 1] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  const size_t total = static_cast<size_t>(R) * N;
-  for (size_t i = t; i < total; i += kDnGradThreads) {
-    const int r = static_cast<int>(i / N), p = static_cast<int>(i % N);
-    const float g = dout[(static_cast<size_t>(r) * cout + o) * N + p];
-    const float* x = in + (static_cast<size_t>(r) * cin + c) * N;
-#pragma unroll
-    for (int k = 0; k < kDnK; ++k) {
-      const int q = p + k - 2;
-      float v = (q >= 0 && q < N) ? x[q] : 0.f;
-      if (relu_in) v = fmaxf(v, 0.f);
-      acc[k] = fmaf(g, v, acc[k]);
+// 32 -> 32 channels: layers 2 and 3 (bias and ReLU) or their data gradients
+// (masked).  Bound by the FMA pipe (5120 FMAs a position).  A thread keeps 8
+// outputs x 4 positions: per input channel two 16-byte loads give its 8-value
+// window and ten broadcast ones its 40 weights, for 160 FMAs issued as 80
+// packed ones (output pairs; the input value in both halves: 60 us where
+// scalar ones took 70, before the copies were asynchronous).  Blocks walk the
+// tiles, four on an SM, the weights loaded once and the next tile's rows
+// copied under the current one's FMAs.  256 rows of 1024: 51 us (floor 33)
+// against 104 us for 32 outputs x 1 position with one shared-memory operand
+// per FMA.
+constexpr int kCvWBytes = 32 * kDnK * 32 * 4;                  // weights [c][k][o]
+constexpr int kCvRow = kDnPos + kDnK - 1;                       // position q0 - 2 + j
+constexpr int kCvStage = 32 * kCvRow * 4;
+constexpr int kCvSmem = kCvWBytes + 2 * kCvStage;
+template <bool BWD>
+__global__ void __launch_bounds__(128, 4) dn_conv32_kernel(const float* __restrict__ in,
+                                                           const float* __restrict__ wt,
+                                                           const float* __restrict__ bias,
+                                                           const float* __restrict__ mask,
+                                                           float* __restrict__ out, int R, int N) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  const float* ws = reinterpret_cast<const float*>(smem);
+  const int tiles_row = N / kDnPos, tiles = R * tiles_row;
+  const int t = threadIdx.x, lane = t & 31, o0 = (t >> 5) * 8;
+  auto fetch = [&](int tile, int b) {
+    if (tile < tiles) {
+      const int r = tile / tiles_row, q0 = (tile % tiles_row) * kDnPos;
+      const uint32_t x = smem_u32(smem + kCvWBytes + b * kCvStage);
+      constexpr int kHalf = kCvRow / 2;
+      for (int i = t; i < 32 * kHalf; i += 128) {
+        const int c = i / kHalf, j = 2 * (i % kHalf), p = q0 + j - 2;
+        const bool on = p >= 0 && p < N;
+        cp_async(x + (c * kCvRow + j) * 4, in + (static_cast<size_t>(r) * 32 + c) * N + (on ? p : 0), on, 8);
+      }
     }
-    acc[kDnK] += g;
-  }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  for (int i = t; i < kCvWBytes / 16; i += 128) cp_async(smem_u32(smem) + 16 * i, wt + 4 * i, true, 16);
+  fetch(blockIdx.x, 0);
+  float2 bs[4];
 #pragma unroll
-  for (int k = 0; k <= kDnK; ++k) red[k][t] = acc[k];
-  __syncthreads();
-  for (int s = kDnGradThreads / 2; s > 0; s >>= 1) {
-    if (t < s) {
-#pragma unroll
-      for (int k = 0; k <= kDnK; ++k) red[k][t] += red[k][t + s];
-    }
+  for (int o = 0; o < 4; ++o)
+    bs[o] = BWD ? make_float2(0.f, 0.f) : make_float2(bias[o0 + 2 * o], bias[o0 + 2 * o + 1]);
+  int b = 0;
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, b ^= 1) {
+    fetch(tile + gridDim.x, b ^ 1);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
     __syncthreads();
+    const float* xs = reinterpret_cast<const float*>(smem + kCvWBytes + b * kCvStage) + 4 * lane;
+    float2 acc[4][4];   // [position][output pair]
+#pragma unroll
+    for (int o = 0; o < 4; ++o)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[i][o] = bs[o];
+#pragma unroll 2
+    for (int c = 0; c < 32; ++c) {
+      const float4 x0 = *reinterpret_cast<const float4*>(xs + c * kCvRow);
+      const float4 x1 = *reinterpret_cast<const float4*>(xs + c * kCvRow + 4);
+      const float x[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+#pragma unroll
+      for (int k = 0; k < kDnK; ++k) {
+        const float4 wa = *reinterpret_cast<const float4*>(ws + (c * kDnK + k) * 32 + o0);
+        const float4 wb = *reinterpret_cast<const float4*>(ws + (c * kDnK + k) * 32 + o0 + 4);
+        const float2 w[4] = {make_float2(wa.x, wa.y), make_float2(wa.z, wa.w), make_float2(wb.x, wb.y),
+                             make_float2(wb.z, wb.w)};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float2 xx = make_float2(x[i + k], x[i + k]);
+#pragma unroll
+          for (int o = 0; o < 4; ++o) acc[i][o] = __ffma2_rn(w[o], xx, acc[i][o]);
+        }
+      }
+    }
+    const int r = tile / tiles_row, q0 = (tile % tiles_row) * kDnPos;
+#pragma unroll
+    for (int o = 0; o < 8; ++o) {
+      const size_t at = (static_cast<size_t>(r) * 32 + o0 + o) * N + q0 + 4 * lane;
+      float4 v = (o & 1) ? make_float4(acc[0][o / 2].y, acc[1][o / 2].y, acc[2][o / 2].y, acc[3][o / 2].y)
+                         : make_float4(acc[0][o / 2].x, acc[1][o / 2].x, acc[2][o / 2].x, acc[3][o / 2].x);
+      v = BWD ? mask4(v, *reinterpret_cast<const float4*>(mask + at)) : relu4(v);
+      *reinterpret_cast<float4*>(out + at) = v;
+    }
+    __syncthreads();   // the stage is consumed before the next copies into it
   }
-  if (t < kDnK) dW[(o * cin + c) * kDnK + t] = red[t][0];
-  if (t == 0 && c == 0) db[o] = red[kDnK][0];
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+template <bool BWD>
+static cudaError_t conv32(const float* in, const float* wt, const float* bias, const float* mask,
+                          float* out, int R, int N, int sms, cudaStream_t st) {
+  const cudaError_t e = cudaFuncSetAttribute(dn_conv32_kernel<BWD>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, kCvSmem);
+  if (e != cudaSuccess) return e;
+  const int tiles = R * (N / kDnPos);
+  dn_conv32_kernel<BWD><<<tiles < 4 * sms ? tiles : 4 * sms, 128, kCvSmem, st>>>(in, wt, bias, mask, out,
+                                                                               R, N);
+  return cudaSuccess;
+}
+
+// 32 -> 2 channels (layer 4) with the network's output: y = x0 + conv, then
+// TRAIN: dy = 2 (y - t) / n and the tile's sum of (y - t)^2, else
+// Hout = (y[0] + j y[1]) rms.  Bound by reading the 32 channels: a warp takes
+// four of them and a lane four positions; the eight warps' sums meet in shared
+// memory, added in warp order.  256 rows of 1024: 11 us; before, 23 us and
+// a launch of 6 us for the loss.
+struct DnOutArgs {
+  const float* in;     // r3 [R][32][N]
+  const float* wt;     // [c][j][k]
+  const float* bias;   // two
+  const float* x0;     // [R][2][N]
+  const float* tt;     // TRAIN: [R][2][N]
+  float* dy;           // TRAIN: [R][2][N]
+  float* part;         // TRAIN: one per tile
+  float inv_n;         // TRAIN: 2 / n
+  const float* rms;    // else
+  float2* Hout;        // else
+  int N;
+};
+template <bool TRAIN>
+__global__ void __launch_bounds__(256) dn_conv_out_kernel(const DnOutArgs a) {
+  __shared__ float ws[320];
+  __shared__ __align__(16) float red[8][2][kDnPos];
+  __shared__ float se[8];
+  const int N = a.N, tiles_row = N / kDnPos;
+  const int r = blockIdx.x / tiles_row, q0 = (blockIdx.x % tiles_row) * kDnPos;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  for (int i = t; i < 320; i += 256) ws[i] = a.wt[i];
+  __syncthreads();
+  float acc[2][4];
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[j][i] = 0.f;
+#pragma unroll
+  for (int cc = 0; cc < 4; ++cc) {
+    const int c = 4 * warp + cc;
+    float w[8];
+    window8(a.in + (static_cast<size_t>(r) * 32 + c) * N, q0 + 4 * lane, N, w);
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int k = 0; k < kDnK; ++k) {
+        const float v = ws[c * 10 + j * kDnK + k];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[j][i] = fmaf(v, w[i + k], acc[j][i]);
+      }
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+    *reinterpret_cast<float4*>(&red[warp][j][4 * lane]) =
+        make_float4(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
+  __syncthreads();
+  const int j = t >> 7, p = t & 127;
+  float y = a.bias[j];
+#pragma unroll
+  for (int w = 0; w < 8; ++w) y += red[w][j][p];
+  const size_t at = (static_cast<size_t>(r) * 2 + j) * N + q0 + p;
+  y += a.x0[at];
+  if (TRAIN) {
+    const float d = y - a.tt[at];
+    a.dy[at] = d * a.inv_n;
+    float e = d * d;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) e += __shfl_xor_sync(0xffffffffu, e, off);
+    if (lane == 0) se[warp] = e;
+    __syncthreads();
+    if (t == 0) {
+      float sum = se[0];
+#pragma unroll
+      for (int w = 1; w < 8; ++w) sum += se[w];
+      a.part[blockIdx.x] = sum;
+    }
+  } else {
+    reinterpret_cast<float*>(a.Hout)[2 * (static_cast<size_t>(r) * N + q0 + p) + j] = y * a.rms[r];
+  }
+}
+
+// Weight gradient of a 32 -> 32 layer, FP32: dW[o][c][k] = sum_p G[o][p]
+// A[c][p + k - 2] and db[o] = sum_p G[o][p], as a product with the positions
+// as the inner dimension.  Bound by the FMA pipe (5120 FMAs a position).  A
+// tile's G and A rows come to shared memory by asynchronous copies, one tile
+// ahead; a thread keeps 4 outputs x 2 inputs x 5 taps and takes the tile four
+// positions at a time: six 16-byte loads (A slides in registers) for 160 FMAs.
+// The two halves of a block take the tile's halves.  Blocks walk the tiles
+// (two blocks fit on an SM) and write one row of partial sums each.  256 rows
+// of 1024: 58 us a layer (packed FMAs over even and odd positions, whose
+// operand pairs share no register from one to the next: 71); one block per
+// (o, c) that re-read both tensors took about 1900 us.
+constexpr int kFwThreads = 256;
+constexpr int kFwRow = kDnPos + 4;                     // floats; rows 4 banks apart
+constexpr int kFwStage = 2 * 32 * kFwRow * 4;          // bytes of G and A
+constexpr int kFwSmem = 2 * kFwStage;
+constexpr int kWgPart = 5 * 32 * 32 + 32;              // one block's partials (floats)
+static_assert(kFwSmem >= 128 * 40 * 4, "the halves meet in the stages");
+
+__global__ void __launch_bounds__(kFwThreads, 2) dn_wgrad32_kernel(const float* __restrict__ G,
+                                                                   const float* __restrict__ A, int R,
+                                                                   int N, float* __restrict__ part) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int t = threadIdx.x, lane = t & 31;
+  const int half = t >> 7, u = t & 127;
+  const int og = u & 7, cg = u >> 3;                   // o = og + 8 i, c = cg + 16 j
+  const int tiles_row = N / kDnPos, tiles = R * tiles_row;
+  auto fetch = [&](int tile, int b) {
+    if (tile < tiles) {
+      const int r = tile / tiles_row, q0 = (tile % tiles_row) * kDnPos;
+      const uint32_t g = smem_u32(smem + b * kFwStage), x = g + 32 * kFwRow * 4;
+      for (int i = t; i < 32 * 32; i += kFwThreads) {
+        const int o = i >> 5, p = 4 * (i & 31);
+        cp_async(g + (o * kFwRow + p) * 4, G + (static_cast<size_t>(r) * 32 + o) * N + q0 + p, true, 16);
+      }
+      constexpr int kHalf = (kDnPos + 4) / 2;
+      for (int i = t; i < 32 * kHalf; i += kFwThreads) {
+        const int c = i / kHalf, jj = 2 * (i % kHalf), p = q0 + jj - 2;
+        const bool on = p >= 0 && p < N;
+        cp_async(x + (c * kFwRow + jj) * 4, A + (static_cast<size_t>(r) * 32 + c) * N + (on ? p : 0), on, 8);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float acc[4][2][kDnK];
+  float bacc = 0.f;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int k = 0; k < kDnK; ++k) acc[i][j][k] = 0.f;
+  fetch(blockIdx.x, 0);
+  int b = 0;
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, b ^= 1) {
+    fetch(tile + gridDim.x, b ^ 1);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();
+    const float* g = reinterpret_cast<const float*>(smem + b * kFwStage);
+    const float* x = g + 32 * kFwRow;
+    {   // bias: eight threads an output, 16 positions each
+      const float4* gb = reinterpret_cast<const float4*>(g + (t >> 3) * kFwRow) + (t & 7);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float4 v = gb[8 * i];
+        bacc += (v.x + v.y) + (v.z + v.w);
+      }
+    }
+    const float* gt = g + og * kFwRow + 64 * half;
+    const float* xt = x + cg * kFwRow + 64 * half;
+    float4 lo[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) lo[j] = *reinterpret_cast<const float4*>(xt + 16 * j * kFwRow);
+#pragma unroll 2
+    for (int p = 0; p < 64; p += 4) {
+      float gv[4][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        *reinterpret_cast<float4*>(gv[i]) = *reinterpret_cast<const float4*>(gt + 8 * i * kFwRow + p);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const float4 hi = *reinterpret_cast<const float4*>(xt + 16 * j * kFwRow + p + 4);
+        const float w[8] = {lo[j].x, lo[j].y, lo[j].z, lo[j].w, hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int k = 0; k < kDnK; ++k)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i][j][k] = fmaf(gv[i][q], w[k + q], acc[i][j][k]);
+        lo[j] = hi;
+      }
+    }
+    __syncthreads();   // the stage is consumed before the next copies into it
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  // the halves' sums meet, the first half writes
+  float* out = part + static_cast<size_t>(blockIdx.x) * kWgPart;
+  float* comb = reinterpret_cast<float*>(smem);
+  if (half == 1) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int k = 0; k < kDnK; ++k)
+          comb[((i * 2 + j) * kDnK + k) * 128 + u] = acc[i][j][k];
+  }
+  __syncthreads();
+  if (half == 0) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int k = 0; k < kDnK; ++k)
+          out[(k * 32 + cg + 16 * j) * 32 + og + 8 * i] =
+              acc[i][j][k] + comb[((i * 2 + j) * kDnK + k) * 128 + u];
+  }
+#pragma unroll
+  for (int off = 4; off > 0; off >>= 1) bacc += __shfl_xor_sync(0xffffffffu, bacc, off);
+  if ((lane & 7) == 0) out[5120 + (t >> 3)] = bacc;
+}
+
+// Weight gradients of the layers with a two-channel side, FP32, in one launch
+// (blockIdx.y 0: layer 4 with T = dy, B = r3; 1: layer 1 with T = x0, B = g1):
+//   layer 4: dW[j][c][k] = sum_q B[c][q] T[j][q + 2 - k], db[j] = sum_q T[j][q]
+//   layer 1: dW[c][j][k] = sum_q B[c][q] T[j][q + k - 2], db[c] = sum_q B[c][q]
+// Bound by one pass over B.  A warp takes four channels and a lane four
+// positions of each tile, 40 sums in registers; blocks walk the tiles and
+// write one row of partial sums each ([j][k][c], then the biases).  256 rows of
+// 1024: 23 us (30 without the loads one tile ahead).
+constexpr int kSdPart = 320 + 32;
+__global__ void __launch_bounds__(256, 2) dn_side32_kernel(const float* __restrict__ dy,
+                                                        const float* __restrict__ r3,
+                                                        const float* __restrict__ x0,
+                                                        const float* __restrict__ g1, int R, int N,
+                                                        float* __restrict__ part4,
+                                                        float* __restrict__ part1) {
+  const bool layer4 = blockIdx.y == 0;
+  const float* __restrict__ T = layer4 ? dy : x0;
+  const float* __restrict__ B = layer4 ? r3 : g1;
+  const int lane = threadIdx.x & 31, ch = (threadIdx.x >> 5) * 4;
+  const int tiles_row = N / kDnPos, tiles = R * tiles_row;
+  float acc[4][2][kDnK], bacc[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    bacc[c] = 0.f;
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int k = 0; k < kDnK; ++k) acc[c][j][k] = 0.f;
+  }
+  float wn[2][8];
+  float4 bn[4];
+  auto fetch = [&](int tile) {   // one tile's loads, a tile ahead of their use
+    const int r = tile / tiles_row, q = (tile % tiles_row) * kDnPos + 4 * lane;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) window8(T + (static_cast<size_t>(r) * 2 + j) * N, q, N, wn[j]);
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      bn[c] = *reinterpret_cast<const float4*>(B + (static_cast<size_t>(r) * 32 + ch + c) * N + q);
+  };
+  if (blockIdx.x < tiles) fetch(blockIdx.x);
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    float w[2][8];
+    float4 bv[4];
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) w[j][i] = wn[j][i];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) bv[c] = bn[c];
+    if (tile + static_cast<int>(gridDim.x) < tiles) fetch(tile + gridDim.x);
+    if (layer4) {
+#pragma unroll
+      for (int j = 0; j < 2; ++j) bacc[j] += (w[j][2] + w[j][3]) + (w[j][4] + w[j][5]);
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const float x[4] = {bv[c].x, bv[c].y, bv[c].z, bv[c].w};
+      if (!layer4) bacc[c] += (x[0] + x[1]) + (x[2] + x[3]);
+      // kk walks the window upwards: tap 4 - kk for layer 4, kk for layer 1
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int kk = 0; kk < kDnK; ++kk)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) acc[c][j][kk] = fmaf(x[i], w[j][i + kk], acc[c][j][kk]);
+    }
+  }
+  auto lanes = [&](float v) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    return v;
+  };
+  float* out = (layer4 ? part4 : part1) + static_cast<size_t>(blockIdx.x) * kSdPart;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int kk = 0; kk < kDnK; ++kk) {
+        const float v = lanes(acc[c][j][kk]);
+        if (lane == 0) out[(j * kDnK + (layer4 ? 4 - kk : kk)) * 32 + ch + c] = v;
+      }
+    const float v = lanes(bacc[c]);
+    if (lane == 0) {
+      if (!layer4) out[320 + ch + c] = v;
+      else if (ch == 0 && c < 2) out[320 + c] = v;
+    }
+  }
 }
 
 // x0 = [Re H, Im H] / rms and, when Ht is given, t = [Re Ht, Im Ht] / rms;
@@ -154,48 +565,17 @@ __device__ __forceinline__ void prepare_row(const float2* H, const float2* Ht, i
   }
 }
 
-__global__ void dn_prepare_kernel(const float2* H, const float2* Ht, int N, float* x0, float* tt,
-                                  float* rms) {
-  prepare_row(H, Ht, blockIdx.x, N, x0, tt, rms);
-}
-
-// H = (y[0] + j y[1]) rms
-__global__ void dn_finish_kernel(const float* y, const float* rms, int R, int N, float2* H) {
-  const size_t n = static_cast<size_t>(R) * N;
-  for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < n;
-       i += static_cast<size_t>(gridDim.x) * blockDim.x) {
-    const int r = static_cast<int>(i / N), k = static_cast<int>(i % N);
-    const float* yr = y + static_cast<size_t>(r) * 2 * N;
-    H[i] = make_float2(yr[k] * rms[r], yr[N + k] * rms[r]);
-  }
-}
-
-// dy = 2 (y - t) / n, per-block partial sums of (y - t)^2
-constexpr int kDnLossBlocks = 256;
-__global__ void dn_loss_kernel(const float* y, const float* tt, size_t n, float* dy, float* part) {
-  __shared__ float red[256];
-  const int t = threadIdx.x;
-  float s = 0.f;
-  const float sc = 2.0f / static_cast<float>(n);
-  for (size_t i = blockIdx.x * static_cast<size_t>(256) + t; i < n; i += static_cast<size_t>(gridDim.x) * 256) {
-    const float d = y[i] - tt[i];
-    dy[i] = sc * d;
-    s = fmaf(d, d, s);
-  }
-  red[t] = s;
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if (t < w) red[t] += red[t + w];
-    __syncthreads();
-  }
-  if (t == 0) part[blockIdx.x] = red[0];
-}
-__global__ void dn_loss_final_kernel(const float* part, int nb, size_t n, float* loss) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    float s = 0.f;
-    for (int i = 0; i < nb; ++i) s += part[i];
-    *loss = s / static_cast<float>(n);
-  }
+// The FP32 kernels' weights (the first kSetupBlocks blocks) and the
+// normalised rows (a block each), in one launch.
+constexpr int kSetupBlocks = 32;
+template <typename WT>
+__global__ void __launch_bounds__(256) dn_setup_kernel(const WT* __restrict__ P, float* wt,
+                                                       const float2* H, const float2* Ht, int N,
+                                                       float* x0, float* tt, float* rms) {
+  if (blockIdx.x < kSetupBlocks)
+    fp32_weights(P, wt, blockIdx.x * 256 + threadIdx.x, kSetupBlocks * 256);
+  else
+    prepare_row(H, Ht, blockIdx.x - kSetupBlocks, N, x0, tt, rms);
 }
 
 __global__ void dn_adam_kernel(float* p, const float* g, float* m, float* v, int n, float lr,
@@ -543,7 +923,6 @@ __device__ __forceinline__ void tc_bimage(const float* __restrict__ P, float* __
 // blocks: the weight images (the first kSetupBlocks blocks an image; bimg
 // null: forward image only) and the normalised rows (a block each).  The four
 // launches it replaces took 10.3 us at 256 rows of 1024 and their gaps.
-constexpr int kSetupBlocks = 32;
 template <typename PT>
 __global__ void __launch_bounds__(256) dn_tc_setup_kernel(const PT* __restrict__ P, float* img,
                                                           float* bimg, const float2* H,
@@ -796,8 +1175,6 @@ constexpr int kWgStage = kWgG + 8 * kWgGChunk;
 constexpr int kWgStages = 4;
 constexpr int kWgBars = kWgStages * kWgStage;              // full, empty, done
 constexpr int kWgSmem = kWgBars + (2 * kWgStages + 1) * 8 + 8;
-constexpr int kWgPart = 5 * 32 * 32 + 32;                  // one block's partials (floats)
-constexpr int kSdPart = 320 + 32;
 // warp 0 copies, 1 MMAs, 2 and 3 bias sums, 4-11 layers 1 and 4: twelve warps
 // leave 168 registers a thread, which the loads one tile ahead need
 constexpr int kWgSideWarp = 4;
@@ -1061,10 +1438,10 @@ __global__ void __launch_bounds__(kWgThreads, 1) dn_tc_wgrad_kernel(const DnWgra
 
 // Sums the blocks' partial rows of every weight gradient and the loss
 // partials, in a fixed order, in one launch.  A block takes 32 columns of one
-// layer's rows: 8 slices of consecutive rows are added side by side (a serial
-// chain of rows / 8 coalesced loads), then the slices in order.  (One thread
+// layer's rows: 16 slices of consecutive rows are added side by side (a serial
+// chain of rows / 16 coalesced loads), then the slices in order.  (One thread
 // per column over 1024 rows took 78 us a layer and one thread over every tile
-// 32 us for the loss; this launch takes 9 us at 512 rows.)
+// 32 us for the loss; this launch takes 3.6 us at 152 rows and 8.6 at 304.)
 struct DnReduceLayer {
   const float* part;   // [rows][stride]
   int rows, stride;
@@ -1078,19 +1455,20 @@ struct DnReduceArgs {
   size_t n;
   float* loss;
 };
+constexpr int kRdSlices = 16, kRdThreads = 32 * kRdSlices;
 constexpr int kRdBig = (5120 + 32) / 32, kRdSide = kSdPart / 32;
 constexpr int kRdBlocks = 2 * kRdBig + 2 * kRdSide + 1;
-__global__ void __launch_bounds__(256) dn_reduce_kernel(const DnReduceArgs a) {
-  __shared__ float red[8][33];
+__global__ void __launch_bounds__(kRdThreads) dn_reduce_kernel(const DnReduceArgs a) {
+  __shared__ float red[kRdSlices][33];
   const int t = threadIdx.x, col32 = t & 31, slice = t >> 5;
   int b = blockIdx.x;
   if (b == kRdBlocks - 1) {   // the loss: strided sums, then a tree
-    __shared__ float ls[256];
+    __shared__ float ls[kRdThreads];
     float s = 0.f;
-    for (int i = t; i < a.loss_n; i += 256) s += a.loss_part[i];
+    for (int i = t; i < a.loss_n; i += kRdThreads) s += a.loss_part[i];
     ls[t] = s;
     __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
+    for (int w = kRdThreads / 2; w > 0; w >>= 1) {
       if (t < w) ls[t] += ls[t + w];
       __syncthreads();
     }
@@ -1108,16 +1486,16 @@ __global__ void __launch_bounds__(256) dn_reduce_kernel(const DnReduceArgs a) {
   }
   const DnReduceLayer l = a.l[layer];
   const int col = b * 32 + col32;
-  const int per = (l.rows + 7) / 8;
+  const int per = (l.rows + kRdSlices - 1) / kRdSlices;
   const int lo = slice * per, hi = min(l.rows, lo + per);
   float s = 0.f;
-#pragma unroll 8
+#pragma unroll 10
   for (int i = lo; i < hi; ++i) s += l.part[static_cast<size_t>(i) * l.stride + col];
   red[slice][col32] = s;
   __syncthreads();
   if (slice != 0) return;
 #pragma unroll
-  for (int i = 1; i < 8; ++i) s += red[i][col32];
+  for (int i = 1; i < kRdSlices; ++i) s += red[i][col32];
   if (layer < 2) {
     if (col < 5120) {
       const int k = col / 1024, c = (col / 32) % 32, o = col % 32;
@@ -1310,18 +1688,20 @@ __global__ void __launch_bounds__(128 * kTcSlots, 1) dn_ls_tc_kernel(const KPara
 
 // ------------------------------------------------------------- host side
 
-// Work buffer (floats): the tensor-core weight image [kTcImgFloats] (first,
-// so that it keeps the buffer's alignment); x0, t, y, dy [R][2][N]; a1, a2,
-// a3, g1, g2 [R][32][N]; rms [R]; transposed weights [5120]; loss partials.
-// The tensor-core training pass also keeps the backward weight image, the
-// block partials of the weight gradients (wp: two
-// 32 -> 32 layers, then the two with two-channel sides), and stores its bf16 tensors r1..r3 from a1 on and g3, g2, g1
-// from g1 on (tr_plane elements each, three to a pair of fp32 regions: 192 of
-// the pair's 256 R N bytes plus the pads' 768 R); its per-tile
-// loss partials go to y.
+// Work buffer (floats): the tensor-core weight images, forward and backward
+// [kTcImgFloats each] (first, so that they keep the buffer's alignment), whose
+// place the FP32 kernels' weights take in their passes; the block partials of
+// the weight gradients (wp: two 32 -> 32 layers, then the two with
+// two-channel sides); x0, t, y, dy [R][2][N]; a1, a2, a3, g1, g2 [R][32][N];
+// rms [R].  The tensor-core training pass stores its bf16 tensors r1..r3 from
+// a1 on and g3, g2, g1 from g1 on (tr_plane elements each, three to a pair of
+// fp32 regions: 192 of the pair's 256 R N bytes plus the pads' 768 R).  The
+// loss partials, one per tile, go to y.
 struct DnWork {
-  float *img, *bimg, *wp, *x0, *tt, *y, *dy, *a1, *a2, *a3, *g1, *g2, *rms, *wt, *part;
+  float *img, *bimg, *wt, *wp, *x0, *tt, *y, *dy, *a1, *a2, *a3, *g1, *g2, *rms;
 };
+constexpr int kHeadFloats = (2 * kTcImgFloats > kWtFloats ? 2 * kTcImgFloats : kWtFloats);
+static_assert(kHeadFloats % 4 == 0, "16-byte alignment of what follows");
 // partial rows of each weight gradient: one per block
 constexpr int kMaxParts = 512;
 static int wg_blocks(int R, int N) {
@@ -1332,44 +1712,51 @@ static size_t part_floats(int R, int N) {
   return 2 * static_cast<size_t>(wg_blocks(R, N)) * (kWgPart + kSdPart);
 }
 size_t dn_work_floats(int R, int N) {
-  return 2 * kTcImgFloats + part_floats(R, N) +
-         static_cast<size_t>(R) * N * (4 * 2 + 5 * 32) + R + 5120 + kDnLossBlocks;
+  // three more than the layout takes: a buffer that is not 16-byte aligned
+  // (the FP32 passes accept one) is used from its first aligned float on
+  return kHeadFloats + part_floats(R, N) + static_cast<size_t>(R) * N * (4 * 2 + 5 * 32) + R + 3;
 }
 static DnWork dn_work(float* w, int R, int N) {
+  w = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(w) + 15) & ~static_cast<uintptr_t>(15));
   DnWork d;
   const size_t s2 = static_cast<size_t>(R) * 2 * N, s32 = static_cast<size_t>(R) * 32 * N;
-  d.img = w; d.bimg = w + kTcImgFloats;
-  d.wp = d.bimg + kTcImgFloats; d.x0 = d.wp + part_floats(R, N);
+  d.img = w; d.bimg = w + kTcImgFloats; d.wt = w;
+  d.wp = w + kHeadFloats; d.x0 = d.wp + part_floats(R, N);
   d.tt = d.x0 + s2; d.y = d.tt + s2; d.dy = d.y + s2;
   d.a1 = d.dy + s2; d.a2 = d.a1 + s32; d.a3 = d.a2 + s32; d.g1 = d.a3 + s32; d.g2 = d.g1 + s32;
-  d.rms = d.g2 + s32; d.wt = d.rms + R; d.part = d.wt + 5120;
+  d.rms = d.g2 + s32;
   return d;
 }
 
-template <int CIN, int COUT, typename WT>
-static void conv(const float* in, const WT* W, const WT* b, int relu_in, const float* pre,
-                 const float* res, float* out, int R, int N, cudaStream_t st) {
-  dn_conv_kernel<CIN, COUT, WT><<<dim3(R, N / kDnPos), kDnPos, 0, st>>>(in, W, b, relu_in, pre, res,
-                                                                       out, N);
-}
-
-template <typename WT>
-static void forward(const WT* P, const DnWork& d, int R, int N, cudaStream_t st) {
-  conv<2, 32, WT>(d.x0, P + kOffW1, P + kOffB1, 0, nullptr, nullptr, d.a1, R, N, st);
-  conv<32, 32, WT>(d.a1, P + kOffW2, P + kOffB2, 1, nullptr, nullptr, d.a2, R, N, st);
-  conv<32, 32, WT>(d.a2, P + kOffW3, P + kOffB3, 1, nullptr, nullptr, d.a3, R, N, st);
-  conv<32, 2, WT>(d.a3, P + kOffW4, P + kOffB4, 1, nullptr, d.x0, d.y, R, N, st);
+// layers 1 to 3 on the CUDA cores (biases b1, b2, b3 in fp32)
+static cudaError_t forward(const float* b, const DnWork& d, int R, int N, int sms, cudaStream_t st) {
+  dn_conv_in_kernel<false><<<R * (N / kDnPos), 256, 0, st>>>(d.x0, d.wt + kFw1, b, nullptr, d.a1, N);
+  cudaError_t e = conv32<false>(d.a1, d.wt + kFw2, b + 32, nullptr, d.a2, R, N, sms, st);
+  if (e == cudaSuccess) e = conv32<false>(d.a2, d.wt + kFw3, b + 64, nullptr, d.a3, R, N, sms, st);
+  return e;
 }
 
 cudaError_t dn_apply(const void* params, bool bf16, const float2* H, int R, int N, float* work,
                      float2* Hout, int sms, cudaStream_t st) {
   const DnWork d = dn_work(work, R, N);
-  dn_prepare_kernel<<<R, 256, 0, st>>>(H, nullptr, N, d.x0, nullptr, d.rms);
-  if (bf16) forward(static_cast<const __nv_bfloat16*>(params), d, R, N, st);
-  else forward(static_cast<const float*>(params), d, R, N, st);
-  const size_t n = static_cast<size_t>(R) * N;
-  const int fg = static_cast<int>((n + 255) / 256 < static_cast<size_t>(sms) * 8 ? (n + 255) / 256 : sms * 8);
-  dn_finish_kernel<<<fg, 256, 0, st>>>(d.y, d.rms, R, N, Hout);
+  if (bf16)
+    dn_setup_kernel<<<kSetupBlocks + R, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(params), d.wt,
+                                                      H, nullptr, N, d.x0, nullptr, d.rms);
+  else
+    dn_setup_kernel<<<kSetupBlocks + R, 256, 0, st>>>(static_cast<const float*>(params), d.wt, H,
+                                                      nullptr, N, d.x0, nullptr, d.rms);
+  const float* b = d.wt + kBias;
+  const cudaError_t e = forward(b, d, R, N, sms, st);
+  if (e != cudaSuccess) return e;
+  DnOutArgs a{};
+  a.in = d.a3;
+  a.wt = d.wt + kFw4;
+  a.bias = b + 96;
+  a.x0 = d.x0;
+  a.rms = d.rms;
+  a.Hout = Hout;
+  a.N = N;
+  dn_conv_out_kernel<false><<<R * (N / kDnPos), 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -1417,31 +1804,54 @@ cudaError_t dn_ls_tc(const KParams& k, const void* params_bf16, int n_frames, fl
 }
 
 cudaError_t dn_grad(const float* P, const float2* Hls, const float2* Ht, int R, int N, float* work,
-                    float* grad, float* loss, cudaStream_t st) {
+                    float* grad, float* loss, int sms, cudaStream_t st) {
   const DnWork d = dn_work(work, R, N);
-  dn_prepare_kernel<<<R, 256, 0, st>>>(Hls, Ht, N, d.x0, d.tt, d.rms);
-  forward(P, d, R, N, st);
+  cudaError_t e =
+      cudaFuncSetAttribute(dn_wgrad32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwSmem);
+  if (e != cudaSuccess) return e;
+  dn_setup_kernel<<<kSetupBlocks + R, 256, 0, st>>>(P, d.wt, Hls, Ht, N, d.x0, d.tt, d.rms);
+  const float* b = d.wt + kBias;
+  e = forward(b, d, R, N, sms, st);
+  if (e != cudaSuccess) return e;
   const size_t n = static_cast<size_t>(R) * 2 * N;
-  dn_loss_kernel<<<kDnLossBlocks, 256, 0, st>>>(d.y, d.tt, n, d.dy, d.part);
-  dn_loss_final_kernel<<<1, 32, 0, st>>>(d.part, kDnLossBlocks, n, loss);
-  // layer 4: input relu(a3); dy -> g1 = d a3 (masked by a3 > 0)
-  dn_wgrad_kernel<<<dim3(2, 32), kDnGradThreads, 0, st>>>(d.dy, d.a3, 1, 32, 2, R, N, grad + kOffW4,
-                                                          grad + kOffB4);
-  dn_wt_kernel<<<8, 256, 0, st>>>(P + kOffW4, d.wt, 32, 2);
-  conv<2, 32, float>(d.dy, d.wt, nullptr, 0, d.a3, nullptr, d.g1, R, N, st);
-  // layer 3: input relu(a2); g1 -> g2 = d a2
-  dn_wgrad_kernel<<<dim3(32, 32), kDnGradThreads, 0, st>>>(d.g1, d.a2, 1, 32, 32, R, N,
-                                                           grad + kOffW3, grad + kOffB3);
-  dn_wt_kernel<<<20, 256, 0, st>>>(P + kOffW3, d.wt, 32, 32);
-  conv<32, 32, float>(d.g1, d.wt, nullptr, 0, d.a2, nullptr, d.g2, R, N, st);
-  // layer 2: input relu(a1); g2 -> g1 = d a1
-  dn_wgrad_kernel<<<dim3(32, 32), kDnGradThreads, 0, st>>>(d.g2, d.a1, 1, 32, 32, R, N,
-                                                           grad + kOffW2, grad + kOffB2);
-  dn_wt_kernel<<<20, 256, 0, st>>>(P + kOffW2, d.wt, 32, 32);
-  conv<32, 32, float>(d.g2, d.wt, nullptr, 0, d.a1, nullptr, d.g1, R, N, st);
-  // layer 1: input x0
-  dn_wgrad_kernel<<<dim3(32, 2), kDnGradThreads, 0, st>>>(d.g1, d.x0, 0, 2, 32, R, N,
-                                                          grad + kOffW1, grad + kOffB1);
+  const int tiles = R * (N / kDnPos);
+  DnOutArgs o{};
+  o.in = d.a3;
+  o.wt = d.wt + kFw4;
+  o.bias = b + 96;
+  o.x0 = d.x0;
+  o.tt = d.tt;
+  o.dy = d.dy;
+  o.part = d.y;
+  o.inv_n = 2.0f / static_cast<float>(n);
+  o.N = N;
+  dn_conv_out_kernel<true><<<tiles, 256, 0, st>>>(o);
+  // two blocks of the weight-gradient kernels per SM
+  const int parts = wg_blocks(R, N);
+  const int wgb = 2 * sms < parts ? 2 * sms : parts;
+  float* wp3 = d.wp;
+  float* wp2 = wp3 + static_cast<size_t>(parts) * kWgPart;
+  float* sp4 = wp2 + static_cast<size_t>(parts) * kWgPart;
+  float* sp1 = sp4 + static_cast<size_t>(parts) * kSdPart;
+  // layer 3: g3 = conv(dy; W4') masked -> g1; layer 2: g2 -> g2; layer 1: g1 -> g1
+  dn_conv_in_kernel<true><<<tiles, 256, 0, st>>>(d.dy, d.wt + kBw4, nullptr, d.a3, d.g1, N);
+  dn_wgrad32_kernel<<<wgb, kFwThreads, kFwSmem, st>>>(d.g1, d.a2, R, N, wp3);
+  e = conv32<true>(d.g1, d.wt + kBw3, nullptr, d.a2, d.g2, R, N, sms, st);
+  if (e != cudaSuccess) return e;
+  dn_wgrad32_kernel<<<wgb, kFwThreads, kFwSmem, st>>>(d.g2, d.a1, R, N, wp2);
+  e = conv32<true>(d.g2, d.wt + kBw2, nullptr, d.a1, d.g1, R, N, sms, st);
+  if (e != cudaSuccess) return e;
+  dn_side32_kernel<<<dim3(wgb, 2), 256, 0, st>>>(d.dy, d.a3, d.x0, d.g1, R, N, sp4, sp1);
+  DnReduceArgs a;
+  a.l[0] = {wp3, wgb, kWgPart, grad + kOffW3, grad + kOffB3};
+  a.l[1] = {wp2, wgb, kWgPart, grad + kOffW2, grad + kOffB2};
+  a.l[2] = {sp4, wgb, kSdPart, grad + kOffW4, grad + kOffB4};
+  a.l[3] = {sp1, wgb, kSdPart, grad + kOffW1, grad + kOffB1};
+  a.loss_part = d.y;
+  a.loss_n = tiles;
+  a.n = n;
+  a.loss = loss;
+  dn_reduce_kernel<<<kRdBlocks, kRdThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -1503,7 +1913,7 @@ cudaError_t dn_grad_tc(const float* P32, const float2* Hls, const float2* Ht, in
   a.loss_n = tiles;
   a.n = n;
   a.loss = loss;
-  dn_reduce_kernel<<<kRdBlocks, 256, 0, st>>>(a);
+  dn_reduce_kernel<<<kRdBlocks, kRdThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -1567,7 +1977,7 @@ lsas_status lsas_dn_grad(const float* d_params, const float* d_Hls, const float*
   if (s != LSAS_OK) return s;
   if (!d_params || !d_Hls || !d_Htrue || !d_work || !d_grad || !d_loss) return LSAS_ERR_INVALID_ARG;
   if (lsas::dn_grad(d_params, reinterpret_cast<const float2*>(d_Hls),
-                    reinterpret_cast<const float2*>(d_Htrue), R, N, d_work, d_grad, d_loss,
+                    reinterpret_cast<const float2*>(d_Htrue), R, N, d_work, d_grad, d_loss, dn_sms(),
                     static_cast<cudaStream_t>(stream)) != cudaSuccess)
     return LSAS_ERR_CUDA;
   return LSAS_OK;
