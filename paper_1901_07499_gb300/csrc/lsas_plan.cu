@@ -39,11 +39,10 @@ int tc_smem_bytes(int N);
 cudaError_t dn_ls_tc(const KParams& k, const void* params_bf16, int n_frames, float* work,
                      float2* Hout, int* status, int sms, cudaStream_t st);
 size_t dn_work_floats(int R, int N);
-cudaError_t launch_pn(const KParams&, bool fc32, int n_frames, cudaStream_t);
-cudaError_t launch_extract(const KParams&, bool fc32, int n_frames, cudaStream_t);
+cudaError_t launch_pn(const KParams&, bool fc32, int n_frames, int sms, cudaStream_t);
+cudaError_t launch_extract(const KParams&, bool fc32, int n_frames, int sms, cudaStream_t);
 cudaError_t launch_shift(void* buf, int kind, size_t rows, int N, int rowbytes, int sms,
                          cudaStream_t);
-int pn_smem_bytes(int pn_len);
 bool tc_tables(int N, std::vector<uint16_t>& w1, std::vector<uint16_t>& w2,
                std::vector<float2>& tw);
 }  // namespace lsas
@@ -1021,7 +1020,7 @@ lsas_status lsas_pn_sync(lsas_plan p, const void* d_capture, int n_frames, int c
   k.offsets = d_offset;
   k.peaks = d_peak;
   ProfScope prof(p, "lsas_pn_sync", stream);
-  if (launch_pn(k, p->fmt == LSAS_IN_FC32, n_frames, static_cast<cudaStream_t>(stream)) !=
+  if (launch_pn(k, p->fmt == LSAS_IN_FC32, n_frames, p->sms, static_cast<cudaStream_t>(stream)) !=
       cudaSuccess)
     return LSAS_ERR_CUDA;
   return LSAS_OK;
@@ -1042,10 +1041,11 @@ lsas_status lsas_pn_extract(lsas_plan p, const void* d_capture, int n_frames, in
   k.offsets_in = d_offset;
   k.pn_len = p->pn_len;
   k.backoff = backoff;
+  k.nframes = n_frames;
   k.cap_len = capture_len;
   k.Y_out = static_cast<float2*>(d_frames);
   ProfScope prof(p, "lsas_pn_extract", stream);
-  if (launch_extract(k, p->fmt == LSAS_IN_FC32, n_frames, static_cast<cudaStream_t>(stream)) !=
+  if (launch_extract(k, p->fmt == LSAS_IN_FC32, n_frames, p->sms, static_cast<cudaStream_t>(stream)) !=
       cudaSuccess)
     return LSAS_ERR_CUDA;
   return LSAS_OK;
