@@ -138,6 +138,8 @@ lsas_status lsas_estimate(lsas_plan plan, const void* d_in, int n_frames,
  * MRC demodulation of the data symbols with a given channel d_H (Sec. II-C):
  * writes d_bits and, if d_eq is not NULL, the combined symbols z.  d_H may
  * come from lsas_estimate or from any other estimator.  Asynchronous.
+ * Batches are split into antenna shards as by lsas_run_frame (except while
+ * the stream is being captured into a graph: one launch then).
  */
 lsas_status lsas_demodulate(lsas_plan plan, const void* d_in,
                             const float* d_H, int n_frames, uint8_t* d_bits,

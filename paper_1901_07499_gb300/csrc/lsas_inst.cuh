@@ -16,7 +16,10 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
   int threads = Geo<LOG2N>::TW;
   int slot = kind;   // entry of the shared-memory attribute cache below
   if (kind == kKindFrame) {
-    // fused receiver: from aligned sc16 rows, two symbols per step for
+    // fused receiver (the two-symbol kernels in a form of their own for a
+    // given channel: 200 frames of 64 antennas at N = 1024 demodulate in 355 us
+    // there and split, 499 in the one-symbol kernel; 16 frames 50 against 250):
+    // from aligned sc16 rows, two symbols per step for
     // N = 1024 (and N = 256, 512 with enough antennas; per-warp pipelines)
     // and N = 2048 (pipelines of warp pairs), or, opt-in at N = 1024, the
     // second FFT pass on the tensor cores; otherwise one symbol per step: per-warp pipelines up to
@@ -28,9 +31,9 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
         threads = kHyThreads;
         smem = kHySmem;
         slot = 3;
-      } else if (p.twin && p.use_tma && (p.mode == kModeRun || p.mode == kModePartial)) {
-        fn = twin_kernel<LOG2N>;
-        slot = 4;
+      } else if (p.twin && p.use_tma) {
+        fn = p.H_in ? twin_kernel<LOG2N, true> : twin_kernel<LOG2N, false>;
+        slot = p.H_in ? 5 : 4;
         threads = kTwThreads;
         smem = make_twlayout().total;
       } else {
@@ -39,9 +42,9 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
       }
     } else if constexpr ((LOG2N == 8 || LOG2N == 9) && !FC32) {
       // p.twin is set by the plan only with enough antennas at these sizes
-      if (p.twin && p.use_tma && (p.mode == kModeRun || p.mode == kModePartial)) {
-        fn = twin_kernel<LOG2N>;
-        slot = 4;
+      if (p.twin && p.use_tma) {
+        fn = p.H_in ? twin_kernel<LOG2N, true> : twin_kernel<LOG2N, false>;
+        slot = p.H_in ? 5 : 4;
         threads = kTwThreads;
         smem = make_twlayout().total;
       } else {
@@ -52,11 +55,11 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
       fn = warp_kernel<LOG2N, FC32>;
       threads = 32 * wgeo_warps(FC32 ? 8 : 4);
     } else if constexpr (!FC32) {
-      if (p.twin && p.use_tma && (p.mode == kModeRun || p.mode == kModePartial)) {
-        fn = twinpair_kernel<LOG2N>;
+      if (p.twin && p.use_tma) {
+        fn = p.H_in ? twinpair_kernel<LOG2N, true> : twinpair_kernel<LOG2N, false>;
         threads = kTpThreads;
         smem = make_tplayout().total;
-        slot = 4;
+        slot = p.H_in ? 5 : 4;
       } else {
         fn = pair_kernel<LOG2N>;
         threads = kPThreads;
@@ -71,7 +74,7 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
     fn = fft_kernel<LOG2N, FC32>;
   }
   // raise the kernel's dynamic shared memory limit once per device
-  static int limit[5][64] = {};
+  static int limit[6][64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -82,7 +85,7 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
   }
   // group layers (partial mode, small batches): the two-symbol kernel groups
   // the data symbols its own way
-  const int gz = !p.group_z ? 1 : (slot == 4 ? twin_groups(p.D) : p.groups);
+  const int gz = !p.group_z ? 1 : (slot >= 4 ? twin_groups(p.D) : p.groups);
   fn<<<dim3(grid, p.grid_y > 1 ? p.grid_y : 1, gz), threads, smem, st>>>(p);
   return cudaGetLastError();
 }

@@ -46,7 +46,7 @@ constexpr int kMaxThresholds = 15;   // 256-QAM: 16 levels per axis
 struct KParams {
   const void* in;        // [F][M][S][N+CP] samples (sc16 or fc32)
   float2* H_out;         // [F][M][N]
-  const float2* H_in;    // [F][M][N] (demodulate)
+  const float2* H_in;    // [F][M][N] given channel (demodulate), or null: LS estimate
   uint8_t* bits;         // [F][D*N*q/8]
   float2* eq;            // [F][D][N] or null
   float2* Y_out;         // [F][M][S][N] (fft)
@@ -809,10 +809,8 @@ __device__ __forceinline__ void reduce_scatter(float2* v, int alpha) {
 // ------------------------------------------------------- staging pipeline
 
 // Whether the frame kernel transforms the pilot itself (LS estimate) rather
-// than reading a given channel.
-__device__ __forceinline__ bool fft_pilot(const KParams& p) {
-  return p.mode == kModeRun || p.mode == kModePartial;
-}
+// than reading a given channel (whole frames or, kModePartial, a shard).
+__device__ __forceinline__ bool fft_pilot(const KParams& p) { return p.H_in == nullptr; }
 
 // Items per antenna chunk in data-symbol group g: the pilot first (group 0 of
 // the fused modes), then the group's data symbols.

@@ -500,12 +500,12 @@ int tail_shards(lsas_plan p, int nf) {
   return best_shards(p, nf, p->tail_units);
 }
 
-// Frames [f0, f0 + nf) of a lsas_run_frame batch as G antenna shards: the
-// fused kernel's partial mode writes the shards' partial sums and H, the
-// combine kernel forms z and the bits.  Calls on different streams share
+// Frames [f0, f0 + nf) of a batch as G antenna shards: the fused kernel's
+// partial mode writes the shards' partial sums and H (d_Hin null) or reads
+// the given channel d_Hin, the combine kernel forms z and the bits.  Calls on different streams share
 // d_tail: each waits for the previous split's combine.
 lsas_status run_split_tail(lsas_plan p, const void* d_in, int f0, int nf, int G, float* d_H,
-                           uint8_t* d_bits, float* d_eq, cudaStream_t st) {
+                           const float* d_Hin, uint8_t* d_bits, float* d_eq, cudaStream_t st) {
   const size_t in_b = in_bytes_per_frame(p->M, p->N, p->cp, p->S, p->fmt);
   const size_t bits_b = bits_bytes_per_frame(p->N, p->S, p->Q);
   const unsigned char* in = static_cast<const unsigned char*>(d_in) + f0 * in_b;
@@ -516,7 +516,9 @@ lsas_status run_split_tail(lsas_plan p, const void* d_in, int f0, int nf, int G,
   KParams k;
   base_params(p, &k);
   k.in = in;
-  k.H_out = reinterpret_cast<float2*>(d_H + static_cast<size_t>(f0) * p->M * p->N * 2);
+  const size_t h0 = static_cast<size_t>(f0) * p->M * p->N * 2;
+  if (d_Hin) k.H_in = reinterpret_cast<const float2*>(d_Hin + h0);
+  else k.H_out = reinterpret_cast<float2*>(d_H + h0);
   k.P_out = reinterpret_cast<float2*>(P);
   k.E_out = E;
   k.M = p->M / G;
@@ -547,6 +549,31 @@ lsas_status run_split_tail(lsas_plan p, const void* d_in, int f0, int nf, int G,
   }
   if (cudaEventRecord(p->tail_ev, st) != cudaSuccess) s = LSAS_ERR_CUDA;
   return s;
+}
+
+// A batch through the fused receiver, with its own LS estimate (writes d_H,
+// d_Hin null) or a given channel d_Hin: whole waves of blocks one frame per
+// block, the frames after them possibly split into antenna shards
+// (tail_shards).
+lsas_status run_batch(lsas_plan p, const void* d_in, int n_frames, float* d_H, const float* d_Hin,
+                      uint8_t* d_bits, float* d_eq, cudaStream_t st) {
+  const int mode = d_Hin ? kModeDemod : kModeRun;
+  const int full = (n_frames / p->sms) * p->sms;
+  int G = tail_shards(p, n_frames - full);
+  if (G > 1 && d_Hin) {
+    // a demodulation recorded into a graph stays one launch: the split orders
+    // itself behind other streams' splits by an event, which a capture may not
+    // wait for
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) return LSAS_ERR_CUDA;
+    if (cap != cudaStreamCaptureStatusNone) G = 1;
+  }
+  if (G == 1) return launch_frame(p, d_in, n_frames, d_H, d_Hin, d_bits, d_eq, mode, st);
+  if (full > 0) {
+    const lsas_status s = launch_frame(p, d_in, full, d_H, d_Hin, d_bits, d_eq, mode, st);
+    if (s != LSAS_OK) return s;
+  }
+  return run_split_tail(p, d_in, full, n_frames - full, G, d_H, d_Hin, d_bits, d_eq, st);
 }
 
 }  // namespace
@@ -823,8 +850,7 @@ lsas_status lsas_demodulate(lsas_plan p, const void* d_in, const float* d_H, int
   if (!d_in || !d_H || !d_bits) return LSAS_ERR_INVALID_ARG;
   if (set_device(p) != LSAS_OK) return LSAS_ERR_CUDA;
   ProfScope prof(p, "lsas_demodulate", stream);
-  return launch_frame(p, d_in, n_frames, nullptr, d_H, d_bits, d_eq, kModeDemod,
-                      static_cast<cudaStream_t>(stream));
+  return run_batch(p, d_in, n_frames, nullptr, d_H, d_bits, d_eq, static_cast<cudaStream_t>(stream));
 }
 
 lsas_status lsas_run_frame(lsas_plan p, const void* d_in, int n_frames, float* d_H,
@@ -836,17 +862,7 @@ lsas_status lsas_run_frame(lsas_plan p, const void* d_in, int n_frames, float* d
   if (!d_in || !d_H || !d_bits) return LSAS_ERR_INVALID_ARG;
   if (set_device(p) != LSAS_OK) return LSAS_ERR_CUDA;
   ProfScope prof(p, "lsas_run_frame", stream);
-  const cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // whole waves of blocks run one frame per block; the frames after them may
-  // run split into antenna shards (tail_shards)
-  const int full = (n_frames / p->sms) * p->sms;
-  const int G = tail_shards(p, n_frames - full);
-  if (G == 1) return launch_frame(p, d_in, n_frames, d_H, nullptr, d_bits, d_eq, kModeRun, st);
-  if (full > 0) {
-    s = launch_frame(p, d_in, full, d_H, nullptr, d_bits, d_eq, kModeRun, st);
-    if (s != LSAS_OK) return s;
-  }
-  return run_split_tail(p, d_in, full, n_frames - full, G, d_H, d_bits, d_eq, st);
+  return run_batch(p, d_in, n_frames, d_H, nullptr, d_bits, d_eq, static_cast<cudaStream_t>(stream));
 }
 
 lsas_status lsas_mrc_partial(lsas_plan p, const void* d_in, int n_frames, int m_begin,
@@ -963,7 +979,7 @@ lsas_status lsas_run_frame_refined(lsas_plan p, const void* d_in, int n_frames,
   if (dn_ls_tc(k, d_params_bf16, n_frames, d_work, reinterpret_cast<float2*>(d_H), d_status,
                p->sms, st) != cudaSuccess)
     return LSAS_ERR_CUDA;
-  return launch_frame(p, d_in, n_frames, nullptr, d_H, d_bits, d_eq, kModeDemod, st);
+  return run_batch(p, d_in, n_frames, nullptr, d_H, d_bits, d_eq, st);
 }
 
 lsas_status lsas_receive_y(lsas_plan p, const float* d_Y, int n_frames, float* d_H,

@@ -28,6 +28,9 @@
 //     data symbol: P += conj(H) Y per subcarrier in the warp's tensor-memory
 //     columns (the MRC numerator, Sec. II-C); for two data symbols as four
 //     packed FMAs per subcarrier on their interleaved columns.
+// With a given channel (GIVEN: demodulation) there is no pilot step: the
+// channel is read per antenna and data-symbol group, and group 0 adds its
+// energy.
 // The second pass is radix L: it reads column jt of the exchange (32 rows of
 // L points per team) and takes 32 / L DFTs of L points per symbol.
 // Data-symbol groups: the pilot with the first three data symbols, then four
@@ -318,7 +321,7 @@ __device__ __forceinline__ int twin_block_col(int it, bool pilot, bool* pair, in
   return pilot ? (ip == 0 ? 0 : 64 + 128 * (ip - 1)) : 128 * ip;
 }
 
-template <int LOG2N>
+template <int LOG2N, bool GIVEN>
 __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
   static_assert(LOG2N >= 7 && LOG2N <= 10, "the two-symbol kernel covers N = 128 .. 1024");
   constexpr int N = 1 << LOG2N;
@@ -386,7 +389,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
   for (int g = g_lo; g < g_hi; ++g) {
     const int d0 = g == 0 ? 0 : kTwDg0 + (g - 1) * kTwDg;
     const int nd = min(g == 0 ? kTwDg0 : kTwDg, p.D - d0);
-    const bool pilot_here = g == 0 || p.group_z;
+    const bool pilot_here = !GIVEN && (g == 0 || p.group_z);
     const bool energy_here = g == 0;
     const int items = nd + (pilot_here ? 1 : 0);
     const int npairs = (items + 1) / 2;
@@ -427,11 +430,21 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
       const size_t hrow = (static_cast<size_t>(f) * p.Mtot + p.m0 + blockIdx.y * p.shard_y + m) * N;
       float2 h[32];
       if (!pilot_here) {
-        // channel written in group 0 (zero for a team without an antenna, so
-        // that its stale rows add nothing)
+        // channel written in group 0, or given (zero for a team without an
+        // antenna, so that its stale rows add nothing)
+        const float2* Hs = GIVEN ? p.H_in : p.H_out;
 #pragma unroll
         for (int e = 0; e < 32; ++e)
-          h[e] = valid ? p.H_out[hrow + bin_of<LOG2N>(jt, e)] : make_float2(0.f, 0.f);
+          h[e] = valid ? Hs[hrow + bin_of<LOG2N>(jt, e)] : make_float2(0.f, 0.f);
+        if (GIVEN && energy_here) {
+          float acc[OWN];
+          tmem_wait_st();
+          TmE::ld(tE, acc);
+          tmem_wait_ld();
+#pragma unroll
+          for (int e = 0; e < 32; ++e) acc[e] = fmaf(h[e].x, h[e].x, fmaf(h[e].y, h[e].y, acc[e]));
+          TmE::st(tE, acc);
+        }
       }
       for (int ip = 0; ip < npairs; ++ip) {
         float2 re[32], im[32];

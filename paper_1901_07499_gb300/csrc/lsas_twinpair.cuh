@@ -120,7 +120,7 @@ __device__ __forceinline__ void tp_twiddle(float2& xr, float2& xi, float2 w) {
   xi = i;
 }
 
-template <int LOG2N>
+template <int LOG2N, bool GIVEN>
 __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p) {
   static_assert(LOG2N == 11, "the two-symbol pair kernel is written for N = 2048");
   constexpr int N = 1 << LOG2N;
@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
   for (int g = g_lo; g < g_hi; ++g) {
     const int d0 = g == 0 ? 0 : kTwDg0 + (g - 1) * kTwDg;
     const int nd = min(g == 0 ? kTwDg0 : kTwDg, p.D - d0);
-    const bool pilot_here = g == 0 || p.group_z;
+    const bool pilot_here = !GIVEN && (g == 0 || p.group_z);
     const bool energy_here = g == 0;
     const int items = nd + (pilot_here ? 1 : 0);
     const int npairs = (items + 1) / 2;
@@ -221,8 +221,18 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
       const size_t hrow = (static_cast<size_t>(f) * p.Mtot + p.m0 + blockIdx.y * p.shard_y + m) * N;
       float2 h[32];
       if (!pilot_here) {
+        const float2* Hs = GIVEN ? p.H_in : p.H_out;
 #pragma unroll
-        for (int e = 0; e < 32; ++e) h[e] = p.H_out[hrow + bin_of<LOG2N>(jt, e)];
+        for (int e = 0; e < 32; ++e) h[e] = Hs[hrow + bin_of<LOG2N>(jt, e)];
+        if (GIVEN && energy_here) {
+          float acc[OWN];
+          tmem_wait_st();
+          TmE::ld(tE, acc);
+          tmem_wait_ld();
+#pragma unroll
+          for (int e = 0; e < 32; ++e) acc[e] = fmaf(h[e].x, h[e].x, fmaf(h[e].y, h[e].y, acc[e]));
+          TmE::st(tE, acc);
+        }
       }
       for (int ip = 0; ip < npairs; ++ip) {
         float2 re[32], im[32];
