@@ -68,13 +68,25 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
       fn = frame_kernel<LOG2N, FC32>;
       threads = Geo<LOG2N>::T;
     }
-  } else if (kind == kKindEstimate) {
-    fn = estimate_kernel<LOG2N, FC32>;
   } else {
-    fn = fft_kernel<LOG2N, FC32>;
+    // symbol rows to memory: two rows at once where the bulk copies can bring
+    // them (aligned sc16 rows), at most one block per SM
+    bool two_rows = false;
+    if constexpr (LOG2N >= 7 && LOG2N <= 10 && !FC32) two_rows = p.use_tma != 0;
+    if constexpr (LOG2N >= 7 && LOG2N <= 10 && !FC32) {
+      if (two_rows) {
+        fn = kind == kKindEstimate ? twin_rows_kernel<LOG2N, true> : twin_rows_kernel<LOG2N, false>;
+        slot = kind == kKindEstimate ? 6 : 7;
+        threads = kTwThreads;
+        smem = make_twlayout().total;
+        grid = p.rows_grid;
+      }
+    }
+    if (!two_rows)
+      fn = kind == kKindEstimate ? estimate_kernel<LOG2N, FC32> : fft_kernel<LOG2N, FC32>;
   }
   // raise the kernel's dynamic shared memory limit once per device
-  static int limit[6][64] = {};
+  static int limit[8][64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -85,7 +97,7 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
   }
   // group layers (partial mode, small batches): the two-symbol kernel groups
   // the data symbols its own way
-  const int gz = !p.group_z ? 1 : (slot >= 4 ? twin_groups(p.D) : p.groups);
+  const int gz = !p.group_z ? 1 : ((slot == 4 || slot == 5) ? twin_groups(p.D) : p.groups);
   fn<<<dim3(grid, p.grid_y > 1 ? p.grid_y : 1, gz), threads, smem, st>>>(p);
   return cudaGetLastError();
 }

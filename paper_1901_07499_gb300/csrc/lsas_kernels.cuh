@@ -60,6 +60,9 @@ struct KParams {
   int M;                 // antennas this call processes
   int m0, Mtot;          // first of them, antennas per frame in the arrays
   int N, S, cp, pilot_idx, D;
+  long nrows, row_stride;   // row batches (twin_rows_kernel): rows, samples between their
+  long row_off;             //   starts, sample of the first one
+  int rows_grid;            //   blocks
   int shards, nframes;   // combine: partials per frame, frames; tensor-core FFT: rows
   const void* tc_w1;     // tensor-core FFT: 32-point DFT operand images (hi, lo)
   const void* tc_w2;     //   N/32-point DFT operand images (hi, lo)

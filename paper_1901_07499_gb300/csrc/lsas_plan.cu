@@ -34,7 +34,7 @@ cudaError_t launch_n1024(int, bool, const KParams&, int, int, cudaStream_t);
 cudaError_t launch_n2048(int, bool, const KParams&, int, int, cudaStream_t);
 cudaError_t launch_combine(const KParams&, cudaStream_t);
 cudaError_t launch_tcfft(const KParams&, int N, int grid, cudaStream_t);
-cudaError_t launch_yrx(const KParams&, int n_frames, cudaStream_t);
+cudaError_t launch_yrx(const KParams&, int n_frames, int sms, cudaStream_t);
 int tc_smem_bytes(int N);
 cudaError_t dn_ls_tc(const KParams& k, const void* params_bf16, int n_frames, float* work,
                      float2* Hout, int* status, int sms, cudaStream_t st);
@@ -432,6 +432,19 @@ bool tma_ok(lsas_plan p, const void* d_in) {
   return aligned16(d_in) && ((p->N + p->cp) * bps) % 16 == 0 && (p->cp * bps) % 16 == 0;
 }
 
+// Row batch of lsas_fft (every symbol of every antenna) or lsas_estimate (the
+// pilots) for the two-rows-at-once kernel.
+void row_batch(lsas_plan p, int n_frames, bool pilots, KParams* k) {
+  const long sym = p->N + p->cp, ant = static_cast<long>(n_frames) * p->M;
+  k->nrows = pilots ? ant : ant * p->S;
+  k->row_stride = pilots ? sym * p->S : sym;
+  k->row_off = (pilots ? sym * p->pilot_idx : 0) + p->cp;
+  // a step takes 64 / (N / 32) rows; eight warps a block, one block per SM
+  const long per_block = 8L * 2048 / p->N;
+  const long blocks = (k->nrows + per_block - 1) / per_block;
+  k->rows_grid = static_cast<int>(blocks < p->sms ? blocks : p->sms);
+}
+
 lsas_status set_device(lsas_plan p) {
   int cur = -1;
   if (cudaGetDevice(&cur) != cudaSuccess) return LSAS_ERR_CUDA;
@@ -811,6 +824,7 @@ lsas_status lsas_fft(lsas_plan p, const void* d_in, int n_frames, float* d_Y, vo
   k.Y_out = reinterpret_cast<float2*>(d_Y);
   k.nslots = p->geo.fft_slots;
   k.use_tma = tma_ok(p, d_in) ? 1 : 0;
+  row_batch(p, n_frames, false, &k);
   const int grid = n_frames * k.chunks;
   ProfScope prof(p, "lsas_fft", stream);
   if (p->launch(kKindFft, p->fmt == LSAS_IN_FC32, k, grid, p->geo.smem_fft,
@@ -833,6 +847,7 @@ lsas_status lsas_estimate(lsas_plan p, const void* d_in, int n_frames, float* d_
   k.H_out = reinterpret_cast<float2*>(d_H);
   k.mode = kModeEstimate;
   k.use_tma = tma_ok(p, d_in) ? 1 : 0;
+  row_batch(p, n_frames, true, &k);
   const int grid = n_frames * k.chunks;
   ProfScope prof(p, "lsas_estimate", stream);
   if (p->launch(kKindEstimate, p->fmt == LSAS_IN_FC32, k, grid, p->geo.smem_est,
@@ -997,7 +1012,7 @@ lsas_status lsas_receive_y(lsas_plan p, const float* d_Y, int n_frames, float* d
   k.bits = d_bits;
   k.eq = reinterpret_cast<float2*>(d_eq);
   ProfScope prof(p, "lsas_receive_y", stream);
-  if (launch_yrx(k, n_frames, static_cast<cudaStream_t>(stream)) != cudaSuccess)
+  if (launch_yrx(k, n_frames, p->sms, static_cast<cudaStream_t>(stream)) != cudaSuccess)
     return LSAS_ERR_CUDA;
   return LSAS_OK;
 }

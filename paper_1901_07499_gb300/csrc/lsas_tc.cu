@@ -440,62 +440,99 @@ cudaError_t launch_tcfft(const KParams& p, int N, int grid, cudaStream_t st) {
 // ---------------------------------------------------------------- staged receiver
 
 constexpr int kYrxMaxThreads = 128;
-constexpr int kYrxMaxD = 63;
 
 // LS, MRC and demap from transformed symbols Y [F][M][S][N] (unitary): one
-// thread per subcarrier k of one frame, the antenna loop in the thread (the
-// MRC sum over antennas in a fixed order), packed bits through shared memory.
+// thread per subcarrier k of one frame and DG data symbols (blockIdx.y takes
+// the next DG), the antenna loop in the thread (the MRC sum over antennas in a
+// fixed order), packed bits through shared memory.  Bound by reading Y once,
+// so a thread keeps its DG sums in registers and has the DG + 1 loads of an
+// antenna, and the next one's, in flight; the energy is formed by every group,
+// H written by the first.  120 frames of 48 antennas, 13 data symbols, N = 512:
+// 67 us (floor 54); with the sums of up to 63 symbols in local memory, 309.
+template <int DG>
 __global__ void __launch_bounds__(kYrxMaxThreads) yrx_kernel(const KParams p) {
-  __shared__ uint8_t codes[kYrxMaxD * kYrxMaxThreads];
+  __shared__ uint8_t codes[DG * kYrxMaxThreads];
   const int N = p.N;
   const int T = blockDim.x;   // min(N, 128) subcarriers per block
   const int per = N / T;
   const int f = blockIdx.x / per;
   const int k0 = (blockIdx.x % per) * T;
   const int k = k0 + threadIdx.x;
+  const int d0 = blockIdx.y * DG;
+  const int nd = min(DG, p.D - d0);
   const float2 xs = p.xinv[k];                       // conj(X)/|X|^2/sqrt(N)
   const float sq = 1.0f / p.inv_sqrtN;
   const float2 xi = make_float2(xs.x * sq, xs.y * sq);   // conj(X)/|X|^2
-  float2 P[kYrxMaxD];
-  for (int d = 0; d < p.D; ++d) P[d] = make_float2(0.f, 0.f);
+  const size_t ant = static_cast<size_t>(p.S) * N;   // Y of one antenna
+  const float2* Y = p.Y_out + static_cast<size_t>(f) * p.M * ant + k;
+  const float2* Yp = Y + static_cast<size_t>(p.pilot_idx) * N;
+  float2* H = p.H_out + static_cast<size_t>(f) * p.M * N + k;
+  // data symbols before and after the pilot: symbol d0 + d at Y + (d0 + d + (d >= split)) N
+  const int split = p.pilot_idx - d0;
+  const float2* Yd = Y + static_cast<size_t>(d0) * N;
+  float2 P[DG];
+#pragma unroll
+  for (int d = 0; d < DG; ++d) P[d] = make_float2(0.f, 0.f);
   float E = 0.f;
+  float2 yn[DG], pn = make_float2(0.f, 0.f);   // the next antenna's loads
+  auto fetch = [&](int m) {
+    pn = __ldg(Yp + m * ant);
+#pragma unroll
+    for (int d = 0; d < DG; ++d)
+      if (d < nd) yn[d] = __ldg(Yd + m * ant + static_cast<size_t>(d >= split ? d + 1 : d) * N);
+  };
+  fetch(0);
   for (int m = 0; m < p.M; ++m) {
-    const float2* Ym = p.Y_out + (static_cast<size_t>(f) * p.M + m) * p.S * N;
-    const float2 h = cmul(Ym[static_cast<size_t>(p.pilot_idx) * N + k], xi);
-    p.H_out[(static_cast<size_t>(f) * p.M + m) * N + k] = h;
+    const float2 yp = pn;
+    float2 y[DG];
+#pragma unroll
+    for (int d = 0; d < DG; ++d) y[d] = yn[d];
+    if (m + 1 < p.M) fetch(m + 1);
+    const float2 h = cmul(yp, xi);
+    if (d0 == 0) H[static_cast<size_t>(m) * N] = h;
     E = fmaf(h.x, h.x, fmaf(h.y, h.y, E));
-    for (int d = 0; d < p.D; ++d) {
-      const int s = d < p.pilot_idx ? d : d + 1;
-      const float2 y = Ym[static_cast<size_t>(s) * N + k];
-      P[d].x = fmaf(h.x, y.x, fmaf(h.y, y.y, P[d].x));
-      P[d].y = fmaf(h.x, y.y, fmaf(-h.y, y.x, P[d].y));
+#pragma unroll
+    for (int d = 0; d < DG; ++d) {
+      P[d].x = fmaf(h.x, y[d].x, fmaf(h.y, y[d].y, P[d].x));
+      P[d].y = fmaf(h.x, y[d].y, fmaf(-h.y, y[d].x, P[d].y));
     }
   }
   const bool ok = (E > 0.f) && (E <= FLT_MAX);
   if (!ok) latch(p.status, kStDevice);
   const float ie = ok ? 1.0f / E : 0.f;
-  for (int d = 0; d < p.D; ++d) {
+#pragma unroll
+  for (int d = 0; d < DG; ++d) {
+    if (d >= nd) break;
     const float2 z = ok ? make_float2(P[d].x * ie, P[d].y * ie) : make_float2(0.f, 0.f);
-    if (p.eq) p.eq[(static_cast<size_t>(f) * p.D + d) * N + k] = z;
+    if (p.eq) p.eq[(static_cast<size_t>(f) * p.D + d0 + d) * N + k] = z;
     uint32_t code = gray(axis_level(z.x, p));
     if (p.axes == 2) code = (code << p.wbits) | gray(axis_level(z.y, p));
     codes[d * T + threadIdx.x] = static_cast<uint8_t>(code);
   }
   __syncthreads();
   const size_t frame_bytes = static_cast<size_t>(p.D) * N * p.q / 8;
-  for (int it = threadIdx.x; it < p.D * (T / 8); it += T) {
+  for (int it = threadIdx.x; it < nd * (T / 8); it += T) {
     const int d = it / (T / 8);
     const int c8 = (it % (T / 8)) * 8;
     uint64_t acc = 0;
     for (int j = 0; j < 8; ++j) acc = (acc << p.q) | codes[d * T + c8 + j];
-    uint8_t* dst = p.bits + f * frame_bytes + (static_cast<size_t>(d) * N + k0 + c8) * p.q / 8;
+    uint8_t* dst = p.bits + f * frame_bytes + (static_cast<size_t>(d0 + d) * N + k0 + c8) * p.q / 8;
     for (int j = 0; j < p.q; ++j) dst[j] = static_cast<uint8_t>(acc >> (8 * (p.q - 1 - j)));
   }
 }
 
-cudaError_t launch_yrx(const KParams& p, int n_frames, cudaStream_t st) {
+cudaError_t launch_yrx(const KParams& p, int n_frames, int sms, cudaStream_t st) {
   const int T = p.N < kYrxMaxThreads ? p.N : kYrxMaxThreads;
-  yrx_kernel<<<n_frames * (p.N / T), T, 0, st>>>(p);
+  const int blocks = n_frames * (p.N / T);
+  // seven symbols a block (70 registers, so seven blocks share an SM; fourteen
+  // in 162 registers left a second wave nearly empty: 105 against 67 us at 120
+  // frames of N = 512, 72 with the registers capped), or four, which re-read
+  // the pilots more often, where seven would leave SMs idle.  Results do not
+  // depend on it.
+  if (p.D <= 4 || static_cast<long>(blocks) * ((p.D + 6) / 7) < 2L * sms)
+    yrx_kernel<4><<<dim3(blocks, (p.D + 3) / 4), T, 0, st>>>(p);
+  else
+    yrx_kernel<7><<<dim3(blocks, (p.D + 6) / 7), T, 0, st>>>(p);
   return cudaGetLastError();
 }
 

@@ -235,6 +235,81 @@ __device__ __forceinline__ void twin_pass2(float2 (&re)[32], float2 (&im)[32]) {
   }
 }
 
+// Both rows of a step: sc16 -> float v + 2^23 + 32768 exactly (sign bits
+// flipped to offset binary, each half placed under the exponent bytes of
+// 2^23; the offset leaves where pass 1 first adds two samples).
+template <int L>
+__device__ __forceinline__ void twin_convert(float2 (&re)[32], float2 (&im)[32], const uint32_t* sa,
+                                             const uint32_t* sb, int jt) {
+#pragma unroll
+  for (int r = 0; r < 32; ++r) {
+    const uint32_t ua = sa[jt + L * r] ^ 0x80008000u;
+    const uint32_t ub = sb[jt + L * r] ^ 0x80008000u;
+    re[r] = make_float2(__uint_as_float(__byte_perm(ua, 0x4b000000u, 0x7610)),
+                        __uint_as_float(__byte_perm(ub, 0x4b000000u, 0x7610)));
+    im[r] = make_float2(__uint_as_float(__byte_perm(ua, 0x4b000000u, 0x7632)),
+                        __uint_as_float(__byte_perm(ub, 0x4b000000u, 0x7632)));
+  }
+}
+
+// The transpose between the passes: one round of 16-byte stores, rows n2 < 16
+// in the slot just read (lo), the others in the exchange region (hi).
+__device__ __forceinline__ void twin_exchange_write(const float2 (&re)[32], const float2 (&im)[32],
+                                                    unsigned char* lo, unsigned char* hi, int lane) {
+  unsigned char* wrow = (lane < 16 ? lo : hi) + (lane & 15) * kTwXRow;
+#pragma unroll
+  for (int r = 0; r < 32; ++r)
+    *reinterpret_cast<float4*>(wrow + 16 * r) = make_float4(re[r].x, re[r].y, im[r].x, im[r].y);
+}
+
+// Row R = lane holds the pass-1 outputs k1 of team R / L, its thread n2 =
+// R % L; this lane reads k1 = jt + L i, n2 = 0 .. L - 1 of its team into
+// register i L + n2.
+template <int L>
+__device__ __forceinline__ void twin_exchange_read(float2 (&re)[32], float2 (&im)[32],
+                                                   const unsigned char* lo, const unsigned char* hi,
+                                                   int lane) {
+  if constexpr (L == 32) {
+#pragma unroll
+    for (int r = 0; r < 32; ++r) {
+      const float4 v =
+          *reinterpret_cast<const float4*>((r < 16 ? lo : hi) + (r & 15) * kTwXRow + 16 * lane);
+      re[r] = make_float2(v.x, v.y);
+      im[r] = make_float2(v.z, v.w);
+    }
+  } else {
+    // a team's L rows lie in one of the two places (L divides 16)
+    const int team = lane / L, jt = lane % L;
+    const unsigned char* trow = (team * L < 16 ? lo : hi) + ((team * L) & 15) * kTwXRow + 16 * jt;
+#pragma unroll
+    for (int i = 0; i < 32 / L; ++i) {
+#pragma unroll
+      for (int n2 = 0; n2 < L; ++n2) {
+        const float4 v = *reinterpret_cast<const float4*>(trow + n2 * kTwXRow + 16 * L * i);
+        re[i * L + n2] = make_float2(v.x, v.y);
+        im[i * L + n2] = make_float2(v.z, v.w);
+      }
+    }
+  }
+}
+
+// Pass twiddles W_N^(n2 k1) of register i L + n2, k1 = jt + L i.
+template <int L>
+__device__ __forceinline__ void twin_twiddles(float2 (&re)[32], float2 (&im)[32], const float2* tws,
+                                              int jt) {
+#pragma unroll
+  for (int i = 0; i < 32 / L; ++i) {
+#pragma unroll
+    for (int n2 = 1; n2 < L; ++n2) {
+      const float2 w = tws[n2 * 32 + jt + L * i];
+      const int e = i * L + n2;
+      const float2 xr = re[e], xi = im[e];
+      re[e] = __ffma2_rn(xi, f2(-w.y), __fmul2_rn(xr, f2(w.x)));
+      im[e] = __ffma2_rn(xr, f2(w.y), __fmul2_rn(xi, f2(w.x)));
+    }
+  }
+}
+
 // Issue the bulk copies of one step: items ia and ia + 1 of a group (the
 // second may be absent) for the A antennas of chunk c.  Lane h A + t copies
 // the row of symbol item ia + h of antenna c A + t to half h of the slot,
@@ -454,20 +529,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
         const uint32_t* sa =
             reinterpret_cast<const uint32_t*>(stage + slot * slot_bytes) + team * (N + L);
         const uint32_t* sb = sa + kTwHalfB / 4;
-        {
-#pragma unroll
-          for (int r = 0; r < 32; ++r) {
-            // sc16 -> float v + 2^23 + 32768 exactly: sign bits flipped to
-            // offset binary, each half placed under the exponent bytes of
-            // 2^23 (the offset leaves where pass 1 first adds two samples)
-            const uint32_t ua = sa[jt + L * r] ^ 0x80008000u;
-            const uint32_t ub = sb[jt + L * r] ^ 0x80008000u;
-            re[r] = make_float2(__uint_as_float(__byte_perm(ua, 0x4b000000u, 0x7610)),
-                                __uint_as_float(__byte_perm(ub, 0x4b000000u, 0x7610)));
-            im[r] = make_float2(__uint_as_float(__byte_perm(ua, 0x4b000000u, 0x7632)),
-                                __uint_as_float(__byte_perm(ub, 0x4b000000u, 0x7632)));
-          }
-        }
+        twin_convert<L>(re, im, sa, sb, jt);
         unsigned char* const yslot = stage + slot * slot_bytes;
         const uint32_t ybar = smem_u32(&bars[slot]);
         if (++slot == K) {
@@ -480,38 +542,9 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
         // this step's slot): transpose in one round of 16-byte stores, rows
         // n2 < 16 in the slot just read, the others in the exchange region
         __syncwarp();
-        {
-          unsigned char* wrow = (lane < 16 ? yslot : reinterpret_cast<unsigned char*>(ex)) + (lane & 15) * kTwXRow;
-#pragma unroll
-          for (int r = 0; r < 32; ++r)
-            *reinterpret_cast<float4*>(wrow + 16 * r) = make_float4(re[r].x, re[r].y, im[r].x, im[r].y);
-        }
+        twin_exchange_write(re, im, yslot, reinterpret_cast<unsigned char*>(ex), lane);
         __syncwarp();
-        // row R = lane holds the pass-1 outputs k1 of team R / L, its thread
-        // n2 = R % L; this lane reads k1 = jt + L i, n2 = 0 .. L - 1 of its
-        // team into register i L + n2
-        if constexpr (L == 32) {
-#pragma unroll
-          for (int r = 0; r < 32; ++r) {
-            const float4 v = *reinterpret_cast<const float4*>(
-                (r < 16 ? yslot : reinterpret_cast<const unsigned char*>(ex)) + (r & 15) * kTwXRow + 16 * lane);
-            re[r] = make_float2(v.x, v.y);
-            im[r] = make_float2(v.z, v.w);
-          }
-        } else {
-          // a team's L rows lie in one of the two places (L divides 16)
-          const unsigned char* trow = (team * L < 16 ? yslot : reinterpret_cast<const unsigned char*>(ex)) +
-                                      ((team * L) & 15) * kTwXRow + 16 * jt;
-#pragma unroll
-          for (int i = 0; i < 32 / L; ++i) {
-#pragma unroll
-            for (int n2 = 0; n2 < L; ++n2) {
-              const float4 v = *reinterpret_cast<const float4*>(trow + n2 * kTwXRow + 16 * L * i);
-              re[i * L + n2] = make_float2(v.x, v.y);
-              im[i * L + n2] = make_float2(v.z, v.w);
-            }
-          }
-        }
+        twin_exchange_read<L>(re, im, yslot, reinterpret_cast<const unsigned char*>(ex), lane);
         __syncwarp();
         if (to_issue > 0 && !*abort_flag) {
           ++issued;
@@ -524,18 +557,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
             ++ic;
           }
         }
-        // pass twiddles W_N^(n2 k1) of register i L + n2, k1 = jt + L i
-#pragma unroll
-        for (int i = 0; i < 32 / L; ++i) {
-#pragma unroll
-          for (int n2 = 1; n2 < L; ++n2) {
-            const float2 w = tws[n2 * 32 + jt + L * i];
-            const int e = i * L + n2;
-            const float2 xr = re[e], xi = im[e];
-            re[e] = __ffma2_rn(xi, f2(-w.y), __fmul2_rn(xr, f2(w.x)));
-            im[e] = __ffma2_rn(xr, f2(w.y), __fmul2_rn(xi, f2(w.x)));
-          }
-        }
+        twin_twiddles<L>(re, im, tws, jt);
         // pass 2: radix-L DFTs over n2; register e holds bin bin_of(jt, e)
         twin_pass2<L>(re, im);
         const int ia = 2 * ip;
@@ -733,6 +755,111 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
   __syncthreads();
   tmem_fence_after();
   if (warp == 0) tmem_dealloc(*tmem_base, kWTmemCols);
+}
+
+// Transform of a batch of symbol rows (lsas_fft, lsas_estimate): row r of
+// p.nframes rows starts at sample r * p.row_stride + p.row_off and its N bins
+// go to out + r N, scaled to the unitary transform (every symbol of every
+// antenna) or as the LS estimate H = Y conj(X) / |X|^2 (EST: the pilots).
+// Bound by memory once the FFTs run at twin_kernel's rate (8 bytes out and 4
+// in per sample).  The same warp pipelines and two-rows-at-once arithmetic as
+// twin_kernel, but a step's 2 A rows are simply consecutive rows, and the
+// blocks (one per SM) walk the steps with nothing to hand over between them.
+// fft_kernel and estimate_kernel, whose blocks put three barriers in every
+// symbol or pay their set-up for one, stay for the rows this kernel does not
+// take (float or unaligned samples, N = 64 and 2048).  120 frames of 48
+// antennas, 14 symbols, N = 512: FFT 127 -> 82 us (floor 73); the pilots of 200
+// frames of 64 antennas, N = 1024: 40.5 -> 29 us (floor 23).
+template <int LOG2N, bool EST>
+__global__ void __launch_bounds__(kTwThreads, 1) twin_rows_kernel(const KParams p) {
+  constexpr int N = 1 << LOG2N, L = N / 32, A = 32 / L, K = kTwSlots;
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int team = lane / L, jt = lane % L;
+  const TwLayout lay = make_twlayout();
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem) + warp * kMaxSlots;
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kWAbort);
+  float2* tws = reinterpret_cast<float2*>(smem + lay.tw_off);
+  unsigned char* stage = smem + lay.warp_off + warp * lay.warp_bytes;
+  unsigned char* ex = stage + lay.stage_bytes;
+  for (int i = threadIdx.x; i < N; i += kTwThreads) tws[i] = __ldg(p.twP + i);
+  if (threadIdx.x == 0) *abort_flag = 0;
+  if (lane == 0) {
+    for (int s = 0; s < K; ++s) mbar_init(smem_u32(&bars[s]), 1);
+    fence_mbar_init();
+  }
+  __syncthreads();
+  const uint64_t pol = evict_first_policy();
+  const long rows = p.nrows, steps = (rows + 2 * A - 1) / (2 * A);
+  const long stride = static_cast<long>(gridDim.x) * kTwWarps;
+  const long first = static_cast<long>(warp) * gridDim.x + blockIdx.x;
+  const uint32_t* in = static_cast<const uint32_t*>(p.in) + p.row_off;
+  // lane h A + t copies row 2 A step + h A + t to team t's place in half h
+  auto issue = [&](long step, int sl) {
+    const long r0 = step * 2 * A;
+    const int n = static_cast<int>(rows - r0 < 2 * A ? rows - r0 : 2 * A);
+    const uint32_t bar = smem_u32(&bars[sl]);
+    if (lane == 0) mbar_expect_tx(bar, N * 4 * n);
+    __syncwarp();
+    if (lane < n)
+      bulk_load(smem_u32(stage + sl * kTwSlotB + (lane / A) * kTwHalfB + (lane % A) * (N + L) * 4),
+                in + (r0 + lane) * p.row_stride, N * 4, bar, pol);
+  };
+  long next = first;
+  int issued = 0;
+  for (int s = 0; s < K && next < steps; ++s, next += stride, ++issued) issue(next, s);
+  int slot = 0, phase = 0;
+  for (long step = first; step < steps; step += stride) {
+    float2 re[32], im[32];
+    wait_slot(smem_u32(&bars[slot]), phase, abort_flag, p.status);
+    unsigned char* const yslot = stage + slot * kTwSlotB;
+    // a missing row leaves earlier contents of the slot, whose transform is
+    // not written
+    const uint32_t* sa = reinterpret_cast<const uint32_t*>(yslot) + team * (N + L);
+    twin_convert<L>(re, im, sa, sa + kTwHalfB / 4, jt);
+    twin_dft32_sr<true>(re, im);
+    __syncwarp();
+    twin_exchange_write(re, im, yslot, ex, lane);
+    __syncwarp();
+    twin_exchange_read<L>(re, im, yslot, ex, lane);
+    __syncwarp();
+    if (next < steps && !*abort_flag) {
+      fence_proxy_async();
+      issue(next, slot);
+      next += stride;
+      ++issued;
+    }
+    if (++slot == K) {
+      slot = 0;
+      phase ^= 1;
+    }
+    twin_twiddles<L>(re, im, tws, jt);
+    twin_pass2<L>(re, im);
+    const long ra = step * 2 * A + team, rb = ra + A;
+    float2* oa = (EST ? p.H_out : p.Y_out) + ra * N;
+    float2* ob = (EST ? p.H_out : p.Y_out) + rb * N;
+    const bool va = ra < rows, vb = rb < rows;
+#pragma unroll
+    for (int e = 0; e < 32; ++e) {
+      const int k = bin_of<LOG2N>(jt, e);
+      if constexpr (EST) {
+        const float2 w = __ldg(p.xinv + k);
+        if (va) oa[k] = cmul(make_float2(re[e].x, im[e].x), w);
+        if (vb) ob[k] = cmul(make_float2(re[e].y, im[e].y), w);
+      } else {
+        if (va) oa[k] = make_float2(re[e].x * p.inv_sqrtN, im[e].x * p.inv_sqrtN);
+        if (vb) ob[k] = make_float2(re[e].y * p.inv_sqrtN, im[e].y * p.inv_sqrtN);
+      }
+    }
+  }
+  if (lane == 0 && *abort_flag) {
+    // a wait gave up: the last copy issued into each slot gets a bounded
+    // chance to land before the block's shared memory is released
+    for (int s = 0; s < K && s < issued; ++s) {
+      const int last = issued - 1 - ((issued - 1 - s) % K);
+      (void)mbar_wait_bounded(smem_u32(&bars[last % K]), (last / K) & 1);
+    }
+  }
 }
 
 #endif  // __CUDACC__
