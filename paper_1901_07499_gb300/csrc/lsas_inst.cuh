@@ -10,6 +10,46 @@
 
 namespace lsas {
 
+// warp_kernel: the largest number of data symbols and pilots any warp of a
+// block transforms for nd data symbols of `chunks` antenna chunks, with its
+// pairs cut evenly over the warps (share) or as whole chunks.
+inline int warp_steps_as(int chunks, int nd, bool share) {
+  constexpr int NW = wgeo_warps(4);
+  int most = 0;
+  for (int w = 0; w < NW; ++w) {
+    const int lo = w * chunks * nd / NW, hi = (w + 1) * chunks * nd / NW;
+    const int whole = w < chunks ? (chunks - 1 - w) / NW + 1 : 0;
+    const int n = share ? (hi > lo ? hi - lo + (hi - 1) / nd - lo / nd + 1 : 0) : whole * (nd + 1);
+    most = n > most ? n : most;
+  }
+  return most;
+}
+// Cut evenly only where the chunks leave warps idle (no warp then holds two
+// chunks' sums of one symbol) and it saves steps.
+inline int warp_share(int chunks, int nd) {
+  return chunks < wgeo_warps(4) && warp_steps_as(chunks, nd, true) < warp_steps_as(chunks, nd, false) ? 1 : 0;
+}
+
+// Forms of the two-symbol kernels: the channel given or estimated, and, at
+// N <= 1024, whole frames or partial sums.  Compile-time, since these kernels
+// are sensitive to what else they carry: with the grid layers' arithmetic in
+// the whole-frame kernel the scale workload took 1524 us instead of 1519.  (At
+// N = 2048 the opposite: 3566 us with the partial form in the same kernel,
+// 3658 without.)
+inline int two_symbol_form(const KParams& p) {
+  return (p.H_in ? 1 : 0) + (p.mode == kModePartial ? 2 : 0);
+}
+template <int LOG2N>
+static auto two_symbol_kernel(const KParams& p) -> void (*)(const KParams) {
+  if constexpr (LOG2N == 11) {
+    return p.H_in ? twinpair_kernel<LOG2N, true> : twinpair_kernel<LOG2N, false>;
+  } else {
+    void (*const k[4])(const KParams) = {twin_kernel<LOG2N, false, false>, twin_kernel<LOG2N, true, false>,
+                                         twin_kernel<LOG2N, false, true>, twin_kernel<LOG2N, true, true>};
+    return k[two_symbol_form(p)];
+  }
+}
+
 template <int LOG2N, bool FC32>
 static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cudaStream_t st) {
   void (*fn)(const KParams) = nullptr;
@@ -26,14 +66,14 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
     // N = 1024, pipelines of warp pairs for N = 2048 from sc16 rows and the
     // warp-specialised producer/consumer kernel for N = 2048 from fc32 rows
     if constexpr (LOG2N == 10 && !FC32) {
-      if (p.hybrid && p.use_tma) {
+      if (p.hybrid && p.use_tma == 1) {
         fn = hyb_kernel<false>;
         threads = kHyThreads;
         smem = kHySmem;
         slot = 3;
-      } else if (p.twin && p.use_tma) {
-        fn = p.H_in ? twin_kernel<LOG2N, true> : twin_kernel<LOG2N, false>;
-        slot = p.H_in ? 5 : 4;
+      } else if (p.twin && p.use_tma == 1) {
+        fn = two_symbol_kernel<LOG2N>(p);
+        slot = 4 + two_symbol_form(p);
         threads = kTwThreads;
         smem = make_twlayout().total;
       } else {
@@ -42,9 +82,9 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
       }
     } else if constexpr ((LOG2N == 8 || LOG2N == 9) && !FC32) {
       // p.twin is set by the plan only with enough antennas at these sizes
-      if (p.twin && p.use_tma) {
-        fn = p.H_in ? twin_kernel<LOG2N, true> : twin_kernel<LOG2N, false>;
-        slot = p.H_in ? 5 : 4;
+      if (p.twin && p.use_tma == 1) {
+        fn = two_symbol_kernel<LOG2N>(p);
+        slot = 4 + two_symbol_form(p);
         threads = kTwThreads;
         smem = make_twlayout().total;
       } else {
@@ -55,11 +95,11 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
       fn = warp_kernel<LOG2N, FC32>;
       threads = 32 * wgeo_warps(FC32 ? 8 : 4);
     } else if constexpr (!FC32) {
-      if (p.twin && p.use_tma) {
-        fn = p.H_in ? twinpair_kernel<LOG2N, true> : twinpair_kernel<LOG2N, false>;
+      if (p.twin && p.use_tma == 1) {
+        fn = two_symbol_kernel<LOG2N>(p);
         threads = kTpThreads;
         smem = make_tplayout().total;
-        slot = p.H_in ? 5 : 4;
+        slot = 4 + two_symbol_form(p);
       } else {
         fn = pair_kernel<LOG2N>;
         threads = kPThreads;
@@ -72,11 +112,11 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
     // symbol rows to memory: two rows at once where the bulk copies can bring
     // them (aligned sc16 rows), at most one block per SM
     bool two_rows = false;
-    if constexpr (LOG2N >= 7 && LOG2N <= 10 && !FC32) two_rows = p.use_tma != 0;
+    if constexpr (LOG2N >= 7 && LOG2N <= 10 && !FC32) two_rows = p.use_tma == 1;
     if constexpr (LOG2N >= 7 && LOG2N <= 10 && !FC32) {
       if (two_rows) {
         fn = kind == kKindEstimate ? twin_rows_kernel<LOG2N, true> : twin_rows_kernel<LOG2N, false>;
-        slot = kind == kKindEstimate ? 6 : 7;
+        slot = kind == kKindEstimate ? 8 : 9;
         threads = kTwThreads;
         smem = make_twlayout().total;
         grid = p.rows_grid;
@@ -85,8 +125,37 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
     if (!two_rows)
       fn = kind == kKindEstimate ? estimate_kernel<LOG2N, FC32> : fft_kernel<LOG2N, FC32>;
   }
+  // rows staged from the boundary before them: the per-warp kernel only
+  KParams q = p;
+  q.nf = q.full = grid;
+  q.zsplit = 1;
+  if constexpr (LOG2N <= 10) {
+    if (q.use_tma == 2 && fn != warp_kernel<LOG2N, FC32>) q.use_tma = 0;
+    if (fn == warp_kernel<LOG2N, FC32>) {
+      q.share = warp_share(q.chunks, q.dg < q.D ? q.dg : q.D);
+      if (q.mode == kModeRun || q.mode == kModeDemod) {
+        // symbol-split the frames after the last whole wave where the parts
+        // fit one data-symbol group and fewer steps a warp
+        const int tail = q.nf % q.sms;
+        int best = warp_steps_as(q.chunks, q.D, q.share != 0);
+        for (int z = 2; z <= q.D && static_cast<long>(tail) * z <= q.sms; ++z) {
+          const int part = (q.D + z - 1) / z;
+          const int steps = warp_steps_as(q.chunks, part, q.share != 0);
+          if (tail == 0 || part > q.dg || steps >= best) continue;
+          best = steps;
+          q.zsplit = z;
+        }
+        if (q.zsplit > 1) {
+          q.full = q.nf - tail;
+          grid = q.full + tail * q.zsplit;
+        }
+      }
+    }
+  } else {
+    if (q.use_tma == 2) q.use_tma = 0;
+  }
   // raise the kernel's dynamic shared memory limit once per device
-  static int limit[8][64] = {};
+  static int limit[10][64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -95,10 +164,8 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) limit[slot][dev] = smem;
   }
-  // group layers (partial mode, small batches): the two-symbol kernel groups
-  // the data symbols its own way
-  const int gz = !p.group_z ? 1 : ((slot == 4 || slot == 5) ? twin_groups(p.D) : p.groups);
-  fn<<<dim3(grid, p.grid_y > 1 ? p.grid_y : 1, gz), threads, smem, st>>>(p);
+  const int gz = q.group_z > 0 ? q.group_z : 1;
+  fn<<<dim3(grid, p.grid_y > 1 ? p.grid_y : 1, gz), threads, smem, st>>>(q);
   return cudaGetLastError();
 }
 

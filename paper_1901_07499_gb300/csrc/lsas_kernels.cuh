@@ -55,25 +55,37 @@ struct KParams {
   int* status;           // latched device status
   float2* P_out;         // [F][D][N] shard partial sum conj(H) Y (partial)
   float* E_out;          // [F][N]    shard partial sum |H|^2 (partial)
-  const float2* P_in;    // [G][F][D][N] partials to combine
-  const float* E_in;     // [G][F][N]
   int M;                 // antennas this call processes
   int m0, Mtot;          // first of them, antennas per frame in the arrays
   int N, S, cp, pilot_idx, D;
-  long nrows, row_stride;   // row batches (twin_rows_kernel): rows, samples between their
-  long row_off;             //   starts, sample of the first one
-  int rows_grid;            //   blocks
-  int shards, nframes;   // combine: partials per frame, frames; tensor-core FFT: rows
-  const void* tc_w1;     // tensor-core FFT: 32-point DFT operand images (hi, lo)
-  const void* tc_w2;     //   N/32-point DFT operand images (hi, lo)
-  const float2* tc_tw;   //   inter-stage twiddles W_N^(n2 k1), [n2][k1]
-  int terms;             //   1: plain operands; 3: hi+lo split operands
-  int tc_bf16;           //   0: fp16 operands; 1: bf16
-  const float* pn;       // packet detection: PN chips (real), pn_len of them
-  int pn_len, cap_len, window, backoff;
-  int* offsets;          //   per frame: detected preamble start (out)
-  float* peaks;          //   per frame: correlation power at it (out, nullable)
-  const int* offsets_in; //   per frame: preamble start (extraction)
+  int nframes;           // combine, extraction: frames; tensor-core FFT: rows
+  // what only one kind of kernel reads shares its place
+  union {
+    struct {                 // combine
+      const float2* P_in;    // [G][F][D][N] partials to combine
+      const float* E_in;     // [G][F][N]
+      int shards;            // partials per frame
+    };
+    struct {                 // tensor-core FFT (tc_w1 also hyb_kernel)
+      const void* tc_w1;     // 32-point DFT operand images (hi, lo)
+      const void* tc_w2;     // N/32-point DFT operand images (hi, lo)
+      const float2* tc_tw;   // inter-stage twiddles W_N^(n2 k1), [n2][k1]
+      int terms;             // 1: plain operands; 3: hi+lo split operands
+      int tc_bf16;           // 0: fp16 operands; 1: bf16
+    };
+    struct {                 // row batches (twin_rows_kernel)
+      long nrows, row_stride;   // rows, samples between their starts
+      long row_off;          // sample of the first one
+      int rows_grid;         // blocks
+    };
+    struct {                 // packet detection and extraction
+      const float* pn;       // PN chips (real), pn_len of them
+      int pn_len, cap_len, window, backoff;
+      int* offsets;          // per frame: detected preamble start (out)
+      float* peaks;          // per frame: correlation power at it (out, nullable)
+      const int* offsets_in; // per frame: preamble start (extraction)
+    };
+  };
   int fault;             // test hook: 1 = block 0 waits for 16 bytes that never come
   int hybrid;            // N = 1024, sc16, staged: second FFT pass on the tensor cores
   int twin;              // N = 1024, sc16, staged: two symbols per step (twin_kernel)
@@ -81,12 +93,17 @@ struct KParams {
                          // blockIdx.y (its first antenna is m0 + blockIdx.y * shard_y, its
                          // partials start at shard blockIdx.y of [G][F][...]); 0 otherwise
   int grid_y;            // grid rows (shards) of the launch; 0 or 1 for a 1-D grid
-  int group_z;           // partial mode of the per-warp kernel: 1 = grid z index g runs
-                         // data-symbol group g alone (groups grid layers); 0 otherwise
+  int group_z;           // partial mode: grid layers, layer z runs the z-th even part of the
+                         // data symbols alone (hyb_kernel: data-symbol group z); 0: none
   int chunks;            // ceil(M / A)
   int groups, dg;        // data-symbol groups per frame, data symbols per group
   int mode;              // kModeDemod, kModeRun or kModePartial (frame_kernel)
-  int use_tma, nslots;
+  int use_tma, nslots;   // use_tma: 0 plain loads, 1 bulk copies of the rows, 2 (warp_kernel)
+                         // bulk copies from the 16-byte boundary before each row
+  int share;             // warp_kernel: 1 = the (chunk, data symbol) pairs cut evenly over warps
+  int nf, sms;           // frames of the launch, SMs of the device
+  int full, zsplit;      // warp_kernel: frames that are one block each; blocks of each other
+                         // frame (an even part of the data symbols each)
   int tmem_cols, tmem_cth;   // TMEM allocation (columns) and columns per thread
   int q, wbits, axes, nthr;
   float inv_sqrtN;

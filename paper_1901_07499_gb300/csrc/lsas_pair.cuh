@@ -134,17 +134,17 @@ __global__ void __launch_bounds__(kPThreads, 1) pair_kernel(const KParams p) {
   int issued = 0;  // steps whose copies this pair has issued (issuer only)
   int slot = 0;    // ring slot of the next step to consume ...
   int phase = 0;   // ... and its mbarrier phase
-  // one data-symbol group per grid z index (partial mode, small batches):
-  // every group's block transforms the pilot itself; group 0 alone writes H
-  // and the channel energy
-  const int g_lo = p.group_z ? static_cast<int>(blockIdx.z) : 0;
-  const int g_hi = p.group_z ? g_lo + 1 : p.groups;
-  for (int g = g_lo; g < g_hi; ++g) {
-    const int nd = min(p.dg, p.D - g * p.dg);
-    const int d0 = g * p.dg;
-    const bool pilot_here = fft_pilot(p) && (g == 0 || p.group_z);
+  // one part of the data symbols per grid z index (partial mode, small
+  // batches): every part's block transforms the pilot itself; part 0 alone
+  // writes H and the channel energy
+  const int d_begin = p.group_z ? static_cast<int>(blockIdx.z) * p.D / p.group_z : 0;
+  const int d_end = p.group_z ? (static_cast<int>(blockIdx.z) + 1) * p.D / p.group_z : p.D;
+  for (int d0 = d_begin; d0 < d_end; d0 += p.dg) {
+    const int nd = min(p.dg, d_end - d0);
+    const bool first = d0 == d_begin;
+    const bool pilot_here = fft_pilot(p) && first;
     const int items = nd + (pilot_here ? 1 : 0);
-    if (g == g_lo) {
+    if (first) {
 #pragma unroll
       for (int q0 = 0; q0 < OWN; q0 += 16) Tmem<16>::st(tE + q0, zero);
     }
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kPThreads, 1) pair_kernel(const KParams p) {
                   kRow, bar, pol);
         // test hook: the first staging phase of block 0 also waits for 16
         // bytes that no copy delivers, so its bounded wait runs out
-        if (p.fault == 1 && blockIdx.x == 0 && q == 0 && g == g_lo && s == 0)
+        if (p.fault == 1 && blockIdx.x == 0 && q == 0 && first && s == 0)
           mbar_expect_tx_only(bar, 16);
         ++issued;
         is = (is + 1 == K) ? 0 : is + 1;
@@ -184,11 +184,11 @@ __global__ void __launch_bounds__(kPThreads, 1) pair_kernel(const KParams p) {
       const size_t hrow = (static_cast<size_t>(f) * p.Mtot + p.m0 + blockIdx.y * p.shard_y + m) * N;
       float2 h[32];
       if (!pilot_here) {
-        // channel from memory: given (demodulate) or written in group 0
+        // channel from memory: given (demodulate) or written in the first group
         const float2* Hs = fft_pilot(p) ? p.H_out : p.H_in;
 #pragma unroll
         for (int e = 0; e < 32; ++e) h[e] = Hs[hrow + bin_of<LOG2N>(jt, e)];
-        if (g == 0) {
+        if (first) {
           float acc[OWN];
           tmem_wait_st();
           TmE::ld(tE, acc);
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kPThreads, 1) pair_kernel(const KParams p) {
           for (int e = 0; e < 32; ++e) {
             const int k = bin_of<LOG2N>(jt, e);
             h[e] = cmul(v[e], __ldg(p.xinv + k));
-            if (g == 0) p.H_out[hrow + k] = h[e];
+            if (d0 == 0) p.H_out[hrow + k] = h[e];
           }
           float acc[OWN];
           tmem_wait_st();
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(kPThreads, 1) pair_kernel(const KParams p) {
     // ---- group end: every pair's steps are done, every copy of the group
     // has landed; the per-pair regions are free for the reduction
     __syncthreads();
-    if (g == 0) {
+    if (d0 == 0) {
       float* RE = reinterpret_cast<float*>(smem + lay.pair_off);   // [pairs][N]
       float e[OWN];
       TmE::ld(tE, e);

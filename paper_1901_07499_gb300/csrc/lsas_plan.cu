@@ -24,6 +24,7 @@
 #include "lsas_kernels.cuh"
 #include "lsas_hyb.cuh"
 #include "lsas_pair.cuh"
+#include "lsas_twin.cuh"
 
 namespace lsas {
 cudaError_t launch_n64(int, bool, const KParams&, int, int, cudaStream_t);
@@ -399,6 +400,7 @@ void base_params(lsas_plan p, KParams* k) {
              (p->N >= 1024 || (p->N == 512 && p->M >= 32) || (p->N == 256 && p->M >= 128)))
                 ? 1 : 0;
   k->tc_w1 = p->d_tc_w1;
+  k->sms = p->sms;
   k->M = p->M;
   k->m0 = 0;
   k->Mtot = p->M;
@@ -452,6 +454,17 @@ lsas_status set_device(lsas_plan p) {
   return LSAS_OK;
 }
 
+// How rows reach shared memory (KParams::use_tma): bulk copies where every row
+// starts on 16 bytes; from the boundary before each row where that lies
+// within the buffer (an aligned buffer, or a prefix of three samples or more)
+// and the samples are aligned to themselves; plain loads otherwise.
+int staging(lsas_plan p, const void* d_in) {
+  if (tma_ok(p, d_in)) return 1;
+  const uintptr_t a = reinterpret_cast<uintptr_t>(d_in);
+  const bool whole = a % (p->fmt == LSAS_IN_SC16 ? 4 : 8) == 0;
+  return whole && (aligned16(d_in) || p->cp >= 3) ? 2 : 0;
+}
+
 lsas_status check_frames(lsas_plan p, int n_frames) {
   if (n_frames < 0) return LSAS_ERR_INVALID_ARG;
   if (n_frames > p->max_frames) return LSAS_ERR_CAPACITY;
@@ -470,11 +483,36 @@ lsas_status launch_frame(lsas_plan p, const void* d_in, int n_frames, float* d_H
   k.eq = reinterpret_cast<float2*>(d_eq);
   k.mode = mode;
   k.chunks = (p->M + p->geo.Af - 1) / p->geo.Af;
-  k.use_tma = tma_ok(p, d_in) ? 1 : 0;
+  k.use_tma = staging(p, d_in);
   if (p->launch(kKindFrame, p->fmt == LSAS_IN_FC32, k, n_frames, p->geo.smem_frame, st) !=
       cudaSuccess)
     return LSAS_ERR_CUDA;
   return LSAS_OK;
+}
+
+// Grid layers of a split launch (KParams::group_z) of nf frames in G shards
+// each: as many even parts of the data symbols as leave every block an SM of
+// its own, each repeating the pilot transform, and no more than shorten the
+// longest part's steps.  Where the kernel's data-symbol groups alone exceed
+// one wave, they become the layers while they fit two (the blocks' steps fall
+// from all groups' to one's).  A single frame of 64 antennas at N = 1024: 8 x 13
+// blocks of one step 11 us, 8 x 4 of up to three 17.
+int grid_layers(lsas_plan p, const KParams& k, int nf, int G) {
+  if (p->N > 1024 && p->fmt != LSAS_IN_SC16) return 0;   // frame_kernel
+  const long blocks = static_cast<long>(nf) * G;
+  const bool twin = k.twin && k.use_tma == 1;
+  const int groups = p->geo.hybrid ? p->geo.groups : twin ? twin_groups(p->D) : p->geo.groups;
+  const int pilot = k.H_in ? 0 : 1;
+  auto steps = [&](int z) {   // of the longest part
+    const int items = (p->D + z - 1) / z + pilot;
+    return twin ? (items + 1) / 2 : items;
+  };
+  int z = static_cast<int>(p->sms / blocks < p->D ? p->sms / blocks : p->D);
+  if (!p->geo.hybrid && z >= groups && z >= 2) {
+    while (z > groups && z > 2 && steps(z - 1) == steps(z)) --z;
+    return steps(z) < steps(1) ? z : 0;
+  }
+  return groups > 1 && blocks * 2 <= p->sms ? groups : 0;
 }
 
 // Antenna shards G for nf frames that do not fill a whole wave of blocks
@@ -537,14 +575,10 @@ lsas_status run_split_tail(lsas_plan p, const void* d_in, int f0, int nf, int G,
   k.M = p->M / G;
   k.shard_y = k.M;
   k.grid_y = G;
-  // small batches: one block per data-symbol group as well (each repeats
-  // the pilot transform), so a frame's groups also run side by side, as in
-  // the one-launch static split
-  k.group_z = ((p->N <= 1024 || p->fmt == LSAS_IN_SC16) && p->geo.groups > 1 &&
-               nf * G * 2 <= p->sms) ? 1 : 0;
   k.chunks = (k.M + p->geo.Af - 1) / p->geo.Af;
   k.mode = kModePartial;
-  k.use_tma = tma_ok(p, in) ? 1 : 0;
+  k.use_tma = staging(p, in);
+  k.group_z = grid_layers(p, k, nf, G);
   lsas_status s = LSAS_OK;
   if (p->launch(kKindFrame, p->fmt == LSAS_IN_FC32, k, nf, p->geo.smem_frame, st) != cudaSuccess) {
     s = LSAS_ERR_CUDA;
@@ -823,7 +857,7 @@ lsas_status lsas_fft(lsas_plan p, const void* d_in, int n_frames, float* d_Y, vo
   k.in = d_in;
   k.Y_out = reinterpret_cast<float2*>(d_Y);
   k.nslots = p->geo.fft_slots;
-  k.use_tma = tma_ok(p, d_in) ? 1 : 0;
+  k.use_tma = staging(p, d_in);
   row_batch(p, n_frames, false, &k);
   const int grid = n_frames * k.chunks;
   ProfScope prof(p, "lsas_fft", stream);
@@ -846,7 +880,7 @@ lsas_status lsas_estimate(lsas_plan p, const void* d_in, int n_frames, float* d_
   k.in = d_in;
   k.H_out = reinterpret_cast<float2*>(d_H);
   k.mode = kModeEstimate;
-  k.use_tma = tma_ok(p, d_in) ? 1 : 0;
+  k.use_tma = staging(p, d_in);
   row_batch(p, n_frames, true, &k);
   const int grid = n_frames * k.chunks;
   ProfScope prof(p, "lsas_estimate", stream);
@@ -900,7 +934,7 @@ lsas_status lsas_mrc_partial(lsas_plan p, const void* d_in, int n_frames, int m_
   k.chunks = (m_count + p->geo.Af - 1) / p->geo.Af;
   ProfScope prof(p, "lsas_mrc_partial", stream);
   k.mode = kModePartial;
-  k.use_tma = tma_ok(p, d_in) ? 1 : 0;
+  k.use_tma = staging(p, d_in);
   if (p->launch(kKindFrame, p->fmt == LSAS_IN_FC32, k, n_frames, p->geo.smem_frame,
                 static_cast<cudaStream_t>(stream)) != cudaSuccess)
     return LSAS_ERR_CUDA;
@@ -1360,13 +1394,10 @@ lsas_status lsas_run_frame_split_static(lsas_plan p, const void* d_in, int n_fra
     k.M = p->M / n_shards;
     k.shard_y = k.M;
     k.grid_y = n_shards;
-    // small batches: one block per data-symbol group as well (each repeats
-    // the pilot transform), so a frame's groups also run side by side
-    k.group_z = ((p->N <= 1024 || p->fmt == LSAS_IN_SC16) && p->geo.groups > 1 &&
-                 n_frames * n_shards * 2 <= p->sms) ? 1 : 0;
     k.chunks = (k.M + p->geo.Af - 1) / p->geo.Af;
     k.mode = kModePartial;
-    k.use_tma = tma_ok(p, d_in) ? 1 : 0;
+    k.use_tma = staging(p, d_in);
+    k.group_z = grid_layers(p, k, n_frames, n_shards);
     if (p->launch(kKindFrame, p->fmt == LSAS_IN_FC32, k, n_frames, p->geo.smem_frame,
                   static_cast<cudaStream_t>(stream)) != cudaSuccess)
       return LSAS_ERR_CUDA;

@@ -396,7 +396,7 @@ __device__ __forceinline__ int twin_block_col(int it, bool pilot, bool* pair, in
   return pilot ? (ip == 0 ? 0 : 64 + 128 * (ip - 1)) : 128 * ip;
 }
 
-template <int LOG2N, bool GIVEN>
+template <int LOG2N, bool GIVEN, bool PART>
 __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
   static_assert(LOG2N >= 7 && LOG2N <= 10, "the two-symbol kernel covers N = 128 .. 1024");
   constexpr int N = 1 << LOG2N;
@@ -452,19 +452,20 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
   const int nch = warp < p.chunks ? (p.chunks - 1 - warp) / NW + 1 : 0;
   // start the warps of the upper half a little later, so that the two warps
   // sharing a scheduler tend to be in different phases of their steps
-  if (warp >= 4) __nanosleep(1400);
+  // (not in a short launch, whose time it would lengthen)
+  if (warp >= 4 && nch > 2) __nanosleep(1400);
   int issued = 0;  // steps whose copies this warp has issued
   int slot = 0;    // ring slot of the next step to consume ...
   int phase = 0;   // ... and its mbarrier phase
-  // one data-symbol group per grid z index (partial mode, small batches):
-  // every group's block transforms the pilot itself; group 0 alone writes H
-  // and the channel energy
-  const int g_lo = p.group_z ? static_cast<int>(blockIdx.z) : 0;
-  const int g_hi = p.group_z ? g_lo + 1 : twin_groups(p.D);
+  // one part of the data symbols per grid z index (partial mode, small
+  // batches; no part is larger than its group): every part's block transforms
+  // the pilot itself; part 0 alone writes H and the channel energy
+  const int g_lo = PART && p.group_z ? static_cast<int>(blockIdx.z) : 0;
+  const int g_hi = PART && p.group_z ? g_lo + 1 : twin_groups(p.D);
   for (int g = g_lo; g < g_hi; ++g) {
-    const int d0 = g == 0 ? 0 : kTwDg0 + (g - 1) * kTwDg;
-    const int nd = min(g == 0 ? kTwDg0 : kTwDg, p.D - d0);
-    const bool pilot_here = !GIVEN && (g == 0 || p.group_z);
+    const int d0 = PART && p.group_z ? g * p.D / p.group_z : g == 0 ? 0 : kTwDg0 + (g - 1) * kTwDg;
+    const int nd = PART && p.group_z ? (g + 1) * p.D / p.group_z - d0 : min(g == 0 ? kTwDg0 : kTwDg, p.D - d0);
+    const bool pilot_here = !GIVEN && (g == 0 || (PART && p.group_z));
     const bool energy_here = g == 0;
     const int items = nd + (pilot_here ? 1 : 0);
     const int npairs = (items + 1) / 2;
@@ -619,7 +620,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
         float E = 0.f;
 #pragma unroll
         for (int w = 0; w < 4 * A; ++w) E += RE[w * N + k];
-        if (p.mode == kModePartial) {
+        if constexpr (PART) {
           p.E_out[(static_cast<size_t>(blockIdx.y) * gridDim.x + f) * N + k] = E;
         } else {
           // zero or non-finite energy flags the frame; z = 0 there
@@ -704,7 +705,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
             const int k = idx & (N - 1);
             const float2 s = sv[u];
             const int dl = dl0 + j;
-            if (p.mode == kModePartial) {
+            if constexpr (PART) {
               p.P_out[((static_cast<size_t>(blockIdx.y) * gridDim.x + f) * p.D + d0 + dl) * N + k] =
                   make_float2(s.x * p.inv_sqrtN, s.y * p.inv_sqrtN);
             } else {
@@ -718,15 +719,19 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
           }
         }
       };
-      switch (p.nthr) {
-        case 1: demap_items(std::integral_constant<int, 1>{}); break;
-        case 3: demap_items(std::integral_constant<int, 3>{}); break;
-        case 7: demap_items(std::integral_constant<int, 7>{}); break;
-        default: demap_items(std::integral_constant<int, kMaxThresholds>{}); break;
+      if constexpr (PART) {
+        demap_items(std::integral_constant<int, 1>{});
+      } else {
+        switch (p.nthr) {
+          case 1: demap_items(std::integral_constant<int, 1>{}); break;
+          case 3: demap_items(std::integral_constant<int, 3>{}); break;
+          case 7: demap_items(std::integral_constant<int, 7>{}); break;
+          default: demap_items(std::integral_constant<int, kMaxThresholds>{}); break;
+        }
       }
       __syncthreads();
     }
-    if (p.mode != kModePartial) {
+    if constexpr (!PART) {
       // pack: 8 consecutive subcarriers -> q bytes
       const int items8 = nd * (N / 8);
       const size_t frame_bytes = static_cast<size_t>(p.D) * N * p.q / 8;

@@ -145,56 +145,37 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
   unsigned char* stage = smem + lay.pair_off + q * lay.pair_bytes;
   unsigned char* const X = stage + lay.stage_bytes;
 
-  for (int i = tid; i < kTpTwl; i += kTpThreads) twl[i] = __ldg(p.twP + 512 + i);
-  for (int i = tid; i < 7 * 32; i += kTpThreads) mtw[i] = __ldg(p.twP + 32 + i);
-  if (tid == 0) *abort_flag = 0;
   if (jt == 0) {
     for (int s = 0; s < K; ++s) mbar_init(smem_u32(&bars[s]), 1);
     fence_mbar_init();
   }
-  if (warp == 0) tmem_alloc(smem_u32(tmem_base), kWTmemCols);
-  tmem_fence_before();
-  __syncthreads();
-  tmem_fence_after();
-  // this warp's columns: 256 columns of its lane quarter; warp w + 4 holds
-  // the same subcarriers (same jt) in the other half of the quarter
-  const uint32_t tE = *tmem_base + (static_cast<uint32_t>(32 * (warp & 3)) << 16) +
-                      static_cast<uint32_t>((warp >> 2) * kTwTmemWarp);
+  uint32_t tE = 0;
   const uint64_t pol = jt < 2 ? evict_first_policy() : 0;
   float zero[16];
 #pragma unroll
   for (int i = 0; i < 16; ++i) zero[i] = 0.f;
 
   const int nch = q < p.chunks ? (p.chunks - 1 - q) / kTpPairs + 1 : 0;
-  // start the pairs of the upper half a little later, so that the two warps
-  // sharing a scheduler tend to be in different phases of their steps
-  if (warp >= 4) __nanosleep(1400);
   int issued = 0;  // steps whose copies this pair has issued
   int slot = 0;    // ring slot of the next step to consume ...
   int phase = 0;   // ... and its mbarrier phase
-  // one data-symbol group per grid z index (partial mode, small batches):
-  // every group's block transforms the pilot itself; group 0 alone writes H
-  // and the channel energy
+  // one part of the data symbols per grid z index (partial mode, small
+  // batches; no part is larger than its group): every part's block transforms
+  // the pilot itself; part 0 alone writes H and the channel energy
   const int g_lo = p.group_z ? static_cast<int>(blockIdx.z) : 0;
   const int g_hi = p.group_z ? g_lo + 1 : twin_groups(p.D);
   for (int g = g_lo; g < g_hi; ++g) {
-    const int d0 = g == 0 ? 0 : kTwDg0 + (g - 1) * kTwDg;
-    const int nd = min(g == 0 ? kTwDg0 : kTwDg, p.D - d0);
+    const int d0 = p.group_z ? g * p.D / p.group_z : g == 0 ? 0 : kTwDg0 + (g - 1) * kTwDg;
+    const int nd = p.group_z ? (g + 1) * p.D / p.group_z - d0 : min(g == 0 ? kTwDg0 : kTwDg, p.D - d0);
     const bool pilot_here = !GIVEN && (g == 0 || p.group_z);
     const bool energy_here = g == 0;
     const int items = nd + (pilot_here ? 1 : 0);
     const int npairs = (items + 1) / 2;
-    const uint32_t tP = energy_here ? tE + OWN : tE;
-    if (energy_here) {
-#pragma unroll
-      for (int q0 = 0; q0 < OWN; q0 += 16) Tmem<16>::st(tE + q0, zero);
-    }
-    for (uint32_t c = tP; c < tE + kTwTmemWarp; c += 16) Tmem<16>::st(c, zero);
     // issue cursor: local chunk and pair of the next step to stage, and how
     // many steps of this group are still to be staged
     int ic = 0, ipi = 0;
     int to_issue = nch * npairs;
-    if (!*abort_flag) {
+    if (g == g_lo || !*abort_flag) {
       // the ring held generic data (last group's reduction): order it before
       // the copies, then fill the first K slots of this group
       fence_proxy_async();
@@ -214,6 +195,30 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
         }
       }
     }
+    if (g == g_lo) {
+      // the block's set-up, under the first copies
+      for (int i = tid; i < kTpTwl; i += kTpThreads) twl[i] = __ldg(p.twP + 512 + i);
+      for (int i = tid; i < 7 * 32; i += kTpThreads) mtw[i] = __ldg(p.twP + 32 + i);
+      if (tid == 0) *abort_flag = 0;
+      if (warp == 0) tmem_alloc(smem_u32(tmem_base), kWTmemCols);
+      tmem_fence_before();
+      __syncthreads();
+      tmem_fence_after();
+      // this warp's columns: 256 columns of its lane quarter; warp w + 4 holds
+      // the same subcarriers (same jt) in the other half of the quarter
+      tE = *tmem_base + (static_cast<uint32_t>(32 * (warp & 3)) << 16) +
+           static_cast<uint32_t>((warp >> 2) * kTwTmemWarp);
+      // start the pairs of the upper half a little later, so that the two warps
+      // sharing a scheduler tend to be in different phases of their steps
+      // (not in a short launch, whose time it would lengthen)
+      if (warp >= 4 && nch > 2) __nanosleep(1400);
+    }
+    const uint32_t tP = energy_here ? tE + OWN : tE;
+    if (energy_here) {
+#pragma unroll
+      for (int q0 = 0; q0 < OWN; q0 += 16) Tmem<16>::st(tE + q0, zero);
+    }
+    for (uint32_t c = tP; c < tE + kTwTmemWarp; c += 16) Tmem<16>::st(c, zero);
     unsigned char* prev_slot = nullptr;   // slot of the pair's previous step in this group
     uint32_t prev_bar = 0;
     for (int lc = 0; lc < nch; ++lc) {

@@ -15,17 +15,41 @@
 //     data symbol: conj(H) Y (Sec. II-C), summed over the chunk's antennas
 //     with shuffles,
 //   * accumulates per subcarrier in the warp's own tensor-memory columns.
+// A warp's work is a list of (chunk, data symbol) pairs.  With at least as many
+// chunks as warps they are whole chunks, w, w + NW, ....  With fewer (p.share),
+// the chunk-major list of all pairs is cut into NW even pieces: a warp then
+// transforms the pilot of each chunk it touches and takes only its own data
+// symbols, and the warp with a chunk's first data symbol alone writes its H
+// and adds its energy.  No warp holds two chunks' sums of one symbol then, so
+// the sums over antennas are those of one chunk per warp, bit for bit.  16
+// frames of 8 antennas at N = 64, 15 symbols (one chunk): 25.2 -> 9.4 us.
+// The frames after the last whole wave may run as p.zsplit blocks each, with an
+// even part of the data symbols (p.full whole frames come first in the grid);
+// every block transforms the pilots itself, the first writes H, and the
+// results are the same bits again.  Together with the even pieces: 200 frames
+// of 24 antennas, N = 256, CP 18: 75.7 -> 57.4 us.
+// Rows that do not start on 16 bytes (p.use_tma = 2) are staged from the
+// 16-byte boundary before them and read at their own offset.
 // Warps never wait for each other inside a data-symbol group.  At a group's
 // end the block adds the warps' partial sums in warp order through shared
 // memory (the staging rings are idle then), forms z = P / E and demaps
 // (Sec. II-B), or writes the block's partial sums (antenna split).
 #pragma once
 
+#include <type_traits>
+
 #include "lsas_kernels.cuh"
 
 namespace lsas {
 
 #ifdef __CUDACC__
+
+// Whether a row is the last of the launch's input (its end may be the
+// buffer's).
+__device__ __forceinline__ bool last_row(const KParams& p, int f, int m, int s) {
+  return s == p.S - 1 && f == p.nf - 1 &&
+         p.m0 + static_cast<int>(blockIdx.y) * p.shard_y + m == p.Mtot - 1;
+}
 
 // Issue the bulk copies of one warp step (antennas of chunk c, symbol s)
 // into a slot: lane 0 registers the byte count, lane a copies row a.
@@ -36,10 +60,45 @@ __device__ __forceinline__ void wissue(const KParams& p, int f, int c, int s,
   constexpr int N = 1 << LOG2N, A = wgeo_A(N);
   constexpr uint32_t bytes = N * (FC32 ? 8 : 4);
   const int nvalid = min(A, p.M - c * A);
+  if (p.use_tma == 2) {
+    // from the boundary before each row, 16 bytes more than the row where it
+    // does not start on one (the next row's, but past the last row of all)
+    static_assert(A <= 32, "one row a lane");
+    const unsigned char* src = row_ptr<LOG2N, FC32>(p, f, c * A + lane, s);
+    const uint32_t mis = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(src) & 15);
+    const uint32_t n = lane >= nvalid ? 0u : (mis != 0 && !last_row(p, f, c * A + lane, s)) ? bytes + 16 : bytes;
+    const uint32_t total = __reduce_add_sync(0xffffffffu, n);
+    if (lane == 0) mbar_expect_tx(bar, total);
+    __syncwarp();
+    if (n) bulk_load(smem_u32(slot + lane * team_stage), src - mis, n, bar, pol);
+    return;
+  }
   if (lane == 0) mbar_expect_tx(bar, bytes * nvalid);
   for (int a = lane; a < nvalid; a += 32)
     bulk_load(smem_u32(slot + a * team_stage), row_ptr<LOG2N, FC32>(p, f, c * A + a, s), bytes,
               bar, pol);
+}
+
+// Pass-1 inputs of a row staged from the 16-byte boundary before it: sample n
+// sits (row mod 16) bytes further on.  The last row of all is staged without
+// the piece that would reach past the buffer; its last samples come from
+// memory.
+template <int LOG2N, bool FC32>
+__device__ __forceinline__ void wload_shifted(float2 (&v)[32], const unsigned char* staged,
+                                              const unsigned char* row, bool last, int jt) {
+  constexpr int N = 1 << LOG2N, L = N / 32, bps = FC32 ? 8 : 4;
+  const int mis = static_cast<int>(reinterpret_cast<uintptr_t>(row) & 15);
+  load_row<LOG2N, FC32>(v, staged + mis, jt, false);
+  if (last) {
+#pragma unroll
+    for (int r = 0; r < 32; ++r) {
+      const int n = jt + r * L;
+      if ((r + 1) * L > N - 4 && (n + 1) * bps + mis > N * bps) {
+        if constexpr (FC32) v[r] = __ldg(reinterpret_cast<const float2*>(row) + n);
+        else v[r] = sc16_to_float2(__ldg(reinterpret_cast<const uint32_t*>(row) + n));
+      }
+    }
+  }
 }
 
 // Symbol index of item `it` of a chunk in a data-symbol group starting at
@@ -86,7 +145,9 @@ __global__ void __launch_bounds__(32 * wgeo_warps(FC32 ? 8 : 4), 1) warp_kernel(
   using TmP = Tmem<2 * OWN>;   // one data symbol of partial sums (complex)
   using TmE = Tmem<OWN>;       // channel energy
   extern __shared__ __align__(128) unsigned char smem[];
-  const int f = blockIdx.x;
+  // whole frames first, then the symbol-split ones, p.zsplit blocks each
+  const int bx = blockIdx.x, sx = bx - p.full;
+  const int f = sx < 0 ? bx : p.full + sx / p.zsplit;
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
   const int lane = tid & 31;
@@ -132,25 +193,42 @@ __global__ void __launch_bounds__(32 * wgeo_warps(FC32 ? 8 : 4), 1) warp_kernel(
 #pragma unroll
   for (int i = 0; i < ZC; ++i) zero[i] = 0.f;
 
-  const int nch = warp < p.chunks ? (p.chunks - 1 - warp) / NW + 1 : 0;
   // start the warps of the upper half a little later, so that the two warps
   // sharing a scheduler tend to be in different phases of their steps
-  if (warp >= 4) __nanosleep(1400);
+  // (not in a short launch, whose time it would lengthen)
+  if (warp >= 4 && p.chunks >= NW) __nanosleep(1400);
   int step = 0;    // this warp's step counter over the whole frame
   int issued = 0;  // steps whose copies this warp has issued
   int slot = 0;    // ring slot of the next step to consume (step % K) ...
   int phase = 0;   // ... and its mbarrier phase ((step / K) & 1)
-  // one data-symbol group per grid z index (partial mode, small batches):
-  // every group's block transforms the pilot itself; group 0 alone writes H
-  // and the channel energy
-  const int g_lo = p.group_z ? static_cast<int>(blockIdx.z) : 0;
-  const int g_hi = p.group_z ? g_lo + 1 : p.groups;
-  for (int g = g_lo; g < g_hi; ++g) {
-    const int nd = min(p.dg, p.D - g * p.dg);
-    const int d0 = g * p.dg;
-    const bool pilot_here = fft_pilot(p) && (g == 0 || p.group_z);
-    const int items = nd + (pilot_here ? 1 : 0);
-    if (g == g_lo) {
+  // the block's data symbols: all, or an even part (per grid z index in partial
+  // mode for small batches, or in a symbol split); every block transforms
+  // the pilots itself, and the one with data symbol 0 writes H (and, in
+  // partial mode, the channel energy)
+  int d_begin = 0, d_end = p.D;
+  if (p.group_z) {
+    const int z = blockIdx.z;
+    d_begin = z * p.D / p.group_z;
+    d_end = (z + 1) * p.D / p.group_z;
+  } else if (sx >= 0) {
+    const int z = sx % p.zsplit;
+    d_begin = z * p.D / p.zsplit;
+    d_end = (z + 1) * p.D / p.zsplit;
+  }
+  for (int d0 = d_begin; d0 < d_end; d0 += p.dg) {
+    const int nd = min(p.dg, d_end - d0);
+    const bool first = d0 == d_begin;
+    const bool pilot_here = fft_pilot(p) && first;
+    const int pil = pilot_here ? 1 : 0;
+    // this warp's pairs (chunk-major), whole chunks warp, warp + NW, ... unless shared
+    const int lo = warp * p.chunks * nd / NW, hi = (warp + 1) * p.chunks * nd / NW;
+    const int nch = p.share ? (hi > lo ? (hi - 1) / nd - lo / nd + 1 : 0)
+                            : (warp < p.chunks ? (p.chunks - 1 - warp) / NW + 1 : 0);
+    // local chunk lc: its number, and its first and past-the-last data symbol of the group
+    auto chunk_of = [&](int lc) { return p.share ? lo / nd + lc : warp + lc * NW; };
+    auto sym_lo = [&](int lc) { return p.share && lc == 0 ? lo % nd : 0; };
+    auto sym_hi = [&](int lc) { return p.share ? min(nd, hi - (lo / nd + lc) * nd) : nd; };
+    if (first) {
 #pragma unroll
       for (int q0 = 0; q0 < OWN; q0 += ZC) Tmem<ZC>::st(tE + q0, zero);
     }
@@ -161,41 +239,49 @@ __global__ void __launch_bounds__(32 * wgeo_warps(FC32 ? 8 : 4), 1) warp_kernel(
     // issue cursor: local chunk and item of the next step to stage, and how
     // many steps of this group are still to be staged
     int ic = 0, iit = 0;
-    int to_issue = nch * items;
+    int ia = sym_lo(0), iitems = sym_hi(0) - ia + pil;   // of chunk ic
+    int to_issue = p.share ? hi - lo + nch * pil : nch * (nd + pil);
+    auto advance = [&]() {
+      if (++iit == iitems) {
+        iit = 0;
+        ++ic;
+        ia = sym_lo(ic);
+        iitems = sym_hi(ic) - ia + pil;
+      }
+    };
     if (p.use_tma && !*abort_flag) {
       // the ring held generic data (last group's reduction): order it before
       // the copies, then fill the first K slots of this group
       fence_proxy_async();
       int is = slot;
       for (int s = 0; s < K && to_issue > 0; ++s, --to_issue) {
-        wissue<LOG2N, FC32>(p, f, warp + ic * NW, witem_symbol(p, pilot_here, d0, iit),
+        wissue<LOG2N, FC32>(p, f, chunk_of(ic), witem_symbol(p, pilot_here, d0 + ia, iit),
                             stage + is * slot_bytes, lay.team_stage, smem_u32(&bars[is]), pol,
                             lane);
         // test hook: the first staging phase of block 0 also waits for 16
         // bytes that no copy delivers, so its bounded wait runs out
-        if (p.fault == 1 && blockIdx.x == 0 && warp == 0 && g == 0 && s == 0 && lane == 0)
+        if (p.fault == 1 && blockIdx.x == 0 && warp == 0 && d0 == 0 && s == 0 && lane == 0)
           mbar_expect_tx_only(smem_u32(&bars[is]), 16);
         ++issued;
         is = (is + 1 == K) ? 0 : is + 1;
-        if (++iit == items) {
-          iit = 0;
-          ++ic;
-        }
+        advance();
       }
     }
     for (int lc = 0; lc < nch; ++lc) {
-      const int c = warp + lc * NW;
+      const int c = chunk_of(lc);
+      const int sa = sym_lo(lc), items = sym_hi(lc) - sa + pil;
+      const bool lead = sa == 0;   // writes the chunk's H and adds its energy
       const int m = c * A + alpha;
       const bool valid = m < p.M;
       const size_t hrow = (static_cast<size_t>(f) * p.Mtot + p.m0 + blockIdx.y * p.shard_y + m) * N;
       float2 h[32];
       if (!pilot_here) {
-        // channel from memory: given (demodulate) or written in group 0
+        // channel from memory: given (demodulate) or written in the first group
         const float2* Hs = fft_pilot(p) ? p.H_out : p.H_in;
 #pragma unroll
         for (int e = 0; e < 32; ++e)
           h[e] = valid ? Hs[hrow + bin_of<LOG2N>(jt, e)] : make_float2(0.f, 0.f);
-        if (g == 0) {
+        if (first && lead) {
           float2 e2[32];
 #pragma unroll
           for (int e = 0; e < 32; ++e) e2[e] = make_float2(h[e].x * h[e].x + h[e].y * h[e].y, 0.f);
@@ -214,14 +300,21 @@ __global__ void __launch_bounds__(32 * wgeo_warps(FC32 ? 8 : 4), 1) warp_kernel(
         if (p.use_tma) {
           wait_slot(smem_u32(&bars[slot]), phase, abort_flag, p.status);
           if (valid) {
-            load_row<LOG2N, FC32>(v, stage + slot * slot_bytes + alpha * lay.team_stage, jt, false);
+            const unsigned char* row = stage + slot * slot_bytes + alpha * lay.team_stage;
+            if (p.use_tma == 2) {
+              const int sym = witem_symbol(p, pilot_here, d0 + sa, it);
+              wload_shifted<LOG2N, FC32>(v, row, row_ptr<LOG2N, FC32>(p, f, m, sym),
+                                         last_row(p, f, m, sym), jt);
+            } else {
+              load_row<LOG2N, FC32>(v, row, jt, false);
+            }
           } else {
 #pragma unroll
             for (int r = 0; r < 32; ++r) v[r] = make_float2(0.f, 0.f);
           }
         } else {
           if (valid) {
-            load_row<LOG2N, FC32>(v, row_ptr<LOG2N, FC32>(p, f, m, witem_symbol(p, pilot_here, d0, it)),
+            load_row<LOG2N, FC32>(v, row_ptr<LOG2N, FC32>(p, f, m, witem_symbol(p, pilot_here, d0 + sa, it)),
                                   jt, true);
           } else {
 #pragma unroll
@@ -234,14 +327,11 @@ __global__ void __launch_bounds__(32 * wgeo_warps(FC32 ? 8 : 4), 1) warp_kernel(
         if (p.use_tma && to_issue > 0 && !*abort_flag) {
           ++issued;
           fence_proxy_async();
-          wissue<LOG2N, FC32>(p, f, warp + ic * NW, witem_symbol(p, pilot_here, d0, iit),
+          wissue<LOG2N, FC32>(p, f, chunk_of(ic), witem_symbol(p, pilot_here, d0 + ia, iit),
                               stage + slot * slot_bytes, lay.team_stage, smem_u32(&bars[slot]),
                               pol, lane);
           --to_issue;
-          if (++iit == items) {
-            iit = 0;
-            ++ic;
-          }
+          advance();
         }
         if (++slot == K) {
           slot = 0;
@@ -259,20 +349,22 @@ __global__ void __launch_bounds__(32 * wgeo_warps(FC32 ? 8 : 4), 1) warp_kernel(
             const int k = bin_of<LOG2N>(jt, e);
             const float2 hv = cmul(v[e], __ldg(p.xinv + k));
             h[e] = valid ? hv : make_float2(0.f, 0.f);
-            if (valid && g == 0) p.H_out[hrow + k] = hv;
+            if (valid && lead && d0 == 0) p.H_out[hrow + k] = hv;
             v[e] = make_float2(h[e].x * h[e].x + h[e].y * h[e].y, 0.f);
           }
-          reduce_scatter<A, 16>(v, alpha);
-          float acc[OWN];
-          tmem_wait_st();
-          TmE::ld(tE, acc);
-          tmem_wait_ld();
+          if (lead) {
+            reduce_scatter<A, 16>(v, alpha);
+            float acc[OWN];
+            tmem_wait_st();
+            TmE::ld(tE, acc);
+            tmem_wait_ld();
 #pragma unroll
-          for (int cc = 0; cc < OWN; ++cc) acc[cc] += v[cc].x;
-          TmE::st(tE, acc);
+            for (int cc = 0; cc < OWN; ++cc) acc[cc] += v[cc].x;
+            TmE::st(tE, acc);
+          }
         } else {
           // MRC numerator: conj(H) Y summed over the chunk's antennas
-          const int dl = it - (pilot_here ? 1 : 0);
+          const int dl = sa + it - pil;
           const uint32_t tp = tP + 2 * OWN * dl;
           if constexpr (A == 1) {
             // one antenna per step: fuse the product into the accumulation,
@@ -318,7 +410,7 @@ __global__ void __launch_bounds__(32 * wgeo_warps(FC32 ? 8 : 4), 1) warp_kernel(
     // ---- group end: every warp's steps are done, every copy of the group
     // has landed; the per-warp regions are free for the reduction
     __syncthreads();
-    if (g == 0) {
+    if (first && (d0 == 0 || p.mode != kModePartial)) {
       float* RE = reinterpret_cast<float*>(smem + lay.warp_off);   // [NW][N]
       float e[OWN];
       TmE::ld(tE, e);
@@ -355,24 +447,49 @@ __global__ void __launch_bounds__(32 * wgeo_warps(FC32 ? 8 : 4), 1) warp_kernel(
           dst[bin_of<LOG2N>(jt, alpha * OWN + cc)] = make_float2(acc[2 * cc], acc[2 * cc + 1]);
       }
       __syncthreads();
-      for (int idx = tid; idx < n * N; idx += NT) {
-        const int j = idx >> LOG2N;
-        const int k = idx & (N - 1);
-        float2 s = make_float2(0.f, 0.f);
+      // four items per thread at a time (their shared-memory sums all loaded
+      // before the first is demapped), one copy of the loop per constellation,
+      // so that the slicer inside it has no branches
+      auto demap_items = [&](auto tcount) {
+        constexpr int TC = decltype(tcount)::value;
+        for (int idx0 = tid; idx0 < n * N; idx0 += 4 * NT) {
+          float2 sv[4];
 #pragma unroll
-        for (int w = 0; w < NW; ++w) s = cadd(s, RP[static_cast<size_t>(w * dlc + j) * N + k]);
-        const int dl = dl0 + j;
-        if (p.mode == kModePartial) {
-          p.P_out[((static_cast<size_t>(blockIdx.y) * gridDim.x + f) * p.D + d0 + dl) * N + k] =
-              make_float2(s.x * p.inv_sqrtN, s.y * p.inv_sqrtN);
-        } else {
-          const float ie = ie_s[k];
-          const float2 z = (ie != 0.f) ? make_float2(s.x * ie, s.y * ie) : make_float2(0.f, 0.f);
-          if (p.eq) p.eq[(static_cast<size_t>(f) * p.D + d0 + dl) * N + k] = z;
-          uint32_t code = gray(axis_level(z.x, p));
-          if (p.axes == 2) code = (code << p.wbits) | gray(axis_level(z.y, p));
-          codes[dl * N + k] = static_cast<uint8_t>(code);
+          for (int u = 0; u < 4; ++u) {
+            const int idx = min(idx0 + u * NT, n * N - 1);
+            const int j = idx >> LOG2N;
+            const int k = idx & (N - 1);
+            sv[u] = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int w = 0; w < NW; ++w) sv[u] = cadd(sv[u], RP[static_cast<size_t>(w * dlc + j) * N + k]);
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int idx = idx0 + u * NT;
+            if (idx >= n * N) break;
+            const int j = idx >> LOG2N;
+            const int k = idx & (N - 1);
+            const float2 s = sv[u];
+            const int dl = dl0 + j;
+            if (p.mode == kModePartial) {
+              p.P_out[((static_cast<size_t>(blockIdx.y) * gridDim.x + f) * p.D + d0 + dl) * N + k] =
+                  make_float2(s.x * p.inv_sqrtN, s.y * p.inv_sqrtN);
+            } else {
+              const float ie = ie_s[k];
+              const float2 z = (ie != 0.f) ? make_float2(s.x * ie, s.y * ie) : make_float2(0.f, 0.f);
+              if (p.eq) p.eq[(static_cast<size_t>(f) * p.D + d0 + dl) * N + k] = z;
+              uint32_t code = gray(count_ge<TC>(z.x, p.thr));
+              if (p.axes == 2) code = (code << p.wbits) | gray(count_ge<TC>(z.y, p.thr));
+              codes[dl * N + k] = static_cast<uint8_t>(code);
+            }
+          }
         }
+      };
+      switch (p.nthr) {
+        case 1: demap_items(std::integral_constant<int, 1>{}); break;
+        case 3: demap_items(std::integral_constant<int, 3>{}); break;
+        case 7: demap_items(std::integral_constant<int, 7>{}); break;
+        default: demap_items(std::integral_constant<int, kMaxThresholds>{}); break;
       }
       __syncthreads();
     }
