@@ -436,9 +436,10 @@ lsas_status lsas_dn_grad_tc(const float* d_params, const float* d_Hls, const flo
 /*
  * The learned form of the receiver with the refinement fused after LS
  * (Sec. II-C's LS estimate is its input): per antenna row, the pilot
- * symbol's FFT, LS and the row normalisation feed the tensor-core refinement
- * (as lsas_dn_apply_tc, bf16 parameters d_params_bf16) on chip, so the
- * unrefined estimate is never written to memory; then MRC and demapping
+ * symbol's FFT, LS and the row normalisation write the refinement's split
+ * input rows into d_work (the unrefined estimate itself is not stored), the
+ * tensor-core refinement (as lsas_dn_apply_tc, bf16 parameters
+ * d_params_bf16) reads them tile by tile; then MRC and demapping
  * with the refined channel (as lsas_demodulate).  Outputs as lsas_run_frame:
  * d_H receives the refined channel.  d_work: lsas_dn_work_size(n_frames * M,
  * N) floats, 16-byte aligned; d_status as lsas_dn_apply_tc.  The plan's
