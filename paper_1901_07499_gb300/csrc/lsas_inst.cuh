@@ -39,10 +39,10 @@ inline int warp_share(int chunks, int nd) {
 inline int two_symbol_form(const KParams& p) {
   return (p.H_in ? 1 : 0) + (p.mode == kModePartial ? 2 : 0);
 }
-template <int LOG2N>
+template <int LOG2N, bool FC32>
 static auto two_symbol_kernel(const KParams& p) -> void (*)(const KParams) {
   if constexpr (LOG2N == 11) {
-    return p.H_in ? twinpair_kernel<LOG2N, true> : twinpair_kernel<LOG2N, false>;
+    return p.H_in ? twinpair_kernel<LOG2N, true, FC32> : twinpair_kernel<LOG2N, false, FC32>;
   } else {
     void (*const k[4])(const KParams) = {twin_kernel<LOG2N, false, false>, twin_kernel<LOG2N, true, false>,
                                          twin_kernel<LOG2N, false, true>, twin_kernel<LOG2N, true, true>};
@@ -59,12 +59,13 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
     // fused receiver (the two-symbol kernels in a form of their own for a
     // given channel: 200 frames of 64 antennas at N = 1024 demodulate in 355 us
     // there and split, 499 in the one-symbol kernel; 16 frames 50 against 250):
-    // from aligned sc16 rows, two symbols per step for
-    // N = 1024 (and N = 256, 512 with enough antennas; per-warp pipelines)
-    // and N = 2048 (pipelines of warp pairs), or, opt-in at N = 1024, the
-    // second FFT pass on the tensor cores; otherwise one symbol per step: per-warp pipelines up to
-    // N = 1024, pipelines of warp pairs for N = 2048 from sc16 rows and the
-    // warp-specialised producer/consumer kernel for N = 2048 from fc32 rows
+    // two symbols per step, from aligned sc16 rows, for N = 1024 (and N = 256,
+    // 512 with enough antennas; per-warp pipelines) and, from aligned rows of
+    // either format, for N = 2048 (pipelines of warp pairs), or, opt-in at
+    // N = 1024, the second FFT pass on the tensor cores; otherwise one symbol
+    // per step: per-warp pipelines up to N = 1024, pipelines of warp pairs for
+    // N = 2048 from sc16 rows and the warp-specialised producer/consumer kernel
+    // for N = 2048 from fc32 rows
     if constexpr (LOG2N == 10 && !FC32) {
       if (p.hybrid && p.use_tma == 1) {
         fn = hyb_kernel<false>;
@@ -72,7 +73,7 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
         smem = kHySmem;
         slot = 3;
       } else if (p.twin && p.use_tma == 1) {
-        fn = two_symbol_kernel<LOG2N>(p);
+        fn = two_symbol_kernel<LOG2N, FC32>(p);
         slot = 4 + two_symbol_form(p);
         threads = kTwThreads;
         smem = make_twlayout().total;
@@ -83,7 +84,7 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
     } else if constexpr ((LOG2N == 8 || LOG2N == 9) && !FC32) {
       // p.twin is set by the plan only with enough antennas at these sizes
       if (p.twin && p.use_tma == 1) {
-        fn = two_symbol_kernel<LOG2N>(p);
+        fn = two_symbol_kernel<LOG2N, FC32>(p);
         slot = 4 + two_symbol_form(p);
         threads = kTwThreads;
         smem = make_twlayout().total;
@@ -94,19 +95,19 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
     } else if constexpr (LOG2N <= 10) {
       fn = warp_kernel<LOG2N, FC32>;
       threads = 32 * wgeo_warps(FC32 ? 8 : 4);
-    } else if constexpr (!FC32) {
+    } else {
       if (p.twin && p.use_tma == 1) {
-        fn = two_symbol_kernel<LOG2N>(p);
+        fn = two_symbol_kernel<LOG2N, FC32>(p);
         threads = kTpThreads;
         smem = make_tplayout().total;
         slot = 4 + two_symbol_form(p);
+      } else if constexpr (FC32) {
+        fn = frame_kernel<LOG2N, FC32>;
+        threads = Geo<LOG2N>::T;
       } else {
         fn = pair_kernel<LOG2N>;
         threads = kPThreads;
       }
-    } else {
-      fn = frame_kernel<LOG2N, FC32>;
-      threads = Geo<LOG2N>::T;
     }
   } else {
     // symbol rows to memory: two rows at once where the bulk copies can bring
@@ -153,6 +154,7 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
     }
   } else {
     if (q.use_tma == 2) q.use_tma = 0;
+    if (kind == kKindFrame && slot >= 4) q.chunks = q.M;   // an antenna a step
   }
   // raise the kernel's dynamic shared memory limit once per device
   static int limit[10][64] = {};

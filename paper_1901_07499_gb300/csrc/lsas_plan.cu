@@ -382,6 +382,14 @@ lsas_status upload_pilot(lsas_plan p, const double* re, const double* im) {
   return LSAS_OK;
 }
 
+// Whether the plan's fused kernel takes two symbols per step (from rows that
+// bulk copies can bring).
+bool two_symbols(lsas_plan p) {
+  if (!p->twin) return false;
+  if (p->fmt != LSAS_IN_SC16) return p->N == 2048;
+  return p->N >= 1024 || (p->N == 512 && p->M >= 32) || (p->N == 256 && p->M >= 128);
+}
+
 bool aligned16(const void* ptr) { return (reinterpret_cast<uintptr_t>(ptr) & 15u) == 0; }
 
 void base_params(lsas_plan p, KParams* k) {
@@ -396,9 +404,7 @@ void base_params(lsas_plan p, KParams* k) {
   // the data symbols take four groups where the one-symbol kernel needs one
   // at N = 256).  Decided per plan on its total antenna count, so that the
   // antenna shards of a split batch run the same arithmetic as a whole frame.
-  k->twin = (p->twin && p->fmt == LSAS_IN_SC16 &&
-             (p->N >= 1024 || (p->N == 512 && p->M >= 32) || (p->N == 256 && p->M >= 128)))
-                ? 1 : 0;
+  k->twin = two_symbols(p) ? 1 : 0;
   k->tc_w1 = p->d_tc_w1;
   k->sms = p->sms;
   k->M = p->M;
@@ -498,9 +504,9 @@ lsas_status launch_frame(lsas_plan p, const void* d_in, int n_frames, float* d_H
 // from all groups' to one's).  A single frame of 64 antennas at N = 1024: 8 x 13
 // blocks of one step 11 us, 8 x 4 of up to three 17.
 int grid_layers(lsas_plan p, const KParams& k, int nf, int G) {
-  if (p->N > 1024 && p->fmt != LSAS_IN_SC16) return 0;   // frame_kernel
   const long blocks = static_cast<long>(nf) * G;
   const bool twin = k.twin && k.use_tma == 1;
+  if (p->N > 1024 && p->fmt != LSAS_IN_SC16 && !twin) return 0;   // frame_kernel
   const int groups = p->geo.hybrid ? p->geo.groups : twin ? twin_groups(p->D) : p->geo.groups;
   const int pilot = k.H_in ? 0 : 1;
   auto steps = [&](int z) {   // of the longest part
@@ -522,9 +528,9 @@ int grid_layers(lsas_plan p, const KParams& k, int nf, int G) {
 // shards only (one launch), each with at least one antenna per pipeline of
 // the fused kernel, nf G within cap; 1 when no split saves 10 % of the wave.
 int best_shards(lsas_plan p, int nf, long cap) {
-  const int pipes = p->N <= 1024 ? wgeo_warps(p->fmt == LSAS_IN_SC16 ? 4 : 8)
-                                  : (p->fmt == LSAS_IN_SC16 ? kPPairs : 1);
-  const int min_ant = pipes * p->geo.Af;
+  const bool pairs = p->N > 1024 && (p->fmt == LSAS_IN_SC16 || two_symbols(p));
+  const int min_ant = pairs ? kPPairs
+                            : (p->N <= 1024 ? wgeo_warps(p->fmt == LSAS_IN_SC16 ? 4 : 8) : 1) * p->geo.Af;
   const double fixed = p->N > 1024 ? kBlockFixedPair : kBlockFixedWarp;
   double best = 0.9;
   int bestG = 1;

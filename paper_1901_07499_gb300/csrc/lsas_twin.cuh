@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int f = blockIdx.x;
   const int tid = threadIdx.x;
-  const int warp = tid >> 5;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // known uniform: see twinpair_kernel
   const int lane = tid & 31;
   const int team = lane / L;    // antenna of the chunk
   const int jt = lane % L;      // FFT team thread
@@ -779,7 +779,7 @@ template <int LOG2N, bool EST>
 __global__ void __launch_bounds__(kTwThreads, 1) twin_rows_kernel(const KParams p) {
   constexpr int N = 1 << LOG2N, L = N / 32, A = 32 / L, K = kTwSlots;
   extern __shared__ __align__(128) unsigned char smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int team = lane / L, jt = lane % L;
   const TwLayout lay = make_twlayout();
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem) + warp * kMaxSlots;

@@ -1,4 +1,4 @@
-// lsas_twinpair.cuh -- fused receiver for N = 2048 from sc16 rows: pairs of
+// lsas_twinpair.cuh -- fused receiver for N = 2048: pairs of
 // warps as pipelines that transform two OFDM symbols of one antenna per step,
 // in split real / imaginary form.
 //
@@ -28,6 +28,12 @@
 // final write -> read.  Middle read -> final write needs only the warp's own
 // order: each warp writes its final-exchange outputs over the cells that it
 // alone read in the middle exchange.
+// Float samples (FC32) fill a slot with one row, so a pair's two slots hold
+// one step: symbol a in the first, b in the second.  The second is refilled
+// for the next step behind the first barrier, as above; the first, half of
+// the exchange, behind a fourth barrier that follows the final reads, and its
+// copy has the last pass and the MRC to land.  60 frames of 64 antennas: 342
+// (frame_kernel) -> 298 us (fetching that row to L2 ahead was slower, 372).
 // Data-symbol groups as in the N = 1024 two-symbol kernel (the pilot with
 // three data symbols, then four); at a group's end warp w < 4 adds the sums
 // of warp w + 4 (same lane quarter, same subcarriers) in tensor memory, the
@@ -97,6 +103,20 @@ __device__ __forceinline__ void tp_issue(const KParams& p, int f, int m, bool pi
   }
 }
 
+// FC32: copy of one row of a step (item `it` of a group; absent: the phase
+// completes without one) into a slot, by thread 0 of the pair.
+__device__ __forceinline__ void tp_issue_row(const KParams& p, int f, int m, bool pilot_here, int d0,
+                                             int items, int it, unsigned char* slot, uint32_t bar,
+                                             uint64_t pol, int jt) {
+  if (jt == 0) {
+    const bool on = it < items;
+    mbar_expect_tx(bar, on ? 2 * kTpRow : 0);
+    if (on)
+      bulk_load(smem_u32(slot), row_ptr<11, true>(p, f, m, witem_symbol(p, pilot_here, d0, it)),
+                2 * kTpRow, bar, pol);
+  }
+}
+
 // Four radix-8 DFTs of both symbols on register groups i * 8 .. i * 8 + 7
 // (split radix, natural order in and out).
 __device__ __forceinline__ void tp_dft8x4(float2 (&re)[32], float2 (&im)[32]) {
@@ -120,7 +140,7 @@ __device__ __forceinline__ void tp_twiddle(float2& xr, float2& xi, float2 w) {
   xi = i;
 }
 
-template <int LOG2N, bool GIVEN>
+template <int LOG2N, bool GIVEN, bool FC32>
 __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p) {
   static_assert(LOG2N == 11, "the two-symbol pair kernel is written for N = 2048");
   constexpr int N = 1 << LOG2N;
@@ -130,7 +150,13 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
   extern __shared__ __align__(128) unsigned char smem[];
   const int f = blockIdx.x;
   const int tid = threadIdx.x;
-  const int warp = tid >> 5;
+  // broadcast, so that the compiler knows the warp index, and with it the
+  // antenna, row and copy addresses, to be uniform and keeps them out of the
+  // threads' registers, all 254 of which the points, the channel and their
+  // temporaries want: precision workload 3566 -> 3457 us, float samples (which
+  // spilled 264 bytes a step) 370 -> 313, and 0.2 to 4 % of the other kernels'
+  // cases
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int q = warp >> 1;          // pair
   const int jt = tid & 63;          // FFT team thread
   const int pbar = 1 + q;           // the pair's named barrier (0 is the block's)
@@ -179,19 +205,34 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
       // the ring held generic data (last group's reduction): order it before
       // the copies, then fill the first K slots of this group
       fence_proxy_async();
-      int is = slot;
-      for (int s = 0; s < K && to_issue > 0; ++s, --to_issue) {
-        tp_issue(p, f, q + ic * kTpPairs, pilot_here, d0, items, 2 * ipi, stage + is * kTpSlotB,
-                 smem_u32(&bars[is]), pol, jt);
-        // test hook: the first staging phase of block 0 also waits for 16
-        // bytes that no copy delivers, so its bounded wait runs out
-        if (p.fault == 1 && blockIdx.x == 0 && q == 0 && g == 0 && s == 0 && jt == 0)
-          mbar_expect_tx_only(smem_u32(&bars[is]), 16);
-        ++issued;
-        is = (is + 1 == K) ? 0 : is + 1;
-        if (++ipi == npairs) {
-          ipi = 0;
-          ++ic;
+      if constexpr (FC32) {
+        if (to_issue > 0) {
+          tp_issue_row(p, f, q, pilot_here, d0, items, 0, stage, smem_u32(&bars[0]), pol, jt);
+          tp_issue_row(p, f, q, pilot_here, d0, items, 1, stage + kTpSlotB, smem_u32(&bars[1]), pol, jt);
+          if (p.fault == 1 && blockIdx.x == 0 && q == 0 && g == 0 && jt == 0)
+            mbar_expect_tx_only(smem_u32(&bars[0]), 16);
+          ++issued;
+          --to_issue;
+          if (++ipi == npairs) {
+            ipi = 0;
+            ++ic;
+          }
+        }
+      } else {
+        int is = slot;
+        for (int s = 0; s < K && to_issue > 0; ++s, --to_issue) {
+          tp_issue(p, f, q + ic * kTpPairs, pilot_here, d0, items, 2 * ipi, stage + is * kTpSlotB,
+                   smem_u32(&bars[is]), pol, jt);
+          // test hook: the first staging phase of block 0 also waits for 16
+          // bytes that no copy delivers, so its bounded wait runs out
+          if (p.fault == 1 && blockIdx.x == 0 && q == 0 && g == 0 && s == 0 && jt == 0)
+            mbar_expect_tx_only(smem_u32(&bars[is]), 16);
+          ++issued;
+          is = (is + 1 == K) ? 0 : is + 1;
+          if (++ipi == npairs) {
+            ipi = 0;
+            ++ic;
+          }
         }
       }
     }
@@ -241,38 +282,62 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
       }
       for (int ip = 0; ip < npairs; ++ip) {
         float2 re[32], im[32];
-        wait_slot(smem_u32(&bars[slot]), phase, abort_flag, p.status);
-        unsigned char* const yslot = stage + slot * kTpSlotB;
+        // (FC32: both slots, one row each)
+        wait_slot(smem_u32(&bars[FC32 ? 0 : slot]), phase, abort_flag, p.status);
+        if constexpr (FC32) wait_slot(smem_u32(&bars[1]), phase, abort_flag, p.status);
+        unsigned char* const yslot = FC32 ? stage : stage + slot * kTpSlotB;
         const uint32_t ybar = smem_u32(&bars[slot]);
-        {
-          // both rows; a missing second row leaves earlier contents of the
-          // slot (finite values), whose transform is not used
-          const uint32_t* sa = reinterpret_cast<const uint32_t*>(yslot);
-          const uint32_t* sb = sa + kTpRow / 4;
+        bool refill = false;   // FC32: the next step's copies are issued in this one
+        if constexpr (FC32) {
+          // both rows; a missing second row leaves earlier samples in its
+          // slot, whose transform is not used
+          const float2* sa = reinterpret_cast<const float2*>(stage);
+          const float2* sb = reinterpret_cast<const float2*>(stage + kTpSlotB);
 #pragma unroll
           for (int r = 0; r < 32; ++r) {
-            // sc16 -> float v + 2^23 + 32768 exactly: sign bits flipped to
-            // offset binary, each half placed under the exponent bytes of
-            // 2^23 (the offset leaves where pass 1 first adds two samples)
-            const uint32_t ua = sa[jt + 64 * r] ^ 0x80008000u;
-            const uint32_t ub = sb[jt + 64 * r] ^ 0x80008000u;
-            re[r] = make_float2(__uint_as_float(__byte_perm(ua, 0x4b000000u, 0x7610)),
-                                __uint_as_float(__byte_perm(ub, 0x4b000000u, 0x7610)));
-            im[r] = make_float2(__uint_as_float(__byte_perm(ua, 0x4b000000u, 0x7632)),
-                                __uint_as_float(__byte_perm(ub, 0x4b000000u, 0x7632)));
+            const float2 a = sa[jt + 64 * r], b = sb[jt + 64 * r];
+            re[r] = make_float2(a.x, b.x);
+            im[r] = make_float2(a.y, b.y);
+          }
+          phase ^= 1;
+        } else {
+          {
+            // both rows; a missing second row leaves earlier contents of the
+            // slot (finite values), whose transform is not used
+            const uint32_t* sa = reinterpret_cast<const uint32_t*>(yslot);
+            const uint32_t* sb = sa + kTpRow / 4;
+#pragma unroll
+            for (int r = 0; r < 32; ++r) {
+              // sc16 -> float v + 2^23 + 32768 exactly: sign bits flipped to
+              // offset binary, each half placed under the exponent bytes of
+              // 2^23 (the offset leaves where pass 1 first adds two samples)
+              const uint32_t ua = sa[jt + 64 * r] ^ 0x80008000u;
+              const uint32_t ub = sb[jt + 64 * r] ^ 0x80008000u;
+              re[r] = make_float2(__uint_as_float(__byte_perm(ua, 0x4b000000u, 0x7610)),
+                                  __uint_as_float(__byte_perm(ub, 0x4b000000u, 0x7610)));
+              im[r] = make_float2(__uint_as_float(__byte_perm(ua, 0x4b000000u, 0x7632)),
+                                  __uint_as_float(__byte_perm(ub, 0x4b000000u, 0x7632)));
+            }
+          }
+          if (++slot == K) {
+            slot = 0;
+            phase ^= 1;
           }
         }
-        if (++slot == K) {
-          slot = 0;
-          phase ^= 1;
-        }
         // pass 1: 32-point DFTs over n1 (n = jt + 64 n1); output k1 = r
-        twin_dft32_sr<true>(re, im);
+        twin_dft32_sr<!FC32>(re, im);
         // B0: both warps have read this step's slot and finished the previous
         // step's reads: the previous slot is refilled, and this step's slot
         // and the exchange region take the middle exchange
         bar_sync(pbar, 64);
-        if (prev_slot && to_issue > 0 && !*abort_flag) {
+        if constexpr (FC32) {
+          refill = to_issue > 0 && !*abort_flag;
+          if (refill) {
+            fence_proxy_async();
+            tp_issue_row(p, f, q + ic * kTpPairs, pilot_here, d0, items, 2 * ipi + 1, stage + kTpSlotB,
+                         smem_u32(&bars[1]), pol, jt);
+          }
+        } else if (prev_slot && to_issue > 0 && !*abort_flag) {
           ++issued;
           fence_proxy_async();
           tp_issue(p, f, q + ic * kTpPairs, pilot_here, d0, items, 2 * ipi, prev_slot, prev_bar, pol,
@@ -343,6 +408,20 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
             re[i * 8 + r] = make_float2(v.x, v.y);
             im[i * 8 + r] = make_float2(v.z, v.w);
             if (r > 0) tp_twiddle(re[i * 8 + r], im[i * 8 + r], twl[(r - 1) * 256 + jt + 64 * i]);
+          }
+        }
+        if constexpr (FC32) {
+          bar_sync(pbar, 64);   // B3: the first slot's exchange half is read
+          if (refill) {
+            ++issued;
+            fence_proxy_async();
+            tp_issue_row(p, f, q + ic * kTpPairs, pilot_here, d0, items, 2 * ipi, stage,
+                         smem_u32(&bars[0]), pol, jt);
+            --to_issue;
+            if (++ipi == npairs) {
+              ipi = 0;
+              ++ic;
+            }
           }
         }
         // last pass: register e holds bin bin_of(jt, e)
@@ -522,9 +601,16 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
     // a wait gave up: give any copy of this pair still in flight a bounded
     // chance to land before the block's shared memory is released (copies
     // stop being issued after the abort: only the issued steps count)
-    for (int s = 0; s < K && s < issued; ++s) {
-      const int last = issued - 1 - ((issued - 1 - s) % K);
-      (void)mbar_wait_bounded(smem_u32(&bars[last % K]), (last / K) & 1);
+    if constexpr (FC32) {
+      if (issued > 0) {
+        (void)mbar_wait_bounded(smem_u32(&bars[0]), (issued - 1) & 1);
+        (void)mbar_wait_bounded(smem_u32(&bars[1]), (issued - 1) & 1);
+      }
+    } else {
+      for (int s = 0; s < K && s < issued; ++s) {
+        const int last = issued - 1 - ((issued - 1 - s) % K);
+        (void)mbar_wait_bounded(smem_u32(&bars[last % K]), (last / K) & 1);
+      }
     }
   }
   tmem_fence_before();

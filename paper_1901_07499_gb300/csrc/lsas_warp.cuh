@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(32 * wgeo_warps(FC32 ? 8 : 4), 1) warp_kernel(
   const int bx = blockIdx.x, sx = bx - p.full;
   const int f = sx < 0 ? bx : p.full + sx / p.zsplit;
   const int tid = threadIdx.x;
-  const int warp = tid >> 5;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // known uniform: see twinpair_kernel
   const int lane = tid & 31;
   const int alpha = lane % A;   // antenna of the chunk
   const int jt = lane / A;      // FFT team thread

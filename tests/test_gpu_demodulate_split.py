@@ -114,3 +114,25 @@ def test_recorded_into_a_graph(L):
     # the unsplit and the split sum over antennas differ in their order only
     assert float((eq - want_eq).abs().max()) <= 1e-5 * float(want_eq.abs().max())
     plan.close()
+
+
+@pytest.mark.parametrize("split", [0, 1])
+@pytest.mark.parametrize("M,cp,S,pilot_idx,F", [(1, 16, 2, 1, 1), (5, 144, 3, 0, 2), (4, 2, 8, 7, 3),
+                                                (32, 144, 14, 0, 2), (9, 4, 17, 5, 1)])
+def test_float_rows_n2048(L, M, cp, S, pilot_idx, F, split):
+    """The two-symbol kernel on float rows: one antenna, antennas that leave
+    pairs idle, even and odd numbers of items in a group, the pilot last."""
+    cfg, b = _case((M, 2048, cp, S, pilot_idx, "fc32", F))
+    plan = _plan(L, cfg, b)
+    plan.set_batch_split(split)
+    H, bits, eq = plan.run_frame(to_torch_frames(b), want_eq=True)
+    plan.sync()
+    ref = oracle_run(cfg, b)
+    if M == 1:   # zero forcing: near a fade only H and the slicer are held
+        from tests.parity_util import rel_err, unpack
+        assert rel_err(H.cpu().numpy(), ref.H, axes=(1, 2)).max() <= 1e-4
+        got, _ = oracle.demap(eq.cpu().numpy(), 16, dtype=np.float32)
+        assert np.array_equal(got, unpack(bits.cpu().numpy(), cfg.D, cfg.N, 4))
+    else:
+        check_frame_outputs(cfg, ref, H.cpu().numpy(), bits.cpu().numpy(), eq.cpu().numpy())
+    plan.close()
