@@ -15,86 +15,101 @@
 
 namespace lsas {
 
-// small blocks: a single frame's 13 x 1024 / 8 threads spread over ~26 SMs
-constexpr int kCombineThreads = 64;
+// small blocks: a single frame's 13 x 1024 / 2 threads spread over 52 SMs
+constexpr int kCombineThreads = 128;
 
-// One thread per 8 consecutive points (data symbol d, subcarriers k0..k0+7)
-// of one frame: it reads 64 B of partial sums and 32 B of energies per shard
-// and writes the q bytes those 8 points pack into.  Partials are streamed
-// (read once); energies are re-read once per data symbol and stay in cache.
+// One thread per two consecutive points (data symbol d, subcarriers k0, k0 +
+// 1) of one frame: 16 bytes of partial sums and 8 of energies per shard, so a
+// warp reads and writes consecutive pieces; four neighbouring threads' codes
+// make the q bytes their 8 points pack into.  Bound by memory, and for one
+// frame by latency: the shards' loads are all in flight, and the launch
+// overlaps the shard pass's end (programmatic dependent launch; the wait below
+// comes before anything the shard pass writes is read).  60 frames of N = 2048
+// in 2 shards with z: 13.6 -> 11 us; one frame of N = 1024 in 8: 5.5 -> 3.1, and
+// the pair of launches 19.5 -> 14.3.
+// (Before, a thread took 8 points, its 64-byte pieces apart from its
+// neighbours'.)
 __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const KParams p) {
-  const size_t per_frame = static_cast<size_t>(p.D) * p.N / 8;
+  const size_t per_frame = static_cast<size_t>(p.D) * p.N / 2;   // a multiple of 32
   const size_t t = static_cast<size_t>(blockIdx.x) * kCombineThreads + threadIdx.x;
-  if (t >= per_frame * static_cast<size_t>(p.nframes)) return;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (t >= per_frame * static_cast<size_t>(p.nframes)) return;   // whole warps
   const int f = static_cast<int>(t / per_frame);
-  const size_t r = t % per_frame;   // points 8r .. 8r+7 of the frame's d*N + k
-  const int k0 = static_cast<int>((r * 8) % p.N);
+  const size_t r = t % per_frame;   // points 2r, 2r + 1 of the frame's d*N + k
+  const int k0 = static_cast<int>((r * 2) % p.N);
   const size_t dn = static_cast<size_t>(p.D) * p.N;
-  float2 P[8];
-  float E[8];
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    P[j] = make_float2(0.f, 0.f);
-    E[j] = 0.f;
-  }
+  const float4* Pg = reinterpret_cast<const float4*>(p.P_in + f * dn) + r;
+  const float2* Eg = reinterpret_cast<const float2*>(p.E_in + static_cast<size_t>(f) * p.N + k0);
+  const size_t ps = static_cast<size_t>(p.nframes) * dn / 2, es = static_cast<size_t>(p.nframes) * p.N / 2;
+  float4 P = make_float4(0.f, 0.f, 0.f, 0.f);
+  float2 E = make_float2(0.f, 0.f);
   // unrolled so that several shards' loads are in flight at once (the sums
   // still run in shard order)
-#pragma unroll 4
+#pragma unroll 8
   for (int g = 0; g < p.shards; ++g) {
-    const size_t gf = static_cast<size_t>(g) * p.nframes + f;
-    const float4* Pg = reinterpret_cast<const float4*>(p.P_in + gf * dn + r * 8);
-    const float4* Eg = reinterpret_cast<const float4*>(p.E_in + gf * p.N + k0);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float4 v = __ldcs(Pg + j);
-      P[2 * j].x += v.x;
-      P[2 * j].y += v.y;
-      P[2 * j + 1].x += v.z;
-      P[2 * j + 1].y += v.w;
-    }
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const float4 e = __ldg(Eg + j);
-      E[4 * j] += e.x;
-      E[4 * j + 1] += e.y;
-      E[4 * j + 2] += e.z;
-      E[4 * j + 3] += e.w;
+    const float4 v = __ldcs(Pg + g * ps);
+    const float2 e = __ldg(Eg + g * es);
+    P.x += v.x;
+    P.y += v.y;
+    P.z += v.z;
+    P.w += v.w;
+    E.x += e.x;
+    E.y += e.y;
+  }
+  // zero or non-finite energy: z = 0 and the frame is flagged
+  auto over = [&](float x, float y, float e) {
+    const bool ok = (e > 0.f) && (e <= FLT_MAX);
+    if (!ok) latch(p.status, kStDevice);
+    const float ie = ok ? 1.0f / e : 0.f;
+    return ok ? make_float2(x * ie, y * ie) : make_float2(0.f, 0.f);
+  };
+  const float2 z0 = over(P.x, P.y, E.x), z1 = over(P.z, P.w, E.y);
+  if (p.eq) {
+    float2* z = p.eq + f * dn + 2 * r;
+    if ((reinterpret_cast<uintptr_t>(p.eq) & 15) == 0) {
+      *reinterpret_cast<float4*>(z) = make_float4(z0.x, z0.y, z1.x, z1.y);
+    } else {
+      z[0] = z0;
+      z[1] = z1;
     }
   }
   // one copy of the slicing per constellation, so that it has no branches
   auto codes_of = [&](auto tcount) {
     constexpr int T = decltype(tcount)::value;
-    uint64_t a = 0;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      // zero or non-finite energy: z = 0 and the frame is flagged
-      const bool ok = (E[j] > 0.f) && (E[j] <= FLT_MAX);
-      if (!ok) latch(p.status, kStDevice);
-      const float ie = ok ? 1.0f / E[j] : 0.f;
-      const float2 z = ok ? make_float2(P[j].x * ie, P[j].y * ie) : make_float2(0.f, 0.f);
-      if (p.eq) p.eq[f * dn + r * 8 + j] = z;
-      uint32_t code = gray(count_ge<T>(z.x, p.thr));
-      if (p.axes == 2) code = (code << p.wbits) | gray(count_ge<T>(z.y, p.thr));
-      a = (a << p.q) | code;
-    }
-    return a;
+    auto code = [&](float2 z) {
+      uint32_t c = gray(count_ge<T>(z.x, p.thr));
+      if (p.axes == 2) c = (c << p.wbits) | gray(count_ge<T>(z.y, p.thr));
+      return c;
+    };
+    return (code(z0) << p.q) | code(z1);
   };
-  uint64_t acc;
+  uint32_t c2;
   switch (p.nthr) {
-    case 1: acc = codes_of(std::integral_constant<int, 1>{}); break;
-    case 3: acc = codes_of(std::integral_constant<int, 3>{}); break;
-    case 7: acc = codes_of(std::integral_constant<int, 7>{}); break;
-    default: acc = codes_of(std::integral_constant<int, kMaxThresholds>{}); break;
+    case 1: c2 = codes_of(std::integral_constant<int, 1>{}); break;
+    case 3: c2 = codes_of(std::integral_constant<int, 3>{}); break;
+    case 7: c2 = codes_of(std::integral_constant<int, 7>{}); break;
+    default: c2 = codes_of(std::integral_constant<int, kMaxThresholds>{}); break;
   }
-  uint8_t* dst = p.bits + f * (dn * p.q / 8) + r * p.q;
-  for (int j = 0; j < p.q; ++j) dst[j] = static_cast<uint8_t>(acc >> (8 * (p.q - 1 - j)));
+  const int j = threadIdx.x & 3;   // of the four threads of 8 points
+  uint64_t acc = static_cast<uint64_t>(c2) << ((3 - j) * 2 * p.q);
+  acc |= __shfl_xor_sync(0xffffffffu, acc, 1);
+  acc |= __shfl_xor_sync(0xffffffffu, acc, 2);
+  uint8_t* dst = p.bits + f * (dn * p.q / 8) + (r / 4) * p.q;
+  for (int i = j; i < p.q; i += 4) dst[i] = static_cast<uint8_t>(acc >> (8 * (p.q - 1 - i)));
 }
 
 cudaError_t launch_combine(const KParams& p, cudaStream_t st) {
-  const size_t n = static_cast<size_t>(p.nframes) * p.D * p.N / 8;
-  const unsigned grid = static_cast<unsigned>((n + kCombineThreads - 1) / kCombineThreads);
-  combine_kernel<<<grid, kCombineThreads, 0, st>>>(p);
-  return cudaGetLastError();
+  const size_t n = static_cast<size_t>(p.nframes) * p.D * p.N / 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>((n + kCombineThreads - 1) / kCombineThreads));
+  cfg.blockDim = dim3(kCombineThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, combine_kernel, p);
 }
 
 }  // namespace lsas
