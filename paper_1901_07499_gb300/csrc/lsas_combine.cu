@@ -23,8 +23,7 @@ constexpr int kCombineThreads = 128;
 // warp reads and writes consecutive pieces; four neighbouring threads' codes
 // make the q bytes their 8 points pack into.  Bound by memory, and for one
 // frame by latency: the shards' loads are all in flight, and the launch
-// overlaps the shard pass's end (programmatic dependent launch; the wait below
-// comes before anything the shard pass writes is read).  60 frames of N = 2048
+// overlaps the shard pass's end (pdl_launch).  60 frames of N = 2048
 // in 2 shards with z: 13.6 -> 11 us; one frame of N = 1024 in 8: 5.5 -> 3.1, and
 // the pair of launches 19.5 -> 14.3.
 // (Before, a thread took 8 points, its 64-byte pieces apart from its
@@ -32,7 +31,7 @@ constexpr int kCombineThreads = 128;
 __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const KParams p) {
   const size_t per_frame = static_cast<size_t>(p.D) * p.N / 2;   // a multiple of 32
   const size_t t = static_cast<size_t>(blockIdx.x) * kCombineThreads + threadIdx.x;
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_wait();
   if (t >= per_frame * static_cast<size_t>(p.nframes)) return;   // whole warps
   const int f = static_cast<int>(t / per_frame);
   const size_t r = t % per_frame;   // points 2r, 2r + 1 of the frame's d*N + k
@@ -100,16 +99,8 @@ __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const KParams 
 
 cudaError_t launch_combine(const KParams& p, cudaStream_t st) {
   const size_t n = static_cast<size_t>(p.nframes) * p.D * p.N / 2;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>((n + kCombineThreads - 1) / kCombineThreads));
-  cfg.blockDim = dim3(kCombineThreads);
-  cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, combine_kernel, p);
+  return pdl_launch(combine_kernel, dim3(static_cast<unsigned>((n + kCombineThreads - 1) / kCombineThreads)),
+                    kCombineThreads, 0, st, p);
 }
 
 }  // namespace lsas

@@ -108,6 +108,7 @@ __global__ void __launch_bounds__(256) dn_conv_in_kernel(const float* __restrict
                                                          const float* __restrict__ bias,
                                                          const float* __restrict__ mask,
                                                          float* __restrict__ out, int N) {
+  pdl_wait();
   __shared__ __align__(16) float ws[320];
   const int tiles_row = N / kDnPos;
   const int r = blockIdx.x / tiles_row;
@@ -163,6 +164,7 @@ __global__ void __launch_bounds__(128, 4) dn_conv32_kernel(const float* __restri
                                                            const float* __restrict__ bias,
                                                            const float* __restrict__ mask,
                                                            float* __restrict__ out, int R, int N) {
+  pdl_wait();
   extern __shared__ __align__(128) unsigned char smem[];
   const float* ws = reinterpret_cast<const float*>(smem);
   const int tiles_row = N / kDnPos, tiles = R * tiles_row;
@@ -236,8 +238,8 @@ static cudaError_t conv32(const float* in, const float* wt, const float* bias, c
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, kCvSmem);
   if (e != cudaSuccess) return e;
   const int tiles = R * (N / kDnPos);
-  dn_conv32_kernel<BWD><<<tiles < 4 * sms ? tiles : 4 * sms, 128, kCvSmem, st>>>(in, wt, bias, mask, out,
-                                                                               R, N);
+  pdl_launch(dn_conv32_kernel<BWD>, dim3(tiles < 4 * sms ? tiles : 4 * sms), 128, kCvSmem, st, in,
+             wt, bias, mask, out, R, N);
   return cudaSuccess;
 }
 
@@ -262,6 +264,7 @@ struct DnOutArgs {
 };
 template <bool TRAIN>
 __global__ void __launch_bounds__(256) dn_conv_out_kernel(const DnOutArgs a) {
+  pdl_wait();
   __shared__ float ws[320];
   __shared__ __align__(16) float red[8][2][kDnPos];
   __shared__ float se[8];
@@ -340,6 +343,7 @@ static_assert(kFwSmem >= 128 * 40 * 4, "the halves meet in the stages");
 __global__ void __launch_bounds__(kFwThreads, 2) dn_wgrad32_kernel(const float* __restrict__ G,
                                                                    const float* __restrict__ A, int R,
                                                                    int N, float* __restrict__ part) {
+  pdl_wait();
   extern __shared__ __align__(128) unsigned char smem[];
   const int t = threadIdx.x, lane = t & 31;
   const int half = t >> 7, u = t & 127;
@@ -457,6 +461,7 @@ __global__ void __launch_bounds__(256, 2) dn_side32_kernel(const float* __restri
                                                         const float* __restrict__ g1, int R, int N,
                                                         float* __restrict__ part4,
                                                         float* __restrict__ part1) {
+  pdl_wait();
   const bool layer4 = blockIdx.y == 0;
   const float* __restrict__ T = layer4 ? dy : x0;
   const float* __restrict__ B = layer4 ? r3 : g1;
@@ -572,6 +577,7 @@ template <typename WT>
 __global__ void __launch_bounds__(256) dn_setup_kernel(const WT* __restrict__ P, float* wt,
                                                        const float2* H, const float2* Ht, int N,
                                                        float* x0, float* tt, float* rms) {
+  pdl_wait();
   if (blockIdx.x < kSetupBlocks)
     fp32_weights(P, wt, blockIdx.x * 256 + threadIdx.x, kSetupBlocks * 256);
   else
@@ -580,6 +586,7 @@ __global__ void __launch_bounds__(256) dn_setup_kernel(const WT* __restrict__ P,
 
 __global__ void dn_adam_kernel(float* p, const float* g, float* m, float* v, int n, float lr,
                                float b1, float b2, float eps, float c1, float c2) {
+  pdl_wait();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.f - b1) * gi;
@@ -591,6 +598,7 @@ __global__ void dn_adam_kernel(float* p, const float* g, float* m, float* v, int
 }
 
 __global__ void dn_bf16_kernel(const float* p, __nv_bfloat16* q, int n) {
+  pdl_wait();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
     q[i] = __float2bfloat16_rn(p[i]);
 }
@@ -724,6 +732,7 @@ __global__ void __launch_bounds__(128 * kTcSlots, 2) dn_tc_kernel(const float* _
                                                        const float* __restrict__ x0,
                                                        const float* __restrict__ rms, int R, int N,
                                                        float2* __restrict__ Hout, int* status) {
+  pdl_wait();
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned char* wimg = smem;
   const int t = threadIdx.x;
@@ -925,6 +934,7 @@ __global__ void __launch_bounds__(256) dn_tc_setup_kernel(const PT* __restrict__
                                                           float* bimg, const float2* H,
                                                           const float2* Ht, int N, float* x0,
                                                           float* tt, float* rms) {
+  pdl_wait();
   int b = blockIdx.x;
   if (b < kSetupBlocks) {
     tc_image(P, img, b * 256 + threadIdx.x, kSetupBlocks * 256);
@@ -960,6 +970,7 @@ __global__ void __launch_bounds__(128 * kTcSlots, 2) dn_tc_train_kernel(
     const float* __restrict__ img_g, const float* __restrict__ in0, const float* __restrict__ tt,
     int R, int N, float inv_n, __nv_bfloat16* __restrict__ acts, __nv_bfloat16* __restrict__ grads,
     float* __restrict__ dy, float* __restrict__ part, int* status) {
+  pdl_wait();
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned char* wimg = smem;
   const int t = threadIdx.x;
@@ -1172,10 +1183,11 @@ constexpr int kWgStage = kWgG + 8 * kWgGChunk;
 constexpr int kWgStages = 4;
 constexpr int kWgBars = kWgStages * kWgStage;              // full, empty, done
 constexpr int kWgSmem = kWgBars + (2 * kWgStages + 1) * 8 + 8;
-// warp 0 copies, 1 MMAs, 2 and 3 bias sums, 4-11 layers 1 and 4: twelve warps
-// leave 168 registers a thread, which the loads one tile ahead need
+// warp 0 copies, 1 MMAs, 2 and 3 bias sums, 4-11 layers 1 and 4, 12 the loss: up
+// to 16 warps leave 128 registers a thread, which the loads one tile ahead need
 constexpr int kWgSideWarp = 4;
-constexpr int kWgThreads = 32 * (kWgSideWarp + 8);
+constexpr int kWgLossWarp = kWgSideWarp + 8;
+constexpr int kWgThreads = 32 * (kWgLossWarp + 1);
 static_assert(kWgSmem <= 232448, "shared memory of one block");
 
 // Weight gradient of a layer with a two-channel side, by eight warps:
@@ -1278,9 +1290,14 @@ struct DnWgradArgs {
   const float* dy;
   int R, N;
   float *part3, *part2, *part4, *part1;   // one row per block: kWgPart, kSdPart floats
+  const float* loss_part;                 // the forward pass's sums of (y - t)^2, one per tile
+  int loss_n;
+  size_t n;
+  float* loss;
   int* status;
 };
 __global__ void __launch_bounds__(kWgThreads, 1) dn_tc_wgrad_kernel(const DnWgradArgs a) {
+  pdl_wait();
   extern __shared__ __align__(128) unsigned char smem[];
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + kWgBars);
@@ -1315,7 +1332,31 @@ __global__ void __launch_bounds__(kWgThreads, 1) dn_tc_wgrad_kernel(const DnWgra
     latch(a.status, kStTimeout);
     return false;
   };
-  if (warp >= kWgSideWarp) {
+  if (warp == kWgLossWarp) {
+    // the loss, by one thread: the forward pass's partials added in tile order
+    // (the order it has always had, so the same bits), loads 64 values ahead
+    if (blockIdx.x == gridDim.x - 1 && lane == 0) {
+      const float4* part = reinterpret_cast<const float4*>(a.loss_part);
+      const int n4 = a.loss_n / 4;
+      float4 v[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) v[i] = i < n4 ? part[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+      float s = 0.f;
+      for (int i0 = 0; i0 < n4; i0 += 16) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {   // (a sum of squares plus zero is itself)
+          s += v[i].x;
+          s += v[i].y;
+          s += v[i].z;
+          s += v[i].w;
+          v[i] = i0 + 16 + i < n4 ? part[i0 + 16 + i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      }
+      for (int i = 4 * n4; i < a.loss_n; ++i) s += a.loss_part[i];
+      *a.loss = s / static_cast<float>(a.n);
+    }
+    __syncwarp();
+  } else if (warp >= kWgSideWarp) {
     side_grad<true>(a.dy, a.acts + 2 * plane, R, N,
                     a.part4 + static_cast<size_t>(blockIdx.x) * kSdPart, warp - kWgSideWarp, lane);
     side_grad<false>(a.x0, a.grads + 2 * plane, R, N,
@@ -1433,7 +1474,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) dn_tc_wgrad_kernel(const DnWgra
   if (warp == 1) tmem_dealloc(tD, 256);
 }
 
-// Sums the blocks' partial rows of every weight gradient and the loss
+// Sums the blocks' partial rows of every weight gradient and (FP32) the loss
 // partials, in a fixed order, in one launch.  A block takes 32 columns of one
 // layer's rows: 16 slices of consecutive rows are added side by side (a serial
 // chain of rows / 16 coalesced loads), then the slices in order.  (One thread
@@ -1456,10 +1497,12 @@ constexpr int kRdSlices = 16, kRdThreads = 32 * kRdSlices;
 constexpr int kRdBig = (5120 + 32) / 32, kRdSide = kSdPart / 32;
 constexpr int kRdBlocks = 2 * kRdBig + 2 * kRdSide + 1;
 __global__ void __launch_bounds__(kRdThreads) dn_reduce_kernel(const DnReduceArgs a) {
+  pdl_wait();
   __shared__ float red[kRdSlices][33];
   const int t = threadIdx.x, col32 = t & 31, slice = t >> 5;
   int b = blockIdx.x;
-  if (b == kRdBlocks - 1) {   // the loss: strided sums, then a tree
+  if (b == kRdBlocks - 1) {   // the loss (when asked for): strided sums, then a tree
+    if (!a.loss) return;
     __shared__ float ls[kRdThreads];
     float s = 0.f;
     for (int i = t; i < a.loss_n; i += kRdThreads) s += a.loss_part[i];
@@ -1536,6 +1579,7 @@ __global__ void __launch_bounds__(32 * kLsWarps) dn_ls_rows_kernel(const KParams
                                                                    float* __restrict__ img,
                                                                    unsigned char* __restrict__ xrows,
                                                                    float* __restrict__ rms) {
+  pdl_wait();
   constexpr int N = kLsN;
   if (blockIdx.x < kLsImgBlocks) {
     tc_image(P, img, blockIdx.x * 32 * kLsWarps + threadIdx.x, kLsImgBlocks * 32 * kLsWarps);
@@ -1586,6 +1630,7 @@ __global__ void __launch_bounds__(128 * kTcSlots, 2) dn_xtc_kernel(const float* 
                                                         const unsigned char* __restrict__ xrows,
                                                         const float* __restrict__ rms, int R,
                                                         float2* __restrict__ Hout, int* status) {
+  pdl_wait();
   constexpr int N = kLsN;
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned char* wimg = smem;
@@ -1772,7 +1817,8 @@ static DnWork dn_work(float* w, int R, int N) {
 
 // layers 1 to 3 on the CUDA cores (biases b1, b2, b3 in fp32)
 static cudaError_t forward(const float* b, const DnWork& d, int R, int N, int sms, cudaStream_t st) {
-  dn_conv_in_kernel<false><<<R * (N / kDnPos), 256, 0, st>>>(d.x0, d.wt + kFw1, b, nullptr, d.a1, N);
+  pdl_launch(dn_conv_in_kernel<false>, dim3(R * (N / kDnPos)), 256, 0, st, d.x0, d.wt + kFw1, b,
+             nullptr, d.a1, N);
   cudaError_t e = conv32<false>(d.a1, d.wt + kFw2, b + 32, nullptr, d.a2, R, N, sms, st);
   if (e == cudaSuccess) e = conv32<false>(d.a2, d.wt + kFw3, b + 64, nullptr, d.a3, R, N, sms, st);
   return e;
@@ -1782,11 +1828,11 @@ cudaError_t dn_apply(const void* params, bool bf16, const float2* H, int R, int 
                      float2* Hout, int sms, cudaStream_t st) {
   const DnWork d = dn_work(work, R, N);
   if (bf16)
-    dn_setup_kernel<<<kSetupBlocks + R, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(params), d.wt,
-                                                      H, nullptr, N, d.x0, nullptr, d.rms);
+    pdl_launch(dn_setup_kernel<__nv_bfloat16>, dim3(kSetupBlocks + R), 256, 0, st,
+               static_cast<const __nv_bfloat16*>(params), d.wt, H, nullptr, N, d.x0, nullptr, d.rms);
   else
-    dn_setup_kernel<<<kSetupBlocks + R, 256, 0, st>>>(static_cast<const float*>(params), d.wt, H,
-                                                      nullptr, N, d.x0, nullptr, d.rms);
+    pdl_launch(dn_setup_kernel<float>, dim3(kSetupBlocks + R), 256, 0, st,
+               static_cast<const float*>(params), d.wt, H, nullptr, N, d.x0, nullptr, d.rms);
   const float* b = d.wt + kBias;
   const cudaError_t e = forward(b, d, R, N, sms, st);
   if (e != cudaSuccess) return e;
@@ -1798,7 +1844,7 @@ cudaError_t dn_apply(const void* params, bool bf16, const float2* H, int R, int 
   a.rms = d.rms;
   a.Hout = Hout;
   a.N = N;
-  dn_conv_out_kernel<false><<<R * (N / kDnPos), 256, 0, st>>>(a);
+  pdl_launch(dn_conv_out_kernel<false>, dim3(R * (N / kDnPos)), 256, 0, st, a);
   return cudaGetLastError();
 }
 
@@ -1813,13 +1859,14 @@ cudaError_t dn_apply_tc(const void* params_bf16, const float2* H, int R, int N, 
     attr = true;
   }
   const auto* P = static_cast<const __nv_bfloat16*>(params_bf16);
-  dn_tc_setup_kernel<<<kSetupBlocks + R, 256, 0, st>>>(P, d.img, nullptr, H, nullptr, N, d.x0,
-                                                       nullptr, d.rms);
+  pdl_launch(dn_tc_setup_kernel<__nv_bfloat16>, dim3(kSetupBlocks + R), 256, 0, st, P, d.img,
+             nullptr, H, nullptr, N, d.x0, nullptr, d.rms);
   // two blocks fit per SM (shared memory and the launch bounds' register cap)
   const int tiles = R * ((N + kTcValid - 1) / kTcValid);
   const int want = (tiles + kTcSlots - 1) / kTcSlots;
   const int grid = want < sms * 2 ? want : sms * 2;
-  dn_tc_kernel<<<grid, 128 * kTcSlots, kTcSmem, st>>>(d.img, d.x0, d.rms, R, N, Hout, status);
+  pdl_launch(dn_tc_kernel, dim3(grid), 128 * kTcSlots, kTcSmem, st, d.img, d.x0, d.rms, R, N, Hout,
+             status);
   return cudaGetLastError();
 }
 
@@ -1843,12 +1890,13 @@ cudaError_t dn_ls_tc(const KParams& k, const void* params_bf16, int n_frames, fl
   }
   const auto* P = static_cast<const __nv_bfloat16*>(params_bf16);
   auto* xrows = reinterpret_cast<unsigned char*>(d.x0);
-  dn_ls_rows_kernel<<<kLsImgBlocks + (R + kLsWarps - 1) / kLsWarps, 32 * kLsWarps, kLsSmem, st>>>(
-      k, R, P, d.img, xrows, d.rms);
+  pdl_launch(dn_ls_rows_kernel, dim3(kLsImgBlocks + (R + kLsWarps - 1) / kLsWarps), 32 * kLsWarps,
+             kLsSmem, st, k, R, P, d.img, xrows, d.rms);
   const int tiles = R * ((kLsN + kTcValid - 1) / kTcValid);
   const int want = (tiles + kTcSlots - 1) / kTcSlots;
   const int grid = want < sms * 2 ? want : sms * 2;
-  dn_xtc_kernel<<<grid, 128 * kTcSlots, kXtSmem, st>>>(d.img, xrows, d.rms, R, Hout, status);
+  pdl_launch(dn_xtc_kernel, dim3(grid), 128 * kTcSlots, kXtSmem, st, d.img, xrows, d.rms, R, Hout,
+             status);
   return cudaGetLastError();
 }
 
@@ -1858,7 +1906,8 @@ cudaError_t dn_grad(const float* P, const float2* Hls, const float2* Ht, int R, 
   cudaError_t e =
       cudaFuncSetAttribute(dn_wgrad32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwSmem);
   if (e != cudaSuccess) return e;
-  dn_setup_kernel<<<kSetupBlocks + R, 256, 0, st>>>(P, d.wt, Hls, Ht, N, d.x0, d.tt, d.rms);
+  pdl_launch(dn_setup_kernel<float>, dim3(kSetupBlocks + R), 256, 0, st, P, d.wt, Hls, Ht, N, d.x0,
+             d.tt, d.rms);
   const float* b = d.wt + kBias;
   e = forward(b, d, R, N, sms, st);
   if (e != cudaSuccess) return e;
@@ -1874,7 +1923,7 @@ cudaError_t dn_grad(const float* P, const float2* Hls, const float2* Ht, int R, 
   o.part = d.y;
   o.inv_n = 2.0f / static_cast<float>(n);
   o.N = N;
-  dn_conv_out_kernel<true><<<tiles, 256, 0, st>>>(o);
+  pdl_launch(dn_conv_out_kernel<true>, dim3(tiles), 256, 0, st, o);
   // two blocks of the weight-gradient kernels per SM
   const int parts = wg_blocks(R, N);
   const int wgb = 2 * sms < parts ? 2 * sms : parts;
@@ -1883,15 +1932,16 @@ cudaError_t dn_grad(const float* P, const float2* Hls, const float2* Ht, int R, 
   float* sp4 = wp2 + static_cast<size_t>(parts) * kWgPart;
   float* sp1 = sp4 + static_cast<size_t>(parts) * kSdPart;
   // layer 3: g3 = conv(dy; W4') masked -> g1; layer 2: g2 -> g2; layer 1: g1 -> g1
-  dn_conv_in_kernel<true><<<tiles, 256, 0, st>>>(d.dy, d.wt + kBw4, nullptr, d.a3, d.g1, N);
-  dn_wgrad32_kernel<<<wgb, kFwThreads, kFwSmem, st>>>(d.g1, d.a2, R, N, wp3);
+  pdl_launch(dn_conv_in_kernel<true>, dim3(tiles), 256, 0, st, d.dy, d.wt + kBw4, nullptr, d.a3,
+             d.g1, N);
+  pdl_launch(dn_wgrad32_kernel, dim3(wgb), kFwThreads, kFwSmem, st, d.g1, d.a2, R, N, wp3);
   e = conv32<true>(d.g1, d.wt + kBw3, nullptr, d.a2, d.g2, R, N, sms, st);
   if (e != cudaSuccess) return e;
-  dn_wgrad32_kernel<<<wgb, kFwThreads, kFwSmem, st>>>(d.g2, d.a1, R, N, wp2);
+  pdl_launch(dn_wgrad32_kernel, dim3(wgb), kFwThreads, kFwSmem, st, d.g2, d.a1, R, N, wp2);
   e = conv32<true>(d.g2, d.wt + kBw2, nullptr, d.a1, d.g1, R, N, sms, st);
   if (e != cudaSuccess) return e;
-  dn_side32_kernel<<<dim3(wgb, 2), 256, 0, st>>>(d.dy, d.a3, d.x0, d.g1, R, N, sp4, sp1);
-  DnReduceArgs a;
+  pdl_launch(dn_side32_kernel, dim3(wgb, 2), 256, 0, st, d.dy, d.a3, d.x0, d.g1, R, N, sp4, sp1);
+  DnReduceArgs a{};
   a.l[0] = {wp3, wgb, kWgPart, grad + kOffW3, grad + kOffB3};
   a.l[1] = {wp2, wgb, kWgPart, grad + kOffW2, grad + kOffB2};
   a.l[2] = {sp4, wgb, kSdPart, grad + kOffW4, grad + kOffB4};
@@ -1900,7 +1950,7 @@ cudaError_t dn_grad(const float* P, const float2* Hls, const float2* Ht, int R, 
   a.loss_n = tiles;
   a.n = n;
   a.loss = loss;
-  dn_reduce_kernel<<<kRdBlocks, kRdThreads, 0, st>>>(a);
+  pdl_launch(dn_reduce_kernel, dim3(kRdBlocks), kRdThreads, 0, st, a);
   return cudaGetLastError();
 }
 
@@ -1921,8 +1971,8 @@ cudaError_t dn_grad_tc(const float* P32, const float2* Hls, const float2* Ht, in
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  dn_tc_setup_kernel<<<2 * kSetupBlocks + R, 256, 0, st>>>(P32, d.img, d.bimg, Hls, Ht, N, d.x0,
-                                                           d.tt, d.rms);
+  pdl_launch(dn_tc_setup_kernel<float>, dim3(2 * kSetupBlocks + R), 256, 0, st, P32, d.img, d.bimg,
+             Hls, Ht, N, d.x0, d.tt, d.rms);
   const size_t n = static_cast<size_t>(R) * 2 * N;
   const int tiles = R * ((N + kTcValid - 1) / kTcValid);
   const int want = (tiles + kTcSlots - 1) / kTcSlots;
@@ -1930,10 +1980,10 @@ cudaError_t dn_grad_tc(const float* P32, const float2* Hls, const float2* Ht, in
   auto* acts = reinterpret_cast<__nv_bfloat16*>(d.a1);
   auto* grads = reinterpret_cast<__nv_bfloat16*>(d.g1);
   const size_t plane = tr_plane(R, N);
-  dn_tc_train_kernel<false><<<grid, 128 * kTcSlots, kTrSmem, st>>>(
-      d.img, d.x0, d.tt, R, N, 2.0f / static_cast<float>(n), acts, nullptr, d.dy, d.y, status);
-  dn_tc_train_kernel<true><<<grid, 128 * kTcSlots, kTrSmem, st>>>(
-      d.bimg, d.dy, nullptr, R, N, 0.f, acts, grads, nullptr, nullptr, status);
+  pdl_launch(dn_tc_train_kernel<false>, dim3(grid), 128 * kTcSlots, kTrSmem, st, d.img, d.x0, d.tt,
+             R, N, 2.0f / static_cast<float>(n), acts, nullptr, d.dy, d.y, status);
+  pdl_launch(dn_tc_train_kernel<true>, dim3(grid), 128 * kTcSlots, kTrSmem, st, d.bimg, d.dy,
+             nullptr, R, N, 0.f, acts, grads, nullptr, nullptr, status);
   const int parts = wg_blocks(R, N);
   float* wp3 = d.wp;
   float* wp2 = wp3 + static_cast<size_t>(parts) * kWgPart;
@@ -1952,17 +2002,18 @@ cudaError_t dn_grad_tc(const float* P32, const float2* Hls, const float2* Ht, in
   w.part4 = sp4;
   w.part1 = sp1;
   w.status = status;
-  dn_tc_wgrad_kernel<<<wgb, kWgThreads, kWgSmem, st>>>(w);
-  DnReduceArgs a;
+  w.loss_part = d.y;
+  w.loss_n = tiles;
+  w.n = n;
+  w.loss = loss;
+  pdl_launch(dn_tc_wgrad_kernel, dim3(wgb), kWgThreads, kWgSmem, st, w);
+  DnReduceArgs a{};
   a.l[0] = {wp3, wgb, kWgPart, grad + kOffW3, grad + kOffB3};
   a.l[1] = {wp2, wgb, kWgPart, grad + kOffW2, grad + kOffB2};
   a.l[2] = {sp4, wgb, kSdPart, grad + kOffW4, grad + kOffB4};
   a.l[3] = {sp1, wgb, kSdPart, grad + kOffW1, grad + kOffB1};
-  a.loss_part = d.y;
-  a.loss_n = tiles;
-  a.n = n;
-  a.loss = loss;
-  dn_reduce_kernel<<<kRdBlocks, kRdThreads, 0, st>>>(a);
+  a.loss = nullptr;   // written by the launch above
+  pdl_launch(dn_reduce_kernel, dim3(kRdBlocks), kRdThreads, 0, st, a);
   return cudaGetLastError();
 }
 
@@ -1970,12 +2021,12 @@ cudaError_t dn_adam(float* p, const float* g, float* m, float* v, int step, floa
                     float b2, float eps, cudaStream_t st) {
   const float c1 = 1.f - powf(b1, static_cast<float>(step));
   const float c2 = 1.f - powf(b2, static_cast<float>(step));
-  dn_adam_kernel<<<44, 256, 0, st>>>(p, g, m, v, kDnParams, lr, b1, b2, eps, c1, c2);
+  pdl_launch(dn_adam_kernel, dim3(44), 256, 0, st, p, g, m, v, kDnParams, lr, b1, b2, eps, c1, c2);
   return cudaGetLastError();
 }
 
 cudaError_t dn_to_bf16(const float* p, void* q, cudaStream_t st) {
-  dn_bf16_kernel<<<44, 256, 0, st>>>(p, static_cast<__nv_bfloat16*>(q), kDnParams);
+  pdl_launch(dn_bf16_kernel, dim3(44), 256, 0, st, p, static_cast<__nv_bfloat16*>(q), kDnParams);
   return cudaGetLastError();
 }
 

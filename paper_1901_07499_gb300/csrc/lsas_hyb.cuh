@@ -142,6 +142,7 @@ struct HyCursor {
 
 template <bool FC32>
 __global__ void __launch_bounds__(kHyThreads, 1) hyb_kernel(const KParams p) {
+  pdl_wait();
   static_assert(!FC32, "the tensor-core kernel stages sc16 rows");
   constexpr int N = 1024;
   extern __shared__ __align__(128) unsigned char smem[];

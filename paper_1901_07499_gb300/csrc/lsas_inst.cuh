@@ -167,7 +167,7 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
     if (dev >= 0 && dev < 64) limit[slot][dev] = smem;
   }
   const int gz = q.group_z > 0 ? q.group_z : 1;
-  fn<<<dim3(grid, p.grid_y > 1 ? p.grid_y : 1, gz), threads, smem, st>>>(q);
+  pdl_launch(fn, dim3(grid, p.grid_y > 1 ? p.grid_y : 1, gz), threads, smem, st, q);
   return cudaGetLastError();
 }
 

@@ -293,6 +293,12 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src,
       "l"(src), "r"(bytes), "r"(bar), "l"(policy)
       : "memory");
 }
+// Programmatic dependent launch: a kernel launched by pdl_launch may be set up
+// while the one before it in the stream still runs its last blocks, and calls
+// pdl_wait before anything else, which returns when every earlier kernel has
+// completed and its writes are visible (every kernel launched so waits, so the
+// order reaches back through all of them).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ uint64_t evict_last_policy() {
   uint64_t pol;
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
@@ -940,6 +946,7 @@ enum { kBarFull0 = 1, kBarEmpty0 = 3, kBarProd = 5 };
 
 template <int LOG2N, bool FC32>
 __global__ void __launch_bounds__(Geo<LOG2N>::T, 1) frame_kernel(const KParams p) {
+  pdl_wait();
   using G = Geo<LOG2N>;
   constexpr int N = G::N, A = G::A, T = G::T, TW = G::TW, F = G::F, W = G::W;
   constexpr int OWN = G::OWN;
@@ -1263,6 +1270,7 @@ __global__ void __launch_bounds__(Geo<LOG2N>::T, 1) frame_kernel(const KParams p
 // One warp group per block: antenna chunk c of frame f.
 template <int LOG2N, bool FC32>
 __global__ void __launch_bounds__(Geo<LOG2N>::TW) estimate_kernel(const KParams p) {
+  pdl_wait();
   using G = Geo<LOG2N>;
   constexpr int N = G::N, A = G::A, F = G::F;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -1324,6 +1332,7 @@ __global__ void __launch_bounds__(Geo<LOG2N>::TW) estimate_kernel(const KParams 
 // One warp group per block: antenna chunk c of frame f, every symbol.
 template <int LOG2N, bool FC32>
 __global__ void __launch_bounds__(Geo<LOG2N>::TW) fft_kernel(const KParams p) {
+  pdl_wait();
   using G = Geo<LOG2N>;
   constexpr int N = G::N, A = G::A, F = G::F;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -1394,6 +1403,24 @@ __global__ void __launch_bounds__(Geo<LOG2N>::TW) fft_kernel(const KParams p) {
 }
 
 #endif  // __CUDACC__
+
+// Launch with programmatic stream serialization (see pdl_wait).  It takes the
+// launch's latency, 1 to 2 us, out of the gap between two kernels.
+template <typename... P, typename... A>
+inline cudaError_t pdl_launch(void (*fn)(P...), dim3 grid, int threads, int smem, cudaStream_t st,
+                              A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
+}
 
 // Host-side launch entry of one FFT length (defined in lsas_inst_n*.cu).
 using LaunchFn = cudaError_t (*)(int kind, bool fc32, const KParams& p, int grid,

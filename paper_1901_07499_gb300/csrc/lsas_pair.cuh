@@ -70,6 +70,7 @@ __host__ __device__ constexpr int pgeo_dg_max() { return (kPTmemWarp - kPOwn) / 
 
 template <int LOG2N>
 __global__ void __launch_bounds__(kPThreads, 1) pair_kernel(const KParams p) {
+  pdl_wait();
   constexpr int N = 1 << LOG2N;
   static_assert(N == kPN, "the pair kernel covers N = 2048");
   constexpr int OWN = kPOwn;

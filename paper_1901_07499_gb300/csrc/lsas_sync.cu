@@ -45,6 +45,7 @@ __host__ __device__ constexpr int pn_smem(int ap) {
 // and one shared-memory operand pair per FMA took 425 us.
 template <bool FC32, int AP>
 __global__ void __launch_bounds__(kPnThreads, 2) pn_kernel(const KParams p) {
+  pdl_wait();
   constexpr int LAGS = pn_lags(AP), ROW = pn_row(AP);
   static_assert(LAGS <= kPnThreads, "one thread per lag adds the powers");
   extern __shared__ __align__(128) unsigned char smem[];
@@ -203,6 +204,7 @@ __global__ void __launch_bounds__(kPnThreads, 2) pn_kernel(const KParams p) {
 // per load.
 template <bool FC32>
 __global__ void __launch_bounds__(256) extract_kernel(const KParams p) {
+  pdl_wait();
   constexpr int WPS = FC32 ? 2 : 1;   // 32-bit words per sample
   const int fm = blockIdx.x;
   const int f = fm / p.M;
@@ -248,6 +250,7 @@ __global__ void __launch_bounds__(256) extract_kernel(const KParams p) {
 
 // fftshift of complex rows of N (swap the halves of every row).
 __global__ void shift_c64_kernel(float2* buf, size_t rows, int N) {
+  pdl_wait();
   const size_t half = static_cast<size_t>(N / 2);
   const size_t n = rows * half;
   for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < n;
@@ -262,6 +265,7 @@ __global__ void shift_c64_kernel(float2* buf, size_t rows, int N) {
 
 // fftshift of packed bit rows (one data symbol = N q bits): swap the halves.
 __global__ void shift_bytes_kernel(uint8_t* buf, size_t rows, int rowbytes) {
+  pdl_wait();
   const size_t half = static_cast<size_t>(rowbytes / 2);
   const size_t n = rows * half;
   for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < n;
@@ -292,11 +296,13 @@ static cudaError_t launch_pn_t(KParams p, int n_frames, int sms, cudaStream_t st
   cfg.blockDim = dim3(kPnThreads);
   cfg.dynamicSmemBytes = pn_smem(AP);
   cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim = {static_cast<unsigned>(blocks), 1, 1};
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim = {static_cast<unsigned>(blocks), 1, 1};
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // as pdl_launch
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, pn_kernel<FC32, AP>, p);
 }
 
@@ -319,16 +325,18 @@ cudaError_t launch_extract(const KParams& p, bool fc32, int n_frames, int sms, c
   const int vecs = p.S * (p.N + p.cp) * (fc32 ? 2 : 1) / 4;
   int split = 1;
   while (static_cast<long>(rows) * split < 8L * sms && split * 2 * 256 <= vecs) split *= 2;
-  if (fc32) extract_kernel<true><<<dim3(rows, split), 256, 0, st>>>(p);
-  else extract_kernel<false><<<dim3(rows, split), 256, 0, st>>>(p);
+  if (fc32) pdl_launch(extract_kernel<true>, dim3(rows, split), 256, 0, st, p);
+  else pdl_launch(extract_kernel<false>, dim3(rows, split), 256, 0, st, p);
   return cudaGetLastError();
 }
 
 cudaError_t launch_shift(void* buf, int kind, size_t rows, int N, int rowbytes, int sms,
                          cudaStream_t st) {
   const int grid = sms * 4;
-  if (kind == 0) shift_c64_kernel<<<grid, 256, 0, st>>>(static_cast<float2*>(buf), rows, N);
-  else shift_bytes_kernel<<<grid, 256, 0, st>>>(static_cast<uint8_t*>(buf), rows, rowbytes);
+  if (kind == 0) pdl_launch(shift_c64_kernel, dim3(grid), 256, 0, st, static_cast<float2*>(buf),
+                            rows, N);
+  else pdl_launch(shift_bytes_kernel, dim3(grid), 256, 0, st, static_cast<uint8_t*>(buf), rows,
+                  rowbytes);
   return cudaGetLastError();
 }
 

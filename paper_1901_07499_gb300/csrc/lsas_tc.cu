@@ -181,6 +181,7 @@ struct TcGeo {
 // -> Y rows (unitary).  Persistent: block b takes batches b, b + grid, ...
 template <int LOG2N, bool FC32>
 __global__ void __launch_bounds__(tc_threads<LOG2N>(), 1) tcfft_kernel(const KParams p) {
+  pdl_wait();
   using G = TcGeo<LOG2N>;
   constexpr int N = G::N, N2 = G::N2, R = G::R, TT = G::TT, PARTS = G::PARTS;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -415,7 +416,7 @@ static cudaError_t launch_tc_t(const KParams& p, int grid, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) limit[dev] = G::SMEM;
   }
-  tcfft_kernel<LOG2N, FC32><<<grid, G::TT, G::SMEM, st>>>(p);
+  pdl_launch(tcfft_kernel<LOG2N, FC32>, dim3(grid), G::TT, G::SMEM, st, p);
   return cudaGetLastError();
 }
 
@@ -451,6 +452,7 @@ constexpr int kYrxMaxThreads = 128;
 // 67 us (floor 54); with the sums of up to 63 symbols in local memory, 309.
 template <int DG>
 __global__ void __launch_bounds__(kYrxMaxThreads) yrx_kernel(const KParams p) {
+  pdl_wait();
   __shared__ uint8_t codes[DG * kYrxMaxThreads];
   const int N = p.N;
   const int T = blockDim.x;   // min(N, 128) subcarriers per block
@@ -530,9 +532,9 @@ cudaError_t launch_yrx(const KParams& p, int n_frames, int sms, cudaStream_t st)
   // the pilots more often, where seven would leave SMs idle.  Results do not
   // depend on it.
   if (p.D <= 4 || static_cast<long>(blocks) * ((p.D + 6) / 7) < 2L * sms)
-    yrx_kernel<4><<<dim3(blocks, (p.D + 3) / 4), T, 0, st>>>(p);
+    pdl_launch(yrx_kernel<4>, dim3(blocks, (p.D + 3) / 4), T, 0, st, p);
   else
-    yrx_kernel<7><<<dim3(blocks, (p.D + 6) / 7), T, 0, st>>>(p);
+    pdl_launch(yrx_kernel<7>, dim3(blocks, (p.D + 6) / 7), T, 0, st, p);
   return cudaGetLastError();
 }
 

@@ -398,6 +398,7 @@ __device__ __forceinline__ int twin_block_col(int it, bool pilot, bool* pair, in
 
 template <int LOG2N, bool GIVEN, bool PART>
 __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
+  pdl_wait();
   static_assert(LOG2N >= 7 && LOG2N <= 10, "the two-symbol kernel covers N = 128 .. 1024");
   constexpr int N = 1 << LOG2N;
   constexpr int L = N / 32;     // lanes of an antenna's FFT team
@@ -777,6 +778,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
 // frames of 64 antennas, N = 1024: 40.5 -> 29 us (floor 23).
 template <int LOG2N, bool EST>
 __global__ void __launch_bounds__(kTwThreads, 1) twin_rows_kernel(const KParams p) {
+  pdl_wait();
   constexpr int N = 1 << LOG2N, L = N / 32, A = 32 / L, K = kTwSlots;
   extern __shared__ __align__(128) unsigned char smem[];
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;

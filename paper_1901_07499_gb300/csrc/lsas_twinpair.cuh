@@ -142,6 +142,7 @@ __device__ __forceinline__ void tp_twiddle(float2& xr, float2& xi, float2 w) {
 
 template <int LOG2N, bool GIVEN, bool FC32>
 __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p) {
+  pdl_wait();
   static_assert(LOG2N == 11, "the two-symbol pair kernel is written for N = 2048");
   constexpr int N = 1 << LOG2N;
   constexpr int OWN = kTwOwn;

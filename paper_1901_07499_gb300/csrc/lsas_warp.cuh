@@ -136,6 +136,7 @@ __device__ __forceinline__ void wfinal_exchange_read(float2 (&v)[32], const floa
 
 template <int LOG2N, bool FC32>
 __global__ void __launch_bounds__(32 * wgeo_warps(FC32 ? 8 : 4), 1) warp_kernel(const KParams p) {
+  pdl_wait();
   constexpr int N = 1 << LOG2N;
   constexpr int NW = wgeo_warps(FC32 ? 8 : 4);   // warps of the block
   constexpr int NT = 32 * NW;
