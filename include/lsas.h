@@ -150,8 +150,9 @@ lsas_status lsas_demodulate(lsas_plan plan, const void* d_in,
  * then demodulation (writes d_bits and optionally d_eq).  Asynchronous.
  * Whole waves of frames (one frame per SM) run in one launch.  The frames
  * after the last whole wave, or all of them for a batch smaller than one
- * wave, may run split into equal antenna shards so that they occupy more
- * SMs: the shards' MRC partial sums go to a scratch array the plan owns
+ * wave, may run split into antenna shards so that they fill the SMs
+ * (equal shards of every frame, or even cuts through all their antennas laid
+ * end to end): the shards' MRC partial sums go to a scratch array the plan owns
  * (lsas_plan_create reserves at most 96 MiB for it), and the combine pass
  * forms z and the bits from them, summing the shards in a fixed order.
  * Outputs agree with the unsplit pass to rounding (the antenna sums are
@@ -478,7 +479,7 @@ lsas_status lsas_plan_set_fault(lsas_plan plan, int kind);
 lsas_status lsas_plan_set_batch_split(lsas_plan plan, int enable);
 
 /*
- * The antenna shards lsas_run_frame would use for the frames after the last
+ * The most antenna shards lsas_run_frame would make of a frame after the last
  * whole wave of an n_frames batch (1: no split), into *out_shards.  The
  * choice depends on the plan's shape, the SM count and the batch split
  * setting only.  INVALID_ARG for null pointers or n_frames < 0.

@@ -44,8 +44,10 @@ __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const KParams 
   float2 E = make_float2(0.f, 0.f);
   // unrolled so that several shards' loads are in flight at once (the sums
   // still run in shard order)
+  // (units: the blocks that touched the frame)
+  const int shards = p.units ? (f * p.upf + p.upf - 1) / p.units - f * p.upf / p.units + 1 : p.shards;
 #pragma unroll 8
-  for (int g = 0; g < p.shards; ++g) {
+  for (int g = 0; g < shards; ++g) {
     const float4 v = __ldcs(Pg + g * ps);
     const float2 e = __ldg(Eg + g * es);
     P.x += v.x;

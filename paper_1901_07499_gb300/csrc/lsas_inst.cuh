@@ -42,7 +42,10 @@ inline int two_symbol_form(const KParams& p) {
 template <int LOG2N, bool FC32>
 static auto two_symbol_kernel(const KParams& p) -> void (*)(const KParams) {
   if constexpr (LOG2N == 11) {
-    return p.H_in ? twinpair_kernel<LOG2N, true, FC32> : twinpair_kernel<LOG2N, false, FC32>;
+    void (*const k[4])(const KParams) = {
+        twinpair_kernel<LOG2N, false, FC32, false>, twinpair_kernel<LOG2N, true, FC32, false>,
+        twinpair_kernel<LOG2N, false, FC32, true>, twinpair_kernel<LOG2N, true, FC32, true>};
+    return k[two_symbol_form(p)];
   } else {
     void (*const k[4])(const KParams) = {twin_kernel<LOG2N, false, false>, twin_kernel<LOG2N, true, false>,
                                          twin_kernel<LOG2N, false, true>, twin_kernel<LOG2N, true, true>};
@@ -128,7 +131,8 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
   }
   // rows staged from the boundary before them: the per-warp kernel only
   KParams q = p;
-  q.nf = q.full = grid;
+  if (!q.units) q.nf = grid;
+  q.full = grid;
   q.zsplit = 1;
   if constexpr (LOG2N <= 10) {
     if (q.use_tma == 2 && fn != warp_kernel<LOG2N, FC32>) q.use_tma = 0;

@@ -102,6 +102,9 @@ struct KParams {
                          // bulk copies from the 16-byte boundary before each row
   int share;             // warp_kernel: 1 = the (chunk, data symbol) pairs cut evenly over warps
   int nf, sms;           // frames of the launch, SMs of the device
+  int units, upf, unit_ant;   // two-symbol kernels and combine, split launches: > 0 = block b takes
+                         // antenna units b * units .. of the frames' consecutive units, upf
+                         // per frame, unit_ant antennas each (one per pipeline)
   int full, zsplit;      // warp_kernel: frames that are one block each; blocks of each other
                          // frame (an even part of the data symbols each)
   int tmem_cols, tmem_cth;   // TMEM allocation (columns) and columns per thread

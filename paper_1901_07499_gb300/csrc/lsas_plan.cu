@@ -547,12 +547,59 @@ int best_shards(lsas_plan p, int nf, long cap) {
   return bestG;
 }
 
+// Antenna units per block for nf frames that do not fill a whole wave of
+// blocks of a two-symbol kernel: the frames' units (one antenna per pipeline:
+// unit_ant antennas, upf per frame) laid end to end and cut into one wave of
+// equal blocks, which may each touch the ends of two frames.  Unlike equal
+// shards of every frame they fill the GPU for any nf.  In fractions of a
+// frame's block time a block takes (1 - f) u / upf plus f per frame it
+// touches, and the partial sums' way through memory is charged to the frame's
+// samples at 3.7 G a second and SM; 0 when that does not save 10 % of a wave, or the
+// scratch is too small.  1000 frames of 64 antennas at N = 1024 (88 after six
+// waves: 5 of 8 units a block) 1517 -> 1485 us; 500 of 128 at N = 2048 (44: 10 of
+// 32) 3447 -> 3403; 60 float frames of 64 (7 of 16) 311 -> 281.
+int unit_antennas(lsas_plan p) { return p->N > 1024 ? kPPairs : 8 * (1024 / p->N); }
+int units_per_frame(lsas_plan p) { return (p->M + unit_antennas(p) - 1) / unit_antennas(p); }
+int best_units(lsas_plan p, int nf) {
+  const int upf = units_per_frame(p);
+  const double fixed = p->N > 1024 ? kBlockFixedPair : kBlockFixedWarp;
+  const double frame_s = static_cast<double>(p->M) * p->S * p->N / 3.7e9;
+  const double sums = (static_cast<double>(p->D) * 2 + 1) * p->N * 4.0;   // bytes of one shard's sums
+  const long total = static_cast<long>(nf) * upf;
+  double best = 0.9;
+  int bestU = 0;
+  for (int u = static_cast<int>((total + p->sms - 1) / p->sms); u < upf; ++u) {
+    const int most = (upf - 1) / u + 2;   // shards of a frame, at most
+    if (static_cast<long>(nf) * (upf % u == 0 ? upf / u : most) > p->tail_units) continue;
+    const int frames = upf % u == 0 ? 1 : 2;   // that a block touches
+    const double moved = 2.0 * sums * (static_cast<double>(total) / u + (frames - 1) * nf) / 4e12;
+    const double t = (1.0 - fixed) * u / upf + fixed * frames + moved / frame_s;
+    if (t < best) {
+      best = t;
+      bestU = u;
+    }
+  }
+  return bestU;
+}
+
+// Whether a batch's rows reach the two-symbol kernels' bulk copies, from the
+// plan alone (an input that is not 16-byte aligned falls back to equal shards).
+bool rows_aligned(lsas_plan p) {
+  const int bps = p->fmt == LSAS_IN_SC16 ? 4 : 8;
+  return ((p->N + p->cp) * bps) % 16 == 0 && (p->cp * bps) % 16 == 0;
+}
+bool split_by_units(lsas_plan p) { return p->batch_split == 1 && two_symbols(p) && rows_aligned(p); }
+
 int tail_shards(lsas_plan p, int nf) {
   if (nf <= 0 || p->batch_split == 0 || p->tail_units == 0 || p->geo.hybrid) return 1;
   if (p->batch_split == 2) {
     // one shard count for every batch: the single frame's choice, among the
     // counts whose scratch holds a batch of max_frames
     return best_shards(p, 1, p->tail_units / (p->max_frames > 0 ? p->max_frames : 1));
+  }
+  if (split_by_units(p)) {
+    const int u = best_units(p, nf), upf = units_per_frame(p);
+    return u == 0 ? 1 : upf % u == 0 ? upf / u : (upf - 1) / u + 2;
   }
   return best_shards(p, nf, p->tail_units);
 }
@@ -566,8 +613,6 @@ lsas_status run_split_tail(lsas_plan p, const void* d_in, int f0, int nf, int G,
   const size_t in_b = in_bytes_per_frame(p->M, p->N, p->cp, p->S, p->fmt);
   const size_t bits_b = bits_bytes_per_frame(p->N, p->S, p->Q);
   const unsigned char* in = static_cast<const unsigned char*>(d_in) + f0 * in_b;
-  float* P = p->d_tail;
-  float* E = P + static_cast<size_t>(G) * nf * p->D * p->N * 2;
   std::lock_guard<std::mutex> lock(p->tail_mu);
   if (cudaStreamWaitEvent(st, p->tail_ev, 0) != cudaSuccess) return LSAS_ERR_CUDA;
   KParams k;
@@ -576,17 +621,33 @@ lsas_status run_split_tail(lsas_plan p, const void* d_in, int f0, int nf, int G,
   const size_t h0 = static_cast<size_t>(f0) * p->M * p->N * 2;
   if (d_Hin) k.H_in = reinterpret_cast<const float2*>(d_Hin + h0);
   else k.H_out = reinterpret_cast<float2*>(d_H + h0);
+  k.use_tma = staging(p, in);
+  int blocks = nf;
+  const int u = split_by_units(p) && k.use_tma == 1 ? best_units(p, nf) : 0;
+  const int upf = units_per_frame(p);
+  if (u > 0 && (upf % u != 0 || p->M % (upf / u) != 0)) {
+    k.units = u;
+    k.upf = upf;
+    k.unit_ant = unit_antennas(p);
+    k.nf = nf;
+    blocks = (nf * upf + u - 1) / u;
+  } else {
+    // equal shards (units that divide the frame are: a grid row each, which
+    // spares a short launch the units' arithmetic, 0.8 us)
+    if (split_by_units(p)) G = u > 0 ? upf / u : best_shards(p, nf, p->tail_units);
+    k.M = p->M / G;
+    k.shard_y = k.M;
+    k.grid_y = G;
+  }
+  float* P = p->d_tail;
+  float* E = P + static_cast<size_t>(G) * nf * p->D * p->N * 2;
   k.P_out = reinterpret_cast<float2*>(P);
   k.E_out = E;
-  k.M = p->M / G;
-  k.shard_y = k.M;
-  k.grid_y = G;
   k.chunks = (k.M + p->geo.Af - 1) / p->geo.Af;
   k.mode = kModePartial;
-  k.use_tma = staging(p, in);
-  k.group_z = grid_layers(p, k, nf, G);
+  k.group_z = k.units ? grid_layers(p, k, blocks, 1) : grid_layers(p, k, nf, G);
   lsas_status s = LSAS_OK;
-  if (p->launch(kKindFrame, p->fmt == LSAS_IN_FC32, k, nf, p->geo.smem_frame, st) != cudaSuccess) {
+  if (p->launch(kKindFrame, p->fmt == LSAS_IN_FC32, k, blocks, p->geo.smem_frame, st) != cudaSuccess) {
     s = LSAS_ERR_CUDA;
   } else {
     KParams c;
@@ -594,6 +655,8 @@ lsas_status run_split_tail(lsas_plan p, const void* d_in, int f0, int nf, int G,
     c.P_in = reinterpret_cast<const float2*>(P);
     c.E_in = E;
     c.shards = G;
+    c.units = k.units;
+    c.upf = k.upf;
     c.nframes = nf;
     c.bits = d_bits + f0 * bits_b;
     c.eq = d_eq ? reinterpret_cast<float2*>(d_eq + static_cast<size_t>(f0) * p->D * p->N * 2)

@@ -314,21 +314,21 @@ __device__ __forceinline__ void twin_twiddles(float2 (&re)[32], float2 (&im)[32]
 // second may be absent) for the A antennas of chunk c.  Lane h A + t copies
 // the row of symbol item ia + h of antenna c A + t to half h of the slot,
 // team t's place (rows L words apart, for conflict-free loads); lane 0
-// registers the bytes.
+// registers the bytes.  The M antennas start at mb of the launch's.
 template <int LOG2N>
 __device__ __forceinline__ void twin_issue(const KParams& p, int f, int c, bool pilot_here, int d0,
                                            int items, int ia, unsigned char* slot, uint32_t bar,
-                                           uint64_t pol, int lane) {
+                                           uint64_t pol, int lane, int mb, int M) {
   constexpr int N = 1 << LOG2N, L = N / 32, A = 32 / L;
   constexpr uint32_t bytes = N * 4;
-  const int nant = min(A, p.M - c * A);
+  const int nant = min(A, M - c * A);
   const int nrow = ia + 1 < items ? 2 : 1;
   if (lane == 0) mbar_expect_tx(bar, bytes * nant * nrow);
   if (lane < 2 * A) {
     const int half = lane / A, t = lane % A;
     if (t < nant && half < nrow)
       bulk_load(smem_u32(slot + half * kTwHalfB + t * (N + L) * 4),
-                row_ptr<LOG2N, false>(p, f, c * A + t, witem_symbol(p, pilot_here, d0, ia + half)),
+                row_ptr<LOG2N, false>(p, f, mb + c * A + t, witem_symbol(p, pilot_here, d0, ia + half)),
                 bytes, bar, pol);
   }
 }
@@ -396,6 +396,42 @@ __device__ __forceinline__ int twin_block_col(int it, bool pilot, bool* pair, in
   return pilot ? (ip == 0 ? 0 : 64 + 128 * (ip - 1)) : 128 * ip;
 }
 
+// The antennas a block of a split launch (PART) works through: an equal shard
+// of one frame (grid row blockIdx.y), or, with p.units, the units
+// blockIdx.x * p.units .. of the frames' consecutive antenna units, one
+// segment per frame they touch; a frame's shards are the blocks that touch it,
+// in block order.  Whole frames: one segment.
+struct Segments {
+  int f, mb, M, shard;
+  int u, uend, ant;
+  __device__ __forceinline__ Segments(const KParams& p, bool part) {
+    f = blockIdx.x;
+    mb = 0;
+    M = p.M;
+    shard = blockIdx.y;
+    u = uend = 0;
+    if (part && p.units) {
+      ant = p.unit_ant;
+      u = blockIdx.x * p.units;
+      uend = min(u + p.units, p.nf * p.upf);
+      set(p);
+    }
+  }
+  __device__ __forceinline__ void set(const KParams& p) {
+    f = u / p.upf;
+    const int um = u - f * p.upf, n = min(uend - u, p.upf - um);
+    mb = um * ant;
+    M = min(n * ant, p.M - mb);
+    shard = blockIdx.x - f * p.upf / p.units;
+    u += n;
+  }
+  __device__ __forceinline__ bool next(const KParams& p) {
+    if (u >= uend) return false;
+    set(p);
+    return true;
+  }
+};
+
 template <int LOG2N, bool GIVEN, bool PART>
 __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
   pdl_wait();
@@ -410,7 +446,6 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
   using TmP = Tmem<2 * OWN>;   // one data symbol of partial sums (complex)
   using TmE = Tmem<OWN>;       // channel energy
   extern __shared__ __align__(128) unsigned char smem[];
-  const int f = blockIdx.x;
   const int tid = threadIdx.x;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // known uniform: see twinpair_kernel
   const int lane = tid & 31;
@@ -450,14 +485,20 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
 #pragma unroll
   for (int i = 0; i < 16; ++i) zero[i] = 0.f;
 
-  const int nch = warp < p.chunks ? (p.chunks - 1 - warp) / NW + 1 : 0;
   // start the warps of the upper half a little later, so that the two warps
   // sharing a scheduler tend to be in different phases of their steps
   // (not in a short launch, whose time it would lengthen)
-  if (warp >= 4 && nch > 2) __nanosleep(1400);
+  if (!PART && warp >= 4 && p.chunks > 2 * NW) __nanosleep(1400);
   int issued = 0;  // steps whose copies this warp has issued
   int slot = 0;    // ring slot of the next step to consume ...
   int phase = 0;   // ... and its mbarrier phase
+  // the antennas of a segment: one frame's, or (units) of each frame that the
+  // block's units touch
+  Segments seg(p, PART);
+  do {
+  const int f = seg.f, mb = seg.mb, M = PART ? seg.M : p.M;
+  const int chunks = PART ? (M + A - 1) / A : p.chunks;
+  const int nch = warp < chunks ? (chunks - 1 - warp) / NW + 1 : 0;
   // one part of the data symbols per grid z index (partial mode, small
   // batches; no part is larger than its group): every part's block transforms
   // the pilot itself; part 0 alone writes H and the channel energy
@@ -488,7 +529,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
       for (int s = 0; s < K && to_issue > 0; ++s, --to_issue) {
         const int ia = 2 * ipi;
         twin_issue<LOG2N>(p, f, warp + ic * NW, pilot_here, d0, items, ia, stage + is * slot_bytes,
-                          smem_u32(&bars[is]), pol, lane);
+                          smem_u32(&bars[is]), pol, lane, mb, M);
         // test hook: the first staging phase of block 0 also waits for 16
         // bytes that no copy delivers, so its bounded wait runs out
         if (p.fault == 1 && blockIdx.x == 0 && warp == 0 && g == 0 && s == 0 && lane == 0)
@@ -503,8 +544,8 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
     }
     for (int lc = 0; lc < nch; ++lc) {
       const int m = (warp + lc * NW) * A + team;   // this lane's antenna
-      const bool valid = m < p.M;                  // a chunk's last teams may have none
-      const size_t hrow = (static_cast<size_t>(f) * p.Mtot + p.m0 + blockIdx.y * p.shard_y + m) * N;
+      const bool valid = m < M;                    // a chunk's last teams may have none
+      const size_t hrow = (static_cast<size_t>(f) * p.Mtot + p.m0 + blockIdx.y * p.shard_y + mb + m) * N;
       float2 h[32];
       if (!pilot_here) {
         // channel written in group 0, or given (zero for a team without an
@@ -552,7 +593,8 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
           ++issued;
           fence_proxy_async();
           const int ia = 2 * ipi;
-          twin_issue<LOG2N>(p, f, warp + ic * NW, pilot_here, d0, items, ia, yslot, ybar, pol, lane);
+          twin_issue<LOG2N>(p, f, warp + ic * NW, pilot_here, d0, items, ia, yslot, ybar, pol,
+                            lane, mb, M);
           --to_issue;
           if (++ipi == npairs) {
             ipi = 0;
@@ -622,7 +664,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
 #pragma unroll
         for (int w = 0; w < 4 * A; ++w) E += RE[w * N + k];
         if constexpr (PART) {
-          p.E_out[(static_cast<size_t>(blockIdx.y) * gridDim.x + f) * N + k] = E;
+          p.E_out[(static_cast<size_t>(seg.shard) * p.nf + f) * N + k] = E;
         } else {
           // zero or non-finite energy flags the frame; z = 0 there
           const bool ok = (E > 0.f) && (E <= 3.4028234663852886e38f);
@@ -707,7 +749,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
             const float2 s = sv[u];
             const int dl = dl0 + j;
             if constexpr (PART) {
-              p.P_out[((static_cast<size_t>(blockIdx.y) * gridDim.x + f) * p.D + d0 + dl) * N + k] =
+              p.P_out[((static_cast<size_t>(seg.shard) * p.nf + f) * p.D + d0 + dl) * N + k] =
                   make_float2(s.x * p.inv_sqrtN, s.y * p.inv_sqrtN);
             } else {
               const float ie = ie_s[k];
@@ -748,6 +790,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
       __syncthreads();   // codes consumed before the next group writes them
     }
   }
+  } while (PART && seg.next(p));
   if (lane == 0 && *abort_flag) {
     // a wait gave up: give any copy of this warp still in flight a bounded
     // chance to land before the block's shared memory is released (copies

@@ -140,7 +140,7 @@ __device__ __forceinline__ void tp_twiddle(float2& xr, float2& xi, float2 w) {
   xi = i;
 }
 
-template <int LOG2N, bool GIVEN, bool FC32>
+template <int LOG2N, bool GIVEN, bool FC32, bool PART>
 __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p) {
   pdl_wait();
   static_assert(LOG2N == 11, "the two-symbol pair kernel is written for N = 2048");
@@ -149,7 +149,6 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
   constexpr int K = 2;
   using TmE = Tmem<OWN>;
   extern __shared__ __align__(128) unsigned char smem[];
-  const int f = blockIdx.x;
   const int tid = threadIdx.x;
   // broadcast, so that the compiler knows the warp index, and with it the
   // antenna, row and copy addresses, to be uniform and keeps them out of the
@@ -182,19 +181,25 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
 #pragma unroll
   for (int i = 0; i < 16; ++i) zero[i] = 0.f;
 
-  const int nch = q < p.chunks ? (p.chunks - 1 - q) / kTpPairs + 1 : 0;
   int issued = 0;  // steps whose copies this pair has issued
   int slot = 0;    // ring slot of the next step to consume ...
   int phase = 0;   // ... and its mbarrier phase
+  // the antennas of a segment: one frame's, or (units) of each frame that the
+  // block's units touch
+  Segments seg(p, PART);
+  bool set_up = false;
+  do {
+  const int f = seg.f, mb = seg.mb, M = PART ? seg.M : p.M;
+  const int nch = q < M ? (M - 1 - q) / kTpPairs + 1 : 0;
   // one part of the data symbols per grid z index (partial mode, small
   // batches; no part is larger than its group): every part's block transforms
   // the pilot itself; part 0 alone writes H and the channel energy
-  const int g_lo = p.group_z ? static_cast<int>(blockIdx.z) : 0;
-  const int g_hi = p.group_z ? g_lo + 1 : twin_groups(p.D);
+  const int g_lo = PART && p.group_z ? static_cast<int>(blockIdx.z) : 0;
+  const int g_hi = PART && p.group_z ? g_lo + 1 : twin_groups(p.D);
   for (int g = g_lo; g < g_hi; ++g) {
-    const int d0 = p.group_z ? g * p.D / p.group_z : g == 0 ? 0 : kTwDg0 + (g - 1) * kTwDg;
-    const int nd = p.group_z ? (g + 1) * p.D / p.group_z - d0 : min(g == 0 ? kTwDg0 : kTwDg, p.D - d0);
-    const bool pilot_here = !GIVEN && (g == 0 || p.group_z);
+    const int d0 = PART && p.group_z ? g * p.D / p.group_z : g == 0 ? 0 : kTwDg0 + (g - 1) * kTwDg;
+    const int nd = PART && p.group_z ? (g + 1) * p.D / p.group_z - d0 : min(g == 0 ? kTwDg0 : kTwDg, p.D - d0);
+    const bool pilot_here = !GIVEN && (g == 0 || (PART && p.group_z));
     const bool energy_here = g == 0;
     const int items = nd + (pilot_here ? 1 : 0);
     const int npairs = (items + 1) / 2;
@@ -202,14 +207,14 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
     // many steps of this group are still to be staged
     int ic = 0, ipi = 0;
     int to_issue = nch * npairs;
-    if (g == g_lo || !*abort_flag) {
+    if (!set_up || !*abort_flag) {
       // the ring held generic data (last group's reduction): order it before
       // the copies, then fill the first K slots of this group
       fence_proxy_async();
       if constexpr (FC32) {
         if (to_issue > 0) {
-          tp_issue_row(p, f, q, pilot_here, d0, items, 0, stage, smem_u32(&bars[0]), pol, jt);
-          tp_issue_row(p, f, q, pilot_here, d0, items, 1, stage + kTpSlotB, smem_u32(&bars[1]), pol, jt);
+          tp_issue_row(p, f, mb + q, pilot_here, d0, items, 0, stage, smem_u32(&bars[0]), pol, jt);
+          tp_issue_row(p, f, mb + q, pilot_here, d0, items, 1, stage + kTpSlotB, smem_u32(&bars[1]), pol, jt);
           if (p.fault == 1 && blockIdx.x == 0 && q == 0 && g == 0 && jt == 0)
             mbar_expect_tx_only(smem_u32(&bars[0]), 16);
           ++issued;
@@ -222,7 +227,7 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
       } else {
         int is = slot;
         for (int s = 0; s < K && to_issue > 0; ++s, --to_issue) {
-          tp_issue(p, f, q + ic * kTpPairs, pilot_here, d0, items, 2 * ipi, stage + is * kTpSlotB,
+          tp_issue(p, f, mb + q + ic * kTpPairs, pilot_here, d0, items, 2 * ipi, stage + is * kTpSlotB,
                    smem_u32(&bars[is]), pol, jt);
           // test hook: the first staging phase of block 0 also waits for 16
           // bytes that no copy delivers, so its bounded wait runs out
@@ -237,8 +242,9 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
         }
       }
     }
-    if (g == g_lo) {
+    if (!set_up) {
       // the block's set-up, under the first copies
+      set_up = true;
       for (int i = tid; i < kTpTwl; i += kTpThreads) twl[i] = __ldg(p.twP + 512 + i);
       for (int i = tid; i < 7 * 32; i += kTpThreads) mtw[i] = __ldg(p.twP + 32 + i);
       if (tid == 0) *abort_flag = 0;
@@ -253,7 +259,7 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
       // start the pairs of the upper half a little later, so that the two warps
       // sharing a scheduler tend to be in different phases of their steps
       // (not in a short launch, whose time it would lengthen)
-      if (warp >= 4 && nch > 2) __nanosleep(1400);
+      if (!PART && warp >= 4 && p.M > 2 * kTpPairs) __nanosleep(1400);
     }
     const uint32_t tP = energy_here ? tE + OWN : tE;
     if (energy_here) {
@@ -265,7 +271,7 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
     uint32_t prev_bar = 0;
     for (int lc = 0; lc < nch; ++lc) {
       const int m = q + lc * kTpPairs;
-      const size_t hrow = (static_cast<size_t>(f) * p.Mtot + p.m0 + blockIdx.y * p.shard_y + m) * N;
+      const size_t hrow = (static_cast<size_t>(f) * p.Mtot + p.m0 + blockIdx.y * p.shard_y + mb + m) * N;
       float2 h[32];
       if (!pilot_here) {
         const float2* Hs = GIVEN ? p.H_in : p.H_out;
@@ -335,13 +341,13 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
           refill = to_issue > 0 && !*abort_flag;
           if (refill) {
             fence_proxy_async();
-            tp_issue_row(p, f, q + ic * kTpPairs, pilot_here, d0, items, 2 * ipi + 1, stage + kTpSlotB,
+            tp_issue_row(p, f, mb + q + ic * kTpPairs, pilot_here, d0, items, 2 * ipi + 1, stage + kTpSlotB,
                          smem_u32(&bars[1]), pol, jt);
           }
         } else if (prev_slot && to_issue > 0 && !*abort_flag) {
           ++issued;
           fence_proxy_async();
-          tp_issue(p, f, q + ic * kTpPairs, pilot_here, d0, items, 2 * ipi, prev_slot, prev_bar, pol,
+          tp_issue(p, f, mb + q + ic * kTpPairs, pilot_here, d0, items, 2 * ipi, prev_slot, prev_bar, pol,
                    jt);
           --to_issue;
           if (++ipi == npairs) {
@@ -416,7 +422,7 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
           if (refill) {
             ++issued;
             fence_proxy_async();
-            tp_issue_row(p, f, q + ic * kTpPairs, pilot_here, d0, items, 2 * ipi, stage,
+            tp_issue_row(p, f, mb + q + ic * kTpPairs, pilot_here, d0, items, 2 * ipi, stage,
                          smem_u32(&bars[0]), pol, jt);
             --to_issue;
             if (++ipi == npairs) {
@@ -483,8 +489,8 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
       __syncthreads();
       for (int k = threadIdx.x; k < N; k += kTpThreads) {
         const float E = RE[k] + RE[N + k];
-        if (p.mode == kModePartial) {
-          p.E_out[(static_cast<size_t>(blockIdx.y) * gridDim.x + f) * N + k] = E;
+        if constexpr (PART) {
+          p.E_out[(static_cast<size_t>(seg.shard) * p.nf + f) * N + k] = E;
         } else {
           // zero or non-finite energy flags the frame; z = 0 there
           const bool ok = (E > 0.f) && (E <= 3.4028234663852886e38f);
@@ -560,8 +566,8 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
             const int dl = idx >> LOG2N;
             const int k = idx & (N - 1);
             const float2 s = sv[u];
-            if (p.mode == kModePartial) {
-              p.P_out[((static_cast<size_t>(blockIdx.y) * gridDim.x + f) * p.D + d0 + dl) * N + k] =
+            if constexpr (PART) {
+              p.P_out[((static_cast<size_t>(seg.shard) * p.nf + f) * p.D + d0 + dl) * N + k] =
                   make_float2(s.x * p.inv_sqrtN, s.y * p.inv_sqrtN);
             } else {
               const float ie = ie_s[k];
@@ -574,15 +580,19 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
           }
         }
       };
-      switch (p.nthr) {
-        case 1: demap_items(std::integral_constant<int, 1>{}); break;
-        case 3: demap_items(std::integral_constant<int, 3>{}); break;
-        case 7: demap_items(std::integral_constant<int, 7>{}); break;
-        default: demap_items(std::integral_constant<int, kMaxThresholds>{}); break;
+      if constexpr (PART) {
+        demap_items(std::integral_constant<int, 1>{});
+      } else {
+        switch (p.nthr) {
+          case 1: demap_items(std::integral_constant<int, 1>{}); break;
+          case 3: demap_items(std::integral_constant<int, 3>{}); break;
+          case 7: demap_items(std::integral_constant<int, 7>{}); break;
+          default: demap_items(std::integral_constant<int, kMaxThresholds>{}); break;
+        }
       }
       __syncthreads();
     }
-    if (p.mode != kModePartial) {
+    if constexpr (!PART) {
       // pack: 8 consecutive subcarriers -> q bytes
       const int items8 = nd * (N / 8);
       const size_t frame_bytes = static_cast<size_t>(p.D) * N * p.q / 8;
@@ -598,6 +608,7 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
       __syncthreads();   // codes consumed before the next group writes them
     }
   }
+  } while (PART && seg.next(p));
   if (jt == 0 && *abort_flag) {
     // a wait gave up: give any copy of this pair still in flight a bounded
     // chance to land before the block's shared memory is released (copies
