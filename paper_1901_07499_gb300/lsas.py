@@ -163,6 +163,11 @@ def _ptr(t) -> Optional[int]:
 def _stream(stream) -> Optional[int]:
     import torch
     if stream is None:
+        # the current stream's handle without a Stream object around it: 0.2 us
+        # of the call instead of 3.0 (a single small frame's call took 8.1)
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is not None and torch.cuda.is_initialized():
+            return raw(torch.cuda.current_device()) or None
         stream = torch.cuda.current_stream()
     return stream.cuda_stream or None
 
