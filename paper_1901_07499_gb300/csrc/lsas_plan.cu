@@ -106,6 +106,8 @@ struct lsas_plan_s {
   int tail_units = 0;               // shard-frames d_tail holds
   int batch_split = 1;              // lsas_plan_set_batch_split: 0 off, 1 per batch, 2 fixed
   cudaEvent_t tail_ev = nullptr;    // the last split's combine has read d_tail
+  bool tail_live = false;           // ... on the stream with this id, outside any capture
+  unsigned long long tail_stream = 0;
   std::mutex tail_mu;
   size_t dev_bytes = 0;             // device memory allocated at creation
   Geometry geo;
@@ -614,7 +616,17 @@ lsas_status run_split_tail(lsas_plan p, const void* d_in, int f0, int nf, int G,
   const size_t bits_b = bits_bytes_per_frame(p->N, p->S, p->Q);
   const unsigned char* in = static_cast<const unsigned char*>(d_in) + f0 * in_b;
   std::lock_guard<std::mutex> lock(p->tail_mu);
-  if (cudaStreamWaitEvent(st, p->tail_ev, 0) != cudaSuccess) return LSAS_ERR_CUDA;
+  // the previous split's combine first, unless it went to this very stream
+  // (by its id, which no later stream takes over), whose order does that: the
+  // wait costs 2 us and keeps the launches from overlapping
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cudaStreamGetId(st, &id) != cudaSuccess)
+    return LSAS_ERR_CUDA;
+  const bool live = cap == cudaStreamCaptureStatusNone;
+  if (!(live && p->tail_live && p->tail_stream == id) &&
+      cudaStreamWaitEvent(st, p->tail_ev, 0) != cudaSuccess)
+    return LSAS_ERR_CUDA;
   KParams k;
   base_params(p, &k);
   k.in = in;
@@ -663,8 +675,10 @@ lsas_status run_split_tail(lsas_plan p, const void* d_in, int f0, int nf, int G,
                 : nullptr;
     if (launch_combine(c, st) != cudaSuccess) s = LSAS_ERR_CUDA;
   }
-  if (cudaEventRecord(p->tail_ev, st) != cudaSuccess) s = LSAS_ERR_CUDA;
-  return s;
+  const bool recorded = cudaEventRecord(p->tail_ev, st) == cudaSuccess;
+  p->tail_live = live && recorded;
+  p->tail_stream = id;
+  return recorded ? s : LSAS_ERR_CUDA;
 }
 
 // A batch through the fused receiver, with its own LS estimate (writes d_H,

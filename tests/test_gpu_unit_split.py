@@ -65,3 +65,38 @@ def test_unit_split(shape, given):
     assert split > 0
     check_frame_outputs(cfg, ref, H0.cpu().numpy(), bits0.cpu().numpy(), eq0.cpu().numpy())
     plan.close()
+
+
+def test_split_scratch_over_streams():
+    """Splits of one plan on one stream, on others in turn and on a stream
+    created after one was destroyed: each must wait for the previous split's
+    combine, by stream order or by event.  Every call has inputs of its own and
+    nothing synchronises in between."""
+    import torch
+    import paper_1901_07499_gb300.lsas as L
+    cfg = FrameConfig(M=64, N=1024, cp=72, S=14, Q=16, taps=4, snr_db=25.0, fmt="sc16", F=6, seed=8)
+    b = synth.generate(cfg)
+    plan = L.Plan(cfg.M, cfg.N, cfg.cp, cfg.S, 0, 16, max_frames=2, pilot=b.pilot)
+    assert plan.batch_split_shards(1) > 1
+    x = torch.from_numpy(np.ascontiguousarray(b.frames)).cuda()
+    want = [[t.clone() for t in plan.run_frame(x[i:i + 1], want_eq=True)] for i in range(6)]
+    torch.cuda.synchronize()
+    a, c = torch.cuda.Stream(), torch.cuda.Stream()
+    order = [a, a, c, a, c, c] * 5
+    outs = []
+    for k, st in enumerate(order):
+        with torch.cuda.stream(st):
+            outs.append((k % 6, plan.run_frame(x[k % 6:k % 6 + 1], want_eq=True)))
+    torch.cuda.synchronize()
+    for _ in range(3):   # ids are not taken over by streams created later
+        d = torch.cuda.Stream()
+        with torch.cuda.stream(d):
+            outs.append((1, plan.run_frame(x[1:2], want_eq=True)))
+        outs.append((2, plan.run_frame(x[2:3], want_eq=True)))
+        del d
+    torch.cuda.synchronize()
+    assert plan.sync_status() == L.LSAS_OK
+    for i, got in outs:
+        for u, v in zip(got, want[i]):
+            assert torch.equal(u, v)
+    plan.close()
