@@ -29,7 +29,8 @@ constexpr int kOffW1 = 0, kOffB1 = 320, kOffW2 = 352, kOffB2 = 5472, kOffW3 = 55
 __device__ __forceinline__ float to_f(float v) { return v; }
 __device__ __forceinline__ float to_f(__nv_bfloat16 v) { return __bfloat162float(v); }
 
-// FP32 network on the CUDA cores.  Activations are stored after their ReLU
+// FP32 network: the two 32 -> 32 layers on the tensor cores in split precision,
+// the rest on the CUDA cores.  Activations are stored after their ReLU
 // (r > 0 is the backward's mask), [R][C][N]; every kernel works on tiles of
 // kDnPos positions of one row.
 //
@@ -144,92 +145,220 @@ __global__ void __launch_bounds__(256) dn_conv_in_kernel(const float* __restrict
   }
 }
 
-// 32 -> 32 channels: layers 2 and 3 (bias and ReLU) or their data gradients
-// (masked).  Bound by the FMA pipe (5120 FMAs a position).  A thread keeps 8
-// outputs x 4 positions: per input channel two 16-byte loads give its 8-value
-// window and ten broadcast ones its 40 weights, for 160 FMAs issued as 80
-// packed ones (output pairs; the input value in both halves: 60 us where
-// scalar ones took 70, before the copies were asynchronous).  Blocks walk the
-// tiles, four on an SM, the weights loaded once and the next tile's rows
-// copied under the current one's FMAs.  256 rows of 1024: 51 us (floor 33)
-// against 104 us for 32 outputs x 1 position with one shared-memory operand
-// per FMA.
-constexpr int kCvWBytes = 32 * kDnK * 32 * 4;                  // weights [c][k][o]
-constexpr int kCvRow = kDnPos + kDnK - 1;                       // position q0 - 2 + j
-constexpr int kCvStage = 32 * kCvRow * 4;
-constexpr int kCvSmem = kCvWBytes + 2 * kCvStage;
+// 32 -> 32 channels in FP32 on tcgen05: layers 2 and 3 (bias and ReLU) or their
+// data gradients (masked).  The FMA pipe would need 33 us for 256 rows of 1024
+// (5120 FMAs a position), so the products go to the tensor cores: inputs and
+// weights are split into three bf16 terms each whose sum is the value
+// (x0 + x1 + x2, nearest even: |x1| <= 2^-9 |x|, |x2| <= 2^-18 |x|), products of
+// terms are exact in FP32, and of the nine the six down to 2^-18 are summed
+// (the others are below 2^-26 of the product).  The tensor cores' own FP32
+// additions do not round to nearest: the products x0 w0 have an accumulator
+// per tap, of two MMAs each, which the CUDA cores add, rounding to nearest; the
+// small products share two.  Relative error (norm) at 256 rows of 1024 against
+// 64 bits: layer output behind all layers 0.55e-7 (FP32 FMAs: 0.64e-7),
+// gradients 0.8e-7 (FMAs 0.7e-7; 1.3e-7 with one accumulator for three taps).
+//
+// Layout: positions as rows 16 bytes (eight channels) apart, so that the
+// operand of tap k is the same buffer k rows on; the weights' terms one after
+// the other as N, so that x0 meets w1 and w2 in one MMA of N = 64.  A block
+// fetches the next tile under a tile's MMAs; two blocks an SM fill each
+// other's gaps.  A tile with a value outside 2^-100 .. 2^120 (but
+// zero), whose split would not be exact, and, after a wait that gave up, every
+// further tile is summed by FMAs.  256 rows of 1024: 26 us, 27 masked (10 and 15 to read and
+// write HBM), against 51 us for packed FMAs from registers (8 outputs x 4
+// positions a thread).
+constexpr int kCvRows = kDnPos + kDnK - 1;           // row j holds position q0 - 2 + j
+constexpr int kCvLbo = kCvRows * 16;                 // bytes between channel chunks
+constexpr int kCvPlane = 4 * kCvLbo;                 // one term of a tile's input
+constexpr int kCvTap = 96 * 64;                      // one tap's weights: three terms x 32 outputs
+constexpr int kCvX = kDnK * kCvTap;
+constexpr int kCvBar = kCvX + 3 * kCvPlane;
+constexpr int kCvSmem = kCvBar + 16;
+constexpr int kCvThreads = 256;
+constexpr int kCvCross = 32 * kDnK, kCvCols = 256;   // TMEM: a sum per tap, then the small products
+static_assert(kCvX % 16 == 0 && kCvBar % 16 == 0, "16-byte operand alignment");
+
+// Eight values as three bf16 terms each (nearest even; the remainders are
+// exact, so the terms' sum is the value).  Returns whether one is outside the
+// range where that holds: zero, and 2^-100 (whose last term is a normal bf16
+// still) up to 2^120.
+__device__ __forceinline__ bool cv_split8(const float (&x)[8], uint4 (&out)[3]) {
+  uint32_t w[3][4];
+  bool off = false;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float a = x[2 * i], b = x[2 * i + 1];
+    const uint32_t ua = __float_as_uint(a) & 0x7fffffffu, ub = __float_as_uint(b) & 0x7fffffffu;
+    constexpr uint32_t kLo = (127u - 100u) << 23, kHi = (127u + 120u) << 23;
+    off |= (ua - kLo >= kHi - kLo && ua != 0) || (ub - kLo >= kHi - kLo && ub != 0);
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+      const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+      w[s][i] = *reinterpret_cast<const uint32_t*>(&h);
+      a -= __low2float(h);
+      b -= __high2float(h);
+    }
+  }
+#pragma unroll
+  for (int s = 0; s < 3; ++s) out[s] = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
+  return off;
+}
+
 template <bool BWD>
-__global__ void __launch_bounds__(128, 4) dn_conv32_kernel(const float* __restrict__ in,
-                                                           const float* __restrict__ wt,
-                                                           const float* __restrict__ bias,
-                                                           const float* __restrict__ mask,
-                                                           float* __restrict__ out, int R, int N) {
+__global__ void __launch_bounds__(kCvThreads, 2) dn_conv32_kernel(const float* __restrict__ in,
+                                                                  const float* __restrict__ wt,
+                                                                  const float* __restrict__ bias,
+                                                                  const float* __restrict__ mask,
+                                                                  float* __restrict__ out, int R, int N) {
   pdl_wait();
   extern __shared__ __align__(128) unsigned char smem[];
-  const float* ws = reinterpret_cast<const float*>(smem);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + kCvBar);
+  uint32_t* tbase = reinterpret_cast<uint32_t*>(bar + 1);
   const int tiles_row = N / kDnPos, tiles = R * tiles_row;
-  const int t = threadIdx.x, lane = t & 31, o0 = (t >> 5) * 8;
-  auto fetch = [&](int tile, int b) {
-    if (tile < tiles) {
-      const int r = tile / tiles_row, q0 = (tile % tiles_row) * kDnPos;
-      const uint32_t x = smem_u32(smem + kCvWBytes + b * kCvStage);
-      constexpr int kHalf = kCvRow / 2;
-      for (int i = t; i < 32 * kHalf; i += 128) {
-        const int c = i / kHalf, j = 2 * (i % kHalf), p = q0 + j - 2;
-        const bool on = p >= 0 && p < N;
-        cp_async(x + (c * kCvRow + j) * 4, in + (static_cast<size_t>(r) * 32 + c) * N + (on ? p : 0), on, 8);
-      }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  for (int i = t; i < kCvWBytes / 16; i += 128) cp_async(smem_u32(smem) + 16 * i, wt + 4 * i, true, 16);
-  fetch(blockIdx.x, 0);
-  float2 bs[4];
-#pragma unroll
-  for (int o = 0; o < 4; ++o)
-    bs[o] = BWD ? make_float2(0.f, 0.f) : make_float2(bias[o0 + 2 * o], bias[o0 + 2 * o + 1]);
-  int b = 0;
-  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, b ^= 1) {
-    fetch(tile + gridDim.x, b ^ 1);
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    __syncthreads();
-    const float* xs = reinterpret_cast<const float*>(smem + kCvWBytes + b * kCvStage) + 4 * lane;
-    float2 acc[4][4];   // [position][output pair]
-#pragma unroll
-    for (int o = 0; o < 4; ++o)
-#pragma unroll
-      for (int i = 0; i < 4; ++i) acc[i][o] = bs[o];
-#pragma unroll 2
-    for (int c = 0; c < 32; ++c) {
-      const float4 x0 = *reinterpret_cast<const float4*>(xs + c * kCvRow);
-      const float4 x1 = *reinterpret_cast<const float4*>(xs + c * kCvRow + 4);
-      const float x[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-#pragma unroll
-      for (int k = 0; k < kDnK; ++k) {
-        const float4 wa = *reinterpret_cast<const float4*>(ws + (c * kDnK + k) * 32 + o0);
-        const float4 wb = *reinterpret_cast<const float4*>(ws + (c * kDnK + k) * 32 + o0 + 4);
-        const float2 w[4] = {make_float2(wa.x, wa.y), make_float2(wa.z, wa.w), make_float2(wb.x, wb.y),
-                             make_float2(wb.z, wb.w)};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float2 xx = make_float2(x[i + k], x[i + k]);
-#pragma unroll
-          for (int o = 0; o < 4; ++o) acc[i][o] = __ffma2_rn(w[o], xx, acc[i][o]);
-        }
-      }
-    }
-    const int r = tile / tiles_row, q0 = (tile % tiles_row) * kDnPos;
-#pragma unroll
-    for (int o = 0; o < 8; ++o) {
-      const size_t at = (static_cast<size_t>(r) * 32 + o0 + o) * N + q0 + 4 * lane;
-      float4 v = (o & 1) ? make_float4(acc[0][o / 2].y, acc[1][o / 2].y, acc[2][o / 2].y, acc[3][o / 2].y)
-                         : make_float4(acc[0][o / 2].x, acc[1][o / 2].x, acc[2][o / 2].x, acc[3][o / 2].x);
-      v = BWD ? mask4(v, *reinterpret_cast<const float4*>(mask + at)) : relu4(v);
-      *reinterpret_cast<float4*>(out + at) = v;
-    }
-    __syncthreads();   // the stage is consumed before the next copies into it
+  const int t = threadIdx.x, u = t & 127, half = t >> 7;
+  const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);
+  if (t == 0) {
+    mbar_init(smem_u32(bar), 1);
+    fence_mbar_init();
   }
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncwarp();
+  if (warp == 0) tmem_alloc(smem_u32(tbase), kCvCols);
+  // a thread's inputs of a tile, fetched one tile ahead: buffer row u of
+  // channel chunks 2 half and 2 half + 1, and, threads 0 to 15, chunk t / 4 of
+  // row 128 + t % 4
+  float xa[2][8], xb[8];
+  auto fetch = [&](int tile) {
+    if (tile >= tiles) return;
+    const int r = tile / tiles_row, q0 = (tile % tiles_row) * kDnPos;
+    const float* row = in + static_cast<size_t>(r) * 32 * N;
+    const int qa = q0 - 2 + u, qb = q0 + 126 + (t & 3);
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        xa[j][i] = qa >= 0 ? row[static_cast<size_t>((2 * half + j) * 8 + i) * N + qa] : 0.f;
+    if (t < 16) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        xb[i] = qb < N ? row[static_cast<size_t>((t >> 2) * 8 + i) * N + qb] : 0.f;
+    }
+  };
+  fetch(blockIdx.x);
+  // the weights' terms: tap k, chunk kc, output o -> rows o, 32 + o, 64 + o
+  bool off = false;
+  for (int e = t; e < kDnK * 4 * 32; e += kCvThreads) {
+    const int k = e / 128, kc = (e / 32) % 4, o = e % 32;
+    float w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = wt[((kc * 8 + i) * kDnK + k) * 32 + o];
+    uint4 s[3];
+    off |= cv_split8(w, s);
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+      *reinterpret_cast<uint4*>(smem + k * kCvTap + (4 * p + (o >> 3)) * 512 + kc * 128 + (o & 7) * 16) = s[p];
+  }
+  tmem_fence_before();
+  bool plain = __syncthreads_or(off);   // this block's tiles on the CUDA cores
+  tmem_fence_after();
+  const uint32_t tmm = *tbase;
+  const uint32_t tm = tmm + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + 16 * half;
+  const uint64_t dx = umma_desc(smem_u32(smem + kCvX), kCvLbo, 128);
+  const uint64_t dw = umma_desc(smem_u32(smem), 128, 512);
+  bool ok = true;
+  uint32_t phase = 0;
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int r = tile / tiles_row, q0 = (tile % tiles_row) * kDnPos;
+    const size_t at0 = (static_cast<size_t>(r) * 32 + 16 * half) * N + q0 + u;   // output 16 half
+    off = !ok;
+    unsigned char* xs = smem + kCvX;
+    uint4 s[3];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      off |= cv_split8(xa[j], s);
+#pragma unroll
+      for (int p = 0; p < 3; ++p)
+        *reinterpret_cast<uint4*>(xs + p * kCvPlane + (2 * half + j) * kCvLbo + u * 16) = s[p];
+    }
+    if (t < 16) {
+      off |= cv_split8(xb, s);
+#pragma unroll
+      for (int p = 0; p < 3; ++p)
+        *reinterpret_cast<uint4*>(xs + p * kCvPlane + (t >> 2) * kCvLbo + (128 + (t & 3)) * 16) = s[p];
+    }
+    fence_proxy_async();
+    tmem_fence_before();
+    const bool cores = __syncthreads_or(off || plain);
+    tmem_fence_after();
+    if (t == 0 && !cores) {
+#pragma unroll
+      for (int k = 0; k < kDnK; ++k)
+#pragma unroll
+        for (int kh = 0; kh < 2; ++kh) {
+          const uint64_t a = dx + ((k * 16 + kh * 2 * kCvLbo) >> 4);
+          const uint64_t b = dw + ((k * kCvTap + kh * 256) >> 4);
+          const uint32_t more = k + kh > 0 ? 1u : 0u;
+          umma_f16(tmm + 32 * k, a, b, umma_idesc(32, true), kh);
+          umma_f16(tmm + kCvCross, a, b + (4 * 512 >> 4), umma_idesc(64, true), more);
+          umma_f16(tmm + kCvCross, a + (kCvPlane >> 4), b, umma_idesc(64, true), 1u);
+          umma_f16(tmm + kCvCross + 32, a + (2 * kCvPlane >> 4), b, umma_idesc(32, true), 1u);
+        }
+      umma_commit(smem_u32(bar));
+    }
+    fetch(tile + gridDim.x);
+    float m[16];
+    if (BWD) {
+#pragma unroll
+      for (int o = 0; o < 16; ++o) m[o] = mask[at0 + static_cast<size_t>(o) * N];
+    }
+    float y[16];
+    if (!cores) {
+      ok = __all_sync(0xffffffffu, mbar_wait_bounded(smem_u32(bar), phase));
+      phase ^= 1;
+    }
+    if (!cores && ok) {
+      tmem_fence_after();
+      float a[16], b[16], c[16];
+      Tmem<16>::ld(tm, a);
+      Tmem<16>::ld(tm + 32, b);
+      tmem_wait_ld();
+#pragma unroll
+      for (int o = 0; o < 16; ++o) y[o] = a[o] + b[o];
+      Tmem<16>::ld(tm + 64, a);
+      Tmem<16>::ld(tm + 96, b);
+      tmem_wait_ld();
+#pragma unroll
+      for (int o = 0; o < 16; ++o) y[o] += a[o] + b[o];
+      Tmem<16>::ld(tm + 128, a);
+      Tmem<16>::ld(tm + kCvCross, b);
+      Tmem<16>::ld(tm + kCvCross + 32, c);
+      tmem_wait_ld();
+#pragma unroll
+      for (int o = 0; o < 16; ++o) {
+        y[o] += BWD ? a[o] : a[o] + bias[16 * half + o];
+        y[o] += b[o] + c[o];
+      }
+    } else {
+      // the same sums as FMAs
+#pragma unroll
+      for (int o = 0; o < 16; ++o) y[o] = BWD ? 0.f : bias[16 * half + o];
+#pragma unroll 1
+      for (int ck = 0; ck < 32 * kDnK; ++ck) {
+        const int q = q0 + u + ck % kDnK - 2;
+        const float x = q >= 0 && q < N ? in[(static_cast<size_t>(r) * 32 + ck / kDnK) * N + q] : 0.f;
+#pragma unroll
+        for (int o = 0; o < 16; ++o) y[o] = fmaf(wt[ck * 32 + 16 * half + o], x, y[o]);
+      }
+    }
+#pragma unroll
+    for (int o = 0; o < 16; ++o)
+      out[at0 + static_cast<size_t>(o) * N] = BWD ? (m[o] > 0.f ? y[o] : 0.f) : fmaxf(y[o], 0.f);
+  }
+  // a wait that gave up: its products get a second bounded chance to finish
+  if (!ok) (void)mbar_wait_bounded(smem_u32(bar), phase ^ 1);
+  tmem_fence_before();
+  __syncthreads();
+  tmem_fence_after();
+  if (warp == 0) tmem_dealloc(tmm, kCvCols);
 }
 template <bool BWD>
 static cudaError_t conv32(const float* in, const float* wt, const float* bias, const float* mask,
@@ -238,7 +367,7 @@ static cudaError_t conv32(const float* in, const float* wt, const float* bias, c
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, kCvSmem);
   if (e != cudaSuccess) return e;
   const int tiles = R * (N / kDnPos);
-  pdl_launch(dn_conv32_kernel<BWD>, dim3(tiles < 4 * sms ? tiles : 4 * sms), 128, kCvSmem, st, in,
+  pdl_launch(dn_conv32_kernel<BWD>, dim3(tiles < 2 * sms ? tiles : 2 * sms), kCvThreads, kCvSmem, st, in,
              wt, bias, mask, out, R, N);
   return cudaSuccess;
 }

@@ -70,7 +70,7 @@ class Denoiser:
 
         ``tensor_cores``: the BF16 pass on tcgen05 (bf16 operands and stored
         tensors, fp32 sums; the fp32 parameters are rounded to bf16 for it);
-        otherwise the FP32 pass on the CUDA cores."""
+        otherwise the FP32 pass."""
         R, N = int(Hls.shape[0]), int(Hls.shape[1])
         if tensor_cores:
             L.check(L.lsas_dn_grad_tc(L._ptr(self.params), L._ptr(Hls), L._ptr(Ht), R, N,
