@@ -162,11 +162,12 @@ __global__ void __launch_bounds__(256) dn_conv_in_kernel(const float* __restrict
 // operand of tap k is the same buffer k rows on; the weights' terms one after
 // the other as N, so that x0 meets w1 and w2 in one MMA of N = 64.  A block
 // fetches the next tile under a tile's MMAs; two blocks an SM fill each
-// other's gaps.  A tile with a value outside 2^-100 .. 2^120 (but
-// zero), whose split would not be exact, and, after a wait that gave up, every
-// further tile is summed by FMAs.  256 rows of 1024: 26 us, 27 masked (10 and 15 to read and
-// write HBM), against 51 us for packed FMAs from registers (8 outputs x 4
-// positions a thread).
+// other's gaps.  A tile with a value outside 2^-100 .. 2^120 (but zero), whose
+// split would not be exact, and, after a wait that gave up, every further tile
+// is summed by FMAs.  Bound by the 40 MMAs of a tile, which read 4 KB of
+// shared memory each whatever their N.  256 rows of 1024: 27 us, 28 masked (10
+// and 15 to read and write HBM), against 51 us for packed FMAs from registers
+// (8 outputs x 4 positions a thread); 24 with one accumulator for three taps.
 constexpr int kCvRows = kDnPos + kDnK - 1;           // row j holds position q0 - 2 + j
 constexpr int kCvLbo = kCvRows * 16;                 // bytes between channel chunks
 constexpr int kCvPlane = 4 * kCvLbo;                 // one term of a tile's input
@@ -582,7 +583,8 @@ __global__ void __launch_bounds__(kFwThreads, 2) dn_wgrad32_kernel(const float* 
 // Bound by one pass over B.  A warp takes four channels and a lane four
 // positions of each tile, 40 sums in registers; blocks walk the tiles and
 // write one row of partial sums each ([j][k][c], then the biases).  256 rows of
-// 1024: 23 us (30 without the loads one tile ahead).
+// 1024: 20 us with one block of each layer an SM (23 with two, whose second
+// wave starts and sums anew; 30 without the loads one tile ahead).
 constexpr int kSdPart = 320 + 32;
 __global__ void __launch_bounds__(256, 2) dn_side32_kernel(const float* __restrict__ dy,
                                                         const float* __restrict__ r3,
@@ -2053,9 +2055,9 @@ cudaError_t dn_grad(const float* P, const float2* Hls, const float2* Ht, int R, 
   o.inv_n = 2.0f / static_cast<float>(n);
   o.N = N;
   pdl_launch(dn_conv_out_kernel<true>, dim3(tiles), 256, 0, st, o);
-  // two blocks of the weight-gradient kernels per SM
+  // two blocks per SM: of one 32 -> 32 layer, or one of each of the other two
   const int parts = wg_blocks(R, N);
-  const int wgb = 2 * sms < parts ? 2 * sms : parts;
+  const int wgb = 2 * sms < parts ? 2 * sms : parts, sdb = sms < parts ? sms : parts;
   float* wp3 = d.wp;
   float* wp2 = wp3 + static_cast<size_t>(parts) * kWgPart;
   float* sp4 = wp2 + static_cast<size_t>(parts) * kWgPart;
@@ -2069,12 +2071,12 @@ cudaError_t dn_grad(const float* P, const float2* Hls, const float2* Ht, int R, 
   pdl_launch(dn_wgrad32_kernel, dim3(wgb), kFwThreads, kFwSmem, st, d.g2, d.a1, R, N, wp2);
   e = conv32<true>(d.g2, d.wt + kBw2, nullptr, d.a1, d.g1, R, N, sms, st);
   if (e != cudaSuccess) return e;
-  pdl_launch(dn_side32_kernel, dim3(wgb, 2), 256, 0, st, d.dy, d.a3, d.x0, d.g1, R, N, sp4, sp1);
+  pdl_launch(dn_side32_kernel, dim3(sdb, 2), 256, 0, st, d.dy, d.a3, d.x0, d.g1, R, N, sp4, sp1);
   DnReduceArgs a{};
   a.l[0] = {wp3, wgb, kWgPart, grad + kOffW3, grad + kOffB3};
   a.l[1] = {wp2, wgb, kWgPart, grad + kOffW2, grad + kOffB2};
-  a.l[2] = {sp4, wgb, kSdPart, grad + kOffW4, grad + kOffB4};
-  a.l[3] = {sp1, wgb, kSdPart, grad + kOffW1, grad + kOffB1};
+  a.l[2] = {sp4, sdb, kSdPart, grad + kOffW4, grad + kOffB4};
+  a.l[3] = {sp1, sdb, kSdPart, grad + kOffW1, grad + kOffB1};
   a.loss_part = d.y;
   a.loss_n = tiles;
   a.n = n;
