@@ -165,7 +165,8 @@ __global__ void __launch_bounds__(256) dn_conv_in_kernel(const float* __restrict
 // other's gaps.  A tile with a value outside 2^-100 .. 2^120 (but zero), whose
 // split would not be exact, and, after a wait that gave up, every further tile
 // is summed by FMAs.  Bound by the 40 MMAs of a tile, which read 4 KB of
-// shared memory each whatever their N.  256 rows of 1024: 27 us, 28 masked (10
+// shared memory each whatever their N (with everything else of a tile under
+// the MMAs of the one before, by a warp that only issues: 28 us).  256 rows of 1024: 27 us, 28 masked (10
 // and 15 to read and write HBM), against 51 us for packed FMAs from registers
 // (8 outputs x 4 positions a thread); 24 with one accumulator for three taps.
 constexpr int kCvRows = kDnPos + kDnK - 1;           // row j holds position q0 - 2 + j
