@@ -80,9 +80,12 @@ __device__ __forceinline__ void window8(const float* __restrict__ row, int q, in
 }
 
 __device__ __forceinline__ void cp_async(uint32_t dst, const void* src, bool on, int bytes) {
-  // bytes is 8 or 16; zero-fills when off
+  // bytes is 4, 8 or 16; zero-fills when off
   if (bytes == 16)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(on ? 16 : 0)
+                 : "memory");
+  else if (bytes == 4)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(on ? 4 : 0)
                  : "memory");
   else
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(on ? 8 : 0)
@@ -457,16 +460,23 @@ __global__ void __launch_bounds__(256) dn_conv_out_kernel(const DnOutArgs a) {
 // A[c][p + k - 2] and db[o] = sum_p G[o][p], as a product with the positions
 // as the inner dimension.  Bound by the FMA pipe (5120 FMAs a position).  A
 // tile's G and A rows come to shared memory by asynchronous copies, one tile
-// ahead; a thread keeps 4 outputs x 2 inputs x 5 taps and takes the tile four
-// positions at a time: six 16-byte loads (A slides in registers) for 160 FMAs.
-// The two halves of a block take the tile's halves.  Blocks walk the tiles
-// (two blocks fit on an SM) and write one row of partial sums each.  256 rows
-// of 1024: 58 us a layer (packed FMAs over even and odd positions, whose
-// operand pairs share no register from one to the next: 71); one block per
-// (o, c) that re-read both tensors took about 1900 us.
+// ahead, G with the values of two outputs side by side (4-byte copies: the
+// copies' 16-byte pieces would need a transpose); a thread keeps 2 output pairs
+// x 2 inputs x 5 taps and takes the tile four positions at a time: six 16-byte
+// loads (A slides in registers, each value in both halves of a pair) for 160
+// FMAs, issued as 80 packed ones.  The two halves of a block take the tile's
+// halves.  Blocks walk the tiles (two blocks fit on an SM) and write one row of
+// partial sums each.  256 rows of 1024: 53 us a layer, FMA pipe 67 % busy
+// (scalar FMAs: 58, issue 75 %; packed over even and odd positions, whose
+// operand pairs share no register from one to the next: 71; on the tensor cores
+// with operands split as above, their sums read out every 32 positions for
+// FP32 accuracy: 117); one block per (o, c) that re-read both tensors took
+// about 1900 us.
 constexpr int kFwThreads = 256;
-constexpr int kFwRow = kDnPos + 4;                     // floats; rows 4 banks apart
-constexpr int kFwStage = 2 * 32 * kFwRow * 4;          // bytes of G and A
+constexpr int kFwRow = kDnPos + 4;                     // floats of a row of A; rows 4 banks apart
+constexpr int kFwGRow = 2 * kDnPos + 4;                // of two rows of G, output pairs side by side
+constexpr int kFwG = 16 * kFwGRow * 4;                 // bytes of G, then A
+constexpr int kFwStage = kFwG + 32 * kFwRow * 4;
 constexpr int kFwSmem = 2 * kFwStage;
 constexpr int kWgPart = 5 * 32 * 32 + 32;              // one block's partials (floats)
 static_assert(kFwSmem >= 128 * 40 * 4, "the halves meet in the stages");
@@ -478,15 +488,17 @@ __global__ void __launch_bounds__(kFwThreads, 2) dn_wgrad32_kernel(const float* 
   extern __shared__ __align__(128) unsigned char smem[];
   const int t = threadIdx.x, lane = t & 31;
   const int half = t >> 7, u = t & 127;
-  const int og = u & 7, cg = u >> 3;                   // o = og + 8 i, c = cg + 16 j
+  const int og = u & 7, cg = u >> 3;                   // o = 2 (og + 8 i) + {0, 1}, c = cg + 16 j
   const int tiles_row = N / kDnPos, tiles = R * tiles_row;
   auto fetch = [&](int tile, int b) {
     if (tile < tiles) {
       const int r = tile / tiles_row, q0 = (tile % tiles_row) * kDnPos;
-      const uint32_t g = smem_u32(smem + b * kFwStage), x = g + 32 * kFwRow * 4;
-      for (int i = t; i < 32 * 32; i += kFwThreads) {
-        const int o = i >> 5, p = 4 * (i & 31);
-        cp_async(g + (o * kFwRow + p) * 4, G + (static_cast<size_t>(r) * 32 + o) * N + q0 + p, true, 16);
+      const uint32_t g = smem_u32(smem + b * kFwStage), x = g + kFwG;
+#pragma unroll 4
+      for (int i = t; i < 32 * kDnPos; i += kFwThreads) {
+        const int o = i / kDnPos, p = i % kDnPos;
+        cp_async(g + ((o >> 1) * kFwGRow + 2 * p + (o & 1)) * 4,
+                 G + (static_cast<size_t>(r) * 32 + o) * N + q0 + p, true, 4);
       }
       constexpr int kHalf = (kDnPos + 4) / 2;
       for (int i = t; i < 32 * kHalf; i += kFwThreads) {
@@ -497,14 +509,14 @@ __global__ void __launch_bounds__(kFwThreads, 2) dn_wgrad32_kernel(const float* 
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  float acc[4][2][kDnK];
-  float bacc = 0.f;
+  float2 acc[2][2][kDnK];   // [output pair][input][tap]
+  float2 bacc = make_float2(0.f, 0.f);
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 2; ++j)
 #pragma unroll
-      for (int k = 0; k < kDnK; ++k) acc[i][j][k] = 0.f;
+      for (int k = 0; k < kDnK; ++k) acc[i][j][k] = make_float2(0.f, 0.f);
   fetch(blockIdx.x, 0);
   int b = 0;
   for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, b ^= 1) {
@@ -512,37 +524,51 @@ __global__ void __launch_bounds__(kFwThreads, 2) dn_wgrad32_kernel(const float* 
     asm volatile("cp.async.wait_group 1;" ::: "memory");
     __syncthreads();
     const float* g = reinterpret_cast<const float*>(smem + b * kFwStage);
-    const float* x = g + 32 * kFwRow;
-    {   // bias: eight threads an output, 16 positions each
-      const float4* gb = reinterpret_cast<const float4*>(g + (t >> 3) * kFwRow) + (t & 7);
+    const float* x = g + kFwG / 4;
+    {   // bias: sixteen threads an output pair, 8 positions each
+      const float4* gb = reinterpret_cast<const float4*>(g + (t >> 4) * kFwGRow) + (t & 15);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const float4 v = gb[8 * i];
-        bacc += (v.x + v.y) + (v.z + v.w);
+        const float4 v = gb[16 * i];
+        bacc = __fadd2_rn(bacc, __fadd2_rn(make_float2(v.x, v.y), make_float2(v.z, v.w)));
       }
     }
-    const float* gt = g + og * kFwRow + 64 * half;
+    const float* gt = g + og * kFwGRow + 128 * half;
     const float* xt = x + cg * kFwRow + 64 * half;
-    float4 lo[2];
+    float2 lo[2][4];   // {x, x} of the window's first four positions
 #pragma unroll
-    for (int j = 0; j < 2; ++j) lo[j] = *reinterpret_cast<const float4*>(xt + 16 * j * kFwRow);
+    for (int j = 0; j < 2; ++j) {
+      const float4 v = *reinterpret_cast<const float4*>(xt + 16 * j * kFwRow);
+      lo[j][0] = make_float2(v.x, v.x);
+      lo[j][1] = make_float2(v.y, v.y);
+      lo[j][2] = make_float2(v.z, v.z);
+      lo[j][3] = make_float2(v.w, v.w);
+    }
 #pragma unroll 2
     for (int p = 0; p < 64; p += 4) {
-      float gv[4][4];
+      float2 gv[2][4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        *reinterpret_cast<float4*>(gv[i]) = *reinterpret_cast<const float4*>(gt + 8 * i * kFwRow + p);
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float4 v = *reinterpret_cast<const float4*>(gt + 8 * i * kFwGRow + 2 * p + 4 * h);
+          gv[i][2 * h] = make_float2(v.x, v.y);
+          gv[i][2 * h + 1] = make_float2(v.z, v.w);
+        }
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         const float4 hi = *reinterpret_cast<const float4*>(xt + 16 * j * kFwRow + p + 4);
-        const float w[8] = {lo[j].x, lo[j].y, lo[j].z, lo[j].w, hi.x, hi.y, hi.z, hi.w};
+        const float2 w[8] = {lo[j][0], lo[j][1], lo[j][2], lo[j][3],
+                             make_float2(hi.x, hi.x), make_float2(hi.y, hi.y),
+                             make_float2(hi.z, hi.z), make_float2(hi.w, hi.w)};
 #pragma unroll
         for (int q = 0; q < 4; ++q)
 #pragma unroll
           for (int k = 0; k < kDnK; ++k)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) acc[i][j][k] = fmaf(gv[i][q], w[k + q], acc[i][j][k]);
-        lo[j] = hi;
+            for (int i = 0; i < 2; ++i) acc[i][j][k] = __ffma2_rn(gv[i][q], w[k + q], acc[i][j][k]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) lo[j][q] = w[4 + q];
       }
     }
     __syncthreads();   // the stage is consumed before the next copies into it
@@ -552,29 +578,33 @@ __global__ void __launch_bounds__(kFwThreads, 2) dn_wgrad32_kernel(const float* 
   // the halves' sums meet, the first half writes
   float* out = part + static_cast<size_t>(blockIdx.x) * kWgPart;
   float* comb = reinterpret_cast<float*>(smem);
+  float2* comb2 = reinterpret_cast<float2*>(comb);
   if (half == 1) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
       for (int j = 0; j < 2; ++j)
 #pragma unroll
         for (int k = 0; k < kDnK; ++k)
-          comb[((i * 2 + j) * kDnK + k) * 128 + u] = acc[i][j][k];
+          comb2[((i * 2 + j) * kDnK + k) * 128 + u] = acc[i][j][k];
   }
   __syncthreads();
   if (half == 0) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
       for (int j = 0; j < 2; ++j)
 #pragma unroll
         for (int k = 0; k < kDnK; ++k)
-          out[(k * 32 + cg + 16 * j) * 32 + og + 8 * i] =
-              acc[i][j][k] + comb[((i * 2 + j) * kDnK + k) * 128 + u];
+          *reinterpret_cast<float2*>(out + (k * 32 + cg + 16 * j) * 32 + 2 * (og + 8 * i)) =
+              __fadd2_rn(acc[i][j][k], comb2[((i * 2 + j) * kDnK + k) * 128 + u]);
   }
 #pragma unroll
-  for (int off = 4; off > 0; off >>= 1) bacc += __shfl_xor_sync(0xffffffffu, bacc, off);
-  if ((lane & 7) == 0) out[5120 + (t >> 3)] = bacc;
+  for (int off = 8; off > 0; off >>= 1) {
+    bacc.x += __shfl_xor_sync(0xffffffffu, bacc.x, off);
+    bacc.y += __shfl_xor_sync(0xffffffffu, bacc.y, off);
+  }
+  if ((lane & 15) == 0) *reinterpret_cast<float2*>(out + 5120 + 2 * (t >> 4)) = bacc;
 }
 
 // Weight gradients of the layers with a two-channel side, FP32, in one launch
