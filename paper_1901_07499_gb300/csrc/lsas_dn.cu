@@ -1641,7 +1641,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) dn_tc_wgrad_kernel(const DnWgra
 // layer's rows: 16 slices of consecutive rows are added side by side (a serial
 // chain of rows / 16 coalesced loads), then the slices in order.  (One thread
 // per column over 1024 rows took 78 us a layer and one thread over every tile
-// 32 us for the loss; this launch takes 3.6 us at 152 rows and 8.6 at 304.)
+// 32 us for the loss; this launch takes 3.5 us at 152 rows and 5.9 at 304; 8.7 with the
+// rows past the last ten of a slice one after the other.)
 struct DnReduceLayer {
   const float* part;   // [rows][stride]
   int rows, stride;
@@ -1691,8 +1692,16 @@ __global__ void __launch_bounds__(kRdThreads) dn_reduce_kernel(const DnReduceArg
   const int per = (l.rows + kRdSlices - 1) / kRdSlices;
   const int lo = slice * per, hi = min(l.rows, lo + per);
   float s = 0.f;
-#pragma unroll 10
-  for (int i = lo; i < hi; ++i) s += l.part[static_cast<size_t>(i) * l.stride + col];
+  // ten rows in flight, the last ones too, added in order
+  for (int i = lo; i < hi; i += 10) {
+    float v[10];
+#pragma unroll
+    for (int j = 0; j < 10; ++j)
+      v[j] = i + j < hi ? l.part[static_cast<size_t>(i + j) * l.stride + col] : 0.f;
+#pragma unroll
+    for (int j = 0; j < 10; ++j)
+      if (i + j < hi) s += v[j];
+  }
   red[slice][col32] = s;
   __syncthreads();
   if (slice != 0) return;
