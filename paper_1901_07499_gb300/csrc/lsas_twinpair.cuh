@@ -175,6 +175,9 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
     for (int s = 0; s < K; ++s) mbar_init(smem_u32(&bars[s]), 1);
     fence_mbar_init();
   }
+  // the first copies stand before the block's barrier, and thread 1 of the pair
+  // issues one of them; the pair's second warp meets the barriers behind it
+  __syncwarp();
   uint32_t tE = 0;
   const uint64_t pol = jt < 2 ? evict_first_policy() : 0;
   float zero[16];
