@@ -43,8 +43,9 @@
  * at pilot_idx, D = S - 1 data symbols), q = log2(Q) bits per data symbol.
  *
  * Ownership: the caller owns every buffer passed in.  A plan owns only its own
- * device tables (twiddles, pilot inverse, a status word) and, after the first
- * lsas_run_frame_host call, its host-transfer staging buffers.
+ * device tables (twiddles, pilot inverse, a status word), the scratch of its
+ * batch split (see lsas_run_frame) and, after the first lsas_run_frame_host
+ * call, its host-transfer staging buffers.
  *
  * Errors: argument checks run on the host before any launch; a failing check
  * returns its code and enqueues nothing.  A CUDA launch or copy failure
@@ -138,8 +139,7 @@ lsas_status lsas_estimate(lsas_plan plan, const void* d_in, int n_frames,
  * MRC demodulation of the data symbols with a given channel d_H (Sec. II-C):
  * writes d_bits and, if d_eq is not NULL, the combined symbols z.  d_H may
  * come from lsas_estimate or from any other estimator.  Asynchronous.
- * Batches are split into antenna shards as by lsas_run_frame (except while
- * the stream is being captured into a graph: one launch then).
+ * Batches are split into antenna shards as by lsas_run_frame.
  */
 lsas_status lsas_demodulate(lsas_plan plan, const void* d_in,
                             const float* d_H, int n_frames, uint8_t* d_bits,
@@ -157,7 +157,11 @@ lsas_status lsas_demodulate(lsas_plan plan, const void* d_in,
  * forms z and the bits from them, summing the shards in a fixed order.
  * Outputs agree with the unsplit pass to rounding (the antenna sums are
  * ordered differently).  Calls on one plan from several streams take turns
- * on the scratch array: a split waits for the previous split's combine.
+ * on the scratch array: a split waits for the previous split's combine.  A
+ * split recorded into a graph (stream capture) has scratch of its own, kept
+ * until the plan is destroyed, so its replays run beside other calls; the
+ * graph must not be replayed after that, nor overlap itself.  A plan keeps at
+ * most 96 MiB for recorded splits; past that the frames are recorded unsplit.
  * lsas_plan_set_batch_split turns the split off.
  */
 lsas_status lsas_run_frame(lsas_plan plan, const void* d_in, int n_frames,

@@ -53,7 +53,8 @@ using namespace lsas;
 namespace {
 
 constexpr int kSmemLimit = 232448;   // opt-in dynamic shared memory per block
-constexpr size_t kTailBytes = 96u << 20;   // cap of a plan's split-tail partial sums
+constexpr size_t kTailBytes = 96u << 20;   // cap of a plan's split-tail partial sums (and
+                                           // of those of its splits recorded into graphs)
 // Share of a fused block's time that does not shrink with its antenna count
 // (the group-end reductions, demap and pack), for the split decision, from
 // single-frame timings on GB300: about 0.08 for the per-warp kernel
@@ -106,8 +107,11 @@ struct lsas_plan_s {
   int tail_units = 0;               // shard-frames d_tail holds
   int batch_split = 1;              // lsas_plan_set_batch_split: 0 off, 1 per batch, 2 fixed
   cudaEvent_t tail_ev = nullptr;    // the last split's combine has read d_tail
-  bool tail_live = false;           // ... on the stream with this id, outside any capture
+  bool tail_live = false;           // ... on the stream with this id
   unsigned long long tail_stream = 0;
+  // splits recorded into graphs: scratch of their own, for the plan's lifetime
+  std::vector<float*> graph_tails;
+  size_t graph_tail_bytes = 0;
   std::mutex tail_mu;
   size_t dev_bytes = 0;             // device memory allocated at creation
   Geometry geo;
@@ -606,27 +610,50 @@ int tail_shards(lsas_plan p, int nf) {
   return best_shards(p, nf, p->tail_units);
 }
 
+// Scratch of a split that is being recorded into a graph, null when the plan's
+// limit is reached.  The capture may not wait for the event that hands d_tail
+// on from split to split, nor a live split for one recorded in a capture, and a
+// replay could not take its turn; so each recorded split has partial sums of
+// its own, which only replays of that call touch (they share its outputs, so
+// they cannot overlap anyway).
+float* graph_tail(lsas_plan p, size_t bytes) {
+  if (p->graph_tail_bytes + bytes > kTailBytes) return nullptr;
+  // an allocation does not enter the capture, whatever the capture's mode
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return nullptr;
+  float* t = nullptr;
+  if (cudaMalloc(&t, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    t = nullptr;
+  }
+  try {
+    if (t) p->graph_tails.push_back(t);
+  } catch (...) {   // out of host memory
+    cudaFree(t);
+    t = nullptr;
+  }
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (t) p->graph_tail_bytes += bytes;
+  return t;
+}
+
 // Frames [f0, f0 + nf) of a batch as G antenna shards: the fused kernel's
 // partial mode writes the shards' partial sums and H (d_Hin null) or reads
 // the given channel d_Hin, the combine kernel forms z and the bits.  Calls on different streams share
-// d_tail: each waits for the previous split's combine.
+// d_tail: each waits for the previous split's combine.  While st is being
+// captured the partial sums go to scratch of the recorded call's own, and the
+// frames run whole where there is none.
 lsas_status run_split_tail(lsas_plan p, const void* d_in, int f0, int nf, int G, float* d_H,
                            const float* d_Hin, uint8_t* d_bits, float* d_eq, cudaStream_t st) {
   const size_t in_b = in_bytes_per_frame(p->M, p->N, p->cp, p->S, p->fmt);
   const size_t bits_b = bits_bytes_per_frame(p->N, p->S, p->Q);
   const unsigned char* in = static_cast<const unsigned char*>(d_in) + f0 * in_b;
   std::lock_guard<std::mutex> lock(p->tail_mu);
-  // the previous split's combine first, unless it went to this very stream
-  // (by its id, which no later stream takes over), whose order does that: the
-  // wait costs 2 us and keeps the launches from overlapping
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   unsigned long long id = 0;
-  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cudaStreamGetId(st, &id) != cudaSuccess)
-    return LSAS_ERR_CUDA;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) return LSAS_ERR_CUDA;
   const bool live = cap == cudaStreamCaptureStatusNone;
-  if (!(live && p->tail_live && p->tail_stream == id) &&
-      cudaStreamWaitEvent(st, p->tail_ev, 0) != cudaSuccess)
-    return LSAS_ERR_CUDA;
+  if (live && cudaStreamGetId(st, &id) != cudaSuccess) return LSAS_ERR_CUDA;
   KParams k;
   base_params(p, &k);
   k.in = in;
@@ -651,8 +678,23 @@ lsas_status run_split_tail(lsas_plan p, const void* d_in, int f0, int nf, int G,
     k.shard_y = k.M;
     k.grid_y = G;
   }
+  const size_t sums = static_cast<size_t>(G) * nf * p->D * p->N * 2;   // floats of P, then E
   float* P = p->d_tail;
-  float* E = P + static_cast<size_t>(G) * nf * p->D * p->N * 2;
+  if (!live) {
+    P = graph_tail(p, (sums + static_cast<size_t>(G) * nf * p->N) * sizeof(float));
+    if (!P)
+      return launch_frame(p, in, nf, d_Hin ? nullptr : d_H + h0, d_Hin ? d_Hin + h0 : nullptr,
+                          d_bits + f0 * bits_b,
+                          d_eq ? d_eq + static_cast<size_t>(f0) * p->D * p->N * 2 : nullptr,
+                          d_Hin ? kModeDemod : kModeRun, st);
+  } else if (!(p->tail_live && p->tail_stream == id) &&
+             cudaStreamWaitEvent(st, p->tail_ev, 0) != cudaSuccess) {
+    // the previous split's combine first, unless it went to this very stream
+    // (by its id, which no later stream takes over), whose order does that: the
+    // wait costs 2 us and keeps the launches from overlapping
+    return LSAS_ERR_CUDA;
+  }
+  float* E = P + sums;
   k.P_out = reinterpret_cast<float2*>(P);
   k.E_out = E;
   k.chunks = (k.M + p->geo.Af - 1) / p->geo.Af;
@@ -675,8 +717,9 @@ lsas_status run_split_tail(lsas_plan p, const void* d_in, int f0, int nf, int G,
                 : nullptr;
     if (launch_combine(c, st) != cudaSuccess) s = LSAS_ERR_CUDA;
   }
+  if (!live) return s;
   const bool recorded = cudaEventRecord(p->tail_ev, st) == cudaSuccess;
-  p->tail_live = live && recorded;
+  p->tail_live = recorded;
   p->tail_stream = id;
   return recorded ? s : LSAS_ERR_CUDA;
 }
@@ -689,15 +732,7 @@ lsas_status run_batch(lsas_plan p, const void* d_in, int n_frames, float* d_H, c
                       uint8_t* d_bits, float* d_eq, cudaStream_t st) {
   const int mode = d_Hin ? kModeDemod : kModeRun;
   const int full = (n_frames / p->sms) * p->sms;
-  int G = tail_shards(p, n_frames - full);
-  if (G > 1 && d_Hin) {
-    // a demodulation recorded into a graph stays one launch: the split orders
-    // itself behind other streams' splits by an event, which a capture may not
-    // wait for
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) return LSAS_ERR_CUDA;
-    if (cap != cudaStreamCaptureStatusNone) G = 1;
-  }
+  const int G = tail_shards(p, n_frames - full);
   if (G == 1) return launch_frame(p, d_in, n_frames, d_H, d_Hin, d_bits, d_eq, mode, st);
   if (full > 0) {
     const lsas_status s = launch_frame(p, d_in, full, d_H, d_Hin, d_bits, d_eq, mode, st);
@@ -1420,6 +1455,7 @@ lsas_status lsas_plan_destroy(lsas_plan p) {
   cudaFree(p->d_tc_tw);
   cudaFree(p->d_pn);
   cudaFree(p->d_tail);
+  for (float* t : p->graph_tails) cudaFree(t);
   if (p->tail_ev) cudaEventDestroy(p->tail_ev);
   for (int i = 0; i < 2; ++i) {
     cudaFree(p->d_in_stage[i]);
