@@ -439,13 +439,6 @@ void base_params(lsas_plan p, KParams* k) {
   }
 }
 
-// Bulk copies need 16-byte aligned rows: every row start
-// ((f M + m) S + s)(N + CP) + CP samples from a 16-byte aligned base.
-bool tma_ok(lsas_plan p, const void* d_in) {
-  const int bps = p->fmt == LSAS_IN_SC16 ? 4 : 8;
-  return aligned16(d_in) && ((p->N + p->cp) * bps) % 16 == 0 && (p->cp * bps) % 16 == 0;
-}
-
 // Row batch of lsas_fft (every symbol of every antenna) or lsas_estimate (the
 // pilots) for the two-rows-at-once kernel.
 void row_batch(lsas_plan p, int n_frames, bool pilots, KParams* k) {
@@ -466,15 +459,11 @@ lsas_status set_device(lsas_plan p) {
   return LSAS_OK;
 }
 
-// How rows reach shared memory (KParams::use_tma): bulk copies where every row
-// starts on 16 bytes; from the boundary before each row where that lies
-// within the buffer (an aligned buffer, or a prefix of three samples or more)
-// and the samples are aligned to themselves; plain loads otherwise.
-int staging(lsas_plan p, const void* d_in) {
-  if (tma_ok(p, d_in)) return 1;
-  const uintptr_t a = reinterpret_cast<uintptr_t>(d_in);
-  const bool whole = a % (p->fmt == LSAS_IN_SC16 ? 4 : 8) == 0;
-  return whole && (aligned16(d_in) || p->cp >= 3) ? 2 : 0;
+// KParams::use_tma for the plan's rows in d_in; shard: the call reads some of the
+// antennas only.
+int staging(lsas_plan p, const void* d_in, bool shard = false) {
+  return row_staging(reinterpret_cast<uintptr_t>(d_in), p->N, p->cp,
+                     p->fmt == LSAS_IN_SC16 ? 4 : 8, shard);
 }
 
 lsas_status check_frames(lsas_plan p, int n_frames) {
@@ -1052,7 +1041,7 @@ lsas_status lsas_mrc_partial(lsas_plan p, const void* d_in, int n_frames, int m_
   k.chunks = (m_count + p->geo.Af - 1) / p->geo.Af;
   ProfScope prof(p, "lsas_mrc_partial", stream);
   k.mode = kModePartial;
-  k.use_tma = staging(p, d_in);
+  k.use_tma = staging(p, d_in, m_count < p->M);
   if (p->launch(kKindFrame, p->fmt == LSAS_IN_FC32, k, n_frames, p->geo.smem_frame,
                 static_cast<cudaStream_t>(stream)) != cudaSuccess)
     return LSAS_ERR_CUDA;

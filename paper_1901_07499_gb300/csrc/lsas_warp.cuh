@@ -42,14 +42,35 @@
 
 namespace lsas {
 
+// How a plan's rows (N samples of bps bytes behind a prefix of cp) reach shared
+// memory from an input at address `at` (KParams::use_tma): 1, bulk copies, where
+// every row starts on 16 bytes; 2, bulk copies from the boundary before each
+// row, where the samples are aligned to themselves and that boundary lies
+// within what the call may read; 0, plain loads, otherwise.  It lies there
+// behind a prefix of three samples (the longest step back is 12 bytes of sc16
+// or 8 of fc32), and for an aligned input read whole; the first row of an
+// antenna shard (`shard`) with a shorter prefix would reach into the antenna
+// before.
+inline int row_staging(uintptr_t at, int N, int cp, int bps, bool shard) {
+  if (at % 16 == 0 && ((N + cp) * bps) % 16 == 0 && (cp * bps) % 16 == 0) return 1;
+  if (at % bps != 0) return 0;
+  return cp >= 3 || (at % 16 == 0 && !shard) ? 2 : 0;
+}
+
+// Bytes that a copy from the boundary `mis` bytes before a row of `row` bytes
+// takes: 16 more than the row, so that it ends in the next one.  The last row
+// of a frame's antennas (the shard's, in a split launch) is staged without
+// that piece, which the call may not read; its last samples come from memory.
+__host__ __device__ constexpr int staged_bytes(int row, int mis, bool last) {
+  return mis != 0 && !last ? row + 16 : row;
+}
+// Whether row s of antenna m of the M that the block takes is that last row.
+__host__ __device__ constexpr bool last_row(int M, int S, int m, int s) {
+  return m == M - 1 && s == S - 1;
+}
+
 #ifdef __CUDACC__
 
-// Whether a row is the last of the launch's input (its end may be the
-// buffer's).
-__device__ __forceinline__ bool last_row(const KParams& p, int f, int m, int s) {
-  return s == p.S - 1 && f == p.nf - 1 &&
-         p.m0 + static_cast<int>(blockIdx.y) * p.shard_y + m == p.Mtot - 1;
-}
 
 // Issue the bulk copies of one warp step (antennas of chunk c, symbol s)
 // into a slot: lane 0 registers the byte count, lane a copies row a.
@@ -61,12 +82,11 @@ __device__ __forceinline__ void wissue(const KParams& p, int f, int c, int s,
   constexpr uint32_t bytes = N * (FC32 ? 8 : 4);
   const int nvalid = min(A, p.M - c * A);
   if (p.use_tma == 2) {
-    // from the boundary before each row, 16 bytes more than the row where it
-    // does not start on one (the next row's, but past the last row of all)
+    // from the boundary before each row (staged_bytes)
     static_assert(A <= 32, "one row a lane");
     const unsigned char* src = row_ptr<LOG2N, FC32>(p, f, c * A + lane, s);
     const uint32_t mis = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(src) & 15);
-    const uint32_t n = lane >= nvalid ? 0u : (mis != 0 && !last_row(p, f, c * A + lane, s)) ? bytes + 16 : bytes;
+    const uint32_t n = lane >= nvalid ? 0u : staged_bytes(bytes, mis, last_row(p.M, p.S, c * A + lane, s));
     const uint32_t total = __reduce_add_sync(0xffffffffu, n);
     if (lane == 0) mbar_expect_tx(bar, total);
     __syncwarp();
@@ -80,9 +100,8 @@ __device__ __forceinline__ void wissue(const KParams& p, int f, int c, int s,
 }
 
 // Pass-1 inputs of a row staged from the 16-byte boundary before it: sample n
-// sits (row mod 16) bytes further on.  The last row of all is staged without
-// the piece that would reach past the buffer; its last samples come from
-// memory.
+// sits (row mod 16) bytes further on.  A last row's last samples, which were
+// not staged, come from memory.
 template <int LOG2N, bool FC32>
 __device__ __forceinline__ void wload_shifted(float2 (&v)[32], const unsigned char* staged,
                                               const unsigned char* row, bool last, int jt) {
@@ -305,7 +324,7 @@ __global__ void __launch_bounds__(32 * wgeo_warps(FC32 ? 8 : 4), 1) warp_kernel(
             if (p.use_tma == 2) {
               const int sym = witem_symbol(p, pilot_here, d0 + sa, it);
               wload_shifted<LOG2N, FC32>(v, row, row_ptr<LOG2N, FC32>(p, f, m, sym),
-                                         last_row(p, f, m, sym), jt);
+                                         last_row(p.M, p.S, m, sym), jt);
             } else {
               load_row<LOG2N, FC32>(v, row, jt, false);
             }
