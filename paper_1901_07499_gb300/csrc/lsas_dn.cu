@@ -1661,8 +1661,12 @@ __global__ void __launch_bounds__(kWgThreads, 1) dn_tc_wgrad_kernel(const DnWgra
 
 // Sums the blocks' partial rows of every weight gradient and (FP32) the loss
 // partials, in a fixed order, in one launch.  A block takes 32 columns of one
-// layer's rows: 16 slices of consecutive rows are added side by side (a serial
-// chain of rows / 16 coalesced loads), then the slices in order.  (One thread
+// layer's rows: 16 slices of consecutive rows are added side by side (rows / 16
+// coalesced loads each, ten at a time as a tree), then the slices as a tree: the
+// blocks' sums are of one sign where a gradient is large, so additions one
+// after the other at nearly its full size would set its error (1.26 times as
+// large against 64 bits, geometric mean of 80 FP32 gradients of 8 x 128 to 500 x
+// 512 and 256 x 1024 rows).  (One thread
 // per column over 1024 rows took 78 us a layer and one thread over every tile
 // 32 us for the loss; this launch takes 3.5 us at 152 rows and 5.9 at 304; 8.7 with the
 // rows past the last ten of a slice one after the other.)
@@ -1715,21 +1719,25 @@ __global__ void __launch_bounds__(kRdThreads) dn_reduce_kernel(const DnReduceArg
   const int per = (l.rows + kRdSlices - 1) / kRdSlices;
   const int lo = slice * per, hi = min(l.rows, lo + per);
   float s = 0.f;
-  // ten rows in flight, the last ones too, added in order
+  // ten rows in flight, the last ones too, added as a tree
   for (int i = lo; i < hi; i += 10) {
     float v[10];
 #pragma unroll
     for (int j = 0; j < 10; ++j)
       v[j] = i + j < hi ? l.part[static_cast<size_t>(i + j) * l.stride + col] : 0.f;
-#pragma unroll
-    for (int j = 0; j < 10; ++j)
-      if (i + j < hi) s += v[j];
+    s += (((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]))) + (v[8] + v[9]);
   }
   red[slice][col32] = s;
   __syncthreads();
   if (slice != 0) return;
+  float q[kRdSlices];
 #pragma unroll
-  for (int i = 1; i < kRdSlices; ++i) s += red[i][col32];
+  for (int i = 0; i < kRdSlices; ++i) q[i] = red[i][col32];
+#pragma unroll
+  for (int w = kRdSlices / 2; w > 0; w /= 2)
+#pragma unroll
+    for (int i = 0; i < w; ++i) q[i] += q[i + w];
+  s = q[0];
   if (layer < 2) {
     if (col < 5120) {
       const int k = col / 1024, c = (col / 32) % 32, o = col % 32;
