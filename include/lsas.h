@@ -397,9 +397,10 @@ lsas_status lsas_server_destroy(lsas_server server);
  *   lsas_dn_apply  d_H [R][N] complex -> d_Hout [R][N] complex (may not
  *                  alias d_H); bf16 != 0 reads bf16 parameters; fp32 sums.
  *                  (Here and in lsas_dn_grad the two 32 -> 32 layers run on
- *                  the tensor cores on operands split into three bf16 terms:
- *                  FP32 precision; values outside 2^-100 .. 2^120, and after a
- *                  bounded wait that gave up, on the FMA units.)
+ *                  the tensor cores on operands split into four bf16 terms:
+ *                  FP32 precision; tiles with values outside 2^-100 .. 2^60
+ *                  of their channel's scale, and after a bounded wait that
+ *                  gave up, on the FMA units, several times slower.)
  *   lsas_dn_grad   mean squared error between the network output and the
  *                  true rows d_Htrue normalised by the same RMS -> d_loss[0]
  *                  and the gradient d_grad [LSAS_DN_PARAMS].

@@ -150,63 +150,84 @@ __global__ void __launch_bounds__(256) dn_conv_in_kernel(const float* __restrict
 
 // 32 -> 32 channels in FP32 on tcgen05: layers 2 and 3 (bias and ReLU) or their
 // data gradients (masked).  The FMA pipe would need 33 us for 256 rows of 1024
-// (5120 FMAs a position), so the products go to the tensor cores: inputs and
-// weights are split into three bf16 terms each whose sum is the value
-// (x0 + x1 + x2, nearest even: |x1| <= 2^-9 |x|, |x2| <= 2^-18 |x|), products of
-// terms are exact in FP32, and of the nine the six down to 2^-18 are summed
-// (the others are below 2^-26 of the product).  The tensor cores' own FP32
-// additions do not round to nearest: the products x0 w0 have an accumulator
-// per tap, of two MMAs each, which the CUDA cores add, rounding to nearest; the
-// small products share two.  Relative error (norm) at 256 rows of 1024 against
-// 64 bits: layer output behind all layers 0.55e-7 (FP32 FMAs: 0.64e-7),
-// gradients 0.8e-7 (FMAs 0.7e-7; 1.3e-7 with one accumulator for three taps).
+// (5120 FMAs a position), so the products go to the tensor cores.  Their FP32
+// additions truncate: a sum of plain bf16 terms is always too small, and weight
+// gradients, which add many outputs, keep that (1.2 times their error).  So the
+// leading terms are small integers: x0 is the value rounded to a grid 2^-8 of
+// the power of two above the largest of its position's 32 channels (at most 256
+// steps, exact in bf16), w0 likewise with the 32 weights of an output and tap.
+// A tap's 32 products x0 w0 are then multiples of one step, at most 2^21 of
+// them, and their sum is exact in any order.  The remainder is exact too and
+// goes into three more bf16 terms, nearest even, which hold all of it.  Products
+// of terms are exact in FP32; those beside x0 w0 share three sums by order (x0
+// w1 + x1 w0; x0 w2 + x1 w1 + x2 w0; the four of the third), 2^-8 of the largest
+// product and less, where truncation does not count; the rest is below 2^-34 of
+// it.  Channels are scaled by powers of two so that each one's largest weight is
+// 1 to 2, which keeps a channel of small values and large weights as exact as
+// the others.  The CUDA cores add the taps' and the small sums, rounding to
+// nearest.  Relative error (norm) against 64 bits, geometric means over 80 sets
+// of 8 x 128 to 500 x 512 and 256 x 1024 rows: output 0.87 and gradients 0.67 of
+// the same layers as FMAs (tests/test_gpu_split_conv_rounding.py).
 //
 // Layout: positions as rows 16 bytes (eight channels) apart, so that the
 // operand of tap k is the same buffer k rows on; the weights' terms one after
-// the other as N, so that x0 meets w1 and w2 in one MMA of N = 64.  A block
+// the other as N, so that x0 meets w1, w2 and w3 in one MMA of N = 96.  A block
 // fetches the next tile under a tile's MMAs; two blocks an SM fill each
-// other's gaps.  A tile with a value outside 2^-100 .. 2^120 (but zero), whose
-// split would not be exact, and, after a wait that gave up, every further tile
-// is summed by FMAs.  Bound by the 40 MMAs of a tile, which read 4 KB of
-// shared memory each whatever their N (with everything else of a tile under
-// the MMAs of the one before, by a warp that only issues: 28 us).  256 rows of 1024: 27 us, 28 masked (10
-// and 15 to read and write HBM), against 51 us for packed FMAs from registers
-// (8 outputs x 4 positions a thread); 24 with one accumulator for three taps.
+// other's gaps.  A tile with a scaled value outside 2^-100 .. 2^60 (but zero),
+// whose last term may be no normal number or whose products may overflow on the
+// way, and, after a wait that gave up, every further tile is summed by FMAs from
+// memory, 160 loads an output one after the other: slow, and right.  Bound by
+// the 50 MMAs of a tile (4 KB of shared memory each whatever their N; tensor
+// pipe 55 to 60 % busy) and the splitting between them.  256 rows of 1024: 34
+// us, 35 masked (10 and 15 to read and write HBM), against 51 us for packed FMAs
+// from registers (8 outputs x 4 positions a thread) and 27 with three plain
+// bf16 terms, whose sums shrink by 1.6e-8.
 constexpr int kCvRows = kDnPos + kDnK - 1;           // row j holds position q0 - 2 + j
 constexpr int kCvLbo = kCvRows * 16;                 // bytes between channel chunks
 constexpr int kCvPlane = 4 * kCvLbo;                 // one term of a tile's input
-constexpr int kCvTap = 96 * 64;                      // one tap's weights: three terms x 32 outputs
+constexpr int kCvTerms = 4;
+constexpr int kCvTap = kCvTerms * 32 * 64;           // one tap's weights: four terms x 32 outputs
 constexpr int kCvX = kDnK * kCvTap;
-constexpr int kCvBar = kCvX + 3 * kCvPlane;
+constexpr int kCvMax = kCvX + kCvTerms * kCvPlane;   // [2][128]: largest of half a position's channels
+constexpr int kCvScale = kCvMax + 2 * kDnPos * 4;    // [32]: a channel's power of two
+constexpr int kCvBar = kCvScale + 32 * 4;
 constexpr int kCvSmem = kCvBar + 16;
 constexpr int kCvThreads = 256;
-constexpr int kCvCross = 32 * kDnK, kCvCols = 256;   // TMEM: a sum per tap, then the small products
+constexpr int kCvSmall = 32 * kDnK, kCvCols = 256;   // TMEM: a sum per tap, then three of small products
 static_assert(kCvX % 16 == 0 && kCvBar % 16 == 0, "16-byte operand alignment");
 
-// Eight values as three bf16 terms each (nearest even; the remainders are
-// exact, so the terms' sum is the value).  Returns whether one is outside the
-// range where that holds: zero, and 2^-100 (whose last term is a normal bf16
-// still) up to 2^120.
-__device__ __forceinline__ bool cv_split8(const float (&x)[8], uint4 (&out)[3]) {
-  uint32_t w[3][4];
-  bool off = false;
+// Whether a value is outside the range of the split: zero, and 2^-100 (whose
+// last term is a normal bf16 still) up to 2^60 (whose products' sums stay finite).
+__device__ __forceinline__ bool cv_off(float x) {
+  constexpr uint32_t kLo = (127u - 100u) << 23, kHi = (127u + 60u) << 23;
+  const uint32_t u = __float_as_uint(x) & 0x7fffffffu;
+  return u - kLo >= kHi - kLo && u != 0;
+}
+// The number whose addition and subtraction round a value to the grid of a
+// group with this largest magnitude: 1.5 * 2^16 times its power of two, so that
+// one unit in the last place of the sum is 2^-7 of that power.
+__device__ __forceinline__ float cv_grid(float most) {
+  return 1.5f * __uint_as_float((__float_as_uint(most) & 0x7f800000u) + (16u << 23));
+}
+// Eight values as four bf16 terms each whose sum is the value: the multiple of
+// the grid, then the remainder's three (nearest even; every remainder is exact).
+__device__ __forceinline__ void cv_split8(const float (&x)[8], float grid, uint4 (&out)[kCvTerms]) {
+  uint32_t w[kCvTerms][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     float a = x[2 * i], b = x[2 * i + 1];
-    const uint32_t ua = __float_as_uint(a) & 0x7fffffffu, ub = __float_as_uint(b) & 0x7fffffffu;
-    constexpr uint32_t kLo = (127u - 100u) << 23, kHi = (127u + 120u) << 23;
-    off |= (ua - kLo >= kHi - kLo && ua != 0) || (ub - kLo >= kHi - kLo && ub != 0);
 #pragma unroll
-    for (int s = 0; s < 3; ++s) {
-      const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    for (int s = 0; s < kCvTerms; ++s) {
+      const __nv_bfloat162 h =
+          s == 0 ? __floats2bfloat162_rn(__fsub_rn(__fadd_rn(a, grid), grid), __fsub_rn(__fadd_rn(b, grid), grid))
+                 : __floats2bfloat162_rn(a, b);
       w[s][i] = *reinterpret_cast<const uint32_t*>(&h);
       a -= __low2float(h);
       b -= __high2float(h);
     }
   }
 #pragma unroll
-  for (int s = 0; s < 3; ++s) out[s] = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
-  return off;
+  for (int s = 0; s < kCvTerms; ++s) out[s] = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
 }
 
 template <bool BWD>
@@ -217,6 +238,8 @@ __global__ void __launch_bounds__(kCvThreads, 2) dn_conv32_kernel(const float* _
                                                                   float* __restrict__ out, int R, int N) {
   pdl_wait();
   extern __shared__ __align__(128) unsigned char smem[];
+  float* most = reinterpret_cast<float*>(smem + kCvMax);
+  float* scale = reinterpret_cast<float*>(smem + kCvScale);
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + kCvBar);
   uint32_t* tbase = reinterpret_cast<uint32_t*>(bar + 1);
   const int tiles_row = N / kDnPos, tiles = R * tiles_row;
@@ -249,18 +272,50 @@ __global__ void __launch_bounds__(kCvThreads, 2) dn_conv32_kernel(const float* _
     }
   };
   fetch(blockIdx.x);
-  // the weights' terms: tap k, chunk kc, output o -> rows o, 32 + o, 64 + o
+  // the weights, a thread a tap k and output o
   bool off = false;
-  for (int e = t; e < kDnK * 4 * 32; e += kCvThreads) {
-    const int k = e / 128, kc = (e / 32) % 4, o = e % 32;
-    float w[8];
+  float w[4][8];
+  if (t < 32) reinterpret_cast<uint32_t*>(scale)[t] = 0u;
+  __syncthreads();
+  if (t < kDnK * 32) {
+    const int k = t / 32, o = t % 32;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) w[i] = wt[((kc * 8 + i) * kDnK + k) * 32 + o];
-    uint4 s[3];
-    off |= cv_split8(w, s);
+    for (int c = 0; c < 32; ++c) w[c / 8][c % 8] = wt[(c * kDnK + k) * 32 + o];
 #pragma unroll
-    for (int p = 0; p < 3; ++p)
-      *reinterpret_cast<uint4*>(smem + k * kCvTap + (4 * p + (o >> 3)) * 512 + kc * 128 + (o & 7) * 16) = s[p];
+    for (int c = 0; c < 32; ++c) {
+      const uint32_t big =
+          __reduce_max_sync(0xffffffffu, __float_as_uint(w[c / 8][c % 8]) & 0x7fffffffu);
+      if (o == 0) atomicMax(reinterpret_cast<uint32_t*>(scale) + c, big);
+    }
+  }
+  __syncthreads();
+  // a channel's largest weight becomes 1 to 2, its inputs are scaled inversely
+  if (t < 32) {
+    const float big = scale[t];
+    off |= cv_off(big);
+    scale[t] = big > 0.f ? __uint_as_float(__float_as_uint(big) & 0x7f800000u) : 1.f;
+  }
+  __syncthreads();
+  // the weights' terms: rows o, 32 + o, 64 + o, 96 + o
+  if (t < kDnK * 32) {
+    const int k = t / 32, o = t % 32;
+    float big = 0.f;
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+      float& v = w[c / 8][c % 8];
+      v *= __uint_as_float((254u << 23) - __float_as_uint(scale[c]));   // its inverse
+      off |= cv_off(v);
+      big = fmaxf(big, fabsf(v));
+    }
+    const float grid = cv_grid(big);
+    uint4 s[kCvTerms];
+#pragma unroll
+    for (int kc = 0; kc < 4; ++kc) {
+      cv_split8(w[kc], grid, s);
+#pragma unroll
+      for (int p = 0; p < kCvTerms; ++p)
+        *reinterpret_cast<uint4*>(smem + k * kCvTap + (4 * p + (o >> 3)) * 512 + kc * 128 + (o & 7) * 16) = s[p];
+    }
   }
   tmem_fence_before();
   bool plain = __syncthreads_or(off);   // this block's tiles on the CUDA cores
@@ -275,19 +330,42 @@ __global__ void __launch_bounds__(kCvThreads, 2) dn_conv32_kernel(const float* _
     const int r = tile / tiles_row, q0 = (tile % tiles_row) * kDnPos;
     const size_t at0 = (static_cast<size_t>(r) * 32 + 16 * half) * N + q0 + u;   // output 16 half
     off = !ok;
+    // the largest of the position's channels: this thread's sixteen, the other
+    // half's from the warp that holds them
+    float big = 0.f;
+    auto scaled = [&](float (&x)[8], int chunk) {
+      const float4 lo = *reinterpret_cast<const float4*>(scale + 8 * chunk);
+      const float4 hi = *reinterpret_cast<const float4*>(scale + 8 * chunk + 4);
+      const float f[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        x[i] *= f[i];
+        off |= cv_off(x[i]);
+        big = fmaxf(big, fabsf(x[i]));
+      }
+    };
+    scaled(xa[0], 2 * half);
+    scaled(xa[1], 2 * half + 1);
+    most[half * kDnPos + u] = big;
+    named_sync(1 + (warp & 3), 64);
+    float grid = cv_grid(fmaxf(big, most[(half ^ 1) * kDnPos + u]));
     unsigned char* xs = smem + kCvX;
-    uint4 s[3];
+    uint4 s[kCvTerms];
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      off |= cv_split8(xa[j], s);
+      cv_split8(xa[j], grid, s);
 #pragma unroll
-      for (int p = 0; p < 3; ++p)
+      for (int p = 0; p < kCvTerms; ++p)
         *reinterpret_cast<uint4*>(xs + p * kCvPlane + (2 * half + j) * kCvLbo + u * 16) = s[p];
     }
     if (t < 16) {
-      off |= cv_split8(xb, s);
+      big = 0.f;
+      scaled(xb, t >> 2);
+      big = fmaxf(big, __shfl_xor_sync(0xffffu, big, 4));
+      grid = cv_grid(fmaxf(big, __shfl_xor_sync(0xffffu, big, 8)));
+      cv_split8(xb, grid, s);
 #pragma unroll
-      for (int p = 0; p < 3; ++p)
+      for (int p = 0; p < kCvTerms; ++p)
         *reinterpret_cast<uint4*>(xs + p * kCvPlane + (t >> 2) * kCvLbo + (128 + (t & 3)) * 16) = s[p];
     }
     fence_proxy_async();
@@ -303,9 +381,10 @@ __global__ void __launch_bounds__(kCvThreads, 2) dn_conv32_kernel(const float* _
           const uint64_t b = dw + ((k * kCvTap + kh * 256) >> 4);
           const uint32_t more = k + kh > 0 ? 1u : 0u;
           umma_f16(tmm + 32 * k, a, b, umma_idesc(32, true), kh);
-          umma_f16(tmm + kCvCross, a, b + (4 * 512 >> 4), umma_idesc(64, true), more);
-          umma_f16(tmm + kCvCross, a + (kCvPlane >> 4), b, umma_idesc(64, true), 1u);
-          umma_f16(tmm + kCvCross + 32, a + (2 * kCvPlane >> 4), b, umma_idesc(32, true), 1u);
+          umma_f16(tmm + kCvSmall, a, b + (4 * 512 >> 4), umma_idesc(96, true), more);
+          umma_f16(tmm + kCvSmall, a + (kCvPlane >> 4), b, umma_idesc(96, true), 1u);
+          umma_f16(tmm + kCvSmall + 32, a + (2 * kCvPlane >> 4), b, umma_idesc(64, true), 1u);
+          umma_f16(tmm + kCvSmall + 64, a + (3 * kCvPlane >> 4), b, umma_idesc(32, true), 1u);
         }
       umma_commit(smem_u32(bar));
     }
@@ -322,26 +401,28 @@ __global__ void __launch_bounds__(kCvThreads, 2) dn_conv32_kernel(const float* _
     }
     if (!cores && ok) {
       tmem_fence_after();
-      float a[16], b[16], c[16];
+      float a[16], b[16];
+      // the small sums first, then the taps
+      Tmem<16>::ld(tm + kCvSmall, y);
+      Tmem<16>::ld(tm + kCvSmall + 32, a);
+      Tmem<16>::ld(tm + kCvSmall + 64, b);
+      tmem_wait_ld();
+#pragma unroll
+      for (int o = 0; o < 16; ++o) y[o] += a[o] + b[o];
       Tmem<16>::ld(tm, a);
       Tmem<16>::ld(tm + 32, b);
       tmem_wait_ld();
 #pragma unroll
-      for (int o = 0; o < 16; ++o) y[o] = a[o] + b[o];
+      for (int o = 0; o < 16; ++o) y[o] += a[o] + b[o];
       Tmem<16>::ld(tm + 64, a);
       Tmem<16>::ld(tm + 96, b);
       tmem_wait_ld();
 #pragma unroll
       for (int o = 0; o < 16; ++o) y[o] += a[o] + b[o];
       Tmem<16>::ld(tm + 128, a);
-      Tmem<16>::ld(tm + kCvCross, b);
-      Tmem<16>::ld(tm + kCvCross + 32, c);
       tmem_wait_ld();
 #pragma unroll
-      for (int o = 0; o < 16; ++o) {
-        y[o] += BWD ? a[o] : a[o] + bias[16 * half + o];
-        y[o] += b[o] + c[o];
-      }
+      for (int o = 0; o < 16; ++o) y[o] += BWD ? a[o] : a[o] + bias[16 * half + o];
     } else {
       // the same sums as FMAs
 #pragma unroll
@@ -1668,7 +1749,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) dn_tc_wgrad_kernel(const DnWgra
 // large against 64 bits, geometric mean of 80 FP32 gradients of 8 x 128 to 500 x
 // 512 and 256 x 1024 rows).  (One thread
 // per column over 1024 rows took 78 us a layer and one thread over every tile
-// 32 us for the loss; this launch takes 3.5 us at 152 rows and 5.9 at 304; 8.7 with the
+// 32 us for the loss; this launch takes 3.2 us at 152 rows and 5.1 at 304; 8.7 with the
 // rows past the last ten of a slice one after the other.)
 struct DnReduceLayer {
   const float* part;   // [rows][stride]
@@ -2017,7 +2098,7 @@ static DnWork dn_work(float* w, int R, int N) {
   return d;
 }
 
-// layers 1 to 3 on the CUDA cores (biases b1, b2, b3 in fp32)
+// layers 1 to 3 (biases b1, b2, b3 in fp32)
 static cudaError_t forward(const float* b, const DnWork& d, int R, int N, int sms, cudaStream_t st) {
   pdl_launch(dn_conv_in_kernel<false>, dim3(R * (N / kDnPos)), 256, 0, st, d.x0, d.wt + kFw1, b,
              nullptr, d.a1, N);
