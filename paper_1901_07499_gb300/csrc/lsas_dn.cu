@@ -2098,6 +2098,18 @@ static DnWork dn_work(float* w, int R, int N) {
   return d;
 }
 
+// Raises a kernel's dynamic shared memory limit on the current device, once for
+// each device; done: the kernel's flags, one a device (past 64 every call).
+template <typename K>
+static cudaError_t raise_smem(K* kernel, int bytes, bool (&done)[64]) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess || (dev < 64 && done[dev])) return e;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess && dev < 64) done[dev] = true;
+  return e;
+}
+
 // layers 1 to 3 (biases b1, b2, b3 in fp32)
 static cudaError_t forward(const float* b, const DnWork& d, int R, int N, int sms, cudaStream_t st) {
   pdl_launch(dn_conv_in_kernel<false>, dim3(R * (N / kDnPos)), 256, 0, st, d.x0, d.wt + kFw1, b,
@@ -2134,13 +2146,9 @@ cudaError_t dn_apply(const void* params, bool bf16, const float2* H, int R, int 
 cudaError_t dn_apply_tc(const void* params_bf16, const float2* H, int R, int N, float* work,
                         float2* Hout, int* status, int sms, cudaStream_t st) {
   const DnWork d = dn_work(work, R, N);
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(dn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static bool done[64] = {};
+  const cudaError_t e = raise_smem(dn_tc_kernel, kTcSmem, done);
+  if (e != cudaSuccess) return e;
   const auto* P = static_cast<const __nv_bfloat16*>(params_bf16);
   pdl_launch(dn_tc_setup_kernel<__nv_bfloat16>, dim3(kSetupBlocks + R), 256, 0, st, P, d.img,
              nullptr, H, nullptr, N, d.x0, nullptr, d.rms);
@@ -2162,15 +2170,10 @@ cudaError_t dn_ls_tc(const KParams& k, const void* params_bf16, int n_frames, fl
   static_assert(kLsXRows * 4 <= 4 * 2 * kLsN, "the input rows fit x0 to dy");
   const int R = n_frames * k.M;
   const DnWork d = dn_work(work, R, kLsN);
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e =
-        cudaFuncSetAttribute(dn_xtc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kXtSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(dn_ls_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kLsSmem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static bool done[2][64] = {};
+  cudaError_t e = raise_smem(dn_xtc_kernel, kXtSmem, done[0]);
+  if (e == cudaSuccess) e = raise_smem(dn_ls_rows_kernel, kLsSmem, done[1]);
+  if (e != cudaSuccess) return e;
   const auto* P = static_cast<const __nv_bfloat16*>(params_bf16);
   auto* xrows = reinterpret_cast<unsigned char*>(d.x0);
   pdl_launch(dn_ls_rows_kernel, dim3(kLsImgBlocks + (R + kLsWarps - 1) / kLsWarps), 32 * kLsWarps,
@@ -2242,18 +2245,11 @@ cudaError_t dn_grad(const float* P, const float2* Hls, const float2* Ht, int R, 
 cudaError_t dn_grad_tc(const float* P32, const float2* Hls, const float2* Ht, int R, int N,
                        float* work, float* grad, float* loss, int* status, int sms, cudaStream_t st) {
   const DnWork d = dn_work(work, R, N);
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(dn_tc_train_kernel<false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kTrSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(dn_tc_train_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               kTrSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(dn_tc_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static bool done[3][64] = {};
+  cudaError_t e = raise_smem(dn_tc_train_kernel<false>, kTrSmem, done[0]);
+  if (e == cudaSuccess) e = raise_smem(dn_tc_train_kernel<true>, kTrSmem, done[1]);
+  if (e == cudaSuccess) e = raise_smem(dn_tc_wgrad_kernel, kWgSmem, done[2]);
+  if (e != cudaSuccess) return e;
   pdl_launch(dn_tc_setup_kernel<float>, dim3(2 * kSetupBlocks + R), 256, 0, st, P32, d.img, d.bimg,
              Hls, Ht, N, d.x0, d.tt, d.rms);
   const size_t n = static_cast<size_t>(R) * 2 * N;
@@ -2320,14 +2316,11 @@ lsas_status dn_check(int R, int N) {
   if (R < 1 || N < 128 || N > 2048 || N % 128 != 0) return LSAS_ERR_INVALID_ARG;
   return LSAS_OK;
 }
-int dn_sms() {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      sms = 1;
-  }
+int dn_sms() {   // of the current device
+  int dev = 0, sms = 1;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 1;
   return sms;
 }
 }  // namespace
