@@ -400,7 +400,7 @@ lsas_status lsas_server_destroy(lsas_server server);
  *                  the tensor cores on operands split into four bf16 terms:
  *                  FP32 precision; tiles with values outside 2^-100 .. 2^60
  *                  of their channel's scale, and after a bounded wait that
- *                  gave up, on the FMA units, several times slower.)
+ *                  gave up, on the FMA units, 2.5 times slower.)
  *   lsas_dn_grad   mean squared error between the network output and the
  *                  true rows d_Htrue normalised by the same RMS -> d_loss[0]
  *                  and the gradient d_grad [LSAS_DN_PARAMS].

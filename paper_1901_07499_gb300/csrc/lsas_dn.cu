@@ -175,11 +175,11 @@ __global__ void __launch_bounds__(256) dn_conv_in_kernel(const float* __restrict
 // fetches the next tile under a tile's MMAs; two blocks an SM fill each
 // other's gaps.  A tile with a scaled value outside 2^-100 .. 2^60 (but zero),
 // whose last term may be no normal number or whose products may overflow on the
-// way, and, after a wait that gave up, every further tile is summed by FMAs from
-// memory, 160 loads an output one after the other: slow, and right.  Bound by
+// way, and, after a wait that gave up, every further tile is summed by FMAs
+// (cv_fma_tile).  Bound by
 // the 50 MMAs of a tile (4 KB of shared memory each whatever their N; tensor
-// pipe 55 to 60 % busy) and the splitting between them.  256 rows of 1024: 34
-// us, 35 masked (10 and 15 to read and write HBM), against 51 us for packed FMAs
+// pipe 55 to 60 % busy) and the splitting between them.  256 rows of 1024: 36
+// us, 36 masked (10 and 15 to read and write HBM), against 51 us for packed FMAs
 // from registers (8 outputs x 4 positions a thread) and 27 with three plain
 // bf16 terms, whose sums shrink by 1.6e-8.
 constexpr int kCvRows = kDnPos + kDnK - 1;           // row j holds position q0 - 2 + j
@@ -228,6 +228,52 @@ __device__ __forceinline__ void cv_split8(const float (&x)[8], float grid, uint4
   }
 #pragma unroll
   for (int s = 0; s < kCvTerms; ++s) out[s] = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
+}
+
+// A tile's sums as FMAs, for values that the split does not take: the inputs
+// through `raw` ([32][kCvRows], the place of their terms), a warp four outputs
+// and a lane four positions.  A layer of 256 rows of 1024 whose tiles all go
+// this way takes 90 us, against 305 with every warp reading its operands of each
+// FMA from memory; the main path's launches take 1 to 2 us more beside it.
+template <bool BWD>
+__device__ __noinline__ void cv_fma_tile(const float* __restrict__ in, const float* __restrict__ wt,
+                                         const float* __restrict__ bias, const float* __restrict__ mask,
+                                         float* __restrict__ out, int r, int q0, int N, float* raw) {
+  const int lane = threadIdx.x & 31, o0 = 4 * (threadIdx.x >> 5);
+  const float* row = in + static_cast<size_t>(r) * 32 * N;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < 32 * kCvRows; i += kCvThreads) {
+    const int c = i / kCvRows, q = q0 - 2 + i % kCvRows;
+    raw[i] = q >= 0 && q < N ? row[static_cast<size_t>(c) * N + q] : 0.f;
+  }
+  __syncthreads();
+  float acc[4][4];   // [output][position]
+#pragma unroll
+  for (int o = 0; o < 4; ++o)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[o][i] = BWD ? 0.f : bias[o0 + o];
+#pragma unroll 2
+  for (int c = 0; c < 32; ++c) {
+    const float4 lo = *reinterpret_cast<const float4*>(raw + c * kCvRows + 4 * lane);
+    const float4 hi = *reinterpret_cast<const float4*>(raw + c * kCvRows + 4 * lane + 4);
+    const float x[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+    for (int k = 0; k < kDnK; ++k) {
+      const float4 v = __ldg(reinterpret_cast<const float4*>(wt + (c * kDnK + k) * 32 + o0));
+      const float w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int o = 0; o < 4; ++o)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[o][i] = fmaf(w[o], x[i + k], acc[o][i]);
+    }
+  }
+#pragma unroll
+  for (int o = 0; o < 4; ++o) {
+    const size_t at = (static_cast<size_t>(r) * 32 + o0 + o) * N + q0 + 4 * lane;
+    const float4 v = make_float4(acc[o][0], acc[o][1], acc[o][2], acc[o][3]);
+    *reinterpret_cast<float4*>(out + at) = BWD ? mask4(v, *reinterpret_cast<const float4*>(mask + at)) : relu4(v);
+  }
+  __syncthreads();   // read before the next tile's terms
 }
 
 template <bool BWD>
@@ -423,8 +469,11 @@ __global__ void __launch_bounds__(kCvThreads, 2) dn_conv32_kernel(const float* _
       tmem_wait_ld();
 #pragma unroll
       for (int o = 0; o < 16; ++o) y[o] += BWD ? a[o] : a[o] + bias[16 * half + o];
+    } else if (cores) {
+      cv_fma_tile<BWD>(in, wt, bias, mask, out, r, q0, N, reinterpret_cast<float*>(xs));
+      continue;
     } else {
-      // the same sums as FMAs
+      // the wait gave up: the same sums as FMAs, in the warps that saw it
 #pragma unroll
       for (int o = 0; o < 16; ++o) y[o] = BWD ? 0.f : bias[16 * half + o];
 #pragma unroll 1

@@ -103,3 +103,26 @@ def test_both_forms_in_one_launch(R, N, j):
     want = D.Denoiser(p).apply(Hls, bf16=False)
     got = D.Denoiser(np.ldexp(p, power).astype(np.float32)).apply(Hls, bf16=False)
     assert (got - want).abs().max().item() <= 2e-5 * want.abs().max().item()
+
+
+@pytest.mark.parametrize("R,N", [(3, 128), (400, 256)])
+def test_gradients_where_weights_are_out_of_range(R, N):
+    """Layer 2's weights scaled by 2^62 and layer 1 by the inverse: layer 2 and
+    its data gradient are summed by FMAs throughout.  The gradients differ from
+    the unscaled network's by those powers and the two forms' rounding (bar of
+    tests/test_gpu_split_conv.py: 1e-4 of a block's largest)."""
+    import torch
+    import paper_1901_07499_gb300.denoiser as D
+    H, Hls, _ = synth.ls_pairs(R, N, seed=9 + N)
+    H, Hls = (torch.from_numpy(v.astype(np.complex64)).cuda() for v in (H, Hls))
+    p = _params(10, True)
+    power = np.zeros(p.size, int)
+    power[W1] = power[B1] = -62
+    power[W2] = 62
+    (loss, want), (loss_e, got) = (
+        [t.cpu().numpy() for t in D.Denoiser(q).compute_grad(Hls, H)]
+        for q in (p, np.ldexp(p, power).astype(np.float32)))
+    assert abs(loss_e[0] - loss[0]) <= 1e-4 * loss[0]
+    got = np.ldexp(got, power)
+    for s in (W1, B1, W2, B2, W3, B3, W4, B4):
+        assert np.abs(got[s] - want[s]).max() <= 1e-4 * np.abs(want[s]).max()
