@@ -471,7 +471,8 @@ lsas_status lsas_run_frame_refined(lsas_plan plan, const void* d_in, int n_frame
  * bytes that no copy delivers.  kind = 0 (the default) turns it off.
  * Applies to every fused kernel: the per-warp kernel (N <= 1024), the
  * warp-pair kernel (N = 2048, sc16 input) and the warp-specialised kernel
- * (N = 2048, fc32 input).  INVALID_ARG for other kinds.
+ * (N = 2048, fc32 input), and to the refinement of lsas_run_frame_refined,
+ * which latches into its d_status.  INVALID_ARG for other kinds.
  */
 lsas_status lsas_plan_set_fault(lsas_plan plan, int kind);
 

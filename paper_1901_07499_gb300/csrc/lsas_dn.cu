@@ -1961,7 +1961,7 @@ static_assert(kXtSlotBytes % 16 == 0, "16-byte operand alignment");
 __global__ void __launch_bounds__(128 * kTcSlots, 2) dn_xtc_kernel(const float* __restrict__ img_g,
                                                         const unsigned char* __restrict__ xrows,
                                                         const float* __restrict__ rms, int R,
-                                                        float2* __restrict__ Hout, int* status) {
+                                                        float2* __restrict__ Hout, int* status, int fault) {
   pdl_wait();
   constexpr int N = kLsN;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -1995,7 +1995,9 @@ __global__ void __launch_bounds__(128 * kTcSlots, 2) dn_xtc_kernel(const float* 
   tmem_fence_after();
   const uint64_t pol = evict_first_policy();
   // a tile's input rows, from position s0 - 2 (s0: MMA row 0), into buffer b
-  auto fetch = [&](int tile, int b) {
+  int fetched = 0;
+  auto fetch = [&](int tile) {
+    const int b = fetched++ & 1;
     const uint32_t xb = smem_u32(&xbars[b]);
     mbar_expect_tx(xb, kXtBytes);
     bulk_load(smem_u32(xbuf + b * kXtBytes),
@@ -2004,7 +2006,12 @@ __global__ void __launch_bounds__(128 * kTcSlots, 2) dn_xtc_kernel(const float* 
               kXtBytes, xb, pol);
   };
   int tile = blockIdx.x * kTcSlots + slot;
-  if (u == 0 && tile < tiles) fetch(tile, 0);
+  if (u == 0 && tile < tiles) {
+    fetch(tile);
+    // test hook: block 0's first input rows also wait for 16 bytes that no copy
+    // delivers, so that the bounded wait runs out
+    if (fault == 1 && blockIdx.x == 0 && slot == 0) mbar_expect_tx_only(smem_u32(&xbars[0]), 16);
+  }
   const uint32_t tm = *tbase + 32 * slot + (static_cast<uint32_t>(32 * (warp & 3)) << 16);
   const uint32_t tm_mma = *tbase + 32 * slot;
   const uint32_t id32 = umma_idesc(32, true), id16 = umma_idesc(16, true);
@@ -2037,7 +2044,9 @@ __global__ void __launch_bounds__(128 * kTcSlots, 2) dn_xtc_kernel(const float* 
             ok = false;
             latch(status, kStTimeout);
           }
-          if (tile + stride < tiles) fetch(tile + stride, b ^ 1);
+          // (after a wait that gave up its buffer may still be in flight, and
+          // its barrier takes no further phase)
+          if (ok && tile + stride < tiles) fetch(tile + stride);
         }
         umma_f16(tm_mma, dones, dw1 + ((kTcBias + 1024 * (layer - 1)) >> 4),
                  layer == 4 ? id16 : id32, 0u);
@@ -2095,8 +2104,8 @@ __global__ void __launch_bounds__(128 * kTcSlots, 2) dn_xtc_kernel(const float* 
     }
   }
   if (u == 0 && !ok) {
-    // a wait gave up: an input copy still in flight gets a bounded chance to land
-    for (int i = n > 0 ? n - 1 : 0; i < n; ++i)
+    // a wait gave up: the last copy into each buffer gets a bounded chance to land
+    for (int i = fetched > 2 ? fetched - 2 : 0; i < fetched; ++i)
       (void)mbar_wait_bounded(smem_u32(&xbars[i & 1]), (i >> 1) & 1);
   }
   tmem_fence_before();
@@ -2231,7 +2240,7 @@ cudaError_t dn_ls_tc(const KParams& k, const void* params_bf16, int n_frames, fl
   const int want = (tiles + kTcSlots - 1) / kTcSlots;
   const int grid = want < sms * 2 ? want : sms * 2;
   pdl_launch(dn_xtc_kernel, dim3(grid), 128 * kTcSlots, kXtSmem, st, d.img, xrows, d.rms, R, Hout,
-             status);
+             status, k.fault);
   return cudaGetLastError();
 }
 
