@@ -80,11 +80,8 @@ __device__ __forceinline__ void window8(const float* __restrict__ row, int q, in
 }
 
 __device__ __forceinline__ void cp_async(uint32_t dst, const void* src, bool on, int bytes) {
-  // bytes is 4, 8 or 16; zero-fills when off
-  if (bytes == 16)
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(on ? 16 : 0)
-                 : "memory");
-  else if (bytes == 4)
+  // bytes is 4 or 8; zero-fills when off
+  if (bytes == 4)
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(on ? 4 : 0)
                  : "memory");
   else

@@ -58,6 +58,7 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
   void (*fn)(const KParams) = nullptr;
   int threads = Geo<LOG2N>::TW;
   int slot = kind;   // entry of the shared-memory attribute cache below
+  bool warp = false;   // warp_kernel
   if (kind == kKindFrame) {
     // fused receiver (the two-symbol kernels in a form of their own for a
     // given channel: 200 frames of 64 antennas at N = 1024 demodulate in 355 us
@@ -81,7 +82,7 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
         threads = kTwThreads;
         smem = make_twlayout().total;
       } else {
-        fn = warp_kernel<LOG2N, FC32>;
+        warp = true;
         threads = 32 * wgeo_warps(4);
       }
     } else if constexpr ((LOG2N == 8 || LOG2N == 9) && !FC32) {
@@ -92,11 +93,11 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
         threads = kTwThreads;
         smem = make_twlayout().total;
       } else {
-        fn = warp_kernel<LOG2N, FC32>;
+        warp = true;
         threads = 32 * wgeo_warps(4);
       }
     } else if constexpr (LOG2N <= 10) {
-      fn = warp_kernel<LOG2N, FC32>;
+      warp = true;
       threads = 32 * wgeo_warps(FC32 ? 8 : 4);
     } else {
       if (p.twin && p.use_tma == 1) {
@@ -135,8 +136,8 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
   q.full = grid;
   q.zsplit = 1;
   if constexpr (LOG2N <= 10) {
-    if (q.use_tma == 2 && fn != warp_kernel<LOG2N, FC32>) q.use_tma = 0;
-    if (fn == warp_kernel<LOG2N, FC32>) {
+    if (q.use_tma == 2 && !warp) q.use_tma = 0;
+    if (warp) {
       q.share = warp_share(q.chunks, q.dg < q.D ? q.dg : q.D);
       if (q.mode == kModeRun || q.mode == kModeDemod) {
         // symbol-split the frames after the last whole wave where the parts
@@ -155,13 +156,19 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
           grid = q.full + tail * q.zsplit;
         }
       }
+      if (q.share || q.zsplit > 1 || q.use_tma == 2) {
+        fn = warp_kernel<LOG2N, FC32, true>;
+        slot = 10;
+      } else {
+        fn = warp_kernel<LOG2N, FC32, false>;
+      }
     }
   } else {
     if (q.use_tma == 2) q.use_tma = 0;
     if (kind == kKindFrame && slot >= 4) q.chunks = q.M;   // an antenna a step
   }
   // raise the kernel's dynamic shared memory limit once per device
-  static int limit[10][64] = {};
+  static int limit[11][64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;

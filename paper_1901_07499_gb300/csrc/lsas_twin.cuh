@@ -807,7 +807,7 @@ __global__ void __launch_bounds__(kTwThreads, 1) twin_kernel(const KParams p) {
 }
 
 // Transform of a batch of symbol rows (lsas_fft, lsas_estimate): row r of
-// p.nframes rows starts at sample r * p.row_stride + p.row_off and its N bins
+// p.nrows rows starts at sample r * p.row_stride + p.row_off and its N bins
 // go to out + r N, scaled to the unitary transform (every symbol of every
 // antenna) or as the LS estimate H = Y conj(X) / |X|^2 (EST: the pilots).
 // Bound by memory once the FFTs run at twin_kernel's rate (8 bytes out and 4

@@ -74,14 +74,14 @@ __host__ __device__ constexpr bool last_row(int M, int S, int m, int s) {
 
 // Issue the bulk copies of one warp step (antennas of chunk c, symbol s)
 // into a slot: lane 0 registers the byte count, lane a copies row a.
-template <int LOG2N, bool FC32>
+template <int LOG2N, bool FC32, bool DIV>
 __device__ __forceinline__ void wissue(const KParams& p, int f, int c, int s,
                                        unsigned char* slot, int team_stage, uint32_t bar,
                                        uint64_t pol, int lane) {
   constexpr int N = 1 << LOG2N, A = wgeo_A(N);
   constexpr uint32_t bytes = N * (FC32 ? 8 : 4);
   const int nvalid = min(A, p.M - c * A);
-  if (p.use_tma == 2) {
+  if (DIV && p.use_tma == 2) {
     // from the boundary before each row (staged_bytes)
     static_assert(A <= 32, "one row a lane");
     const unsigned char* src = row_ptr<LOG2N, FC32>(p, f, c * A + lane, s);
@@ -153,7 +153,11 @@ __device__ __forceinline__ void wfinal_exchange_read(float2 (&v)[32], const floa
   }
 }
 
-template <int LOG2N, bool FC32>
+// DIV: the form that divides a frame (p.share, p.zsplit) and takes shifted rows
+// (p.use_tma = 2).  A form of its own, because its address arithmetic in every
+// step costs whole frames: 760 float frames of 64 antennas at N = 1024 take 1288
+// us without it and 1400 with it.
+template <int LOG2N, bool FC32, bool DIV>
 __global__ void __launch_bounds__(32 * wgeo_warps(FC32 ? 8 : 4), 1) warp_kernel(const KParams p) {
   pdl_wait();
   constexpr int N = 1 << LOG2N;
@@ -166,7 +170,7 @@ __global__ void __launch_bounds__(32 * wgeo_warps(FC32 ? 8 : 4), 1) warp_kernel(
   using TmE = Tmem<OWN>;       // channel energy
   extern __shared__ __align__(128) unsigned char smem[];
   // whole frames first, then the symbol-split ones, p.zsplit blocks each
-  const int bx = blockIdx.x, sx = bx - p.full;
+  const int bx = blockIdx.x, sx = DIV ? bx - p.full : -1;
   const int f = sx < 0 ? bx : p.full + sx / p.zsplit;
   const int tid = threadIdx.x;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // known uniform: see twinpair_kernel
@@ -241,13 +245,14 @@ __global__ void __launch_bounds__(32 * wgeo_warps(FC32 ? 8 : 4), 1) warp_kernel(
     const bool pilot_here = fft_pilot(p) && first;
     const int pil = pilot_here ? 1 : 0;
     // this warp's pairs (chunk-major), whole chunks warp, warp + NW, ... unless shared
+    const bool share = DIV && p.share;
     const int lo = warp * p.chunks * nd / NW, hi = (warp + 1) * p.chunks * nd / NW;
-    const int nch = p.share ? (hi > lo ? (hi - 1) / nd - lo / nd + 1 : 0)
+    const int nch = share ? (hi > lo ? (hi - 1) / nd - lo / nd + 1 : 0)
                             : (warp < p.chunks ? (p.chunks - 1 - warp) / NW + 1 : 0);
     // local chunk lc: its number, and its first and past-the-last data symbol of the group
-    auto chunk_of = [&](int lc) { return p.share ? lo / nd + lc : warp + lc * NW; };
-    auto sym_lo = [&](int lc) { return p.share && lc == 0 ? lo % nd : 0; };
-    auto sym_hi = [&](int lc) { return p.share ? min(nd, hi - (lo / nd + lc) * nd) : nd; };
+    auto chunk_of = [&](int lc) { return share ? lo / nd + lc : warp + lc * NW; };
+    auto sym_lo = [&](int lc) { return share && lc == 0 ? lo % nd : 0; };
+    auto sym_hi = [&](int lc) { return share ? min(nd, hi - (lo / nd + lc) * nd) : nd; };
     if (first) {
 #pragma unroll
       for (int q0 = 0; q0 < OWN; q0 += ZC) Tmem<ZC>::st(tE + q0, zero);
@@ -260,7 +265,7 @@ __global__ void __launch_bounds__(32 * wgeo_warps(FC32 ? 8 : 4), 1) warp_kernel(
     // many steps of this group are still to be staged
     int ic = 0, iit = 0;
     int ia = sym_lo(0), iitems = sym_hi(0) - ia + pil;   // of chunk ic
-    int to_issue = p.share ? hi - lo + nch * pil : nch * (nd + pil);
+    int to_issue = share ? hi - lo + nch * pil : nch * (nd + pil);
     auto advance = [&]() {
       if (++iit == iitems) {
         iit = 0;
@@ -275,7 +280,7 @@ __global__ void __launch_bounds__(32 * wgeo_warps(FC32 ? 8 : 4), 1) warp_kernel(
       fence_proxy_async();
       int is = slot;
       for (int s = 0; s < K && to_issue > 0; ++s, --to_issue) {
-        wissue<LOG2N, FC32>(p, f, chunk_of(ic), witem_symbol(p, pilot_here, d0 + ia, iit),
+        wissue<LOG2N, FC32, DIV>(p, f, chunk_of(ic), witem_symbol(p, pilot_here, d0 + ia, iit),
                             stage + is * slot_bytes, lay.team_stage, smem_u32(&bars[is]), pol,
                             lane);
         // test hook: the first staging phase of block 0 also waits for 16
@@ -321,7 +326,7 @@ __global__ void __launch_bounds__(32 * wgeo_warps(FC32 ? 8 : 4), 1) warp_kernel(
           wait_slot(smem_u32(&bars[slot]), phase, abort_flag, p.status);
           if (valid) {
             const unsigned char* row = stage + slot * slot_bytes + alpha * lay.team_stage;
-            if (p.use_tma == 2) {
+            if (DIV && p.use_tma == 2) {
               const int sym = witem_symbol(p, pilot_here, d0 + sa, it);
               wload_shifted<LOG2N, FC32>(v, row, row_ptr<LOG2N, FC32>(p, f, m, sym),
                                          last_row(p.M, p.S, m, sym), jt);
@@ -347,7 +352,7 @@ __global__ void __launch_bounds__(32 * wgeo_warps(FC32 ? 8 : 4), 1) warp_kernel(
         if (p.use_tma && to_issue > 0 && !*abort_flag) {
           ++issued;
           fence_proxy_async();
-          wissue<LOG2N, FC32>(p, f, chunk_of(ic), witem_symbol(p, pilot_here, d0 + ia, iit),
+          wissue<LOG2N, FC32, DIV>(p, f, chunk_of(ic), witem_symbol(p, pilot_here, d0 + ia, iit),
                               stage + slot * slot_bytes, lay.team_stage, smem_u32(&bars[slot]),
                               pol, lane);
           --to_issue;
