@@ -498,12 +498,10 @@ lsas_status launch_frame(lsas_plan p, const void* d_in, int n_frames, float* d_H
 // one wave, they become the layers while they fit two (the blocks' steps fall
 // from all groups' to one's).  A single frame of 64 antennas at N = 1024: 8 x 13
 // blocks of one step 11 us, 8 x 4 of up to three 17.
-int grid_layers(lsas_plan p, const KParams& k, int nf, int G) {
-  const long blocks = static_cast<long>(nf) * G;
-  const bool twin = k.twin && k.use_tma == 1;
+int grid_layers(lsas_plan p, bool twin, bool given, long blocks) {
   if (p->N > 1024 && p->fmt != LSAS_IN_SC16 && !twin) return 0;   // frame_kernel
   const int groups = p->geo.hybrid ? p->geo.groups : twin ? twin_groups(p->D) : p->geo.groups;
-  const int pilot = k.H_in ? 0 : 1;
+  const int pilot = given ? 0 : 1;
   auto steps = [&](int z) {   // of the longest part
     const int items = (p->D + z - 1) / z + pilot;
     return twin ? (items + 1) / 2 : items;
@@ -514,6 +512,9 @@ int grid_layers(lsas_plan p, const KParams& k, int nf, int G) {
     return steps(z) < steps(1) ? z : 0;
   }
   return groups > 1 && blocks * 2 <= p->sms ? groups : 0;
+}
+int grid_layers(lsas_plan p, const KParams& k, long blocks) {
+  return grid_layers(p, k.twin && k.use_tma == 1, k.H_in != nullptr, blocks);
 }
 
 // Antenna shards G for nf frames that do not fill a whole wave of blocks
@@ -542,39 +543,69 @@ int best_shards(lsas_plan p, int nf, long cap) {
   return bestG;
 }
 
-// Antenna units per block for nf frames that do not fill a whole wave of
-// blocks of a two-symbol kernel: the frames' units (one antenna per pipeline:
-// unit_ant antennas, upf per frame) laid end to end and cut into one wave of
-// equal blocks, which may each touch the ends of two frames.  Unlike equal
-// shards of every frame they fill the GPU for any nf.  In fractions of a
-// frame's block time a block takes (1 - f) u / upf plus f per frame it
-// touches, and the partial sums' way through memory is charged to the frame's
-// samples at 3.7 G a second and SM; 0 when that does not save 10 % of a wave, or the
-// scratch is too small.  1000 frames of 64 antennas at N = 1024 (88 after six
-// waves: 5 of 8 units a block) 1517 -> 1485 us; 500 of 128 at N = 2048 (44: 10 of
-// 32) 3447 -> 3403; 60 float frames of 64 (7 of 16) 311 -> 281.
+// How the two-symbol kernels split nf frames that do not fill a wave of blocks:
+// into equal shards of every frame, or as antenna units (one antenna per
+// pipeline: unit_ant antennas, upf per frame) of all frames laid end to end and
+// cut into one wave of equal blocks, which may each touch the ends of two
+// frames.  Units fill the GPU for any nf; equal shards have one group end per
+// data-symbol group where such a block has two.
+struct Split {
+  int shards = 1;   // of a frame (1: whole), the most where units are given
+  int units = 0;    // a block's antenna units; 0: equal shards
+};
 int unit_antennas(lsas_plan p) { return p->N > 1024 ? kPPairs : 8 * (1024 / p->N); }
 int units_per_frame(lsas_plan p) { return (p->M + unit_antennas(p) - 1) / unit_antennas(p); }
-int best_units(lsas_plan p, int nf) {
+
+// The split with the least time of waves x (steps of a warp x kStep + group
+// ends x kEnd), + kSplit for the combine pass; a tie goes to whole frames, then
+// to equal shards.  The constants (us) are least squares over 756 batches (1 to 150
+// frames of 8 to 256 antennas, N = 256 to 2048) in every split each can take.
+// Chosen so, a batch took 1.004 times the fastest split's time on average (1.12 at
+// most), where units alone, without the group ends' count, took 1.04 (1.46): 72 frames of
+// 48 antennas at N = 512 66 us as two shards each, 81 as units of two frames;
+// 1000 of 64 at N = 1024 (88 after six waves: 5 of 8 units a block) 1517 whole,
+// 1485 as units.
+Split best_split(lsas_plan p, int nf) {
+  const bool pair = p->N > 1024;
+  const double kStep = pair ? 4.58 : 3.35, kEnd = pair ? 4.4 : 3.74, kSplit = pair ? 8.0 : 7.5;
+  // at N = 2048 splits that save little cost more than this counts
+  const double margin = pair ? 0.95 : 1.0;
   const int upf = units_per_frame(p);
-  const double fixed = p->N > 1024 ? kBlockFixedPair : kBlockFixedWarp;
-  const double frame_s = static_cast<double>(p->M) * p->S * p->N / 3.7e9;
-  const double sums = (static_cast<double>(p->D) * 2 + 1) * p->N * 4.0;   // bytes of one shard's sums
-  const long total = static_cast<long>(nf) * upf;
-  double best = 0.9;
-  int bestU = 0;
-  for (int u = static_cast<int>((total + p->sms - 1) / p->sms); u < upf; ++u) {
-    const int most = (upf - 1) / u + 2;   // shards of a frame, at most
-    if (static_cast<long>(nf) * (upf % u == 0 ? upf / u : most) > p->tail_units) continue;
-    const int frames = upf % u == 0 ? 1 : 2;   // that a block touches
-    const double moved = 2.0 * sums * (static_cast<double>(total) / u + (frames - 1) * nf) / 4e12;
-    const double t = (1.0 - fixed) * u / upf + fixed * frames + moved / frame_s;
-    if (t < best) {
-      best = t;
-      bestU = u;
+  auto us = [&](int units, int frames, long blocks, bool layered) {
+    const int z = layered ? grid_layers(p, true, false, blocks) : 0;
+    int steps;   // of one antenna, two symbols each
+    if (z) {
+      steps = ((p->D + z - 1) / z + 2) / 2;
+    } else {
+      const int first = p->D < kTwDg0 ? p->D : kTwDg0;
+      steps = (first + 2) / 2;
+      for (int rest = p->D - first; rest > 0; rest -= kTwDg)
+        steps += ((rest < kTwDg ? rest : kTwDg) + 1) / 2;
     }
+    const double waves = std::ceil(static_cast<double>(blocks) * (z ? z : 1) / p->sms);
+    return waves * (units * steps * kStep + frames * (z ? 1 : twin_groups(p->D)) * kEnd);
+  };
+  Split best;
+  double t = us(upf, 1, nf, false) * margin;
+  auto offer = [&](Split s, double v) {
+    if (static_cast<long>(nf) * s.shards > p->tail_units || v + kSplit >= t) return;
+    best = s;
+    t = v + kSplit;
+  };
+  const int ant = unit_antennas(p);
+  for (int G = 2; G <= 32; G *= 2) {
+    if (p->M % G != 0 || p->M / G < ant) continue;
+    offer({G, 0}, us((p->M / G + ant - 1) / ant, 1, static_cast<long>(nf) * G, true));
   }
-  return bestU;
+  const long total = static_cast<long>(nf) * upf;
+  const int u0 = static_cast<int>((total + p->sms - 1) / p->sms);   // one wave
+  for (int u = u0; u < upf && u < u0 + 3; ++u) {
+    const bool even = upf % u == 0;
+    const long blocks = (total + u - 1) / u;
+    if (even && p->M % (upf / u) == 0) offer({upf / u, 0}, us(u, 1, blocks, true));
+    else offer({even ? upf / u : (upf - 1) / u + 2, u}, us(u, even ? 1 : 2, blocks, true));
+  }
+  return best;
 }
 
 // Whether a batch's rows reach the two-symbol kernels' bulk copies, from the
@@ -585,18 +616,14 @@ bool rows_aligned(lsas_plan p) {
 }
 bool split_by_units(lsas_plan p) { return p->batch_split == 1 && two_symbols(p) && rows_aligned(p); }
 
-int tail_shards(lsas_plan p, int nf) {
-  if (nf <= 0 || p->batch_split == 0 || p->tail_units == 0 || p->geo.hybrid) return 1;
-  if (p->batch_split == 2) {
-    // one shard count for every batch: the single frame's choice, among the
-    // counts whose scratch holds a batch of max_frames
-    return best_shards(p, 1, p->tail_units / (p->max_frames > 0 ? p->max_frames : 1));
-  }
-  if (split_by_units(p)) {
-    const int u = best_units(p, nf), upf = units_per_frame(p);
-    return u == 0 ? 1 : upf % u == 0 ? upf / u : (upf - 1) / u + 2;
-  }
-  return best_shards(p, nf, p->tail_units);
+Split tail_split(lsas_plan p, int nf) {
+  if (nf <= 0 || p->batch_split == 0 || p->tail_units == 0 || p->geo.hybrid) return {};
+  if (split_by_units(p)) return best_split(p, nf);
+  // one shard count for every batch (mode 2): the single frame's choice, among the
+  // counts whose scratch holds a batch of max_frames
+  if (p->batch_split == 2)
+    return {best_shards(p, 1, p->tail_units / (p->max_frames > 0 ? p->max_frames : 1)), 0};
+  return {best_shards(p, nf, p->tail_units), 0};
 }
 
 // Scratch of a split that is being recorded into a graph, null when the plan's
@@ -626,13 +653,13 @@ float* graph_tail(lsas_plan p, size_t bytes) {
   return t;
 }
 
-// Frames [f0, f0 + nf) of a batch as G antenna shards: the fused kernel's
+// Frames [f0, f0 + nf) of a batch as antenna shards: the fused kernel's
 // partial mode writes the shards' partial sums and H (d_Hin null) or reads
 // the given channel d_Hin, the combine kernel forms z and the bits.  Calls on different streams share
 // d_tail: each waits for the previous split's combine.  While st is being
 // captured the partial sums go to scratch of the recorded call's own, and the
 // frames run whole where there is none.
-lsas_status run_split_tail(lsas_plan p, const void* d_in, int f0, int nf, int G, float* d_H,
+lsas_status run_split_tail(lsas_plan p, const void* d_in, int f0, int nf, Split split, float* d_H,
                            const float* d_Hin, uint8_t* d_bits, float* d_eq, cudaStream_t st) {
   const size_t in_b = in_bytes_per_frame(p->M, p->N, p->cp, p->S, p->fmt);
   const size_t bits_b = bits_bytes_per_frame(p->N, p->S, p->Q);
@@ -651,18 +678,16 @@ lsas_status run_split_tail(lsas_plan p, const void* d_in, int f0, int nf, int G,
   else k.H_out = reinterpret_cast<float2*>(d_H + h0);
   k.use_tma = staging(p, in);
   int blocks = nf;
-  const int u = split_by_units(p) && k.use_tma == 1 ? best_units(p, nf) : 0;
-  const int upf = units_per_frame(p);
-  if (u > 0 && (upf % u != 0 || p->M % (upf / u) != 0)) {
-    k.units = u;
-    k.upf = upf;
+  // an input that bulk copies cannot bring runs on the one-symbol kernels
+  if (split_by_units(p) && k.use_tma != 1) split = {best_shards(p, nf, p->tail_units), 0};
+  const int G = split.shards;
+  if (split.units) {
+    k.units = split.units;
+    k.upf = units_per_frame(p);
     k.unit_ant = unit_antennas(p);
     k.nf = nf;
-    blocks = (nf * upf + u - 1) / u;
+    blocks = (nf * k.upf + k.units - 1) / k.units;
   } else {
-    // equal shards (units that divide the frame are: a grid row each, which
-    // spares a short launch the units' arithmetic, 0.8 us)
-    if (split_by_units(p)) G = u > 0 ? upf / u : best_shards(p, nf, p->tail_units);
     k.M = p->M / G;
     k.shard_y = k.M;
     k.grid_y = G;
@@ -688,7 +713,7 @@ lsas_status run_split_tail(lsas_plan p, const void* d_in, int f0, int nf, int G,
   k.E_out = E;
   k.chunks = (k.M + p->geo.Af - 1) / p->geo.Af;
   k.mode = kModePartial;
-  k.group_z = k.units ? grid_layers(p, k, blocks, 1) : grid_layers(p, k, nf, G);
+  k.group_z = grid_layers(p, k, static_cast<long>(blocks) * (k.units ? 1 : G));
   lsas_status s = LSAS_OK;
   if (p->launch(kKindFrame, p->fmt == LSAS_IN_FC32, k, blocks, p->geo.smem_frame, st) != cudaSuccess) {
     s = LSAS_ERR_CUDA;
@@ -716,18 +741,18 @@ lsas_status run_split_tail(lsas_plan p, const void* d_in, int f0, int nf, int G,
 // A batch through the fused receiver, with its own LS estimate (writes d_H,
 // d_Hin null) or a given channel d_Hin: whole waves of blocks one frame per
 // block, the frames after them possibly split into antenna shards
-// (tail_shards).
+// (tail_split).
 lsas_status run_batch(lsas_plan p, const void* d_in, int n_frames, float* d_H, const float* d_Hin,
                       uint8_t* d_bits, float* d_eq, cudaStream_t st) {
   const int mode = d_Hin ? kModeDemod : kModeRun;
   const int full = (n_frames / p->sms) * p->sms;
-  const int G = tail_shards(p, n_frames - full);
-  if (G == 1) return launch_frame(p, d_in, n_frames, d_H, d_Hin, d_bits, d_eq, mode, st);
+  const Split split = tail_split(p, n_frames - full);
+  if (split.shards == 1) return launch_frame(p, d_in, n_frames, d_H, d_Hin, d_bits, d_eq, mode, st);
   if (full > 0) {
     const lsas_status s = launch_frame(p, d_in, full, d_H, d_Hin, d_bits, d_eq, mode, st);
     if (s != LSAS_OK) return s;
   }
-  return run_split_tail(p, d_in, full, n_frames - full, G, d_H, d_Hin, d_bits, d_eq, st);
+  return run_split_tail(p, d_in, full, n_frames - full, split, d_H, d_Hin, d_bits, d_eq, st);
 }
 
 }  // namespace
@@ -1266,7 +1291,7 @@ lsas_status lsas_plan_set_batch_split(lsas_plan p, int enable) {
 
 lsas_status lsas_plan_batch_split_shards(lsas_plan p, int n_frames, int* out_shards) {
   if (!p || !out_shards || n_frames < 0) return LSAS_ERR_INVALID_ARG;
-  *out_shards = tail_shards(p, n_frames - (n_frames / p->sms) * p->sms);
+  *out_shards = tail_split(p, n_frames - (n_frames / p->sms) * p->sms).shards;
   return LSAS_OK;
 }
 
@@ -1505,7 +1530,7 @@ lsas_status lsas_run_frame_split_static(lsas_plan p, const void* d_in, int n_fra
     k.chunks = (k.M + p->geo.Af - 1) / p->geo.Af;
     k.mode = kModePartial;
     k.use_tma = staging(p, d_in);
-    k.group_z = grid_layers(p, k, n_frames, n_shards);
+    k.group_z = grid_layers(p, k, static_cast<long>(n_frames) * n_shards);
     if (p->launch(kKindFrame, p->fmt == LSAS_IN_FC32, k, n_frames, p->geo.smem_frame,
                   static_cast<cudaStream_t>(stream)) != cudaSuccess)
       return LSAS_ERR_CUDA;
