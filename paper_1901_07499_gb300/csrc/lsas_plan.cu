@@ -556,54 +556,61 @@ struct Split {
 int unit_antennas(lsas_plan p) { return p->N > 1024 ? kPPairs : 8 * (1024 / p->N); }
 int units_per_frame(lsas_plan p) { return (p->M + unit_antennas(p) - 1) / unit_antennas(p); }
 
-// The split with the least time of waves x (steps of a warp x kStep + group
-// ends x kEnd), + kSplit for the combine pass; a tie goes to whole frames, then
-// to equal shards.  The constants (us) are least squares over 756 batches (1 to 150
-// frames of 8 to 256 antennas, N = 256 to 2048) in every split each can take.
-// Chosen so, a batch took 1.004 times the fastest split's time on average (1.12 at
-// most), where units alone, without the group ends' count, took 1.04 (1.46): 72 frames of
-// 48 antennas at N = 512 66 us as two shards each, 81 as units of two frames;
-// 1000 of 64 at N = 1024 (88 after six waves: 5 of 8 units a block) 1517 whole,
-// 1485 as units.
-Split best_split(lsas_plan p, int nf) {
+// The split with the least time: waves of blocks x (two-symbol steps of the
+// block's busiest warp x kStep + of its mean warp x kWork, since two warps share
+// a scheduler, + group ends x kEnd, less kSecond for a block's second frame),
+// + kSplit for the combine pass.  A tie goes to whole frames, then to equal
+// shards.  The constants (us) make the choice best over 3179 batches (1 to 150
+// frames of 6 to 256 antennas and 3 to 20 symbols, N = 256 to 2048, channel
+// estimated or given), each timed in every split it can take: the choice takes
+// 1.007 times the fastest's time on average at N <= 1024 (1.17 at most) and 1.005
+// (1.12) at N = 2048; units alone, without the group ends' count, took 1.036 and
+// 1.03 (1.5).  72 frames of 48 antennas at N = 512: 66 us as two shards each, 81
+// as units; 1000 of 64 at N = 1024 (88 after six waves: 5 of 8 units a block): 1517
+// whole, 1485 as units.
+Split best_split(lsas_plan p, int nf, bool given) {
   const bool pair = p->N > 1024;
-  const double kStep = pair ? 4.58 : 3.35, kEnd = pair ? 4.4 : 3.74, kSplit = pair ? 8.0 : 7.5;
-  // at N = 2048 splits that save little cost more than this counts
-  const double margin = pair ? 0.95 : 1.0;
-  const int upf = units_per_frame(p);
-  auto us = [&](int units, int frames, long blocks, bool layered) {
-    const int z = layered ? grid_layers(p, true, false, blocks) : 0;
-    int steps;   // of one antenna, two symbols each
+  const double kStep = pair ? 1.8 : 2.7, kWork = pair ? 3.5 : 1.0, kEnd = pair ? 4.2 : 3.5;
+  const double kSecond = pair ? 2.2 : 2.0, kSplit = pair ? 4.5 : 4.0;
+  const int ant = unit_antennas(p), upf = units_per_frame(p);
+  // of blocks with `antennas` each, from so many frames
+  auto us = [&](double antennas, int frames, long blocks, bool split) {
+    const int z = split ? grid_layers(p, true, given, blocks) : 0;
+    const int pilot = given ? 0 : 1;
+    int steps;   // of one antenna
     if (z) {
-      steps = ((p->D + z - 1) / z + 2) / 2;
+      steps = ((p->D + z - 1) / z + pilot + 1) / 2;
     } else {
       const int first = p->D < kTwDg0 ? p->D : kTwDg0;
-      steps = (first + 2) / 2;
+      steps = (first + pilot + 1) / 2;
       for (int rest = p->D - first; rest > 0; rest -= kTwDg)
         steps += ((rest < kTwDg ? rest : kTwDg) + 1) / 2;
     }
     const double waves = std::ceil(static_cast<double>(blocks) * (z ? z : 1) / p->sms);
-    return waves * (units * steps * kStep + frames * (z ? 1 : twin_groups(p->D)) * kEnd);
+    return waves * (steps * (std::ceil(antennas / ant) * kStep + antennas / ant * kWork) +
+                    frames * (z ? 1 : twin_groups(p->D)) * kEnd - (frames - 1) * kSecond) +
+           (split ? kSplit : 0.0);
   };
   Split best;
-  double t = us(upf, 1, nf, false) * margin;
-  auto offer = [&](Split s, double v) {
-    if (static_cast<long>(nf) * s.shards > p->tail_units || v + kSplit >= t) return;
+  double least = us(p->M, 1, nf, false);
+  auto offer = [&](Split s, double t) {
+    if (static_cast<long>(nf) * s.shards > p->tail_units || t >= least) return;
     best = s;
-    t = v + kSplit;
+    least = t;
   };
-  const int ant = unit_antennas(p);
   for (int G = 2; G <= 32; G *= 2) {
     if (p->M % G != 0 || p->M / G < ant) continue;
-    offer({G, 0}, us((p->M / G + ant - 1) / ant, 1, static_cast<long>(nf) * G, true));
+    offer({G, 0}, us(p->M / G, 1, static_cast<long>(nf) * G, true));
   }
   const long total = static_cast<long>(nf) * upf;
   const int u0 = static_cast<int>((total + p->sms - 1) / p->sms);   // one wave
   for (int u = u0; u < upf && u < u0 + 3; ++u) {
     const bool even = upf % u == 0;
     const long blocks = (total + u - 1) / u;
-    if (even && p->M % (upf / u) == 0) offer({upf / u, 0}, us(u, 1, blocks, true));
-    else offer({even ? upf / u : (upf - 1) / u + 2, u}, us(u, even ? 1 : 2, blocks, true));
+    if (even && p->M % (upf / u) == 0)
+      offer({upf / u, 0}, us(p->M / (upf / u), 1, blocks, true));
+    else
+      offer({even ? upf / u : (upf - 1) / u + 2, u}, us(u * ant, even ? 1 : 2, blocks, true));
   }
   return best;
 }
@@ -616,9 +623,9 @@ bool rows_aligned(lsas_plan p) {
 }
 bool split_by_units(lsas_plan p) { return p->batch_split == 1 && two_symbols(p) && rows_aligned(p); }
 
-Split tail_split(lsas_plan p, int nf) {
+Split tail_split(lsas_plan p, int nf, bool given) {
   if (nf <= 0 || p->batch_split == 0 || p->tail_units == 0 || p->geo.hybrid) return {};
-  if (split_by_units(p)) return best_split(p, nf);
+  if (split_by_units(p)) return best_split(p, nf, given);
   // one shard count for every batch (mode 2): the single frame's choice, among the
   // counts whose scratch holds a batch of max_frames
   if (p->batch_split == 2)
@@ -746,7 +753,7 @@ lsas_status run_batch(lsas_plan p, const void* d_in, int n_frames, float* d_H, c
                       uint8_t* d_bits, float* d_eq, cudaStream_t st) {
   const int mode = d_Hin ? kModeDemod : kModeRun;
   const int full = (n_frames / p->sms) * p->sms;
-  const Split split = tail_split(p, n_frames - full);
+  const Split split = tail_split(p, n_frames - full, d_Hin != nullptr);
   if (split.shards == 1) return launch_frame(p, d_in, n_frames, d_H, d_Hin, d_bits, d_eq, mode, st);
   if (full > 0) {
     const lsas_status s = launch_frame(p, d_in, full, d_H, d_Hin, d_bits, d_eq, mode, st);
@@ -1291,7 +1298,7 @@ lsas_status lsas_plan_set_batch_split(lsas_plan p, int enable) {
 
 lsas_status lsas_plan_batch_split_shards(lsas_plan p, int n_frames, int* out_shards) {
   if (!p || !out_shards || n_frames < 0) return LSAS_ERR_INVALID_ARG;
-  *out_shards = tail_split(p, n_frames - (n_frames / p->sms) * p->sms).shards;
+  *out_shards = tail_split(p, n_frames - (n_frames / p->sms) * p->sms, false).shards;
   return LSAS_OK;
 }
 
