@@ -522,9 +522,10 @@ int grid_layers(lsas_plan p, const KParams& k, long blocks) {
 // ceil(nf G / sms) waves of about (1 - f) / G + f of a frame's block time
 // (f: kBlockFixedWarp or kBlockFixedPair), against one wave unsplit.  Equal
 // shards only (one launch), each with at least one antenna per pipeline of
-// the fused kernel, nf G within cap; 1 when no split saves 10 % of the wave.
-int best_shards(lsas_plan p, int nf, long cap) {
-  const bool pairs = p->N > 1024 && (p->fmt == LSAS_IN_SC16 || two_symbols(p));
+// the fused kernel (two: a two-symbol one), nf G within cap; 1 when no split
+// saves 10 % of the wave.
+int best_shards(lsas_plan p, int nf, long cap, bool two) {
+  const bool pairs = p->N > 1024 && (p->fmt == LSAS_IN_SC16 || two);   // else frame_kernel
   const int min_ant = pairs ? kPPairs
                             : (p->N <= 1024 ? wgeo_warps(p->fmt == LSAS_IN_SC16 ? 4 : 8) : 1) * p->geo.Af;
   const double fixed = p->N > 1024 ? kBlockFixedPair : kBlockFixedWarp;
@@ -626,11 +627,12 @@ bool split_by_units(lsas_plan p) { return p->batch_split == 1 && two_symbols(p) 
 Split tail_split(lsas_plan p, int nf, bool given) {
   if (nf <= 0 || p->batch_split == 0 || p->tail_units == 0 || p->geo.hybrid) return {};
   if (split_by_units(p)) return best_split(p, nf, given);
+  const bool two = two_symbols(p) && rows_aligned(p);
   // one shard count for every batch (mode 2): the single frame's choice, among the
   // counts whose scratch holds a batch of max_frames
   if (p->batch_split == 2)
-    return {best_shards(p, 1, p->tail_units / (p->max_frames > 0 ? p->max_frames : 1)), 0};
-  return {best_shards(p, nf, p->tail_units), 0};
+    return {best_shards(p, 1, p->tail_units / (p->max_frames > 0 ? p->max_frames : 1), two), 0};
+  return {best_shards(p, nf, p->tail_units, two), 0};
 }
 
 // Scratch of a split that is being recorded into a graph, null when the plan's
@@ -686,7 +688,7 @@ lsas_status run_split_tail(lsas_plan p, const void* d_in, int f0, int nf, Split 
   k.use_tma = staging(p, in);
   int blocks = nf;
   // an input that bulk copies cannot bring runs on the one-symbol kernels
-  if (split_by_units(p) && k.use_tma != 1) split = {best_shards(p, nf, p->tail_units), 0};
+  if (split_by_units(p) && k.use_tma != 1) split = {best_shards(p, nf, p->tail_units, false), 0};
   const int G = split.shards;
   if (split.units) {
     k.units = split.units;
