@@ -838,6 +838,14 @@ __device__ __forceinline__ void reduce_scatter(float2* v, int alpha) {
 
 // ------------------------------------------------------- staging pipeline
 
+// Part of the data symbols that a block of a layered launch (p.group_z) takes:
+// the last, largest one first, then the first, which has the energy too, so that
+// blocks past one wave of them are of the others.  10 frames of 100 antennas at
+// N = 2048 in 4 shards x 4 layers (160 blocks): 134 us, 161 in the parts' order.
+__device__ __forceinline__ int grid_layer(const KParams& p) {
+  return blockIdx.z == 0 ? p.group_z - 1 : static_cast<int>(blockIdx.z) - 1;
+}
+
 // Whether the frame kernel transforms the pilot itself (LS estimate) rather
 // than reading a given channel (whole frames or, kModePartial, a shard).
 __device__ __forceinline__ bool fft_pilot(const KParams& p) { return p.H_in == nullptr; }

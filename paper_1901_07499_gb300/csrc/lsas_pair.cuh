@@ -138,8 +138,8 @@ __global__ void __launch_bounds__(kPThreads, 1) pair_kernel(const KParams p) {
   // one part of the data symbols per grid z index (partial mode, small
   // batches): every part's block transforms the pilot itself; part 0 alone
   // writes H and the channel energy
-  const int d_begin = p.group_z ? static_cast<int>(blockIdx.z) * p.D / p.group_z : 0;
-  const int d_end = p.group_z ? (static_cast<int>(blockIdx.z) + 1) * p.D / p.group_z : p.D;
+  const int d_begin = p.group_z ? grid_layer(p) * p.D / p.group_z : 0;
+  const int d_end = p.group_z ? (grid_layer(p) + 1) * p.D / p.group_z : p.D;
   for (int d0 = d_begin; d0 < d_end; d0 += p.dg) {
     const int nd = min(p.dg, d_end - d0);
     const bool first = d0 == d_begin;

@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(kTpThreads, 1) twinpair_kernel(const KParams p
   // one part of the data symbols per grid z index (partial mode, small
   // batches; no part is larger than its group): every part's block transforms
   // the pilot itself; part 0 alone writes H and the channel energy
-  const int g_lo = PART && p.group_z ? static_cast<int>(blockIdx.z) : 0;
+  const int g_lo = PART && p.group_z ? grid_layer(p) : 0;
   const int g_hi = PART && p.group_z ? g_lo + 1 : twin_groups(p.D);
   for (int g = g_lo; g < g_hi; ++g) {
     const int d0 = PART && p.group_z ? g * p.D / p.group_z : g == 0 ? 0 : kTwDg0 + (g - 1) * kTwDg;

@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(32 * wgeo_warps(FC32 ? 8 : 4), 1) warp_kernel(
   // partial mode, the channel energy)
   int d_begin = 0, d_end = p.D;
   if (p.group_z) {
-    const int z = blockIdx.z;
+    const int z = grid_layer(p);
     d_begin = z * p.D / p.group_z;
     d_end = (z + 1) * p.D / p.group_z;
   } else if (sx >= 0) {
