@@ -138,7 +138,11 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
   if constexpr (LOG2N <= 10) {
     if (q.use_tma == 2 && !warp) q.use_tma = 0;
     if (warp) {
-      q.share = warp_share(q.chunks, q.dg < q.D ? q.dg : q.D);
+      // (not an antenna shard in several data-symbol groups: twice the warps
+      // then read its channel back in each; 4 antennas of float rows at N = 1024
+      // 41.2 us shared, 39.8 as whole chunks)
+      if (q.mode != kModePartial || q.group_z || q.D <= q.dg)
+        q.share = warp_share(q.chunks, q.dg < q.D ? q.dg : q.D);
       if (q.mode == kModeRun || q.mode == kModeDemod) {
         // symbol-split the frames after the last whole wave where the parts
         // fit one data-symbol group and fewer steps a warp
