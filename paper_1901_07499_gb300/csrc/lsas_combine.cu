@@ -24,7 +24,7 @@ constexpr int kCombineThreads = 128;
 // make the q bytes their 8 points pack into.  Bound by memory, and for one
 // frame by latency: the shards' loads are all in flight, and the launch
 // overlaps the shard pass's end (pdl_launch).  60 frames of N = 2048
-// in 2 shards with z: 13.6 -> 11 us; one frame of N = 1024 in 8: 5.5 -> 3.1, and
+// in 2 shards with z: 13.6 -> 11 us; one frame of N = 1024 in 8: 5.2 -> 3.6, and
 // the pair of launches 19.5 -> 14.3.
 // (Before, a thread took 8 points, its 64-byte pieces apart from its
 // neighbours'.)

@@ -1,5 +1,6 @@
-// lsas_pair.cuh -- fused receiver kernel for N = 2048 from sc16 rows: pairs
-// of warps as independent pipelines.
+// lsas_pair.cuh -- fused receiver kernel for N = 2048 from sc16 rows that do
+// not start on 16 bytes (the others run twinpair_kernel): pairs of warps as
+// independent pipelines.
 //
 // One block per frame, four pairs of warps.  A pair is the FFT team of one
 // antenna-symbol row (64 threads, 32 points each; Stockham radix 32 x 8 x 8,
