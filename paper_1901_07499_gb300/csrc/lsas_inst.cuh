@@ -181,8 +181,9 @@ static cudaError_t launch_t(int kind, const KParams& p, int grid, int smem, cuda
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) limit[slot][dev] = smem;
   }
-  const int gz = q.group_z > 0 ? q.group_z : 1;
-  pdl_launch(fn, dim3(grid, p.grid_y > 1 ? p.grid_y : 1, gz), threads, smem, st, q);
+  const int gz = q.group_z > 0 ? q.group_z : 1, gy = p.grid_y > 1 ? p.grid_y : 1;
+  q.big_first = static_cast<long>(grid) * gy * gz > q.sms ? 1 : 0;
+  pdl_launch(fn, dim3(grid, gy, gz), threads, smem, st, q);
   return cudaGetLastError();
 }
 

@@ -96,6 +96,7 @@ struct KParams {
   int grid_y;            // grid rows (shards) of the launch; 0 or 1 for a 1-D grid
   int group_z;           // partial mode: grid layers, layer z runs the z-th even part of the
                          // data symbols alone (hyb_kernel: data-symbol group z); 0: none
+  int big_first;         // group_z: 1 = the last, largest part runs first (grid_layer)
   int chunks;            // ceil(M / A)
   int groups, dg;        // data-symbol groups per frame, data symbols per group
   int mode;              // kModeDemod, kModeRun or kModePartial (frame_kernel)
@@ -838,12 +839,15 @@ __device__ __forceinline__ void reduce_scatter(float2* v, int alpha) {
 
 // ------------------------------------------------------- staging pipeline
 
-// Part of the data symbols that a block of a layered launch (p.group_z) takes:
-// the last, largest one first, then the first, which has the energy too, so that
-// blocks past one wave of them are of the others.  10 frames of 100 antennas at
-// N = 2048 in 4 shards x 4 layers (160 blocks): 134 us, 161 in the parts' order.
+// Part of the data symbols that a block of a layered launch (p.group_z) takes.
+// Past one wave of blocks (p.big_first) the last, largest one runs first, then the
+// first, which has the energy too, so that the blocks of the second wave are of
+// the others; within one wave the first, since it has the most to do (one frame
+// 12.5 us, 13.0 the other way).  10 frames of 100 antennas at N = 2048 in 4 shards
+// x 4 layers (160 blocks): 134 us, 161 in the parts' order.
 __device__ __forceinline__ int grid_layer(const KParams& p) {
-  return blockIdx.z == 0 ? p.group_z - 1 : static_cast<int>(blockIdx.z) - 1;
+  const int z = blockIdx.z;
+  return !p.big_first ? z : z == 0 ? p.group_z - 1 : z - 1;
 }
 
 // Whether the frame kernel transforms the pilot itself (LS estimate) rather
